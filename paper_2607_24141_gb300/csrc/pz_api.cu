@@ -242,11 +242,25 @@ static pz_status build_items(pz_ctx *c) {
             kmin = std::min(kmin, kC * (double)c->h_invdv[(size_t)st * c->ns * c->nd + k]);
         const double hw = 20.0 / (kmin * c->lnr) * 1.02 + 4.0;
         for (int t = 0; t < nt; ++t) {
-            const int64_t a = (int64_t)t * T - c->W, b = (int64_t)t * T + T - 1 + c->W;
-            const int lo = (int)(std::lower_bound(b0, b1, (int32_t)std::max<int64_t>(a, INT32_MIN)) - c->h_il.begin());
-            const int hi = (int)(std::upper_bound(b0, b1, (int32_t)std::min<int64_t>(b, INT32_MAX)) - c->h_il.begin());
-            for (int g = 0; g < ngf; ++g)
+            for (int g = 0; g < ngf; ++g) {
+                // lines whose window touches the tile; with the box expansions those in the boxes
+                // nearer than every class of the group's slabs (the kernels gather the few others)
+                int64_t a = (int64_t)t * T - c->W, b = (int64_t)t * T + T - 1 + c->W;
+                if (c->box.B) {
+                    int n0 = 0;
+                    for (int w = 0; w < c->tiling.GW; ++w)
+                        n0 = std::max(n0, c->box.h_nmin[((size_t)st * c->nslab + g * c->tiling.GW + w) * 4]);
+                    if (n0 < kBoxNever) {
+                        a = std::max(a, (int64_t)t * T - (int64_t)(n0 - 1) * c->box.B);
+                        b = std::min(b, (int64_t)t * T + T - 1 + (int64_t)(n0 - 1) * c->box.B);
+                    }
+                }
+                const int lo =
+                    (int)(std::lower_bound(b0, b1, (int32_t)std::max<int64_t>(a, INT32_MIN)) - c->h_il.begin());
+                const int hi =
+                    (int)(std::upper_bound(b0, b1, (int32_t)std::min<int64_t>(b, INT32_MAX)) - c->h_il.begin());
                 fi.push_back({make_int4(st, t * ngf + g, lo, hi), (double)(hi - lo) * std::min(DC, c->nd - g * DC)});
+            }
             double na = (double)t * T - hw, nb_ = (double)t * T + T - 1 + hw;
             na = std::max(na, (double)INT32_MIN / 2);
             nb_ = std::min(nb_, (double)INT32_MAX / 2);
@@ -278,8 +292,7 @@ static pz_status build_items(pz_ctx *c) {
         int4 v, ext;
         double cost;
     };
-    std::vector<FItem> fp;
-    std::vector<Item> bp;
+    std::vector<FItem> fp, bp;
     fp.reserve(fi.size());
     int nslot = 0, nsplit = 0;
     for (const Item &it : fi) {
@@ -292,7 +305,7 @@ static pz_status build_items(pz_ctx *c) {
             const int4 v = make_int4(it.v.x, it.v.y, lo, hi);
             const int4 ext = P > 1 ? make_int4(nslot, P, nsplit, q) : make_int4(-1, 1, -1, 0);
             fp.push_back({v, ext, it.cost / P});
-            if (hi > lo) bp.push_back({v, it.cost / P});
+            if (hi > lo || c->box.B) bp.push_back({v, make_int4(0, P, 0, q), it.cost / P});
         }
         if (P > 1) {
             nslot += P;
@@ -304,6 +317,12 @@ static pz_status build_items(pz_ctx *c) {
     for (size_t k = 0; k < fp.size(); ++k) {
         hf[k] = fp[k].v;
         hx[k] = fp[k].ext;
+    }
+    std::stable_sort(bp.begin(), bp.end(), [](const FItem &x, const FItem &y) { return x.cost > y.cost; });
+    std::vector<int4> hbf(bp.size()), hbx(bp.size());
+    for (size_t k = 0; k < bp.size(); ++k) {
+        hbf[k] = bp[k].v;
+        hbx[k] = bp[k].ext;
     }
     // near-core backward pieces (per-line sums added atomically, as whole items do); the
     // near kernels hold about kNearCtasPerSm CTAs per SM
@@ -321,18 +340,20 @@ static pz_status build_items(pz_ctx *c) {
             if (hi > lo) nbp.push_back({make_int4(it.v.x, it.v.y, lo, hi), it.cost / P});
         }
     }
-    std::vector<int4> hbf = order(bp), hn = order(nf), hb = order(nbp);
+    std::vector<int4> hn = order(nf), hb = order(nbp);
     dfree(c->d_fitems);
     dfree(c->d_fext);
     dfree(c->d_bitems);
+    dfree(c->d_bext);
     dfree(c->d_nitems_f);
     dfree(c->d_nitems_b);
     dfree(c->d_fcnt);
-    c->d_fitems = c->d_fext = c->d_bitems = c->d_nitems_f = c->d_nitems_b = nullptr;
+    c->d_fitems = c->d_fext = c->d_bitems = c->d_bext = c->d_nitems_f = c->d_nitems_b = nullptr;
     c->d_fcnt = nullptr;
     PZ_TRY(upload(&c->d_fitems, hf, "work items"));
     PZ_TRY(upload(&c->d_fext, hx, "work items"));
     PZ_TRY(upload(&c->d_bitems, hbf, "work items"));
+    PZ_TRY(upload(&c->d_bext, hbx, "work items"));
     PZ_TRY(upload(&c->d_nitems_f, hn, "work items"));
     PZ_TRY(upload(&c->d_nitems_b, hb, "work items"));
     PZ_TRY(dalloc(&c->d_fcnt, (size_t)nsplit, "work items"));
@@ -379,7 +400,38 @@ static pz_status build_thresholds(pz_ctx *c) {
     c->d_thr = nullptr;
     PZ_TRY(upload(&c->d_thr, thr, "thresholds"));
     c->nslab = nslab;
+    // box expansions: nearest offset n_c of class c at each (star, slab): the points of boxes n_c
+    // apart lie beyond 2^c times the widest species' threshold; kBoxNever if no whole box or
+    // window end is that far.  Layers past the last one take the bounds of no line.
+    BoxPlan &bx = c->box;
+    bx.h_nmin.assign((size_t)c->S * nslab * 4, kBoxNever);
+    if (bx.B)
+        for (int st = 0; st < c->S; ++st)
+            for (int b = 0; b < nslab; ++b) {
+                float w = 0.0f;
+                for (int s = 0; s < c->ns; ++s) w = std::max(w, thr[((size_t)st * c->ns + s) * nslab + b]);
+                for (int k = 0; k < 4; ++k) {
+                    const int n = std::max(3, 1 + (int)std::ceil(std::ldexp((double)w, k) / bx.B));
+                    if (n <= bx.omax + 1) bx.h_nmin[((size_t)st * nslab + b) * 4 + k] = n;
+                }
+            }
+    dfree(bx.d_nmin);
+    bx.d_nmin = nullptr;
+    PZ_TRY(upload(&bx.d_nmin, bx.h_nmin, "box offsets"));
     return PZ_OK;
+}
+
+// Device tables and workspace of the box expansions (once per context).
+static pz_status build_boxes(pz_ctx *c) {
+    BoxPlan &b = c->box;
+    if (!b.B) return PZ_OK;
+    const size_t K = 14, row = 16;   // moments per box, row of the tables
+    PZ_TRY(dalloc(&b.d_C, (size_t)2 * (b.omax + 3) * K * row, "box tables"));
+    PZ_TRY(dalloc(&b.d_E, (size_t)4 * b.B * b.KE, "box tables"));
+    PZ_TRY(dalloc(&b.d_A, 3 * K * K, "box tables"));
+    PZ_TRY(dalloc(&b.d_start, (size_t)c->S * (b.nbox + 1), "box tables"));
+    PZ_TRY(dalloc(&b.d_ws, box_workspace_floats(c, b.chunk), "box workspace"));
+    return cuda_check(launch_box_tables(c), "box tables");
 }
 
 static void drop_graph(pz_ctx *c) {
@@ -399,12 +451,13 @@ static void destroy_ctx(pz_ctx *c) {
                     c->d_thr, c->d_kc, c->d_B, c->d_stim, c->d_dab, c->d_mdgf, c->d_mdg6, c->d_eos, c->L.orig, c->L.star, c->L.ilf,
                     c->L.il32, c->L.frac, c->L.sp, c->L.E, c->L.lamcm, c->L.grad, c->L.g4, c->L.g6base, c->L.g6,
                     c->L.Q, c->L.Qbase, c->L.x64, c->L.lg_gf, c->L.lg_rad, c->L.lg_4, c->L.lg_6, c->L.dgf, c->L.dg6,
-                    c->d_line_off, c->d_fitems, c->d_fext, c->d_bitems, c->d_fpart, c->d_fcnt, c->d_nitems_f,
+                    c->d_line_off, c->d_fitems, c->d_fext, c->d_bitems, c->d_bext, c->d_fpart, c->d_fcnt, c->d_nitems_f,
                     c->d_nitems_b, c->d_ctr, c->d_knear, c->d_kline,
                     c->d_F, c->d_Fc, c->d_g, c->d_gc, c->d_tap0, c->d_ntap, c->d_tapw, c->d_dFbar, c->d_Gt,
                     c->d_Gt64, c->d_gacc, c->d_gline, c->d_gab, c->d_dLdf, c->d_finfo, c->d_status,
                     c->d_keep, c->L.gradbase, c->L.g4base, c->L.dgrad, c->L.dg4, c->d_mdgrad, c->d_mdg4,
-                    c->d_grp_of, c->d_grp_off, c->d_grp_mem, c->d_sigma};
+                    c->d_grp_of, c->d_grp_off, c->d_grp_mem, c->d_sigma,
+                    c->box.d_nmin, c->box.d_start, c->box.d_A, c->box.d_C, c->box.d_E, c->box.d_ws, c->box.d_wide};
     for (void *p : ptrs) dfree(p);
     destroy_marks(c->marks);
     destroy_marks(c->cap_marks);
@@ -624,6 +677,8 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         }
     }
     c->h_invdv = invdv;
+    // widest near zone (20 Doppler widths, in grid points) over stars, species and layers
+    box_choose(c, 20.0 / (kC * (double)*std::min_element(invdv.begin(), invdv.end()) * c->lnr));
     std::vector<double> dab(1, 0.0);
     std::vector<int32_t> eos(ns, -1);
     if (upload(&c->d_m, c->h_m, "depth") || upload(&c->d_T, c->h_T, "depth") || upload(&c->d_beta_hi, bh, "depth") ||
@@ -659,7 +714,7 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
     if (cuda_check(cudaMemset(c->d_status, 0, sizeof(int32_t)), "status word")) return bail(PZ_ECUDA);
     if (prec == PZ_MIXED && cuda_check(cudaMemset(c->d_knear, 0, sizeof(float) * SD * c->ld), "kappa_line buffer"))
         return bail(PZ_ECUDA);
-    if (build_items(c) != PZ_OK) return bail(PZ_ENOMEM);
+    if (build_boxes(c) != PZ_OK || build_items(c) != PZ_OK) return bail(PZ_ENOMEM);
     if (prec == PZ_MIXED && ensure_far_tables(c) != PZ_OK) return bail(PZ_ENOMEM);
     if (cuda_check(cudaDeviceSynchronize(), who)) return bail(PZ_ECUDA);
     *out = c;
@@ -707,6 +762,14 @@ static pz_status ensure_far_tables(pz_ctx *c) {
         }
         c->finfo_cap = ib;
     }
+    const size_t wb = c->box.B ? box_wide_bytes(c) : 0;
+    if (c->box.wide_cap < wb) {
+        dfree(c->box.d_wide);
+        c->box.d_wide = nullptr;
+        c->box.wide_cap = 0;
+        PZ_TRY(dalloc(&c->box.d_wide, wb / sizeof(uint32_t), "box classes"));
+        c->box.wide_cap = wb;
+    }
     return PZ_OK;
 }
 
@@ -720,6 +783,7 @@ static pz_status apply_tiling(pz_ctx *c, const Tiling &t, const char *who) {
     if (t.LC < 1 || t.LC > 512) return fail(PZ_EINVAL, w + ": lines_per_chunk must be in [1, 512]");
     if (!tiling_fits(t)) return fail(PZ_EINVAL, w + ": shared-memory chunk too large");
     drop_graph(c);
+    c->finfo_valid = false;
     c->tiling = t;
     PZ_TRY(build_thresholds(c));
     PZ_TRY(build_items(c));
@@ -953,6 +1017,7 @@ pz_status pz_set_centre_test(pz_ctx *c, double eta, int64_t *kept_pairs, void *s
     if (!(std::isfinite(eta) && eta >= 0.0)) return fail(PZ_EINVAL, "pz_set_centre_test: eta must be finite and >= 0");
     cudaStream_t s = (cudaStream_t)stream;
     drop_graph(c);
+    c->finfo_valid = false;
     c->have_kline = c->have_flux = c->have_inst = false;
     if (eta == 0.0) {
         PZ_CUDA(cudaStreamSynchronize(s), "pz_set_centre_test");
@@ -1272,6 +1337,7 @@ pz_status pz_calib_step(pz_ctx *c, const float *y, const float *w, int64_t n, fl
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
         if (st != PZ_OK || e != cudaSuccess) {
+            c->finfo_valid = false;   // what was captured has not run
             if (graph) cudaGraphDestroy(graph);
             destroy_marks(c->cap_marks);
             return st != PZ_OK ? st : cuda_check(e, "pz_calib_step: end capture");
@@ -1279,6 +1345,7 @@ pz_status pz_calib_step(pz_ctx *c, const float *y, const float *w, int64_t n, fl
         e = cudaGraphInstantiate(&G.exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
+            c->finfo_valid = false;
             G.exec = nullptr;
             destroy_marks(c->cap_marks);
             return cuda_check(e, "pz_calib_step: instantiate");
@@ -1423,6 +1490,7 @@ pz_status pz_group_eval(pz_ctx *c, const float *y, const float *w, int64_t n, co
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->cap_stream, &graph);
         if (st != PZ_OK || e != cudaSuccess) {
+            c->finfo_valid = false;   // what was captured has not run
             if (graph) cudaGraphDestroy(graph);
             destroy_marks(c->cap_marks);
             return st != PZ_OK ? st : cuda_check(e, "pz_group_eval: end capture");
@@ -1430,6 +1498,7 @@ pz_status pz_group_eval(pz_ctx *c, const float *y, const float *w, int64_t n, co
         e = cudaGraphInstantiate(&G.exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
+            c->finfo_valid = false;
             G.exec = nullptr;
             destroy_marks(c->cap_marks);
             return cuda_check(e, "pz_group_eval: instantiate");

@@ -91,6 +91,25 @@ struct LineTable {
     float *dgrad = nullptr, *dg4 = nullptr;
 };
 
+// Box expansions of the far wings (pz_box.cuh): geometry, tables and workspace.  B = 0: off, the
+// far-wing kernels sum every pair of a line's window.
+struct BoxPlan {
+    int B = 0;                  // grid points per box (a power of two; 32 J is a multiple of it)
+    int sh = 0;                 // log2 B
+    int omax = 0, rem = 0;      // widest whole offset; (W + 1) - (omax + 1) B
+    int s_lo = 0, nbox = 0, ntb = 0;   // first source box, source boxes, target boxes
+    int KE = 0;                 // moments kept per grid index for the window ends
+    int chunk = 0;              // stars per launch (bounds the workspace)
+    int *d_nmin = nullptr;      // [S][nslab][4] nearest offset of each separation class
+    int32_t *d_start = nullptr; // [S][nbox + 1] first line of each box
+    float *d_A = nullptr, *d_C = nullptr, *d_E = nullptr;
+    float *d_ws = nullptr;      // moments and prefixes, or the moments of G
+    uint32_t *d_wide = nullptr; // [4][nslab][words] lines of class >= 1..4, one bit per line
+    size_t wide_cap = 0;
+    std::vector<int> h_nmin;
+};
+constexpr int kBoxNever = 1 << 28;   // offset of a class that does not exist
+
 // A pair of profiler events around one launch and the kernel family it times.
 struct ProfMark {
     cudaEvent_t a, b;
@@ -163,6 +182,7 @@ struct pz_ctx {
     int n_elem = 0;
 
     pz::LineTable L;
+    pz::BoxPlan box;
     int64_t *d_line_off = nullptr;  // [S+1]
     // work items (star, tile * groups + group, lo, hi), longest first
     // (far-wing items with many lines are split into pieces of their line range, so that
@@ -170,6 +190,7 @@ struct pz_ctx {
     int4 *d_fitems = nullptr;       // far-wing forward pieces
     int4 *d_fext = nullptr;         // per forward piece: (first slot, pieces, item counter, piece)
     int4 *d_bitems = nullptr;       // far-wing backward pieces (those holding lines)
+    int4 *d_bext = nullptr;         // per backward piece: (0, pieces, 0, piece)
     int4 *d_nitems_f = nullptr;     // near-core forward
     int4 *d_nitems_b = nullptr;     // near-core backward
     int n_fitems = 0, n_bitems = 0, n_nitems_f = 0, n_nitems_b = 0;
@@ -212,6 +233,7 @@ struct pz_ctx {
     bool have_gt = false;                // G (dL/dkappa_line) holds a reverse pass
     void *d_finfo = nullptr;             // far-wing line records [depth groups][lines]
     size_t finfo_cap = 0;                // its size in bytes
+    bool finfo_valid = false;            // they match the current corrections, centre test and tiling
     int32_t *d_status = nullptr;         // device status word (bounded-wait failures), read by pz_sync_status
     uint32_t *d_keep = nullptr;          // centre test: bit d of word [l][d / 32] set if (l, d) is kept; NULL = off
     double centre_eta = 0.0;             // its selection fraction (0 = off)
@@ -276,5 +298,9 @@ cudaError_t launch_centre_mask(pz_ctx *c, double eta, unsigned long long *d_coun
 bool tiling_supported(int J, int DS, int minb);
 bool tiling_fits(const Tiling &t);   // both far-wing chunks fit in shared memory
 size_t far_info_bytes(const pz_ctx *c);
+size_t box_wide_bytes(const pz_ctx *c);
+size_t box_workspace_floats(const pz_ctx *c, int stars);
+void box_choose(pz_ctx *c, double thr_max);          // geometry of the box expansions (host)
+cudaError_t launch_box_tables(pz_ctx *c);            // fills their device tables
 
 }  // namespace pz

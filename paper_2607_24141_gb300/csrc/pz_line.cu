@@ -131,6 +131,7 @@ pz_status ensure_device_tables() {
 // ---------------------------------------------------------------------------
 
 struct LineInfo;
+constexpr int kBoxClasses = 4;             // box separation classes (class 4: never, pz_box.cuh)
 
 // Kernel arguments.  Line arrays are indexed by absolute line; the per-star tables
 // and buffers point at star 0 and are advanced by star_view().
@@ -151,7 +152,7 @@ struct LineArgs {
     int64_t nl;
     // work queue: items (star, tile * ngroups + group, lo, hi), longest first
     const int4 *items;
-    const int4 *fext;                               // forward pieces: (first slot, pieces, counter, piece)
+    const int4 *fext;                               // pieces: (first slot, pieces, counter, piece)
     float4 *fpart;                                  // partial sums of split forward items [slot][DS][threads][2]
     int *fcnt;                                      // pieces finished per split forward item
     int n_items, ngroups;
@@ -164,6 +165,13 @@ struct LineArgs {
     const uint32_t *keep;                           // centre-test mask [nl][kKeepWords] or NULL (all kept)
     int dsel;                                       // backward: damping family of the second sum
                                                     // (0 van der Waals, 1 radiative, 2 Stark)
+    // box expansions (pz_box.cuh): pairs they sum are skipped by the far-wing kernels
+    int boxB, boxsh, s_lo, nbox;                    // box points (0: off) and log2, first source box, boxes
+    float shrink;                                   // |v| >= |Delta| ln r shrink k over a window
+    const int *nmin;                                // [S][nslab][4] nearest offset of each class
+    const int32_t *bstart;                          // [S][nbox + 1] first line of each box
+    uint32_t *wide;                                 // [4][nslab][wwords] lines of class >= 1..4
+    int64_t wwords;
 };
 
 // Centre-test decision of the pair (l, d): kept unless a mask is set and its bit is clear.
@@ -297,6 +305,36 @@ struct alignas(16) LineInfo {
     int sp, amask;
 };
 
+// Box separation class of a line at slab w of its record's depth group, and the nearest box
+// offset that the expansions take over for it.
+__device__ __forceinline__ int box_class(int amask, int w) { return (amask >> (16 + 3 * w)) & 7; }
+
+// The warp's view of the box expansions: nearest offsets of its slab by class, the tile's boxes
+// and the lane's box.
+struct BoxView {
+    int n0, n1, n2, n3, ta, tb, tl;
+};
+__device__ __forceinline__ BoxView box_view(const LineArgs &g, int st, int slab, int t0, int T, int lam_thr) {
+    BoxView v;
+    const int4 n = *reinterpret_cast<const int4 *>(g.nmin + ((int64_t)st * g.nslab + slab) * 4);
+    v.n0 = n.x;
+    v.n1 = n.y;
+    v.n2 = n.z;
+    v.n3 = n.w;
+    v.ta = t0 >> g.boxsh;
+    v.tb = (t0 + T - 1) >> g.boxsh;
+    v.tl = lam_thr >> g.boxsh;
+    return v;
+}
+__device__ __forceinline__ int box_nmin(const BoxView &v, int cls) {
+    return cls == 0 ? v.n0 : cls == 1 ? v.n1 : cls == 2 ? v.n2 : cls == 3 ? v.n3 : kBoxNever;
+}
+// The lane's points are summed directly for this line (not by the expansions).
+__device__ __forceinline__ bool box_near(const LineArgs &g, const BoxView &v, const LineInfo &info, int w) {
+    return abs(((int)info.ilf >> g.boxsh) - v.tl) < box_nmin(v, box_class(info.amask, w));
+}
+
+
 // ---- packed FP32 pairs ------------------------------------------------------
 // The far-wing kernels evaluate two depths of one (line, lambda) cell with one
 // instruction: a register pair {value at depth d, value at depth d + 1} and the
@@ -396,33 +434,64 @@ constexpr float kFast2V = 5.0f;      // distance threshold factor: |v| >= 5 x 20
 constexpr float kFast3V = 1.5f;      // distance threshold factor: |v| >= 1.5 x 20
 constexpr float kFast2A2 = 1.5f;     // a^2 bound
 
-// One thread per (group, line): the line record, whose amask has bit w set when
+// The line record of every (depth group, line), whose amask has bit w set when
 // a^2 <= kFast2A2 at every layer of slab w (DS layers) of the group, and bit 8 + w when
 // the centre test rejects every layer of slab w (its warp skips the line).
-__global__ void k_far_info(LineArgs gq, int DC, int DS, int ngroups, LineInfo *info) {
-    const int64_t n = (int64_t)ngroups * gq.nl;
-    for (int64_t gl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gl < n; gl += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t l = gl % gq.nl;
-        const int grp = (int)(gl / gq.nl);
-        const LineArgs g = star_view(gq, gq.star[l]);
-        const LineScalars L = load_line(g, l);
-        int amask = 0;
-        for (int w = 0; w < DC / DS; ++w) {
-            bool ok = true, none = true;
-            for (int dd = grp * DC + w * DS; dd < min(grp * DC + (w + 1) * DS, g.nd); ++dd) {
-                float q[16];
+// Bits 16 + 3w..: the line's box separation class at slab w: the smallest c whose nearest
+// distance (n_c - 1) B has |v| >= 9 a at every layer (thresholds of |v| >= 20 are in n_c), or
+// kBoxClasses.  Lines of class >= 1 that keep a layer are also marked in the words of wide.
+// Depth group = blockIdx.y; warp w of each half of the block takes slab w (of at most 4) of 32
+// consecutive lines, one word of wide (one thread per line over all slabs waited four times as
+// long on its chain of table loads: 50 -> 19 us at 2 10^5 lines, 10 -> 4 us at 2,000).
+constexpr int kInfoLines = 64;     // lines per block
+__global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, LineInfo *info) {
+    __shared__ int s_mask[4][kInfoLines];
+    const int grp = blockIdx.y, w = (threadIdx.x >> 5) & 3, col = (threadIdx.x & 31) + (threadIdx.x >> 7) * 32;
+    const int64_t l = (int64_t)blockIdx.x * kInfoLines + col;
+    const bool in = l < gq.nl;
+    const int st = in ? gq.star[l] : 0;
+    const LineArgs g = star_view(gq, st);
+    int amask = 0;
+    if (w < DC / DS) {
+        bool ok = true, none = true;
+        float need = 0.0f;
+        if (in) {
+            const LineScalars L = load_line(g, l);
+            const int d1 = min(grp * DC + (w + 1) * DS, g.nd);
+            for (int dd = grp * DC + w * DS; dd < d1; ++dd) {
+                float q[8];
                 depth_params<8>(g, L, dd, q);
                 ok = ok && q[1] <= kFast2A2;
                 none = none && !pair_kept(g.keep, l, dd);
+                need = fmaxf(need, sqrtf(q[1]) / q[0]);
             }
-            amask |= (ok ? 1 << w : 0) | (none ? 1 << (8 + w) : 0);
         }
+        amask = (ok ? 1 << w : 0) | (none ? 1 << (8 + w) : 0);
+        int cls = kBoxClasses;
+        if (gq.boxB) {
+            if (in) {
+                need *= 9.0f / (gq.lnr * gq.shrink);
+                const int *n = gq.nmin + ((int64_t)st * gq.nslab + grp * (DC / DS) + w) * 4;
+                for (int c = kBoxClasses - 1; c >= 0; --c)
+                    if (n[c] < kBoxNever && (float)((n[c] - 1) * gq.boxB) >= need) cls = c;
+            }
+            for (int c = 1; c <= kBoxClasses; ++c) {
+                const unsigned m = __ballot_sync(0xffffffffu, in && !none && cls >= c);
+                if ((threadIdx.x & 31) == 0 && (l >> 5) < gq.wwords)
+                    gq.wide[((int64_t)(c - 1) * gq.nslab + grp * (DC / DS) + w) * gq.wwords + (l >> 5)] = m;
+            }
+        }
+        amask |= cls << (16 + 3 * w);
+    }
+    s_mask[w][col] = amask;
+    __syncthreads();
+    if (w == 0 && in) {
         LineInfo r;
         r.ilf = g.ilf[l];
         r.frac = g.frac[l];
-        r.sp = L.sp;
-        r.amask = amask;
-        info[gl] = r;
+        r.sp = g.sp[l];
+        r.amask = s_mask[0][col] | s_mask[1][col] | s_mask[2][col] | s_mask[3][col];
+        info[(int64_t)grp * gq.nl + l] = r;
     }
 }
 
@@ -466,6 +535,10 @@ __device__ __forceinline__ void far_depth_prefactors(const LineArgs &g, const Li
         c1 = c2 = 0.0f;
     }
 }
+
+}  // namespace pz
+#include "pz_box.cuh"
+namespace pz {
 
 // Per-warp staging of a chunk of lines.  Each warp keeps, in its own part of shared
 // memory, the layer constants of its slab (dc: DS x {beta_hi, beta_lo, n_e, n_pert}),
@@ -520,6 +593,83 @@ __device__ __forceinline__ int warp_gather(const WarpStage &ws, const LineInfo *
     }
     __syncwarp();
     return count;
+}
+
+// Up to LC lines of [cur, hi) whose bit is set in words (one bit per line), in line order, into
+// ws.idx; returns the count and leaves cur after the last line looked at.
+__device__ __forceinline__ int warp_gather_bits(const WarpStage &ws, const uint32_t *words, int &cur, int hi, int LC,
+                                                int lane) {
+    int count = 0;
+    __syncwarp();
+    while (count < LC && cur < hi) {
+        const int w0 = cur >> 5, first = (w0 + lane) << 5;
+        uint32_t m = first < hi ? words[w0 + lane] : 0u;
+        if (first < cur) m &= ~0u << (cur - first);            // (lane 0 alone holds lines before cur)
+        if (first < hi && hi - first < 32) m &= (1u << (hi - first)) - 1u;
+        const int n = __popc(m);
+        int inc = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, inc, 31);
+        int slot = count + inc - n;
+        for (; m && slot < LC; ++slot) {
+            ws.idx[slot] = first + __ffs(m) - 1;
+            m &= m - 1u;
+        }
+        __syncwarp();
+        if (count + total <= LC) {
+            count += total;
+            cur = (w0 + 32) << 5;
+        } else {
+            count = LC;
+            cur = ws.idx[LC - 1] + 1;
+        }
+    }
+    __syncwarp();
+    return count;
+}
+
+// The lines beyond the tile's near boxes that warp's slab still sums directly, ring by ring:
+// between the nearest offsets of class c - 1 (n0g: that of the whole group) and of class c, the
+// lines of class >= c; beyond class 3, the lines no class takes.  f(lines) runs for every gathered
+// chunk.  Piece q of P takes its share of every ring.
+template <class F>
+__device__ __forceinline__ void box_rings(const LineArgs &g, const BoxView &v, int st, int slab, int n0g, int t0, int T,
+                                          int q, int P, const WarpStage &ws, int LC, int lane, F &&f) {
+    if (!g.boxB || n0g >= kBoxNever) return;
+    const int32_t *bs = g.bstart + (int64_t)st * (g.nbox + 1);
+    int below = n0g;
+    for (int c = 1; c <= kBoxClasses; ++c) {
+        const int n = box_nmin(v, c);
+        const int upto = max(n, below);
+        const uint32_t *words = g.wide + ((int64_t)(c - 1) * g.nslab + slab) * g.wwords;
+        for (int side = 0; side < 2 && upto > below; ++side) {
+            // boxes of the ring, clipped to those the windows reach
+            int s0 = side ? v.ta - upto + 1 : v.tb + below;
+            int s1 = side ? v.ta - below : v.tb + upto - 1;
+            s0 = max(max(s0, (t0 - g.W) >> g.boxsh), g.s_lo);
+            s1 = min(min(s1, (t0 + T - 1 + g.W) >> g.boxsh), g.s_lo + g.nbox - 1);
+            if (s0 > s1) continue;
+            const int a = bs[s0 - g.s_lo], b = bs[s1 - g.s_lo + 1];
+            int cur = a + (int)((int64_t)(b - a) * q / P);
+            const int hi = a + (int)((int64_t)(b - a) * (q + 1) / P);
+            while (cur < hi) {
+                const int nl = warp_gather_bits(ws, words, cur, hi, LC, lane);
+                if (nl > 0) f(nl);
+            }
+        }
+        below = upto;
+    }
+}
+
+// Nearest offset of class 0 over the slabs of a depth group (the group's near boxes).
+__device__ __forceinline__ int box_group_n0(const LineArgs &g, int st, int group, int GW) {
+    int n = 0;
+    for (int w = 0; w < GW; ++w) n = max(n, g.nmin[((int64_t)st * g.nslab + group * GW + w) * 4]);
+    return n;
 }
 
 template <int NQ, int DS>
@@ -580,19 +730,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
 
 
 // Per-warp flags of a line over the tile (4: every layer of the slab rejected by the
-// centre test, nothing to evaluate): bit 0 if the line's window covers the tile
+// centre test, or every pair summed by the box expansions: nothing to evaluate): bit 0 if the line's window covers the tile
 // and every cell of the warp's slab is in the far wing (|v| >= 20); bit 1 if every
 // cell of the slab has |v| >= 100 and a^2 <= kFast2A2 at every layer (reduced form),
 // whether or not the window covers the tile: the reduced form masks the window per
 // point at no cost per cell (a zero reciprocal s = 1/U); bit 3 if instead every cell
 // has |v| >= 30 with the same a^2 bound (three-term reduced form).
 __device__ __forceinline__ int far_flags(const LineArgs &g, const LineInfo &info, float t0f, float tendf, int slab,
-                                         int w) {
+                                         int w, const BoxView &bv) {
     const float dlo = info.ilf - t0f + info.frac;      // x_l - t0
     const float dhi = info.ilf - tendf + info.frac;    // x_l - (t0 + T - 1)
     const float dmin = fmaxf(0.0f, fmaxf(-dlo, dhi));
     const bool full = (info.ilf - (float)g.W <= t0f) && (info.ilf + (float)g.W >= tendf);
     if ((info.amask >> (8 + w)) & 1) return 4;        // the centre test rejects the whole slab
+    const int sbox = (int)info.ilf >> g.boxsh, nb = box_nmin(bv, box_class(info.amask, w));
+    if (sbox <= bv.ta - nb || sbox >= bv.tb + nb) return 4;   // every pair is in the box expansions
     const float thr = __ldg(g.thr + info.sp * g.nslab + slab);
     const bool fast = full && dmin >= thr;
     const bool amask = (info.amask >> w) & 1;
@@ -645,7 +797,8 @@ __device__ __forceinline__ void far_c3456(f2_t a2, f2_t C1, f2_t &C3, f2_t &C4, 
 // Reciprocals s_j = 1/U_j of the squared scaled offsets of one line at the thread's J
 // points (and their squares), for the reduced forms: offsets from the first point's,
 // u_j = u_0 r^-j + (r^-j - 1) scaled by 2^18; points outside the line's window get
-// s = 0 unless the window covers the tile (full).
+// s = 0 unless the window covers the tile (full), points of a lane whose box is left to the
+// box expansions (not near) too.
 template <int J>
 __device__ __forceinline__ void far_scaled_u2(const LineArgs &g, const LineInfo &info, float lamf, float (&U)[J]) {
     // scalar chain: the offsets depend on the line and the point only, not on the depth
@@ -659,13 +812,13 @@ __device__ __forceinline__ void far_scaled_u2(const LineArgs &g, const LineInfo 
 }
 
 template <int J>
-__device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo &info, bool full, float lamf,
-                                              int lam_thr, f2_t (&sp)[J], f2_t (&sq)[J]) {
+__device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo &info, bool full, bool near,
+                                              float lamf, int lam_thr, f2_t (&sp)[J], f2_t (&sq)[J]) {
     float U[J];
     far_scaled_u2<J>(g, info, lamf, U);
-    if (full) {
+    if (full || !near) {
 #pragma unroll
-        for (int j = 0; j < J; ++j) sp[j] = f2_splat(rcp_approx(U[j]));
+        for (int j = 0; j < J; ++j) sp[j] = f2_splat(near ? rcp_approx(U[j]) : 0.0f);
     } else {
         const int il = (int)info.ilf;
 #pragma unroll
@@ -683,9 +836,9 @@ __device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo 
 // k_line_near_fwd into knear, which this kernel adds before applying stim.
 // Returns false if a chunk never arrived (the kernel stops).
 template <int J, int DS, bool GATHER>
-__device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, const int group, const int lo,
-                                             const int hi, const int GW, const int LC, const WarpStage &ws,
-                                             float *s_comp, const int4 ext) {
+__device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, const int tile, const int group,
+                                             const int lo, const int hi, const int GW, const int LC,
+                                             const WarpStage &ws, float *s_comp, const int4 ext) {
     static_assert(J == 2 || J == 4, "J must be 2 or 4");
     static_assert(DS % 2 == 0, "DS must be even (depth pairs)");
     constexpr int DP = DS / 2;          // depth pairs per warp
@@ -702,6 +855,8 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
     const float t0f = (float)t0, tendf = (float)(t0 + T - 1);
     const int lam_thr = t0 + lane * J;
     const float lamf = (float)lam_thr;
+
+    const BoxView bv = box_view(g, st, slab, t0, T, lam_thr);
 
     f2_t acc[DP][J];
 #pragma unroll
@@ -725,7 +880,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
         for (int li = 0; li < nl; ++li) {
             if ((li & 31) == 0) {
                 const int lj = li + lane;
-                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp) : 0;
+                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp, bv) : 0;
                 m_fast = __ballot_sync(0xffffffffu, f & 1);
                 m_red = __ballot_sync(0xffffffffu, (f & 2) != 0);
                 m_red3 = __ballot_sync(0xffffffffu, (f & 8) != 0);
@@ -736,8 +891,8 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
                 // two consecutive two-term lines: their offsets and reciprocals are independent
                 // chains, formed together; the sums take line li's terms, then line li + 1's
                 f2_t spa[J], sqa[J], spb[J], sqb[J];
-                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, lamf, lam_thr, spa, sqa);
-                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, lamf, lam_thr, spb, sqb);
+                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
+                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr, spb, sqb);
                 const ulonglong2 *pa = s_par + (size_t)li * DP * NQ, *pb = pa + DP * NQ;
 #pragma unroll
                 for (int dp = 0; dp < DP; ++dp) {
@@ -755,6 +910,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
             const int fl = (int)((m_fast >> b) & 1u) | (int)(((m_red >> b) & 1u) << 1) | (int)(((m_red3 >> b) & 1u) << 2);
             if ((m_skip >> b) & 1u) continue;        // every layer rejected by the centre test
             const ulonglong2 *par = s_par + (size_t)li * DP * NQ;
+            const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
             // the whole tile in the line's far wing (fl != 0): offsets from the first point's,
             // u_j = u_0 r^-j + (r^-j - 1), scaled by 2^18, and their squares U = 2^36 u^2
             float U[J];
@@ -763,9 +919,9 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
                 // reduced forms (B1 K) s + (B2' K^2) s^2 [+ (B3' K^3) s^3] with s = 1/U; points
                 // outside the window (lines whose window edge crosses the tile) get s = 0
                 f2_t sp[J], sq[J];
-                if (fl & 1) {
+                if ((fl & 1) || !near) {
 #pragma unroll
-                    for (int j = 0; j < J; ++j) sp[j] = f2_splat(rcp_approx(U[j]));
+                    for (int j = 0; j < J; ++j) sp[j] = f2_splat(near ? rcp_approx(U[j]) : 0.0f);
                 } else {
                     const int il = (int)info.ilf;
 #pragma unroll
@@ -817,7 +973,8 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
                         // r = 1/(U + a^2 K) = 2^-36/(u^2 + a^2/k^2), t = 1/(u^2 k^2 + a^2) = K r
-                        const f2_t r = f2_rcp(f2_fma(u2[j], f2_splat(1.0f), ak));
+                        const f2_t rr = f2_rcp(f2_fma(u2[j], f2_splat(1.0f), ak));
+                        const f2_t r = near ? rr : 0ull;
                         const f2_t t = f2_mul(q0.x, r);
                         f2_t h = f2_fma(t, B5, B4);
                         h = f2_fma(t, h, B3);
@@ -837,7 +994,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int di = lam_thr + j - il;
-                    inwin[j] = di >= -g.W && di <= g.W;
+                    inwin[j] = near && di >= -g.W && di <= g.W;
                 }
                 f2_t kp[DP];
                 far_kpairs<DP>(g, info.sp, d0 + warp * DS, kp);
@@ -901,12 +1058,15 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
             }
         }
     };
+    auto listed = [&](const int nl) {
+        warp_fill<NQ, DS>(g, ws, ginfo, 0, nl, d0 + warp * DS, lane, true);
+        chunk(nl);
+    };
     if (GATHER) {
         for (int cur = lo; cur < hi;) {
             const int nl = warp_gather(ws, ginfo, cur, hi, LC, warp, lane);
             if (nl == 0) break;
-            warp_fill<NQ, DS>(g, ws, ginfo, 0, nl, d0 + warp * DS, lane, true);
-            chunk(nl);
+            listed(nl);
         }
     } else {
         const int nch = (hi - lo + LC - 1) / LC;
@@ -916,6 +1076,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int tile, 
             chunk(nl);
         }
     }
+    box_rings(g, bv, st, slab, box_group_n0(g, st, group, GW), t0, T, ext.w, ext.y, ws, LC, lane, listed);
 
     if (ext.y > 1) {
         // one of ext.y pieces of a split item (slots ext.x.., counter ext.z, piece ext.w):
@@ -1001,8 +1162,7 @@ __global__ void __launch_bounds__(128, MINB) k_line_fwd(LineArgs g, int GW, int 
     const WarpStage ws = make_stage(mine, LC, DS, kNQF);
     float *s_comp = reinterpret_cast<float *>(smem4 + (size_t)GW * wq);
     for_each_item(g, [&](const LineArgs &v, int tile, int group, int lo, int hi, int it) {
-        return far_fwd_item<J, DS, GATHER>(v, tile, group, lo, hi, GW, LC, ws, s_comp,
-                                           g.fext ? g.fext[it] : make_int4(-1, 1, -1, 0));
+        return far_fwd_item<J, DS, GATHER>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_comp, g.fext[it]);
     });
 }
 
@@ -1011,16 +1171,16 @@ __global__ void __launch_bounds__(128, MINB) k_line_fwd(LineArgs g, int GW, int 
 // (C1 K, C2' K^2); usq: the scaled squared offsets U = 2^36 u^2 of the thread's points.
 template <int J, int DP, bool THREE>
 __device__ __forceinline__ void far_bwd_line_reduced(const ulonglong2 *par, const float (&usq)[J],
-                                                     const f2_t (&gv)[DP][J], bool full, int di0, int W, f2_t &S1,
-                                                     f2_t &S2) {
+                                                     const f2_t (&gv)[DP][J], bool full, bool near, int di0, int W,
+                                                     f2_t &S1, f2_t &S2) {
     // reduced forms with s = 1/U: per depth pair X1 = sum_j G s_j and X2 = sum_j G s_j^2,
     // then S1 += (B1 K) X1 + (B2' K^2) X2 and S2 += (C1 K) X1 + (C2' K^2) X2 (THREE: also
     // X3 = sum_j G s_j^3 with B3' K^3 and C3' K^3); points outside the window
-    // (di0 + j = i - i_l) get s = 0 unless it covers the tile
+    // (di0 + j = i - i_l) get s = 0 unless it covers the tile, and so do lanes that are not near
     f2_t sp[J], sq[J];
-    if (full) {
+    if (full || !near) {
 #pragma unroll
-        for (int j = 0; j < J; ++j) sp[j] = f2_splat(rcp_approx(usq[j]));
+        for (int j = 0; j < J; ++j) sp[j] = f2_splat(near ? rcp_approx(usq[j]) : 0.0f);
     } else {
 #pragma unroll
         for (int j = 0; j < J; ++j)
@@ -1093,7 +1253,7 @@ __device__ __forceinline__ void far_bwd_two_term(const ulonglong2 *par, const f2
 // only the far cells inside the window (inwin per lambda point) are kept.
 template <int J, int DP, bool MASK>
 __device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (&w)[J], const f2_t (&gv)[DP][J],
-                                             const bool *inwin, const f2_t *kp, f2_t &S1, f2_t &S2) {
+                                             const bool near, const bool *inwin, const f2_t *kp, f2_t &S1, f2_t &S2) {
 #pragma unroll
     for (int dp = 0; dp < DP; ++dp) {
         // (K, a^2) (B1 K, B2' K^2) (C1 K, C2' K^2); the other coefficients from a^2, B1 K and C1 K
@@ -1121,7 +1281,8 @@ __device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (
                 m = t;
             } else {
                 // r = 1/(U + a^2 K), t = K r; the coefficients carry K, so the sums take r
-                m = f2_rcp(f2_fma(w[j], f2_splat(1.0f), ak));
+                const f2_t rr = f2_rcp(f2_fma(w[j], f2_splat(1.0f), ak));
+                m = near ? rr : 0ull;
                 t = f2_mul(q0.x, m);
             }
             f2_t h = f2_fma(t, B5, B4);
@@ -1151,9 +1312,10 @@ __device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (
 // Far-wing kernel (backward): the per-line sums over the tile's far cells of
 // G stim A H and G stim A a6 dH/da, reduced over the CTA and added to gacc.
 template <int J, int DS>
-__device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, const int group, const int lo,
-                                             const int hi, const int GW, const int LC, const WarpStage &ws,
-                                             float2 *s_part, float2 *s_red2, unsigned &cc) {
+__device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, const int tile, const int group,
+                                             const int lo, const int hi, const int GW, const int LC,
+                                             const WarpStage &ws, float2 *s_part, float2 *s_red2, unsigned &cc,
+                                             const int4 ext) {
     static_assert(J == 2 || J == 4, "J must be 2 or 4");
     static_assert(DS % 2 == 0, "DS must be even (depth pairs)");
     constexpr int DP = DS / 2;
@@ -1186,14 +1348,9 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
     }
 
     warp_stage_depths<DS>(g, ws, d0 + warp * DS, lane);
-    const int nch = (hi - lo + LC - 1) / LC;
-    for (int c = 0; c < nch; ++c) {
-        const int c0 = lo + c * LC;
-        const int nl = min(LC, hi - c0);
-        // per-line sums of this chunk go to buffer cc & 1: its previous readers (the
-        // reduction two chunks back) are past the CTA barrier of the previous chunk
-        float2 *s_red = s_red2 + (size_t)((cc + c) & 1) * LC * GW;
-        warp_fill<NQ, DS>(g, ws, ginfo, c0, nl, d0 + warp * DS, lane);
+    const BoxView bv = box_view(g, st, slab, t0, T, lam_thr);
+    // the staged lines of one chunk: the warp's two sums of slot k go to sink(k, S1, S2)
+    auto chunk = [&](const int nl, auto &&sink) {
         const ulonglong2 *s_par = reinterpret_cast<const ulonglong2 *>(ws.par);
         const LineInfo *s_line = ws.info;
         unsigned m_fast = 0u, m_red = 0u, m_red3 = 0u, m_skip = 0u;   // this warp's flags of 32 lines, one per lane
@@ -1201,7 +1358,7 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
             const unsigned b = li & 31;
             if (b == 0) {
                 const int lj = li + lane;
-                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp) : 0;
+                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp, bv) : 0;
                 m_fast = __ballot_sync(0xffffffffu, f & 1);
                 m_red = __ballot_sync(0xffffffffu, (f & 2) != 0);
                 m_red3 = __ballot_sync(0xffffffffu, (f & 8) != 0);
@@ -1212,8 +1369,8 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
                 // two consecutive two-term lines of one batch: independent offset and
                 // reciprocal chains, formed together
                 f2_t spa[J], sqa[J], spb[J], sqb[J];
-                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, lamf, lam_thr, spa, sqa);
-                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, lamf, lam_thr, spb, sqb);
+                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
+                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr, spb, sqb);
                 const ulonglong2 *pa = s_par + (size_t)li * DP * NQ;
                 f2_t S1a = 0ull, S2a = 0ull, S1b = 0ull, S2b = 0ull;
                 far_bwd_two_term<J, DP>(pa, spa, sqa, gv, S1a, S2a);
@@ -1229,19 +1386,20 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
                 f2_t S1 = 0ull, S2 = 0ull;
                 // (a slab whose every layer the centre test rejects keeps zero sums)
                 if (!((m_skip >> b) & 1u)) {
+                    const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
                     float U[J];
                     if (fl != 0) far_scaled_u2<J>(g, info, lamf, U);
                     if (fl & 2) {
-                        far_bwd_line_reduced<J, DP, false>(par, U, gv, (fl & 1) != 0, lam_thr - (int)info.ilf, g.W,
+                        far_bwd_line_reduced<J, DP, false>(par, U, gv, (fl & 1) != 0, near, lam_thr - (int)info.ilf, g.W,
                                                            S1, S2);
                     } else if (fl & 4) {
-                        far_bwd_line_reduced<J, DP, true>(par, U, gv, (fl & 1) != 0, lam_thr - (int)info.ilf, g.W,
+                        far_bwd_line_reduced<J, DP, true>(par, U, gv, (fl & 1) != 0, near, lam_thr - (int)info.ilf, g.W,
                                                           S1, S2);
                     } else if (fl & 1) {
                         f2_t u2[J];
 #pragma unroll
                         for (int j = 0; j < J; ++j) u2[j] = f2_splat(U[j]);
-                        far_bwd_line<J, DP, false>(par, u2, gv, nullptr, nullptr, S1, S2);
+                        far_bwd_line<J, DP, false>(par, u2, gv, near, nullptr, nullptr, S1, S2);
                     } else {
                         // line near the tile or partly outside its window: far cells inside the window only
                         f2_t u2[J];
@@ -1253,11 +1411,11 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
 #pragma unroll
                         for (int j = 0; j < J; ++j) {
                             const int di = lam_thr + j - il;
-                            inwin[j] = di >= -g.W && di <= g.W;
+                            inwin[j] = near && di >= -g.W && di <= g.W;
                         }
                         f2_t kp[DP];
                         far_kpairs<DP>(g, info.sp, d0 + warp * DS, kp);
-                        far_bwd_line<J, DP, true>(par, u2, gv, inwin, kp, S1, S2);
+                        far_bwd_line<J, DP, true>(par, u2, gv, near, inwin, kp, S1, S2);
                     }
                 }
                 const int r = b & (kBwdBatch - 1);
@@ -1283,10 +1441,20 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
                 }
                 a1 += __shfl_xor_sync(0xffffffffu, a1, 1);
                 a2 += __shfl_xor_sync(0xffffffffu, a2, 1);
-                if (h == 0 && base + r < nl) s_red[(base + r) * GW + warp] = make_float2(a1, a2);
+                if (h == 0 && base + r < nl) sink(base + r, a1, a2);
                 __syncwarp();
             }
         }
+    };
+    const int nch = (hi - lo + LC - 1) / LC;
+    for (int c = 0; c < nch; ++c) {
+        const int c0 = lo + c * LC;
+        const int nl = min(LC, hi - c0);
+        // per-line sums of this chunk go to buffer cc & 1: its previous readers (the
+        // reduction two chunks back) are past the CTA barrier of the previous chunk
+        float2 *s_red = s_red2 + (size_t)((cc + c) & 1) * LC * GW;
+        warp_fill<NQ, DS>(g, ws, ginfo, c0, nl, d0 + warp * DS, lane);
+        chunk(nl, [&](int k, float a1, float a2) { s_red[k * GW + warp] = make_float2(a1, a2); });
         __syncthreads();
         // thread k adds sum k & 1 of line k >> 1 over the warps in FP32, in warp order, and
         // converts once for the FP64 accumulator: FP64 arithmetic runs at a small fraction
@@ -1300,6 +1468,14 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int tile, 
         }
     }
     cc += nch;
+    // lines beyond the near boxes: each warp gathers its slab's and adds their sums itself
+    box_rings(g, bv, st, slab, box_group_n0(g, st, group, GW), t0, T, ext.w, ext.y, ws, LC, lane, [&](const int nl) {
+        warp_fill<NQ, DS>(g, ws, ginfo, 0, nl, d0 + warp * DS, lane, true);
+        chunk(nl, [&](int k, float a1, float a2) {
+            atomicAdd(g.gacc + ws.idx[k], (double)a1);
+            atomicAdd(g.gacc + g.nl + ws.idx[k], (double)a2);
+        });
+    });
     return true;
 }
 
@@ -1313,8 +1489,8 @@ __global__ void __launch_bounds__(128, MINB) k_line_bwd(LineArgs g, int GW, int 
     float2 *s_red2 = reinterpret_cast<float2 *>(smem4 + (size_t)GW * wq);
     float2 *s_part = s_red2 + (size_t)2 * LC * GW + (size_t)warp * kBwdBatch * 32;
     unsigned cc = 0;
-    for_each_item(g, [&](const LineArgs &v, int tile, int group, int lo, int hi, int) {
-        return far_bwd_item<J, DS>(v, tile, group, lo, hi, GW, LC, ws, s_part, s_red2, cc);
+    for_each_item(g, [&](const LineArgs &v, int tile, int group, int lo, int hi, int it) {
+        return far_bwd_item<J, DS>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_part, s_red2, cc, g.fext[it]);
     });
 }
 
@@ -1683,6 +1859,15 @@ static LineArgs make_args(pz_ctx *c) {
     g.dstride = c->nd;
     g.bstride = (int64_t)c->nd * c->ld;
     g.tstride = (int64_t)c->ns * c->nslab;
+    g.boxB = c->box.B;
+    g.boxsh = c->box.sh;
+    g.s_lo = c->box.s_lo;
+    g.nbox = c->box.nbox;
+    g.shrink = (float)std::max(0.5, 1.0 - 0.5 * (c->W + 1024.0) * c->lnr);
+    g.nmin = c->box.d_nmin;
+    g.bstart = c->box.d_start;
+    g.wide = c->box.d_wide;
+    g.wwords = (c->L.n + 31) / 32;
     return g;
 }
 
@@ -1755,13 +1940,13 @@ constexpr size_t kFarSmemMax = 200 * 1024;   // the opt-in size the far-wing ker
 bool tiling_fits(const Tiling &t) { return far_fwd_smem(t) <= kFarSmemMax && far_bwd_smem(t) <= kFarSmemMax; }
 
 // Line records of the far-wing kernels for the current tiling, into the context's
-// buffer (sized by ensure_far_tables).
+// buffer (sized by ensure_far_tables).  They depend on the corrections, the centre test and
+// the tiling; the reverse pass after a forward finds the forward's (finfo_valid).
 static cudaError_t launch_far_info(pz_ctx *c, LineArgs &g, int DS, cudaStream_t s) {
     const int DC = c->tiling.depth_per_cta();
-    const int64_t n = (int64_t)g.ngroups * c->L.n;
-    const int grid = (int)std::min<int64_t>((n + 255) / 256, (int64_t)c->n_sm * 16);
+    const dim3 grid((unsigned)((c->L.n + kInfoLines - 1) / kInfoLines), (unsigned)g.ngroups);
     g.finfo = reinterpret_cast<const LineInfo *>(c->d_finfo);
-    k_far_info<<<grid, 256, 0, s>>>(g, DC, DS, g.ngroups, reinterpret_cast<LineInfo *>(c->d_finfo));
+    k_far_info<<<grid, 256, 0, s>>>(g, DC, DS, reinterpret_cast<LineInfo *>(c->d_finfo));
     c->launches++;
     return cudaGetLastError();
 }
@@ -1770,6 +1955,146 @@ size_t far_info_bytes(const pz_ctx *c) {
     const int DC = c->tiling.depth_per_cta();
     const int ng = (c->nd + DC - 1) / DC;
     return (size_t)ng * std::max<int64_t>(c->L.n, 1) * sizeof(LineInfo);
+}
+
+// ---- box expansions: host side -------------------------------------------------
+constexpr size_t kBoxWorkspace = (size_t)1 << 30;   // bytes per launch aimed at (stars are taken in chunks)
+
+// Geometry of the expansions.  A box of B points, a power of two near half the widest near zone
+// (thr_max: 20 Doppler widths in grid points), so that the nearest pairs are 3 or 4 boxes apart:
+// smaller boxes raise the pairs as 1/B^2, larger ones the points left to the direct sum.
+void box_choose(pz_ctx *c, double thr_max) {
+    BoxPlan &b = c->box;
+    b.B = b.sh = 0;
+    if (c->prec != PZ_MIXED || c->L.n == 0) return;
+    int sh = 2;
+    while (sh < 5 && thr_max >= 2.5 * (1 << sh)) ++sh;
+    const int B = 1 << sh;
+    const int64_t omax = (c->W + 1) / B - 1;
+    // the window ends' tables need a wide offset (few moments), and at least some whole boxes
+    if (omax < 8) return;
+    // the expansions cost a fixed amount per (point, layer) and some 0.1 ms of latency per pass:
+    // below about 200 lines per window, or 2e8 (line, point, layer) terms in all, the direct sum
+    // is as fast (574 points x 1,416 lines, 3.5e7 terms: 0.63 ms direct, 0.72 ms with boxes; 4,000 x
+    // 2,000, 2.5e8: 0.22 against 0.18 ms; 2,200 x 12,000, 1.7e9, with the reverse pass: 1.35 against
+    // 0.92 ms; 37,550 x 200,000, 4.3e10: 23.0 against 7.0 ms, near cores aside)
+    const double per_window = (double)c->L.n / c->S / (double)c->nlam * (2.0 * c->W + 1.0);
+    if (per_window < 200.0 || (double)c->n_evals < 2e8) return;
+    b.B = B;
+    b.sh = sh;
+    b.omax = (int)omax;
+    b.rem = c->W + 1 - (int)(omax + 1) * B;
+    b.s_lo = -((c->W + B - 1) / B);
+    b.nbox = (int)((c->nlam - 1 + c->W) / B) - b.s_lo + 1;
+    b.ntb = (int)((c->nlam + B - 1) / B);
+    b.KE = box_order((int)omax + 1) + 1 <= 5 ? 5 : 8;
+    b.chunk = 1;
+    while (b.chunk < c->S && box_workspace_floats(c, b.chunk + 1) * sizeof(float) <= kBoxWorkspace) ++b.chunk;
+}
+
+static size_t box_moment_floats(const pz_ctx *c) { return (size_t)c->box.nbox * kBoxClasses * kBoxK * c->nd; }
+size_t box_workspace_floats(const pz_ctx *c, int stars) {
+    const BoxPlan &b = c->box;
+    const size_t fwd = box_moment_floats(c) + (size_t)b.nbox * b.B * b.KE * c->nd;
+    const size_t bwd = (size_t)b.ntb * kBoxK * c->nd;
+    return std::max(fwd, bwd) * stars;
+}
+size_t box_wide_bytes(const pz_ctx *c) {
+    return (size_t)kBoxClasses * c->nslab * (size_t)((c->L.n + 31) / 32) * sizeof(uint32_t);
+}
+
+cudaError_t launch_box_tables(pz_ctx *c) {
+    const BoxPlan &b = c->box;
+    k_box_tables<<<dim3(b.omax + 2, 2), 256>>>(b.B, c->lnr, b.omax, b.d_C);
+    k_box_edges<<<dim3(b.B, 2, 2), 32>>>(b.B, b.omax, b.KE, b.d_C, b.d_E);
+    k_box_start<<<dim3(b.nbox / 256 + 1, c->S), 256>>>(b.nbox, b.s_lo, b.B, c->L.il32, c->d_line_off, b.d_start);
+    // operators of f^2, f^3, f^4 on the Chebyshev basis: column k of (1/m)(d + p eps)(d + q eps)
+    const double eps = 0.5 * b.B * c->lnr;
+    std::vector<double> cur((size_t)kBoxK * kBoxK, 0.0);   // [k][j]: image of T_k as coefficients of T_j
+    for (int k = 0; k < kBoxK; ++k) cur[k * kBoxK + k] = 1.0;
+    auto apply = [&](double *v, double add) {                // v <- (d/dx + add) v in Chebyshev coefficients
+        double dv[kBoxK + 2] = {0.0};
+        for (int j = kBoxK - 1; j >= 1; --j) dv[j - 1] = dv[j + 1] + 2.0 * j * v[j];
+        dv[0] *= 0.5;
+        for (int j = 0; j < kBoxK; ++j) v[j] = dv[j] + add * v[j];
+    };
+    std::vector<float> A((size_t)3 * kBoxK * kBoxK);
+    const double m[3] = {6.0, 20.0, 42.0};
+    for (int q = 0; q < 3; ++q)
+        for (int k = 0; k < kBoxK; ++k) {
+            double *v = &cur[(size_t)k * kBoxK];
+            apply(v, (2 * q + 2) * eps);
+            apply(v, (2 * q + 3) * eps);
+            for (int j = 0; j < kBoxK; ++j) {
+                v[j] /= m[q];
+                A[((size_t)q * kBoxK + k) * kBoxK + j] = (float)v[j];
+            }
+        }
+    const cudaError_t e = cudaMemcpy(b.d_A, A.data(), A.size() * sizeof(float), cudaMemcpyHostToDevice);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+static BoxArgs box_args(const pz_ctx *c, int star0) {
+    const BoxPlan &p = c->box;
+    BoxArgs b;
+    b.B = p.B;
+    b.omax = p.omax;
+    b.rem = p.rem;
+    b.s_lo = p.s_lo;
+    b.nbox = p.nbox;
+    b.ntb = p.ntb;
+    b.DC = c->tiling.depth_per_cta();
+    b.DS = c->tiling.DS;
+    b.star0 = star0;
+    b.invh = 2.0f / p.B;
+    b.ctr = 0.5f * (p.B - 1);
+    const double eps = 0.5 * p.B * c->lnr;
+    b.kapscale = (float)(1.0 / ((double)kKScale * eps * eps));
+    b.A = p.d_A;
+    b.C = p.d_C;
+    b.E = p.d_E;
+    b.nmin = p.d_nmin;
+    b.M = p.d_ws;
+    b.PM = p.d_ws + (size_t)p.chunk * box_moment_floats(c);
+    b.N = p.d_ws;
+    return b;
+}
+
+// Forward: moments of the lines, then the far field of every point into knear.
+template <int KE>
+static cudaError_t launch_box_fwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+    const int thr = (c->nd + 31) / 32 * 32;
+    for (int st = 0; st < c->S; st += c->box.chunk) {
+        const int n = std::min(c->box.chunk, c->S - st);
+        const BoxArgs b = box_args(c, st);
+        k_box_moments<KE><<<dim3(b.nbox, n), thr, sizeof(float) * 3 * kBoxK * thr, s>>>(g, b);
+        k_box_field<KE><<<dim3(b.ntb, n), (kBoxSplit * c->nd + 31) / 32 * 32,
+                          sizeof(float) * (kBoxSplit * kBoxK * c->nd + b.B * (c->nd + 1)), s>>>(g, b);
+        c->launches += 2;
+    }
+    return cudaGetLastError();
+}
+
+// Backward: moments of G, then every line's sums over the points its boxes reach, into gacc.
+template <int KE>
+static cudaError_t launch_box_bwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+    const int thr = (c->nd + 31) / 32 * 32;
+    const size_t smem = box_grad_smem(c->box.B, KE, c->nd);
+    static std::atomic<bool> attr_set[kMaxDevices];
+    if (!attr_set[c->device].load(std::memory_order_acquire)) {
+        const cudaError_t e = cudaFuncSetAttribute(k_box_grad<KE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)box_grad_smem(32, KE, kMaxDepth));
+        if (e != cudaSuccess) return e;
+        attr_set[c->device].store(true, std::memory_order_release);
+    }
+    for (int st = 0; st < c->S; st += c->box.chunk) {
+        const int n = std::min(c->box.chunk, c->S - st);
+        const BoxArgs b = box_args(c, st);
+        k_box_gmoments<<<dim3(b.ntb, n), thr, sizeof(float) * c->nd * (b.B + 1), s>>>(g, b);
+        k_box_grad<KE><<<dim3(b.nbox, n), 32 * kBoxGradWarps, smem, s>>>(g, b);
+        c->launches += 2;
+    }
+    return cudaGetLastError();
 }
 
 template <int J, int DS, int MINB>
@@ -1796,6 +2121,11 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
     g.ctr = c->d_ctr + 1;
     if (c->L.n > 0) {
         e = launch_far_info(c, g, DS, s);
+        if (e != cudaSuccess) return e;
+        c->finfo_valid = true;
+    }
+    if (c->box.B) {
+        e = c->box.KE == 5 ? launch_box_fwd<5>(c, g, s) : launch_box_fwd<8>(c, g, s);
         if (e != cudaSuccess) return e;
     }
     if (c->n_fsplit > 0) {
@@ -1826,8 +2156,15 @@ static cudaError_t launch_bwd_t(pz_ctx *c, cudaStream_t s) {
         gb.n_items = c->n_bitems;
         gb.ngroups = (c->nd + t.depth_per_cta() - 1) / t.depth_per_cta();
         gb.ctr = c->d_ctr + 2;
-        e = launch_far_info(c, gb, DS, s);
-        if (e != cudaSuccess) return e;
+        gb.fext = c->d_bext;
+        if (!c->finfo_valid) {
+            e = launch_far_info(c, gb, DS, s);
+            if (e != cudaSuccess) return e;
+        }
+        if (c->box.B) {
+            e = c->box.KE == 5 ? launch_box_bwd<5>(c, gb, s) : launch_box_bwd<8>(c, gb, s);
+            if (e != cudaSuccess) return e;
+        }
         int grid = persistent_grid(c, k_line_bwd<J, DS, MINB>, 32 * t.GW, smem, gb.n_items);
         k_line_bwd<J, DS, MINB><<<grid, 32 * t.GW, smem, s>>>(gb, t.GW, t.LCB);
         c->launches++;
@@ -2100,6 +2437,7 @@ __global__ void k_apply_abund(int64_t n, int ns, int nd, const double *Rbase, co
 }
 
 cudaError_t launch_apply_corrections(pz_ctx *c, cudaStream_t s) {
+    c->finfo_valid = false;
     if (c->L.n > 0) {
         CorrArgs a{c->L.n,     c->L.orig,  c->L.Qbase, c->L.g6base, c->L.gradbase, c->L.g4base,
                    c->d_mdgf,  c->d_mdg6,  c->d_mdgrad, c->d_mdg4, c->L.dgf,      c->L.dg6,
