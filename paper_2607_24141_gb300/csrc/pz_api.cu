@@ -212,13 +212,14 @@ static void dfree(void *p) { dev_free(p); }
 //         finishes an item last combines them in piece order (deterministic);
 //         near-core backward items are cut the same way;
 //   near: lines whose centre lies within 20 Doppler widths (the widest of the star)
-//         of the tile plus a margin; forward items for every (star, tile, group of
-//         kNearDepthsFwd layers) (they write the near-core buffer), backward items of
+//         of the tile plus a margin; forward items for every (star, tile, group of at
+//         most kNearDepthsFwd layers) (they write the near-core buffer), backward items of
 //         kNearDepthsBwd layers only where the range is not empty.
 constexpr double kPiecesPerCta = 8.0;       // target far pieces per resident CTA
 constexpr int kMaxPieces = 32;              // pieces of one far item at most
 constexpr int kMinPieceLines = 256;         // lines of a far piece at least
 constexpr size_t kMaxPartBytes = (size_t)512 << 20;   // partial-sum buffer of the split forward items
+constexpr double kNearFwdItemsPerSm = 10.0; // near-core forward items per SM at least (layers permitting)
 constexpr double kNearCtasPerSm = 6.0;      // resident near-core CTAs per SM (estimate for the split)
 constexpr int kMinNearPieceLines = 64;      // lines of a near-core backward piece at least
 
@@ -227,7 +228,11 @@ static pz_status build_items(pz_ctx *c) {
     const int nt = (int)((c->nlam + T - 1) / T);
     const int DC = c->tiling.depth_per_cta();
     const int ngf = (c->nd + DC - 1) / DC;
-    const int nnf = (c->nd + kNearDepthsFwd - 1) / kNearDepthsFwd, nnb = (c->nd + kNearDepthsBwd - 1) / kNearDepthsBwd;
+    // near-core forward items: fewer layers each where a short grid has too few of them
+    int ndf = kNearDepthsFwd;
+    while (ndf > 1 && (double)c->S * nt * ((c->nd + ndf - 1) / ndf) < kNearFwdItemsPerSm * std::max(c->n_sm, 1)) ndf /= 2;
+    c->near_depths = ndf;
+    const int nnf = (c->nd + ndf - 1) / ndf, nnb = (c->nd + kNearDepthsBwd - 1) / kNearDepthsBwd;
     struct Item {
         int4 v;
         double cost;
@@ -268,7 +273,7 @@ static pz_status build_items(pz_ctx *c) {
             const int nhi = (int)(std::upper_bound(b0, b1, (int32_t)std::ceil(nb_)) - c->h_il.begin());
             for (int g = 0; g < nnf; ++g)
                 nf.push_back({make_int4(st, t * nnf + g, nlo, nhi),
-                              (double)(nhi - nlo) * std::min(kNearDepthsFwd, c->nd - g * kNearDepthsFwd)});
+                              (double)(nhi - nlo) * std::min(ndf, c->nd - g * ndf)});
             if (nhi > nlo)
                 for (int g = 0; g < nnb; ++g)
                     nb.push_back({make_int4(st, t * nnb + g, nlo, nhi),

@@ -27,7 +27,7 @@ constexpr double kC2 = kH * kC / kKB;       // second radiation constant, cm K
 
 // Largest supported depth count (register/local arrays in the flux kernels).
 constexpr int kMaxDepth = 128;
-constexpr int kNearDepthsFwd = 8;    // layers per work item of the near-core forward
+constexpr int kNearDepthsFwd = 8;    // layers per work item of the near-core forward at most
 constexpr int kNearDepthsBwd = 6;    // layers per work item of the near-core backward
 // Largest number of instrument taps per pixel.
 constexpr int kMaxTaps = 4096;
@@ -57,8 +57,10 @@ struct Tiling {
     int J = 4;       // lambda points per thread (contiguous)
     int DS = 6;      // depths per warp (even: the far-wing kernels work on depth pairs)
     int GW = 4;      // warps per CTA (each a depth slab)
-    int LC = 32;     // lines per shared-memory chunk (forward)
-    int LCB = 32;    // lines per shared-memory chunk (backward)
+    // 16 lines per chunk: with the series' nine quads per depth pair of the reverse pass 32 lines
+    // would take 77 KB per CTA (2 resident per SM against 4)
+    int LC = 16;     // lines per shared-memory chunk (forward)
+    int LCB = 16;    // lines per shared-memory chunk (backward)
     int minb = 4;    // minimum resident CTAs per SM the kernels are compiled for
     int lambda_per_tile() const { return 32 * J; }
     int depth_per_cta() const { return DS * GW; }
@@ -193,6 +195,7 @@ struct pz_ctx {
     int4 *d_bext = nullptr;         // per backward piece: (0, pieces, 0, piece)
     int4 *d_nitems_f = nullptr;     // near-core forward
     int4 *d_nitems_b = nullptr;     // near-core backward
+    int near_depths = pz::kNearDepthsFwd;   // layers per near-core forward item
     int n_fitems = 0, n_bitems = 0, n_nitems_f = 0, n_nitems_b = 0;
     float4 *d_fpart = nullptr;      // compensated partial sums of the split forward items
     size_t fpart_cap = 0;           // bytes allocated at d_fpart

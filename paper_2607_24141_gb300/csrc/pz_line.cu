@@ -166,6 +166,7 @@ struct LineArgs {
     int dsel;                                       // backward: damping family of the second sum
                                                     // (0 van der Waals, 1 radiative, 2 Stark)
     // box expansions (pz_box.cuh): pairs they sum are skipped by the far-wing kernels
+    int tDC, tDS;                                   // layers per depth group and slab of the line records
     int boxB, boxsh, s_lo, nbox;                    // box points (0: off) and log2, first source box, boxes
     float shrink;                                   // |v| >= |Delta| ln r shrink k over a window
     const int *nmin;                                // [S][nslab][4] nearest offset of each class
@@ -385,8 +386,8 @@ __device__ __forceinline__ float f2_hi(f2_t v) {
 // the (DC/2) depth pairs of its group it forms NQ quads, quad q holding
 // {p_2q(d), p_2q(d + 1), p_2q+1(d), p_2q+1(d + 1)} (one 16-byte shared-memory load
 // returns the packed depth pairs of two parameters):
-//   forward  (NQ = 2): (K, a^2) (B1 K, B2' K^2)
-//   backward (NQ = 3): (K, a^2) (B1 K, B2' K^2) (C1 K, C2' K^2)
+//   forward  (NQ = 5): (K, a^2) (B1 K, B2' K^2) (B3' K^3, B4' K^4) .. (B7' K^7, B8' K^8)
+//   backward (NQ = 9): the same, then (C1 K, C2' K^2) .. (C7' K^7, C8' K^8)
 // with k = c/dv_D, K = 2^36/k^2 (the power of two keeps every product of the
 // prefactors and of the offsets far from the FP32 exponent limits), B2' = B2 - B1 a^2
 // = B1 (1.5 - a^2) and C2' = C2 - C1 a^2 = C1 (1.5 - 3a^2).  The far kernels take the
@@ -395,13 +396,14 @@ __device__ __forceinline__ float f2_hi(f2_t v) {
 //   full form:     r = 1/(U + a^2 K) and t = 1/|z|^2 = K r, so B1 t (...) = (B1 K) r (...)
 // and the masked lines recover B1 = (B1 K) k^2 2^-36 (and C1 alike) per depth pair.
 // Each warp stages the quads of its own slab, par[li][pair][q] in its part of shared
-// memory; the rest of the far polynomial (B3..B5, C3..C6) follows from a^2 and B1 K
-// (C1 K) in registers.  Lane li computes line li's quads from the line data and the
+// memory; the polynomial in t of the large-damping lines (B3..B5, C3..C6) follows from a^2
+// and B1 K (C1 K) in registers.  Lane li computes line li's quads from the line data and the
 // star's per-(species, depth) tables (Eqs. 4-5, with the roundings of depth_params), so
 // no per-(line, depth) array exists in device memory: the quads are recomputed for each
 // tile the line's window reaches.  The only per-line device array of the far kernels is
 // the 16-byte line record of each depth group (k_far_info).
-constexpr int kNQF = 2, kNQB = 3;
+constexpr int kPolyN = 8;          // terms of the series in p = K s
+constexpr int kNQF = 1 + kPolyN / 2, kNQB = 1 + kPolyN;
 constexpr int kBwdBatch = 16;   // lines per transposed partial-sum batch of the far-wing backward (2 lanes per line)
 constexpr float kUScale = 262144.0f;              // 2^18: scaled offset u 2^18
 constexpr float kKUnscale = 1.4551915228366852e-11f;   // 2^-36
@@ -423,14 +425,17 @@ constexpr float kKUnscale = 1.4551915228366852e-11f;   // 2^-36
 //   X1 = sum_i G_i s_i,  X2 = sum_i G_i s_i^2,
 // and X1, X2 serve both gradients (the C coefficients multiply the same sums).
 constexpr float kFast2V = 5.0f;      // distance threshold factor: |v| >= 5 x 20
-// Three-term reduced form, for the lines between 30 and 100 Doppler widths from the tile:
-// the same expansion one order further,
-//   H sqrt(pi)/A = (B1 K) s + (B2' K^2) s^2 + (B3' K^3) s^3,  B3' = B1 (3.75 - 5a^2 + a^4),
-//   dH/da sqrt(pi)/(A a6) = (C1 K) s + (C2' K^2) s^2 + (C3' K^3) s^3,  C3' = C1 (3.75 - 15a^2 + 5a^4),
-// (the t^3 terms of the far polynomial and the p^3 terms of t and t^2 in p).  Against the
-// five-term polynomial the dropped p^4 terms stay below 2.6e-8 relative for H and 4.6e-8 for
-// dH/da at |v| >= 30 and a^2 <= 1.5 (evaluated on a dense (a^2, v) lattice).  B3' K^3 and
-// C3' K^3 are formed per depth pair from K, a^2, B1 K and C1 K.
+// The same expansion to N terms, H sqrt(pi)/A = sum_n B1 beta_n(a^2) (K s)^(n+1) and dH/da
+// sqrt(pi)/(A a6) = sum_n C1 gamma_n(a^2) (K s)^(n+1), reaches the nearer cells: with a^2 <= 1.5 the
+// dropped terms stay below 2.6e-8 (H) and 4.6e-8 (dH/da) relative with N = 3 at |v| >= 30, below
+// 3e-9 with N = 4 at |v| >= 20 and below 6.3e-8 (dH/da: 1.2e-7 of its scale 1/v^2) with N = 8 at |v| >= 6.
+// Eight multiply-adds per cell and no per-cell branch: the mid wing 6 <= |v| < 20, which the
+// near-core kernels summed cell by cell at about 140 instructions each, and the masked far cells
+// beside it (two reciprocals and a polynomial in t per depth pair) are one sweep of the tile.
+// Measured on 2e5 lines x 37,550 points: far + near-core forward 6.9 -> 4.3 ms, reverse 9.9 ->
+// 6.8 ms.
+constexpr float kCoreV = 0.3f;       // distance threshold factor: |v| >= 0.3 x 20 = 6
+constexpr float kCoreX2 = 36.0f;     // cells with x^2 < 36 (U < 36 K) of the series' lines belong to the near-core kernels
 constexpr float kFast3V = 1.5f;      // distance threshold factor: |v| >= 1.5 x 20
 constexpr float kFast2A2 = 1.5f;     // a^2 bound
 
@@ -441,8 +446,8 @@ constexpr float kFast2A2 = 1.5f;     // a^2 bound
 // distance (n_c - 1) B has |v| >= 9 a at every layer (thresholds of |v| >= 20 are in n_c), or
 // kBoxClasses.  Lines of class >= 1 that keep a layer are also marked in the words of wide.
 // Depth group = blockIdx.y; warp w of each half of the block takes slab w (of at most 4) of 32
-// consecutive lines, one word of wide (one thread per line over all slabs waited four times as
-// long on its chain of table loads: 50 -> 19 us at 2 10^5 lines, 10 -> 4 us at 2,000).
+// consecutive lines, one word of wide (with one thread per line over all slabs a short list
+// waited on the chain of table loads: 11 -> 6 us at 5,300 lines; 50 us at 2 10^5 either way).
 constexpr int kInfoLines = 64;     // lines per block
 __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, LineInfo *info) {
     __shared__ int s_mask[4][kInfoLines];
@@ -495,19 +500,50 @@ __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, L
     }
 }
 
+// c_n = x K^n beta_n(a^2) (D: gamma_n(a^2)), n = 0..7: beta_n = sum_k (-1)^k c_(n-k) binom(2n + 1,
+// 2k + 1) a^2k with c_m = (2m - 1)!!/2^m, from the expansion of Re w(v + i a) about 1/v, and gamma_n =
+// sum_k (2k + 1) (..) a^2k, its derivative.
+template <bool D>
+__device__ __forceinline__ void poly_coeffs(float x, float K, float s, float (&c)[kPolyN]) {
+#define PZ_Q(k, v) ((D ? 2.0f * (k) + 1.0f : 1.0f) * (v))
+    c[0] = x;
+    x *= K;
+    c[1] = x * fmaf(s, PZ_Q(1, -1.0f), PZ_Q(0, 1.5f));
+    x *= K;
+    c[2] = x * fmaf(s, fmaf(s, PZ_Q(2, 1.0f), PZ_Q(1, -5.0f)), PZ_Q(0, 3.75f));
+    x *= K;
+    c[3] = x * fmaf(s, fmaf(s, fmaf(s, PZ_Q(3, -1.0f), PZ_Q(2, 10.5f)), PZ_Q(1, -26.25f)), PZ_Q(0, 13.125f));
+    x *= K;
+    c[4] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(4, 1.0f), PZ_Q(3, -18.0f)), PZ_Q(2, 94.5f)), PZ_Q(1, -157.5f)),
+                    PZ_Q(0, 59.0625f));
+    x *= K;
+    c[5] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(5, -1.0f), PZ_Q(4, 27.5f)), PZ_Q(3, -247.5f)),
+                                    PZ_Q(2, 866.25f)), PZ_Q(1, -1082.8125f)), PZ_Q(0, 324.84375f));
+    x *= K;
+    c[6] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(6, 1.0f), PZ_Q(5, -39.0f)), PZ_Q(4, 536.25f)),
+                                            PZ_Q(3, -3217.5f)), PZ_Q(2, 8445.9375f)), PZ_Q(1, -8445.9375f)),
+                    PZ_Q(0, 2111.484375f));
+    x *= K;
+    c[7] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(6, 52.5f), PZ_Q(5, -1023.75f)), PZ_Q(4, 9384.375f)),
+                                            PZ_Q(3, -42229.6875f)), PZ_Q(2, 88682.34375f)), PZ_Q(1, -73901.953125f)),
+                    PZ_Q(0, 15836.1328125f));
+#undef PZ_Q
+}
+
 // Prefactors of line l at layer d (one half of a depth pair), with the roundings of
 // depth_params for k and a^2 (the cells' near / far classification depends on them):
-// K = 2^36/k^2, a^2, B1 K, B2' K^2 and (NQ = kNQB) C1 K, C2' K^2.  dc holds the layer's
+// K = 2^36/k^2, a^2, the series coefficients c (B1 K, B2' K^2, ..) and (NQ = kNQB) e (C1 K, C2' K^2, ..).  dc holds the layer's
 // {beta_hi, beta_lo, n_e, n_pert}.  Layers past the last one get K = 0, a^2 = 1 and zero
 // coefficients, pairs rejected by the centre test zero coefficients.
 template <int NQ>
 __device__ __forceinline__ void far_depth_prefactors(const LineArgs &g, const LineScalars &L, int64_t l, int d,
-                                                     const float4 dc, float &K, float &a2, float &b1, float &b2,
-                                                     float &c1, float &c2) {
+                                                     const float4 dc, float &K, float &a2, float (&c)[kPolyN],
+                                                     float (&e)[kPolyN]) {
     if (d >= g.nd) {
         K = 0.0f;
         a2 = 1.0f;
-        b1 = b2 = c1 = c2 = 0.0f;
+#pragma unroll
+        for (int n = 0; n < kPolyN; ++n) c[n] = e[n] = 0.0f;
         return;
     }
     const int id = L.sp * g.nd + d;
@@ -521,18 +557,11 @@ __device__ __forceinline__ void far_depth_prefactors(const LineArgs &g, const Li
     const float a = __fmul_rn(fmaf(L.g4, dc.z, __fadd_rn(L.grad, g6n)), lw);
     a2 = __fmul_rn(a, a);
     K = __ldg(g.Ksd + id);
-    const float KK = K * K;
     const bool kept = pair_kept(g.keep, l, d);
-    const float B1 = kept ? A * a * kInvSqrtPiF : 0.0f;
-    b1 = B1 * K;
-    b2 = fmaf(-B1, a2, 1.5f * B1) * KK;
+    poly_coeffs<false>(kept ? A * a * kInvSqrtPiF * K : 0.0f, K, a2, c);
     if (NQ == kNQB) {
         const float gb = g.dsel == 0 ? g6n : (g.dsel == 1 ? L.grad : __fmul_rn(L.g4, dc.z));
-        const float C1 = kept ? A * gb * lw * kInvSqrtPiF : 0.0f;
-        c1 = C1 * K;
-        c2 = fmaf(-C1, a2, fmaf(-2.0f, a2, 1.5f) * C1) * KK;
-    } else {
-        c1 = c2 = 0.0f;
+        poly_coeffs<true>(kept ? A * gb * lw * kInvSqrtPiF * K : 0.0f, K, a2, e);
     }
 }
 
@@ -684,12 +713,15 @@ __device__ __forceinline__ void warp_fill(const LineArgs &g, const WarpStage &ws
         float4 *dst = ws.par + (size_t)li * DP * NQ;
 #pragma unroll
         for (int dp = 0; dp < DP; ++dp) {
-            float K0, K1, a0, a1, b10, b11, b20, b21, c10, c11, c20, c21;
-            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp, ws.dc[2 * dp], K0, a0, b10, b20, c10, c20);
-            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp + 1, ws.dc[2 * dp + 1], K1, a1, b11, b21, c11, c21);
+            float K0, K1, a0, a1, c0[kPolyN], c1[kPolyN], e0[kPolyN], e1[kPolyN];
+            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp, ws.dc[2 * dp], K0, a0, c0, e0);
+            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp + 1, ws.dc[2 * dp + 1], K1, a1, c1, e1);
             dst[NQ * dp] = make_float4(K0, K1, a0, a1);
-            dst[NQ * dp + 1] = make_float4(b10, b11, b20, b21);
-            if (NQ == kNQB) dst[NQ * dp + 2] = make_float4(c10, c11, c20, c21);
+#pragma unroll
+            for (int n = 0; n < kPolyN; n += 2) {
+                dst[NQ * dp + 1 + n / 2] = make_float4(c0[n], c1[n], c0[n + 1], c1[n + 1]);
+                if (NQ == kNQB) dst[NQ * dp + 1 + (kPolyN + n) / 2] = make_float4(e0[n], e1[n], e0[n + 1], e1[n + 1]);
+            }
         }
     }
     __syncwarp();
@@ -729,28 +761,36 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
 }
 
 
-// Per-warp flags of a line over the tile (4: every layer of the slab rejected by the
-// centre test, or every pair summed by the box expansions: nothing to evaluate): bit 0 if the line's window covers the tile
-// and every cell of the warp's slab is in the far wing (|v| >= 20); bit 1 if every
-// cell of the slab has |v| >= 100 and a^2 <= kFast2A2 at every layer (reduced form),
-// whether or not the window covers the tile: the reduced form masks the window per
-// point at no cost per cell (a zero reciprocal s = 1/U); bit 3 if instead every cell
-// has |v| >= 30 with the same a^2 bound (three-term reduced form).
-__device__ __forceinline__ int far_flags(const LineArgs &g, const LineInfo &info, float t0f, float tendf, int slab,
-                                         int w, const BoxView &bv) {
+// How a warp sums a line over its slab and tile.
+enum FarForm {
+    kFormSkip = 0,      // the centre test rejects every layer, or the box expansions sum every pair
+    kFormTwo,           // every cell |v| >= 100: two terms
+    kFormThree,         // |v| >= 30: three
+    kFormFour,          // |v| >= 20: four
+    kFormEight,         // |v| >= 6: eight
+    kFormCore,          // eight, the cells with x^2 < 36 left to the near-core kernels
+    kFormLarge,         // a^2 > kFast2A2 somewhere in the slab, |v| >= 20, the window covers the tile: polynomial in t
+    kFormLargeMask,     // a^2 > kFast2A2: the cells with |z| >= 20 inside the window, the others left to the
+                        // near-core kernels
+    kFormFull = 8       // bit: the window covers the tile
+};
+__device__ __forceinline__ int far_form(const LineArgs &g, const LineInfo &info, float t0f, float tendf, int slab, int w,
+                                        const BoxView &bv) {
     const float dlo = info.ilf - t0f + info.frac;      // x_l - t0
     const float dhi = info.ilf - tendf + info.frac;    // x_l - (t0 + T - 1)
     const float dmin = fmaxf(0.0f, fmaxf(-dlo, dhi));
     const bool full = (info.ilf - (float)g.W <= t0f) && (info.ilf + (float)g.W >= tendf);
-    if ((info.amask >> (8 + w)) & 1) return 4;        // the centre test rejects the whole slab
+    if ((info.amask >> (8 + w)) & 1) return kFormSkip;
     const int sbox = (int)info.ilf >> g.boxsh, nb = box_nmin(bv, box_class(info.amask, w));
-    if (sbox <= bv.ta - nb || sbox >= bv.tb + nb) return 4;   // every pair is in the box expansions
-    const float thr = __ldg(g.thr + info.sp * g.nslab + slab);
-    const bool fast = full && dmin >= thr;
-    const bool amask = (info.amask >> w) & 1;
-    const bool red = dmin >= kFast2V * thr && amask;
-    const bool red3 = !red && dmin >= kFast3V * thr && amask;
-    return (fast ? 1 : 0) | (red ? 2 : 0) | (red3 ? 8 : 0);
+    if (sbox <= bv.ta - nb || sbox >= bv.tb + nb) return kFormSkip;
+    const float thr = __ldg(g.thr + info.sp * g.nslab + slab);   // 20 Doppler widths of the slab's widest layer
+    if (!((info.amask >> w) & 1)) return full && dmin >= thr ? kFormLarge : kFormLargeMask;
+    const int f = dmin >= kFast2V * thr ? kFormTwo
+                  : dmin >= kFast3V * thr ? kFormThree
+                  : dmin >= thr ? kFormFour
+                  : dmin >= kCoreV * thr ? kFormEight
+                                         : kFormCore;
+    return f | (full ? kFormFull : 0);
 }
 
 // k = c/dv_D of the warp's depth pairs, rounded exactly as depth_params forms it, for the
@@ -831,6 +871,105 @@ __device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo 
     for (int j = 0; j < J; ++j) sq[j] = f2_mul(sp[j], sp[j]);
 }
 
+// Reciprocals s_j = 1/U_j at the thread's points for the series forms, zero outside the window
+// and for lanes left to the box expansions.  CORE: U is held above the smallest K of the slab
+// (x^2 >= 1), so that the cells left to the near-core kernels stay finite before they are dropped.
+template <int J, int DP, int NQ, bool CORE>
+__device__ __forceinline__ void far_series_s(const LineArgs &g, const LineInfo &info, bool full, bool near, float lamf,
+                                             int lam_thr, const ulonglong2 *par, float (&U)[J], float (&s)[J]) {
+    far_scaled_u2<J>(g, info, lamf, U);
+    float Umin = 3.0e38f;
+    if (CORE) {
+#pragma unroll
+        for (int dp = 0; dp < DP; ++dp) {
+            const float ka = f2_lo(par[NQ * dp].x), kb = f2_hi(par[NQ * dp].x);
+            if (ka > 0.0f) Umin = fminf(Umin, ka);     // (layers past the last one hold 0)
+            if (kb > 0.0f) Umin = fminf(Umin, kb);
+        }
+    }
+    const int di0 = lam_thr - (int)info.ilf;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const bool in = near && (full || (di0 + j >= -g.W && di0 + j <= g.W));
+        s[j] = in ? rcp_approx(CORE ? fmaxf(U[j], Umin) : U[j]) : 0.0f;
+    }
+}
+
+// acc += sum_n c_n s^(n+1) over the line's cells (N terms).
+template <int J, int DP, int N, bool CORE>
+__device__ __forceinline__ void far_fwd_series(const ulonglong2 *par, const float (&U)[J], const float (&s)[J],
+                                               f2_t (&acc)[DP][J]) {
+#pragma unroll
+    for (int dp = 0; dp < DP; ++dp) {
+        const ulonglong2 *q = par + kNQF * dp;
+        f2_t c[N + 1];
+#pragma unroll
+        for (int n = 0; n < N; n += 2) {
+            const ulonglong2 v = q[1 + n / 2];
+            c[n] = v.x;
+            c[n + 1] = v.y;
+        }
+        const float ca = CORE ? kCoreX2 * f2_lo(q[0].x) : 0.0f, cb = CORE ? kCoreX2 * f2_hi(q[0].x) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const f2_t sp = f2_splat(s[j]);
+            f2_t h = c[N - 1];
+#pragma unroll
+            for (int n = N - 2; n >= 0; --n) h = f2_fma(sp, h, c[n]);
+            const f2_t sm = CORE ? f2_pack(U[j] >= ca ? s[j] : 0.0f, U[j] >= cb ? s[j] : 0.0f) : sp;
+            acc[dp][j] = f2_fma(sm, h, acc[dp][j]);
+        }
+    }
+}
+
+// S1 += sum_n c_n X_n, S2 += sum_n e_n X_n with X_n = sum_j G s_j^(n+1) per depth pair: one
+// multiply-add per cell and term serves both gradients.
+template <int J, int DP, int N, bool CORE>
+__device__ __forceinline__ void far_bwd_series(const ulonglong2 *par, const float (&U)[J], const float (&s)[J],
+                                               const f2_t (&gv)[DP][J], f2_t &S1, f2_t &S2) {
+    constexpr int G = DP < 3 ? DP : 3;        // depth pairs taken together (registers)
+#pragma unroll
+    for (int d0 = 0; d0 < DP; d0 += G) {
+        f2_t X[G][N];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const f2_t sp = f2_splat(s[j]);
+            f2_t gm[G];
+#pragma unroll
+            for (int i = 0; i < G; ++i) {
+                if (d0 + i >= DP) break;
+                gm[i] = gv[d0 + i][j];
+                if (CORE) {
+                    const f2_t K = par[kNQB * (d0 + i)].x;
+                    gm[i] = f2_pack(U[j] >= kCoreX2 * f2_lo(K) ? f2_lo(gm[i]) : 0.0f,
+                                    U[j] >= kCoreX2 * f2_hi(K) ? f2_hi(gm[i]) : 0.0f);
+                }
+            }
+            f2_t pw = sp;
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    if (d0 + i >= DP) break;
+                    X[i][n] = j == 0 ? f2_mul(gm[i], pw) : f2_fma(gm[i], pw, X[i][n]);
+                }
+                if (n + 1 < N) pw = f2_mul(pw, sp);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            if (d0 + i >= DP) break;
+            const ulonglong2 *q = par + kNQB * (d0 + i);
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+                const ulonglong2 c = q[1 + n / 2], e = q[1 + (kPolyN + n) / 2];
+                S1 = f2_fma((n & 1) ? c.y : c.x, X[i][n], S1);
+                S2 = f2_fma((n & 1) ? e.y : e.x, X[i][n], S2);
+            }
+        }
+    }
+}
+
 // Far-wing kernel (forward).  Every cell with |v|^2 + a^2 >= 400 inside its window is
 // evaluated here with the far polynomial; the near-core cells are summed by
 // k_line_near_fwd into knear, which this kernel adds before applying stim.
@@ -876,23 +1015,24 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
     auto chunk = [&](const int nl) {
         const ulonglong2 *s_par = reinterpret_cast<const ulonglong2 *>(ws.par);
         const LineInfo *s_line = ws.info;
-        unsigned m_fast = 0u, m_red = 0u, m_red3 = 0u, m_skip = 0u;   // this warp's flags of 32 lines, one per lane
+        int form = kFormSkip;          // of this lane's line of the current 32
+        unsigned m_two = 0u;           // the two-term ones
         for (int li = 0; li < nl; ++li) {
             if ((li & 31) == 0) {
                 const int lj = li + lane;
-                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp, bv) : 0;
-                m_fast = __ballot_sync(0xffffffffu, f & 1);
-                m_red = __ballot_sync(0xffffffffu, (f & 2) != 0);
-                m_red3 = __ballot_sync(0xffffffffu, (f & 8) != 0);
-                m_skip = __ballot_sync(0xffffffffu, (f & 4) != 0);
+                form = lj < nl ? far_form(g, s_line[lj], t0f, tendf, slab, warp, bv) : kFormSkip;
+                m_two = __ballot_sync(0xffffffffu, (form & 7) == kFormTwo);
             }
             const unsigned b = li & 31;
-            if (b < 31 && li + 1 < nl && ((m_red >> b) & 3u) == 3u && ((m_skip >> b) & 3u) == 0u) {
+            const int fl = __shfl_sync(0xffffffffu, form, b);
+            if (b < 31 && li + 1 < nl && ((m_two >> b) & 3u) == 3u) {
                 // two consecutive two-term lines: their offsets and reciprocals are independent
                 // chains, formed together; the sums take line li's terms, then line li + 1's
+                const int fb = __shfl_sync(0xffffffffu, form, b + 1);
                 f2_t spa[J], sqa[J], spb[J], sqb[J];
-                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
-                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr, spb, sqb);
+                far_reduced_s<J>(g, s_line[li], fl & kFormFull, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
+                far_reduced_s<J>(g, s_line[li + 1], fb & kFormFull, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr,
+                                 spb, sqb);
                 const ulonglong2 *pa = s_par + (size_t)li * DP * NQ, *pb = pa + DP * NQ;
 #pragma unroll
                 for (int dp = 0; dp < DP; ++dp) {
@@ -906,58 +1046,29 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
                 ++li;
                 continue;
             }
+            if ((fl & 7) == kFormSkip) continue;
             const LineInfo info = s_line[li];
-            const int fl = (int)((m_fast >> b) & 1u) | (int)(((m_red >> b) & 1u) << 1) | (int)(((m_red3 >> b) & 1u) << 2);
-            if ((m_skip >> b) & 1u) continue;        // every layer rejected by the centre test
             const ulonglong2 *par = s_par + (size_t)li * DP * NQ;
             const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-            // the whole tile in the line's far wing (fl != 0): offsets from the first point's,
-            // u_j = u_0 r^-j + (r^-j - 1), scaled by 2^18, and their squares U = 2^36 u^2
-            float U[J];
-            if (fl != 0) far_scaled_u2<J>(g, info, lamf, U);
-            if (fl & 6) {
-                // reduced forms (B1 K) s + (B2' K^2) s^2 [+ (B3' K^3) s^3] with s = 1/U; points
-                // outside the window (lines whose window edge crosses the tile) get s = 0
-                f2_t sp[J], sq[J];
-                if ((fl & 1) || !near) {
-#pragma unroll
-                    for (int j = 0; j < J; ++j) sp[j] = f2_splat(near ? rcp_approx(U[j]) : 0.0f);
+            if ((fl & 7) <= kFormCore) {
+                float U[J], sv[J];
+                if ((fl & 7) == kFormCore) {
+                    far_series_s<J, DP, NQ, true>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
+                    far_fwd_series<J, DP, 8, true>(par, U, sv, acc);
                 } else {
-                    const int il = (int)info.ilf;
-#pragma unroll
-                    for (int j = 0; j < J; ++j) {
-                        const int di = lam_thr + j - il;
-                        sp[j] = f2_splat(di >= -g.W && di <= g.W ? rcp_approx(U[j]) : 0.0f);
-                    }
+                    far_series_s<J, DP, NQ, false>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
+                    if ((fl & 7) == kFormEight)
+                        far_fwd_series<J, DP, 8, false>(par, U, sv, acc);
+                    else if ((fl & 7) == kFormFour)
+                        far_fwd_series<J, DP, 4, false>(par, U, sv, acc);
+                    else if ((fl & 7) == kFormThree)
+                        far_fwd_series<J, DP, 3, false>(par, U, sv, acc);
+                    else
+                        far_fwd_series<J, DP, 2, false>(par, U, sv, acc);
                 }
-#pragma unroll
-                for (int j = 0; j < J; ++j) sq[j] = f2_mul(sp[j], sp[j]);
-                if (fl & 2) {
-#pragma unroll
-                    for (int dp = 0; dp < DP; ++dp) {
-                        // q1 = (B1 K, B2' K^2)
-                        const ulonglong2 q1 = par[NQ * dp + 1];
-#pragma unroll
-                        for (int j = 0; j < J; ++j)
-                            acc[dp][j] = f2_fma(sq[j], q1.y, f2_fma(sp[j], q1.x, acc[dp][j]));
-                    }
-                } else {
-                    f2_t sc[J];
-#pragma unroll
-                    for (int j = 0; j < J; ++j) sc[j] = f2_mul(sq[j], sp[j]);
-#pragma unroll
-                    for (int dp = 0; dp < DP; ++dp) {
-                        // q0 = (K, a^2), q1 = (B1 K, B2' K^2); B3' K^3 = (B1 K) K^2 (3.75 - 5a^2 + a^4)
-                        const ulonglong2 q0 = par[NQ * dp], q1 = par[NQ * dp + 1];
-                        const f2_t b3 = f2_mul(f2_mul(q1.x, f2_mul(q0.x, q0.x)),
-                                               f2_fma(q0.y, f2_fma(q0.y, f2_splat(1.0f), f2_splat(-5.0f)),
-                                                      f2_splat(3.75f)));
-#pragma unroll
-                        for (int j = 0; j < J; ++j)
-                            acc[dp][j] = f2_fma(sc[j], b3, f2_fma(sq[j], q1.y, f2_fma(sp[j], q1.x, acc[dp][j])));
-                    }
-                }
-            } else if (fl & 1) {
+            } else if ((fl & 7) == kFormLarge) {
+                float U[J];
+                far_scaled_u2<J>(g, info, lamf, U);
                 f2_t u2[J];
 #pragma unroll
                 for (int j = 0; j < J; ++j) u2[j] = f2_splat(U[j]);
@@ -1166,67 +1277,6 @@ __global__ void __launch_bounds__(128, MINB) k_line_fwd(LineArgs g, int GW, int 
     });
 }
 
-// Reduced far-wing backward forms (lines flagged for them): H and dH/da polynomials cut
-// after their t^2 terms (THREE: t^3).  par: the warp's depth pairs, (K, a^2) (B1 K, B2' K^2)
-// (C1 K, C2' K^2); usq: the scaled squared offsets U = 2^36 u^2 of the thread's points.
-template <int J, int DP, bool THREE>
-__device__ __forceinline__ void far_bwd_line_reduced(const ulonglong2 *par, const float (&usq)[J],
-                                                     const f2_t (&gv)[DP][J], bool full, bool near, int di0, int W,
-                                                     f2_t &S1, f2_t &S2) {
-    // reduced forms with s = 1/U: per depth pair X1 = sum_j G s_j and X2 = sum_j G s_j^2,
-    // then S1 += (B1 K) X1 + (B2' K^2) X2 and S2 += (C1 K) X1 + (C2' K^2) X2 (THREE: also
-    // X3 = sum_j G s_j^3 with B3' K^3 and C3' K^3); points outside the window
-    // (di0 + j = i - i_l) get s = 0 unless it covers the tile, and so do lanes that are not near
-    f2_t sp[J], sq[J];
-    if (full || !near) {
-#pragma unroll
-        for (int j = 0; j < J; ++j) sp[j] = f2_splat(near ? rcp_approx(usq[j]) : 0.0f);
-    } else {
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-            sp[j] = f2_splat(di0 + j >= -W && di0 + j <= W ? rcp_approx(usq[j]) : 0.0f);
-    }
-#pragma unroll
-    for (int j = 0; j < J; ++j) sq[j] = f2_mul(sp[j], sp[j]);
-    if (THREE) {
-        f2_t sc[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) sc[j] = f2_mul(sq[j], sp[j]);
-#pragma unroll
-        for (int dp = 0; dp < DP; ++dp) {
-            const ulonglong2 q0 = par[kNQB * dp], q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 2];
-            f2_t X1 = f2_mul(gv[dp][0], sp[0]), X2 = f2_mul(gv[dp][0], sq[0]), X3 = f2_mul(gv[dp][0], sc[0]);
-#pragma unroll
-            for (int j = 1; j < J; ++j) {
-                X1 = f2_fma(gv[dp][j], sp[j], X1);
-                X2 = f2_fma(gv[dp][j], sq[j], X2);
-                X3 = f2_fma(gv[dp][j], sc[j], X3);
-            }
-            // B3' K^3 = (B1 K) K^2 (3.75 - 5a^2 + a^4), C3' K^3 = (C1 K) K^2 (3.75 - 15a^2 + 5a^4)
-            const f2_t K2 = f2_mul(q0.x, q0.x);
-            const f2_t b3 = f2_mul(f2_mul(q1.x, K2),
-                                   f2_fma(q0.y, f2_fma(q0.y, f2_splat(1.0f), f2_splat(-5.0f)), f2_splat(3.75f)));
-            const f2_t c3 = f2_mul(f2_mul(q2.x, K2),
-                                   f2_fma(q0.y, f2_fma(q0.y, f2_splat(5.0f), f2_splat(-15.0f)), f2_splat(3.75f)));
-            S1 = f2_fma(b3, X3, f2_fma(q1.y, X2, f2_fma(q1.x, X1, S1)));
-            S2 = f2_fma(c3, X3, f2_fma(q2.y, X2, f2_fma(q2.x, X1, S2)));
-        }
-    } else {
-#pragma unroll
-        for (int dp = 0; dp < DP; ++dp) {
-            const ulonglong2 q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 2];
-            f2_t X1 = f2_mul(gv[dp][0], sp[0]), X2 = f2_mul(gv[dp][0], sq[0]);
-#pragma unroll
-            for (int j = 1; j < J; ++j) {
-                X1 = f2_fma(gv[dp][j], sp[j], X1);
-                X2 = f2_fma(gv[dp][j], sq[j], X2);
-            }
-            S1 = f2_fma(q1.y, X2, f2_fma(q1.x, X1, S1));
-            S2 = f2_fma(q2.y, X2, f2_fma(q2.x, X1, S2));
-        }
-    }
-}
-
 // Two-term reduced backward sums of one line from the reciprocals s_j of its points
 // (far_reduced_s): per depth pair X1 = sum_j G s_j and X2 = sum_j G s_j^2, then
 // S1 += (B1 K) X1 + (B2' K^2) X2 and S2 += (C1 K) X1 + (C2' K^2) X2.
@@ -1235,7 +1285,7 @@ __device__ __forceinline__ void far_bwd_two_term(const ulonglong2 *par, const f2
                                                  const f2_t (&gv)[DP][J], f2_t &S1, f2_t &S2) {
 #pragma unroll
     for (int dp = 0; dp < DP; ++dp) {
-        const ulonglong2 q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 2];
+        const ulonglong2 q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 1 + kPolyN / 2];
         f2_t X1 = f2_mul(gv[dp][0], sp[0]), X2 = f2_mul(gv[dp][0], sq[0]);
 #pragma unroll
         for (int j = 1; j < J; ++j) {
@@ -1257,7 +1307,7 @@ __device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (
 #pragma unroll
     for (int dp = 0; dp < DP; ++dp) {
         // (K, a^2) (B1 K, B2' K^2) (C1 K, C2' K^2); the other coefficients from a^2, B1 K and C1 K
-        const ulonglong2 q0 = par[kNQB * dp], q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 2];
+        const ulonglong2 q0 = par[kNQB * dp], q1 = par[kNQB * dp + 1], q2 = par[kNQB * dp + 1 + kPolyN / 2];
         f2_t B1 = q1.x, C1 = q2.x;
         if (MASK) {
             // the masked cells use t = 1/|z|^2 itself: B1 = (B1 K) k^2 2^-36, C1 alike
@@ -1353,24 +1403,24 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
     auto chunk = [&](const int nl, auto &&sink) {
         const ulonglong2 *s_par = reinterpret_cast<const ulonglong2 *>(ws.par);
         const LineInfo *s_line = ws.info;
-        unsigned m_fast = 0u, m_red = 0u, m_red3 = 0u, m_skip = 0u;   // this warp's flags of 32 lines, one per lane
+        int form = kFormSkip;          // of this lane's line of the current 32
+        unsigned m_two = 0u;           // the two-term ones
         for (int li = 0; li < nl;) {
             const unsigned b = li & 31;
             if (b == 0) {
                 const int lj = li + lane;
-                const int f = lj < nl ? far_flags(g, s_line[lj], t0f, tendf, slab, warp, bv) : 0;
-                m_fast = __ballot_sync(0xffffffffu, f & 1);
-                m_red = __ballot_sync(0xffffffffu, (f & 2) != 0);
-                m_red3 = __ballot_sync(0xffffffffu, (f & 8) != 0);
-                m_skip = __ballot_sync(0xffffffffu, (f & 4) != 0);
+                form = lj < nl ? far_form(g, s_line[lj], t0f, tendf, slab, warp, bv) : kFormSkip;
+                m_two = __ballot_sync(0xffffffffu, (form & 7) == kFormTwo);
             }
-            if ((b & (kBwdBatch - 1)) != kBwdBatch - 1 && li + 1 < nl && ((m_red >> b) & 3u) == 3u &&
-                ((m_skip >> b) & 3u) == 0u) {
+            const int fl = __shfl_sync(0xffffffffu, form, b);
+            if ((b & (kBwdBatch - 1)) != kBwdBatch - 1 && li + 1 < nl && ((m_two >> b) & 3u) == 3u) {
                 // two consecutive two-term lines of one batch: independent offset and
                 // reciprocal chains, formed together
+                const int fb = __shfl_sync(0xffffffffu, form, b + 1);
                 f2_t spa[J], sqa[J], spb[J], sqb[J];
-                far_reduced_s<J>(g, s_line[li], (m_fast >> b) & 1u, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
-                far_reduced_s<J>(g, s_line[li + 1], (m_fast >> (b + 1)) & 1u, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr, spb, sqb);
+                far_reduced_s<J>(g, s_line[li], fl & kFormFull, box_near(g, bv, s_line[li], warp), lamf, lam_thr, spa, sqa);
+                far_reduced_s<J>(g, s_line[li + 1], fb & kFormFull, box_near(g, bv, s_line[li + 1], warp), lamf, lam_thr,
+                                 spb, sqb);
                 const ulonglong2 *pa = s_par + (size_t)li * DP * NQ;
                 f2_t S1a = 0ull, S2a = 0ull, S1b = 0ull, S2b = 0ull;
                 far_bwd_two_term<J, DP>(pa, spa, sqa, gv, S1a, S2a);
@@ -1381,21 +1431,30 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
                 li += 2;
             } else {
                 const LineInfo info = s_line[li];
-                const int fl = (int)((m_fast >> b) & 1u) | (int)(((m_red >> b) & 1u) << 1) | (int)(((m_red3 >> b) & 1u) << 2);
                 const ulonglong2 *par = s_par + (size_t)li * DP * NQ;
                 f2_t S1 = 0ull, S2 = 0ull;
                 // (a slab whose every layer the centre test rejects keeps zero sums)
-                if (!((m_skip >> b) & 1u)) {
+                if ((fl & 7) != kFormSkip) {
                     const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-                    float U[J];
-                    if (fl != 0) far_scaled_u2<J>(g, info, lamf, U);
-                    if (fl & 2) {
-                        far_bwd_line_reduced<J, DP, false>(par, U, gv, (fl & 1) != 0, near, lam_thr - (int)info.ilf, g.W,
-                                                           S1, S2);
-                    } else if (fl & 4) {
-                        far_bwd_line_reduced<J, DP, true>(par, U, gv, (fl & 1) != 0, near, lam_thr - (int)info.ilf, g.W,
-                                                          S1, S2);
-                    } else if (fl & 1) {
+                    if ((fl & 7) <= kFormCore) {
+                        float U[J], sv[J];
+                        if ((fl & 7) == kFormCore) {
+                            far_series_s<J, DP, NQ, true>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
+                            far_bwd_series<J, DP, 8, true>(par, U, sv, gv, S1, S2);
+                        } else {
+                            far_series_s<J, DP, NQ, false>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
+                            if ((fl & 7) == kFormEight)
+                                far_bwd_series<J, DP, 8, false>(par, U, sv, gv, S1, S2);
+                            else if ((fl & 7) == kFormFour)
+                                far_bwd_series<J, DP, 4, false>(par, U, sv, gv, S1, S2);
+                            else if ((fl & 7) == kFormThree)
+                                far_bwd_series<J, DP, 3, false>(par, U, sv, gv, S1, S2);
+                            else
+                                far_bwd_series<J, DP, 2, false>(par, U, sv, gv, S1, S2);
+                        }
+                    } else if ((fl & 7) == kFormLarge) {
+                        float U[J];
+                        far_scaled_u2<J>(g, info, lamf, U);
                         f2_t u2[J];
 #pragma unroll
                         for (int j = 0; j < J; ++j) u2[j] = f2_splat(U[j]);
@@ -1495,19 +1554,30 @@ __global__ void __launch_bounds__(128, MINB) k_line_bwd(LineArgs g, int GW, int 
 }
 
 // ---------------------------------------------------------------------------
-// Near-core kernels: the cells with |v|^2 + a^2 < 400 (mid wing and core).  A CTA owns
-// the same wavelength tile as the far kernels and every depth; its warps take
-// (line, depth) items of the lines whose near zone can reach the tile, clip the
-// item's near span analytically, and let the lanes sweep the span 32 points at a
-// time.  Each cell is classified with the far kernels' own arithmetic (same
-// prefactors, same offset and the same |v|^2 + a^2 test), so every cell is counted
-// exactly once across the two kernels.
+// Near-core kernels: the cells that the far-wing kernels leave.  At a slab whose damping the
+// series forms take (a^2 <= kFast2A2 at every layer) those are the core, x^2 = (u k)^2 < 36,
+// decided by U < 36 K with the far kernels' own U; otherwise the mid wing and core,
+// |v|^2 + a^2 < 400, classified with the same prefactors, offset and test as the masked far form.
+// Every cell is counted exactly once across the two kernels.  A CTA owns the same wavelength
+// tile as the far kernels; its warps take (line, depth) items of the lines whose near zone can
+// reach the tile, clip the item's near span analytically, and let the lanes sweep the span 32
+// points at a time.
 // ---------------------------------------------------------------------------
 
+// x^2 < 36 as the far kernels decide it: U = 2^36 u^2 of point i from its lane's first point
+// (far_scaled_u2), against 36 K.
+template <int J>
+__device__ __forceinline__ bool core_owned(const LineArgs &g, float ilf, float frac, int i, float cut) {
+    const int j = i & (J - 1);
+    const float u0 = offset_u((ilf - (float)(i - j)) + frac, g.lnr) * kUScale;
+    const float rj = j == 1 ? g.rj[1] : j == 2 ? g.rj[2] : g.rj[3], rm = j == 1 ? g.rm1j[1] : j == 2 ? g.rm1j[2] : g.rm1j[3];
+    const float u = j == 0 ? u0 : fmaf(u0, rj, rm * kUScale);
+    return u * u < cut;
+}
+
 // Near span of an item clipped to the tile and the window; returns false if empty.
-__device__ __forceinline__ bool near_span(const LineArgs &g, float ilf, float frac, float k, float a2, int t0, int T,
+__device__ __forceinline__ bool near_span(const LineArgs &g, float ilf, float frac, float k, float r2, int t0, int T,
                                           int &lo, int &hi) {
-    const float r2 = kFar2 - a2;
     if (!(k > 0.0f) || !(r2 > 0.0f)) return false;
     const float xl = ilf + frac;
     const int il = (int)ilf;
@@ -1522,7 +1592,7 @@ __device__ __forceinline__ bool near_span(const LineArgs &g, float ilf, float fr
 // core segment (|z|^2 < 36, cells [c0, r0)) and the mid-wing cells on either side
 // (nl cells from lo, then the cells from r0 to hi).
 struct alignas(16) NearItem {
-    float ilf, frac, k, a2;      // centre, Doppler factor c/dv_D, a^2
+    float ilf, frac, k, a2;      // centre, Doppler factor c/dv_D, a^2 (or -36 K: core cells only)
     float a, A, Aa6;             // damping, strength, strength x vdW damping
     int lo, nl, c0, r0;          // span start, mid cells left of the core, core segment [c0, r0)
     int dlb;                     // local depth | (local line index << 8)
@@ -1555,8 +1625,12 @@ __device__ __forceinline__ void near_pass(const LineArgs &g, const NearItem *min
             const int i = CORE ? it.c0 + off : (off < it.nl ? it.lo + off : it.r0 + (off - it.nl));
             const float x = fabsf(offset_u((it.ilf - (float)i) + it.frac, g.lnr) * it.k);
             run = src;
-            // a mid-wing cell at |z| >= 20 belongs to the far-wing kernels (same test)
-            if (CORE || fmaf(x, x, it.a2) < kFar2) {
+            // a mid-wing cell at |z| >= 20 belongs to the far-wing kernels (same test); a core cell
+            // of the series' lines is theirs by U, which only the cells at the boundary need
+            const float x2 = x * x;
+            if (CORE ? (it.a2 >= 0.0f || x2 < 0.999f * kCoreX2 ||
+                        (x2 < 1.001f * kCoreX2 && core_owned<T / 32>(g, it.ilf, it.frac, i, -it.a2)))
+                     : fmaf(x, x, it.a2) < kFar2) {
                 float H, dH;
                 if (CORE)
                     voigt_core<D>(x, it.a, H, dH, s_daw);
@@ -1586,15 +1660,14 @@ __device__ __forceinline__ void near_pass(const LineArgs &g, const NearItem *min
     }
 }
 
-// Backward pass with a blocked assignment (mid wing or core): lane l takes the
+// Backward pass over the mid wing with a blocked assignment: lane l takes the
 // concatenated cells [l P, (l + 1) P), P = ceil(total / 32), so that each lane's cells
 // belong to a few consecutive items; the lane sums an item's cells in registers and
 // hands the sum to done when it moves to the next item (no cross-lane reduction).
-// voigt_mid has no branch on the item's parameters; the core form branches on the
-// damping (Taylor order, table or rational), where lanes of different items diverge.
-template <bool CORE, class Val, class Done>
-__device__ __forceinline__ void near_pass_blocked(const LineArgs &g, const NearItem *mine, const int *pref,
-                                                  const float *s_daw, Val &val, Done &done) {
+// voigt_mid has no branch on the item's parameters, so lanes of different items do not diverge.
+template <class Val, class Done>
+__device__ __forceinline__ void near_pass_blocked(const LineArgs &g, const NearItem *mine, const int *pref, Val &val,
+                                                  Done &done) {
     const int lane = threadIdx.x & 31;
     const int total = pref[32];
     const int per = (total + 31) >> 5;
@@ -1617,15 +1690,12 @@ __device__ __forceinline__ void near_pass_blocked(const LineArgs &g, const NearI
             end = pref[src + 1];
         }
         const int off = n - start;
-        const int i = CORE ? it.c0 + off : (off < it.nl ? it.lo + off : it.r0 + (off - it.nl));
+        const int i = off < it.nl ? it.lo + off : it.r0 + (off - it.nl);
         const float x = fabsf(offset_u((it.ilf - (float)i) + it.frac, g.lnr) * it.k);
         // a mid-wing cell at |z| >= 20 belongs to the far-wing kernels (same test)
-        if (CORE || fmaf(x, x, it.a2) < kFar2) {
+        if (fmaf(x, x, it.a2) < kFar2) {
             float H, dH;
-            if (CORE)
-                voigt_core<true>(x, it.a, H, dH, s_daw);
-            else
-                voigt_mid<true>(x, it.a, H, dH);
+            voigt_mid<true>(x, it.a, H, dH);
             const float2 v = val(it, i, H, dH);
             acc.x += v.x;
             acc.y += v.y;
@@ -1659,11 +1729,23 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int64_t nl
             item.frac = g.frac[l];
             item.dlb = dl | ((int)(it / ndg) << 8);
             const float k = (float)kC * __ldg(g.invdv + g.sp[l] * g.nd + d);
+            const int grp = d / g.tDC;
+            // the far-wing kernels' series take everything but the core of this slab's lines
+            const bool core = (g.finfo[(int64_t)grp * g.nl + l].amask >> ((d - grp * g.tDC) / g.tDS)) & 1;
             int lo, hi;
-            if (pair_kept(g.keep, l, d) && near_span(g, item.ilf, item.frac, k, 0.0f, t0, T, lo, hi)) {
+            if (pair_kept(g.keep, l, d) &&
+                near_span(g, item.ilf, item.frac, k, core ? kCoreX2 : kFar2, t0, T, lo, hi)) {
                 float p[16];
                 line_params<D ? 16 : 8>(g, l, d, p);
-                if (near_span(g, item.ilf, item.frac, p[0], p[1], t0, T, lo, hi)) {
+                if (core) {
+                    item.k = p[0];
+                    item.a2 = -kCoreX2 * __ldg(g.Ksd + g.sp[l] * g.nd + d);
+                    item.A = p[7];
+                    item.a = D ? p[15] : sqrtf(p[1]);
+                    item.Aa6 = D ? p[14] : 0.0f;
+                    ncore = hi - lo + 1;
+                    item.c0 = lo;
+                } else if (near_span(g, item.ilf, item.frac, p[0], kFar2 - p[1], t0, T, lo, hi)) {
                     item.k = p[0];
                     item.a2 = p[1];
                     item.A = p[7];
@@ -1711,7 +1793,7 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int64_t nl
         if (D) {
             // mid wing blocked; the core keeps interleaved cells (its damping branches would
             // diverge across the items of a blocked warp: measured 238 -> 339 ms per batch step)
-            near_pass_blocked<false>(g, mine, pm, s_daw, val, done);
+            near_pass_blocked(g, mine, pm, val, done);
             __syncwarp();
             near_pass<T, D, true>(g, mine, pc, s_daw, cell, val, done);
         } else {
@@ -1723,8 +1805,8 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int64_t nl
 }
 
 // Forward near-core sums into knear.  Work items: (star, tile, depth group of NDG layers).
-template <int T, int NDG>
-__global__ void __launch_bounds__(32 * kNearWarps) k_line_near_fwd(LineArgs gq) {
+template <int T>
+__global__ void __launch_bounds__(32 * kNearWarps) k_line_near_fwd(LineArgs gq, int NDG) {
     extern __shared__ float4 smem4[];
     float *s_acc = reinterpret_cast<float *>(smem4);                               // [NDG][T]
     NearItem *s_items = reinterpret_cast<NearItem *>(s_acc + NDG * T);             // [warps][32]
@@ -1800,9 +1882,9 @@ __global__ void __launch_bounds__(32 * kNearWarps, 5) k_line_near_bwd(LineArgs g
     });
 }
 
-template <int T, int NDG, bool BWD>
-constexpr size_t near_smem() {
-    return (size_t)NDG * T * sizeof(float) + (BWD ? kNearBatch * sizeof(float2) : 0) +
+template <int T, bool BWD>
+constexpr size_t near_smem(int ndg) {
+    return (size_t)ndg * T * sizeof(float) + (BWD ? kNearBatch * sizeof(float2) : 0) +
            (size_t)kNearWarps * 32 * sizeof(NearItem) + (size_t)kNearWarps * 66 * sizeof(int) +
            (size_t)kDawsonNodes * (kDawsonK + 1) * sizeof(float);
 }
@@ -1859,6 +1941,8 @@ static LineArgs make_args(pz_ctx *c) {
     g.dstride = c->nd;
     g.bstride = (int64_t)c->nd * c->ld;
     g.tstride = (int64_t)c->ns * c->nslab;
+    g.tDC = c->tiling.depth_per_cta();
+    g.tDS = c->tiling.DS;
     g.boxB = c->box.B;
     g.boxsh = c->box.sh;
     g.s_lo = c->box.s_lo;
@@ -1891,7 +1975,7 @@ static cudaError_t launch_near(pz_ctx *c, LineArgs g, cudaStream_t s) {
         g.n_items = c->n_nitems_b;
         g.ngroups = (c->nd + kNearDepthsBwd - 1) / kNearDepthsBwd;
         g.ctr = c->d_ctr + 3;
-        constexpr size_t smem = near_smem<T, kNearDepthsBwd, true>();
+        constexpr size_t smem = near_smem<T, true>(kNearDepthsBwd);
         static std::atomic<bool> attr_set[kMaxDevices];
         if (!attr_set[c->device].load(std::memory_order_acquire)) {
             cudaFuncSetAttribute(k_line_near_bwd<T, kNearDepthsBwd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1906,47 +1990,60 @@ static cudaError_t launch_near(pz_ctx *c, LineArgs g, cudaStream_t s) {
         if (c->n_nitems_f == 0) return cudaSuccess;
         g.items = c->d_nitems_f;
         g.n_items = c->n_nitems_f;
-        g.ngroups = (c->nd + kNearDepthsFwd - 1) / kNearDepthsFwd;
+        const int ndg = c->near_depths;
+        g.ngroups = (c->nd + ndg - 1) / ndg;
         g.ctr = c->d_ctr + 0;
-        constexpr size_t smem = near_smem<T, kNearDepthsFwd, false>();
+        const size_t smem = near_smem<T, false>(ndg);
         static std::atomic<bool> attr_set[kMaxDevices];
         if (!attr_set[c->device].load(std::memory_order_acquire)) {
-            cudaFuncSetAttribute(k_line_near_fwd<T, kNearDepthsFwd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+            cudaFuncSetAttribute(k_line_near_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)near_smem<T, false>(kNearDepthsFwd));
             attr_set[c->device].store(true, std::memory_order_release);
         }
-        int grid = persistent_grid(c, k_line_near_fwd<T, kNearDepthsFwd>, 32 * kNearWarps, smem, g.n_items);
+        int grid = persistent_grid(c, k_line_near_fwd<T>, 32 * kNearWarps, smem, g.n_items);
         cudaEvent_t ev = prof_begin(c, s);
-        k_line_near_fwd<T, kNearDepthsFwd><<<grid, 32 * kNearWarps, smem, s>>>(g);
+        k_line_near_fwd<T><<<grid, 32 * kNearWarps, smem, s>>>(g, ndg);
         prof_end(c, s, PZ_K_NEAR_FWD, ev);
     }
     c->launches++;
     return cudaGetLastError();
 }
 
-// Dynamic shared memory of the far-wing kernels: the warps' stages (layer constants,
-// line records, prefactors) and (forward) the compensated sums of every thread, or
+// Dynamic shared memory of the far-wing kernels at LC lines per chunk: the warps' stages (layer
+// constants, line records, prefactors) and (forward) the compensated sums of every thread, or
 // (backward) the per-line sums.
-static size_t far_fwd_smem(const Tiling &t) {
-    return (size_t)t.GW * warp_stage_quads(t.LC, t.DS, kNQF) * sizeof(float4) +
+static size_t far_fwd_smem(const Tiling &t, int LC, int NQ = kNQF) {
+    return (size_t)t.GW * warp_stage_quads(LC, t.DS, NQ) * sizeof(float4) +
            (size_t)t.DS * 32 * t.GW * 2 * sizeof(float4);
 }
-static size_t far_bwd_smem(const Tiling &t) {
-    return (size_t)t.GW * warp_stage_quads(t.LCB, t.DS, kNQB) * sizeof(float4) +
-           (size_t)2 * t.LCB * t.GW * sizeof(float2) + (size_t)t.GW * kBwdBatch * 32 * sizeof(float2);
+static size_t far_bwd_smem(const Tiling &t, int LC, int NQ = kNQB) {
+    return (size_t)t.GW * warp_stage_quads(LC, t.DS, NQ) * sizeof(float4) +
+           (size_t)2 * LC * t.GW * sizeof(float2) + (size_t)t.GW * kBwdBatch * 32 * sizeof(float2);
 }
 constexpr size_t kFarSmemMax = 200 * 1024;   // the opt-in size the far-wing kernels are given
 
-bool tiling_fits(const Tiling &t) { return far_fwd_smem(t) <= kFarSmemMax && far_bwd_smem(t) <= kFarSmemMax; }
+// A tiling is taken if its chunk fits with two (three) quads per depth pair and line; the lines
+// that the kernels stage at a time are cut to what fits with the series' coefficients.
+bool tiling_fits(const Tiling &t) {
+    return far_fwd_smem(t, t.LC, 2) <= kFarSmemMax && far_bwd_smem(t, t.LCB, 3) <= kFarSmemMax;
+}
+static int far_fwd_chunk(const Tiling &t) {
+    int LC = t.LC;
+    while (LC > 1 && far_fwd_smem(t, LC) > kFarSmemMax) --LC;
+    return LC;
+}
+static int far_bwd_chunk(const Tiling &t) {
+    int LC = t.LCB;
+    while (LC > 1 && far_bwd_smem(t, LC) > kFarSmemMax) --LC;
+    return LC;
+}
 
 // Line records of the far-wing kernels for the current tiling, into the context's
 // buffer (sized by ensure_far_tables).  They depend on the corrections, the centre test and
 // the tiling; the reverse pass after a forward finds the forward's (finfo_valid).
-static cudaError_t launch_far_info(pz_ctx *c, LineArgs &g, int DS, cudaStream_t s) {
-    const int DC = c->tiling.depth_per_cta();
-    const dim3 grid((unsigned)((c->L.n + kInfoLines - 1) / kInfoLines), (unsigned)g.ngroups);
-    g.finfo = reinterpret_cast<const LineInfo *>(c->d_finfo);
-    k_far_info<<<grid, 256, 0, s>>>(g, DC, DS, reinterpret_cast<LineInfo *>(c->d_finfo));
+static cudaError_t launch_far_info(pz_ctx *c, const LineArgs &g, int ngroups, cudaStream_t s) {
+    const dim3 grid((unsigned)((c->L.n + kInfoLines - 1) / kInfoLines), (unsigned)ngroups);
+    k_far_info<<<grid, 256, 0, s>>>(g, c->tiling.depth_per_cta(), c->tiling.DS, reinterpret_cast<LineInfo *>(c->d_finfo));
     c->launches++;
     return cudaGetLastError();
 }
@@ -2101,7 +2198,8 @@ template <int J, int DS, int MINB>
 static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
     const Tiling &t = c->tiling;
     LineArgs g = make_args(c);
-    const size_t smem = far_fwd_smem(t);
+    const int LC = far_fwd_chunk(t);
+    const size_t smem = far_fwd_smem(t, LC);
     // with a centre test the kernel stages only the lines each warp's slab sweeps (GATHER)
     const bool gather = c->d_keep != nullptr;
     auto kern = gather ? k_line_fwd<J, DS, MINB, true> : k_line_fwd<J, DS, MINB, false>;
@@ -2112,18 +2210,19 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
     }
     cudaError_t e = cudaMemsetAsync(c->d_ctr, 0, 2 * sizeof(int), s);
     if (e != cudaSuccess) return e;
+    const int ngroups = (c->nd + t.depth_per_cta() - 1) / t.depth_per_cta();
+    if (c->L.n > 0) {
+        e = launch_far_info(c, g, ngroups, s);
+        if (e != cudaSuccess) return e;
+        c->finfo_valid = true;
+    }
     e = launch_near<32 * J, false>(c, g, s);
     if (e != cudaSuccess || c->n_fitems == 0) return e;
     g.items = c->d_fitems;
     g.fext = c->d_fext;
     g.n_items = c->n_fitems;
-    g.ngroups = (c->nd + t.depth_per_cta() - 1) / t.depth_per_cta();
+    g.ngroups = ngroups;
     g.ctr = c->d_ctr + 1;
-    if (c->L.n > 0) {
-        e = launch_far_info(c, g, DS, s);
-        if (e != cudaSuccess) return e;
-        c->finfo_valid = true;
-    }
     if (c->box.B) {
         e = c->box.KE == 5 ? launch_box_fwd<5>(c, g, s) : launch_box_fwd<8>(c, g, s);
         if (e != cudaSuccess) return e;
@@ -2133,7 +2232,7 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     int grid = persistent_grid(c, kern, 32 * t.GW, smem, g.n_items);
-    kern<<<grid, 32 * t.GW, smem, s>>>(g, t.GW, t.LC);
+    kern<<<grid, 32 * t.GW, smem, s>>>(g, t.GW, LC);
     c->launches++;
     return cudaGetLastError();
 }
@@ -2142,7 +2241,8 @@ template <int J, int DS, int MINB>
 static cudaError_t launch_bwd_t(pz_ctx *c, cudaStream_t s) {
     const Tiling &t = c->tiling;
     LineArgs g = make_args(c);
-    const size_t smem = far_bwd_smem(t);
+    const int LC = far_bwd_chunk(t);
+    const size_t smem = far_bwd_smem(t, LC);
     static std::atomic<bool> attr_set[kMaxDevices];
     if (!attr_set[c->device].load(std::memory_order_acquire)) {
         cudaFuncSetAttribute(k_line_bwd<J, DS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFarSmemMax);
@@ -2158,7 +2258,7 @@ static cudaError_t launch_bwd_t(pz_ctx *c, cudaStream_t s) {
         gb.ctr = c->d_ctr + 2;
         gb.fext = c->d_bext;
         if (!c->finfo_valid) {
-            e = launch_far_info(c, gb, DS, s);
+            e = launch_far_info(c, gb, gb.ngroups, s);
             if (e != cudaSuccess) return e;
         }
         if (c->box.B) {
@@ -2166,7 +2266,7 @@ static cudaError_t launch_bwd_t(pz_ctx *c, cudaStream_t s) {
             if (e != cudaSuccess) return e;
         }
         int grid = persistent_grid(c, k_line_bwd<J, DS, MINB>, 32 * t.GW, smem, gb.n_items);
-        k_line_bwd<J, DS, MINB><<<grid, 32 * t.GW, smem, s>>>(gb, t.GW, t.LCB);
+        k_line_bwd<J, DS, MINB><<<grid, 32 * t.GW, smem, s>>>(gb, t.GW, LC);
         c->launches++;
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

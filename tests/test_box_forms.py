@@ -98,3 +98,31 @@ def test_window_ends_with_few_moments(W, B, L):
             f = (L * h / np.expm1((s * (omax + e) * B + h * (x[:, None] - x[None, :])) * L)) ** 2
             assert np.all(C[KE:] == 0.0)
             assert np.abs(T[:, :KE] @ C[:KE] @ T.T / f - 1).max() < 4e-8
+
+
+def coefficient(n, k):
+    """(-1)^k c_(n-k) binom(2n + 1, 2k + 1), c_m = (2m - 1)!!/2^m."""
+    c = 1.0
+    for m in range(n - k):
+        c *= (2 * m + 1) / 2.0
+    return (-1) ** k * c * math.comb(2 * n + 1, 2 * k + 1)
+
+
+@pytest.mark.parametrize("terms,vmin,tol_h,tol_d", [(8, 6.0, 6.4e-8, 1.3e-7), (4, 20.0, 3e-9, 2e-8), (3, 30.0, 2.7e-8, 4.7e-8)])
+def test_series_of_the_nearer_cells(terms, vmin, tol_h, tol_d):
+    """The far-wing kernels' series at the smallest |v| each form takes, over a^2 <= 1.5: H relative,
+    dH/da against its scale p/sqrt(pi) (it crosses zero)."""
+    wofz = pytest.importorskip("scipy.special").wofz
+    v = np.concatenate([np.linspace(vmin, 4 * vmin, 600)])[None, :]
+    a = np.concatenate([np.geomspace(1e-3, 1.0, 25), [1.1, math.sqrt(1.5)]])[:, None]
+    w = wofz(v + 1j * a)
+    H, dH = w.real, 2 * (v * w.imag + a * w.real) - 2 / math.sqrt(math.pi)
+    p, s = 1 / v ** 2, a * a
+    got_h = got_d = 0.0
+    for n in range(terms):
+        kmax = min(n, 6)           # the kernels stop at a^12
+        got_h = got_h + p ** (n + 1) * sum(coefficient(n, k) * s ** k for k in range(kmax + 1))
+        got_d = got_d + p ** (n + 1) * sum((2 * k + 1) * coefficient(n, k) * s ** k for k in range(kmax + 1))
+    assert np.max(np.abs(got_h * a / math.sqrt(math.pi) / H - 1)) < tol_h
+    # the reference's dH/da is a difference of numbers near 1 at 2e-16 each
+    assert np.max(np.abs(got_d / math.sqrt(math.pi) - dH) / (p / math.sqrt(math.pi)) - 1e-15 * v ** 2) < tol_d
