@@ -212,14 +212,14 @@ static void dfree(void *p) { dev_free(p); }
 //         finishes an item last combines them in piece order (deterministic);
 //         near-core backward items are cut the same way;
 //   near: lines whose centre lies within 20 Doppler widths (the widest of the star)
-//         of the tile plus a margin; forward items for every (star, tile, group of at
-//         most kNearDepthsFwd layers) (they write the near-core buffer), backward items of
-//         kNearDepthsBwd layers only where the range is not empty.
+//         of the tile plus a margin; forward items for every (star, tile, group of
+//         kNearDepths layers) (they write the near-core buffer), backward items only
+//         where the range is not empty.
 constexpr double kPiecesPerCta = 8.0;       // target far pieces per resident CTA
 constexpr int kMaxPieces = 32;              // pieces of one far item at most
-constexpr int kMinPieceLines = 256;         // lines of a far piece at least
+constexpr int kMinPieceLines = 64;          // lines of a far piece at least
 constexpr size_t kMaxPartBytes = (size_t)512 << 20;   // partial-sum buffer of the split forward items
-constexpr double kNearFwdItemsPerSm = 10.0; // near-core forward items per SM at least (layers permitting)
+constexpr double kNearItemsPerSm = 8.0;     // near-core forward items per SM below which they are cut by lines
 constexpr double kNearCtasPerSm = 6.0;      // resident near-core CTAs per SM (estimate for the split)
 constexpr int kMinNearPieceLines = 64;      // lines of a near-core backward piece at least
 
@@ -228,11 +228,8 @@ static pz_status build_items(pz_ctx *c) {
     const int nt = (int)((c->nlam + T - 1) / T);
     const int DC = c->tiling.depth_per_cta();
     const int ngf = (c->nd + DC - 1) / DC;
-    // near-core forward items: fewer layers each where a short grid has too few of them
-    int ndf = kNearDepthsFwd;
-    while (ndf > 1 && (double)c->S * nt * ((c->nd + ndf - 1) / ndf) < kNearFwdItemsPerSm * std::max(c->n_sm, 1)) ndf /= 2;
-    c->near_depths = ndf;
-    const int nnf = (c->nd + ndf - 1) / ndf, nnb = (c->nd + kNearDepthsBwd - 1) / kNearDepthsBwd;
+    constexpr int ndl = kNearDepths;
+    const int nnf = (c->nd + ndl - 1) / ndl;
     struct Item {
         int4 v;
         double cost;
@@ -273,11 +270,11 @@ static pz_status build_items(pz_ctx *c) {
             const int nhi = (int)(std::upper_bound(b0, b1, (int32_t)std::ceil(nb_)) - c->h_il.begin());
             for (int g = 0; g < nnf; ++g)
                 nf.push_back({make_int4(st, t * nnf + g, nlo, nhi),
-                              (double)(nhi - nlo) * std::min(ndf, c->nd - g * ndf)});
+                              (double)(nhi - nlo) * std::min(ndl, c->nd - g * ndl)});
             if (nhi > nlo)
-                for (int g = 0; g < nnb; ++g)
-                    nb.push_back({make_int4(st, t * nnb + g, nlo, nhi),
-                                  (double)(nhi - nlo) * std::min(kNearDepthsBwd, c->nd - g * kNearDepthsBwd)});
+                for (int g = 0; g < nnf; ++g)
+                    nb.push_back({make_int4(st, t * nnf + g, nlo, nhi),
+                                  (double)(nhi - nlo) * std::min(ndl, c->nd - g * ndl)});
         }
     }
     auto order = [](std::vector<Item> &v) {
@@ -345,7 +342,20 @@ static pz_status build_items(pz_ctx *c) {
             if (hi > lo) nbp.push_back({make_int4(it.v.x, it.v.y, lo, hi), it.cost / P});
         }
     }
-    std::vector<int4> hn = order(nf), hb = order(nbp);
+    // near-core forward pieces on short grids only (their sums meet in knear by atomics); the cut
+    // depends on the grid and the star's lines alone, so a star's sums do not change with its batch
+    std::vector<Item> nfp;
+    const int PF = std::min(8, (int)std::ceil(kNearItemsPerSm * std::max(c->n_sm, 1) / ((double)nt * nnf)));
+    c->near_split = false;
+    for (const Item &it : nf) {
+        const int n = it.v.w - it.v.z;
+        const int P = std::max(1, std::min({PF, kMaxPieces, n / kMinNearPieceLines}));
+        c->near_split = c->near_split || P > 1;
+        for (int q = 0; q < P; ++q)
+            nfp.push_back({make_int4(it.v.x, it.v.y, it.v.z + (int)((int64_t)n * q / P),
+                                     it.v.z + (int)((int64_t)n * (q + 1) / P)), it.cost / P});
+    }
+    std::vector<int4> hn = order(nfp), hb = order(nbp);
     dfree(c->d_fitems);
     dfree(c->d_fext);
     dfree(c->d_bitems);
@@ -390,20 +400,25 @@ static pz_status build_thresholds(pz_ctx *c) {
     const int nslab = ((c->nd + DC - 1) / DC) * c->tiling.GW;
     double shrink = 1.0 - 0.5 * (c->W + 1024.0) * c->lnr;
     if (shrink < 0.5) shrink = 0.5;
-    std::vector<float> thr((size_t)c->S * c->ns * nslab, 0.0f);
+    std::vector<float> thr((size_t)c->S * c->ns * nslab, 0.0f), cut(thr);
     for (int st = 0; st < c->S; ++st)
         for (int s = 0; s < c->ns; ++s)
             for (int b = 0; b < nslab; ++b) {
                 double mn = 1e300;
                 for (int d = b * DS; d < std::min(c->nd, (b + 1) * DS); ++d)
                     mn = std::min(mn, (double)c->h_invdv[((size_t)st * c->ns + s) * c->nd + d]);
-                if (mn < 1e300)
+                if (mn < 1e300) {
                     thr[((size_t)st * c->ns + s) * nslab + b] =
                         (float)(20.0 / (kC * mn * c->lnr * shrink) * (1.0 + 1e-4) + 1e-3);
+                    // U = 2^36 u^2 at x = u k = 6, k = c/dv_D of the widest layer
+                    cut[((size_t)st * c->ns + s) * nslab + b] = (float)(36.0 * (double)kKScale / (kC * mn * kC * mn));
+                }
             }
     dfree(c->d_thr);
-    c->d_thr = nullptr;
+    dfree(c->d_cut);
+    c->d_thr = c->d_cut = nullptr;
     PZ_TRY(upload(&c->d_thr, thr, "thresholds"));
+    PZ_TRY(upload(&c->d_cut, cut, "thresholds"));
     c->nslab = nslab;
     // box expansions: nearest offset n_c of class c at each (star, slab): the points of boxes n_c
     // apart lie beyond 2^c times the widest species' threshold; kBoxNever if no whole box or
@@ -453,7 +468,7 @@ static void destroy_ctx(pz_ctx *c) {
     drop_graph(c);
     void *ptrs[] = {c->d_m, c->d_T, c->d_beta_hi, c->d_beta_lo, c->d_ne, c->d_npert, c->d_c2T, c->d_ne64,
                     c->d_npert64, c->d_rho64, c->d_R, c->d_Rbase, c->d_invdv, c->d_Ksd, c->d_pop64, c->d_mass64, c->d_xi64,
-                    c->d_thr, c->d_kc, c->d_B, c->d_stim, c->d_dab, c->d_mdgf, c->d_mdg6, c->d_eos, c->L.orig, c->L.star, c->L.ilf,
+                    c->d_thr, c->d_cut, c->d_kc, c->d_B, c->d_stim, c->d_dab, c->d_mdgf, c->d_mdg6, c->d_eos, c->L.orig, c->L.star, c->L.ilf,
                     c->L.il32, c->L.frac, c->L.sp, c->L.E, c->L.lamcm, c->L.grad, c->L.g4, c->L.g6base, c->L.g6,
                     c->L.Q, c->L.Qbase, c->L.x64, c->L.lg_gf, c->L.lg_rad, c->L.lg_4, c->L.lg_6, c->L.dgf, c->L.dg6,
                     c->d_line_off, c->d_fitems, c->d_fext, c->d_bitems, c->d_bext, c->d_fpart, c->d_fcnt, c->d_nitems_f,

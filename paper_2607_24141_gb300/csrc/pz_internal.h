@@ -27,8 +27,7 @@ constexpr double kC2 = kH * kC / kKB;       // second radiation constant, cm K
 
 // Largest supported depth count (register/local arrays in the flux kernels).
 constexpr int kMaxDepth = 128;
-constexpr int kNearDepthsFwd = 8;    // layers per work item of the near-core forward at most
-constexpr int kNearDepthsBwd = 6;    // layers per work item of the near-core backward
+constexpr int kNearDepths = 8;       // layers per work item of the near-core kernels
 // Largest number of instrument taps per pixel.
 constexpr int kMaxTaps = 4096;
 // Device ordinals a context may live on (per-device launch-attribute bookkeeping).
@@ -166,6 +165,7 @@ struct pz_ctx {
     double *d_mass64 = nullptr;     // [S][ns]
     double *d_xi64 = nullptr;       // [S]
     float *d_thr = nullptr;         // [S][ns][nslab] fast-path distance threshold (grid units)
+    float *d_cut = nullptr;         // [S][ns][nslab] 36 K of the slab's widest layer (scaled u^2 of x^2 = 36)
     int nslab = 0;                  // depth slabs of DS layers covered by the launch grid
     double *d_kc = nullptr;         // [S][nd][ld] continuum opacity FP64
     double *d_B = nullptr;          // [S][nd][ld] Planck function B_lambda(T_d) per nm, FP64
@@ -195,7 +195,7 @@ struct pz_ctx {
     int4 *d_bext = nullptr;         // per backward piece: (0, pieces, 0, piece)
     int4 *d_nitems_f = nullptr;     // near-core forward
     int4 *d_nitems_b = nullptr;     // near-core backward
-    int near_depths = pz::kNearDepthsFwd;   // layers per near-core forward item
+    bool near_split = false;        // near-core forward items are cut by lines (sums added to knear)
     int n_fitems = 0, n_bitems = 0, n_nitems_f = 0, n_nitems_b = 0;
     float4 *d_fpart = nullptr;      // compensated partial sums of the split forward items
     size_t fpart_cap = 0;           // bytes allocated at d_fpart

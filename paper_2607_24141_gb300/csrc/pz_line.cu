@@ -142,6 +142,7 @@ struct LineArgs {
     const float *ilf, *frac, *E, *lamcm, *grad, *g4, *g6, *Q;
     const int32_t *sp;
     const float *R, *invdv, *thr;                   // [ns][nd], [ns][nd], [ns][nslab] of the star
+    const float *cut;                               // [ns][nslab] 36 K of the slab's widest layer
     const float *Ksd;                               // [ns][nd] K = 2^36/k^2 of the star
     int nslab;
     const float *beta_hi, *beta_lo, *ne, *npert, *c2T;   // [nd] of the star
@@ -186,6 +187,7 @@ __device__ __forceinline__ LineArgs star_view(const LineArgs &g, int s) {
     v.invdv += s * g.sstride;
     v.Ksd += s * g.sstride;
     v.thr += s * g.tstride;
+    v.cut += s * g.tstride;
     v.beta_hi += s * g.dstride;
     v.beta_lo += s * g.dstride;
     v.ne += s * g.dstride;
@@ -429,13 +431,13 @@ constexpr float kFast2V = 5.0f;      // distance threshold factor: |v| >= 5 x 20
 // sqrt(pi)/(A a6) = sum_n C1 gamma_n(a^2) (K s)^(n+1), reaches the nearer cells: with a^2 <= 1.5 the
 // dropped terms stay below 2.6e-8 (H) and 4.6e-8 (dH/da) relative with N = 3 at |v| >= 30, below
 // 3e-9 with N = 4 at |v| >= 20 and below 6.3e-8 (dH/da: 1.2e-7 of its scale 1/v^2) with N = 8 at |v| >= 6.
-// Eight multiply-adds per cell and no per-cell branch: the mid wing 6 <= |v| < 20, which the
+// Eight multiply-adds per cell and no per-cell branch (one cut in U serves all layers of a slab, so the
+// points of the core have s = 0): the mid wing 6 <= |v| < 20, which the
 // near-core kernels summed cell by cell at about 140 instructions each, and the masked far cells
 // beside it (two reciprocals and a polynomial in t per depth pair) are one sweep of the tile.
 // Measured on 2e5 lines x 37,550 points: far + near-core forward 6.9 -> 4.3 ms, reverse 9.9 ->
 // 6.8 ms.
 constexpr float kCoreV = 0.3f;       // distance threshold factor: |v| >= 0.3 x 20 = 6
-constexpr float kCoreX2 = 36.0f;     // cells with x^2 < 36 (U < 36 K) of the series' lines belong to the near-core kernels
 constexpr float kFast3V = 1.5f;      // distance threshold factor: |v| >= 1.5 x 20
 constexpr float kFast2A2 = 1.5f;     // a^2 bound
 
@@ -767,8 +769,8 @@ enum FarForm {
     kFormTwo,           // every cell |v| >= 100: two terms
     kFormThree,         // |v| >= 30: three
     kFormFour,          // |v| >= 20: four
-    kFormEight,         // |v| >= 6: eight
-    kFormCore,          // eight, the cells with x^2 < 36 left to the near-core kernels
+    kFormEight,         // eight, the points with U < cut (x^2 < 36 at the slab's widest layer) left to the
+                        // near-core kernels at every layer of the slab
     kFormLarge,         // a^2 > kFast2A2 somewhere in the slab, |v| >= 20, the window covers the tile: polynomial in t
     kFormLargeMask,     // a^2 > kFast2A2: the cells with |z| >= 20 inside the window, the others left to the
                         // near-core kernels
@@ -788,8 +790,7 @@ __device__ __forceinline__ int far_form(const LineArgs &g, const LineInfo &info,
     const int f = dmin >= kFast2V * thr ? kFormTwo
                   : dmin >= kFast3V * thr ? kFormThree
                   : dmin >= thr ? kFormFour
-                  : dmin >= kCoreV * thr ? kFormEight
-                                         : kFormCore;
+                                : kFormEight;
     return f | (full ? kFormFull : 0);
 }
 
@@ -871,34 +872,24 @@ __device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo 
     for (int j = 0; j < J; ++j) sq[j] = f2_mul(sp[j], sp[j]);
 }
 
-// Reciprocals s_j = 1/U_j at the thread's points for the series forms, zero outside the window
-// and for lanes left to the box expansions.  CORE: U is held above the smallest K of the slab
-// (x^2 >= 1), so that the cells left to the near-core kernels stay finite before they are dropped.
-template <int J, int DP, int NQ, bool CORE>
+// Reciprocals s_j = 1/U_j at the thread's points for the series forms: zero outside the window,
+// below cut (the points left to the near-core kernels) and for lanes left to the box expansions.
+template <int J>
 __device__ __forceinline__ void far_series_s(const LineArgs &g, const LineInfo &info, bool full, bool near, float lamf,
-                                             int lam_thr, const ulonglong2 *par, float (&U)[J], float (&s)[J]) {
+                                             int lam_thr, float cut, f2_t (&sp)[J]) {
+    float U[J];
     far_scaled_u2<J>(g, info, lamf, U);
-    float Umin = 3.0e38f;
-    if (CORE) {
-#pragma unroll
-        for (int dp = 0; dp < DP; ++dp) {
-            const float ka = f2_lo(par[NQ * dp].x), kb = f2_hi(par[NQ * dp].x);
-            if (ka > 0.0f) Umin = fminf(Umin, ka);     // (layers past the last one hold 0)
-            if (kb > 0.0f) Umin = fminf(Umin, kb);
-        }
-    }
     const int di0 = lam_thr - (int)info.ilf;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const bool in = near && (full || (di0 + j >= -g.W && di0 + j <= g.W));
-        s[j] = in ? rcp_approx(CORE ? fmaxf(U[j], Umin) : U[j]) : 0.0f;
+        const bool in = near && U[j] >= cut && (full || (di0 + j >= -g.W && di0 + j <= g.W));
+        sp[j] = f2_splat(in ? rcp_approx(U[j]) : 0.0f);
     }
 }
 
 // acc += sum_n c_n s^(n+1) over the line's cells (N terms).
-template <int J, int DP, int N, bool CORE>
-__device__ __forceinline__ void far_fwd_series(const ulonglong2 *par, const float (&U)[J], const float (&s)[J],
-                                               f2_t (&acc)[DP][J]) {
+template <int J, int DP, int N>
+__device__ __forceinline__ void far_fwd_series(const ulonglong2 *par, const f2_t (&sp)[J], f2_t (&acc)[DP][J]) {
 #pragma unroll
     for (int dp = 0; dp < DP; ++dp) {
         const ulonglong2 *q = par + kNQF * dp;
@@ -909,51 +900,36 @@ __device__ __forceinline__ void far_fwd_series(const ulonglong2 *par, const floa
             c[n] = v.x;
             c[n + 1] = v.y;
         }
-        const float ca = CORE ? kCoreX2 * f2_lo(q[0].x) : 0.0f, cb = CORE ? kCoreX2 * f2_hi(q[0].x) : 0.0f;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const f2_t sp = f2_splat(s[j]);
             f2_t h = c[N - 1];
 #pragma unroll
-            for (int n = N - 2; n >= 0; --n) h = f2_fma(sp, h, c[n]);
-            const f2_t sm = CORE ? f2_pack(U[j] >= ca ? s[j] : 0.0f, U[j] >= cb ? s[j] : 0.0f) : sp;
-            acc[dp][j] = f2_fma(sm, h, acc[dp][j]);
+            for (int n = N - 2; n >= 0; --n) h = f2_fma(sp[j], h, c[n]);
+            acc[dp][j] = f2_fma(sp[j], h, acc[dp][j]);
         }
     }
 }
 
 // S1 += sum_n c_n X_n, S2 += sum_n e_n X_n with X_n = sum_j G s_j^(n+1) per depth pair: one
 // multiply-add per cell and term serves both gradients.
-template <int J, int DP, int N, bool CORE>
-__device__ __forceinline__ void far_bwd_series(const ulonglong2 *par, const float (&U)[J], const float (&s)[J],
-                                               const f2_t (&gv)[DP][J], f2_t &S1, f2_t &S2) {
+template <int J, int DP, int N>
+__device__ __forceinline__ void far_bwd_series(const ulonglong2 *par, const f2_t (&sp)[J], const f2_t (&gv)[DP][J],
+                                               f2_t &S1, f2_t &S2) {
     constexpr int G = DP < 3 ? DP : 3;        // depth pairs taken together (registers)
 #pragma unroll
     for (int d0 = 0; d0 < DP; d0 += G) {
         f2_t X[G][N];
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const f2_t sp = f2_splat(s[j]);
-            f2_t gm[G];
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-                if (d0 + i >= DP) break;
-                gm[i] = gv[d0 + i][j];
-                if (CORE) {
-                    const f2_t K = par[kNQB * (d0 + i)].x;
-                    gm[i] = f2_pack(U[j] >= kCoreX2 * f2_lo(K) ? f2_lo(gm[i]) : 0.0f,
-                                    U[j] >= kCoreX2 * f2_hi(K) ? f2_hi(gm[i]) : 0.0f);
-                }
-            }
-            f2_t pw = sp;
+            f2_t pw = sp[j];
 #pragma unroll
             for (int n = 0; n < N; ++n) {
 #pragma unroll
                 for (int i = 0; i < G; ++i) {
                     if (d0 + i >= DP) break;
-                    X[i][n] = j == 0 ? f2_mul(gm[i], pw) : f2_fma(gm[i], pw, X[i][n]);
+                    X[i][n] = j == 0 ? f2_mul(gv[d0 + i][j], pw) : f2_fma(gv[d0 + i][j], pw, X[i][n]);
                 }
-                if (n + 1 < N) pw = f2_mul(pw, sp);
+                if (n + 1 < N) pw = f2_mul(pw, sp[j]);
             }
         }
 #pragma unroll
@@ -1050,22 +1026,18 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
             const LineInfo info = s_line[li];
             const ulonglong2 *par = s_par + (size_t)li * DP * NQ;
             const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-            if ((fl & 7) <= kFormCore) {
-                float U[J], sv[J];
-                if ((fl & 7) == kFormCore) {
-                    far_series_s<J, DP, NQ, true>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
-                    far_fwd_series<J, DP, 8, true>(par, U, sv, acc);
-                } else {
-                    far_series_s<J, DP, NQ, false>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
-                    if ((fl & 7) == kFormEight)
-                        far_fwd_series<J, DP, 8, false>(par, U, sv, acc);
-                    else if ((fl & 7) == kFormFour)
-                        far_fwd_series<J, DP, 4, false>(par, U, sv, acc);
-                    else if ((fl & 7) == kFormThree)
-                        far_fwd_series<J, DP, 3, false>(par, U, sv, acc);
-                    else
-                        far_fwd_series<J, DP, 2, false>(par, U, sv, acc);
-                }
+            if ((fl & 7) <= kFormEight) {
+                f2_t sp[J];
+                far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
+                                (fl & 7) == kFormEight ? __ldg(g.cut + info.sp * g.nslab + slab) : 0.0f, sp);
+                if ((fl & 7) == kFormEight)
+                    far_fwd_series<J, DP, 8>(par, sp, acc);
+                else if ((fl & 7) == kFormFour)
+                    far_fwd_series<J, DP, 4>(par, sp, acc);
+                else if ((fl & 7) == kFormThree)
+                    far_fwd_series<J, DP, 3>(par, sp, acc);
+                else
+                    far_fwd_series<J, DP, 2>(par, sp, acc);
             } else if ((fl & 7) == kFormLarge) {
                 float U[J];
                 far_scaled_u2<J>(g, info, lamf, U);
@@ -1436,22 +1408,18 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
                 // (a slab whose every layer the centre test rejects keeps zero sums)
                 if ((fl & 7) != kFormSkip) {
                     const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-                    if ((fl & 7) <= kFormCore) {
-                        float U[J], sv[J];
-                        if ((fl & 7) == kFormCore) {
-                            far_series_s<J, DP, NQ, true>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
-                            far_bwd_series<J, DP, 8, true>(par, U, sv, gv, S1, S2);
-                        } else {
-                            far_series_s<J, DP, NQ, false>(g, info, fl & kFormFull, near, lamf, lam_thr, par, U, sv);
-                            if ((fl & 7) == kFormEight)
-                                far_bwd_series<J, DP, 8, false>(par, U, sv, gv, S1, S2);
-                            else if ((fl & 7) == kFormFour)
-                                far_bwd_series<J, DP, 4, false>(par, U, sv, gv, S1, S2);
-                            else if ((fl & 7) == kFormThree)
-                                far_bwd_series<J, DP, 3, false>(par, U, sv, gv, S1, S2);
-                            else
-                                far_bwd_series<J, DP, 2, false>(par, U, sv, gv, S1, S2);
-                        }
+                    if ((fl & 7) <= kFormEight) {
+                        f2_t sp[J];
+                        far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
+                                        (fl & 7) == kFormEight ? __ldg(g.cut + info.sp * g.nslab + slab) : 0.0f, sp);
+                        if ((fl & 7) == kFormEight)
+                            far_bwd_series<J, DP, 8>(par, sp, gv, S1, S2);
+                        else if ((fl & 7) == kFormFour)
+                            far_bwd_series<J, DP, 4>(par, sp, gv, S1, S2);
+                        else if ((fl & 7) == kFormThree)
+                            far_bwd_series<J, DP, 3>(par, sp, gv, S1, S2);
+                        else
+                            far_bwd_series<J, DP, 2>(par, sp, gv, S1, S2);
                     } else if ((fl & 7) == kFormLarge) {
                         float U[J];
                         far_scaled_u2<J>(g, info, lamf, U);
@@ -1555,338 +1523,223 @@ __global__ void __launch_bounds__(128, MINB) k_line_bwd(LineArgs g, int GW, int 
 
 // ---------------------------------------------------------------------------
 // Near-core kernels: the cells that the far-wing kernels leave.  At a slab whose damping the
-// series forms take (a^2 <= kFast2A2 at every layer) those are the core, x^2 = (u k)^2 < 36,
-// decided by U < 36 K with the far kernels' own U; otherwise the mid wing and core,
-// |v|^2 + a^2 < 400, classified with the same prefactors, offset and test as the masked far form.
-// Every cell is counted exactly once across the two kernels.  A CTA owns the same wavelength
-// tile as the far kernels; its warps take (line, depth) items of the lines whose near zone can
-// reach the tile, clip the item's near span analytically, and let the lanes sweep the span 32
-// points at a time.
+// series forms take (a^2 <= kFast2A2 at every layer) those are the points with U < cut (the core
+// x^2 < 36 of the slab's widest layer) by the far kernels' own U; otherwise the mid wing and
+// core, |v|^2 + a^2 < 400, classified with the same prefactors, offset and test as the masked far
+// form.  Every cell is counted exactly once across the two kernels.
+//
+// A CTA takes a (tile, group of ND layers) and a range of lines; its warps take the lines that
+// reach the tile in turn.  In a warp, lane = (layer, point): ND layers of 32 / ND neighbouring points, so a line's
+// prefactors are formed once per layer in the lanes that use them, its core (25 to 60 points,
+// nearly the same at neighbouring layers) is swept 32 / ND points at a step with all lanes busy,
+// and every lane owns its cell: the forward adds into the warp's own [point][layer] sums in
+// shared memory without atomics, the reverse pass sums in registers and reduces once per line.
+// (Before, lanes swept the concatenated cells of 32 (line, layer) items: finding a cell's item,
+// fetching its 48 bytes, the shared-memory float atomics and the segmented scan of the reverse pass
+// cost more than the profile, about 250 instructions per core cell.)
+// Measured on 2e5 lines x 37,550 points: forward 2.11 -> 1.63 ms, reverse 3.50 -> 1.89 ms (5,300
+// lines x 1,500 points, forward items cut by lines: 0.090 -> 0.086, reverse 0.146 -> 0.086 ms).
 // ---------------------------------------------------------------------------
 
-// x^2 < 36 as the far kernels decide it: U = 2^36 u^2 of point i from its lane's first point
-// (far_scaled_u2), against 36 K.
+// U = 2^36 u^2 of point i as the far kernels form it, from their lane's first point (far_scaled_u2).
 template <int J>
-__device__ __forceinline__ bool core_owned(const LineArgs &g, float ilf, float frac, int i, float cut) {
+__device__ __forceinline__ float far_u2(const LineArgs &g, float ilf, float frac, int i) {
     const int j = i & (J - 1);
     const float u0 = offset_u((ilf - (float)(i - j)) + frac, g.lnr) * kUScale;
     const float rj = j == 1 ? g.rj[1] : j == 2 ? g.rj[2] : g.rj[3], rm = j == 1 ? g.rm1j[1] : j == 2 ? g.rm1j[2] : g.rm1j[3];
     const float u = j == 0 ? u0 : fmaf(u0, rj, rm * kUScale);
-    return u * u < cut;
+    return u * u;
 }
 
-// Near span of an item clipped to the tile and the window; returns false if empty.
-__device__ __forceinline__ bool near_span(const LineArgs &g, float ilf, float frac, float k, float r2, int t0, int T,
-                                          int &lo, int &hi) {
-    if (!(k > 0.0f) || !(r2 > 0.0f)) return false;
-    const float xl = ilf + frac;
-    const int il = (int)ilf;
-    const float span = sqrtf(r2) / (k * g.lnr) * 1.01f + 1.0f;
-    lo = max(max(t0, (int)floorf(xl - span)), il - g.W);
-    hi = min(min(t0 + T - 1, (int)ceilf(xl + span)), il + g.W);
-    return lo <= hi;
-}
-
-// One near-core item (a line at one depth) after its lane-parallel set-up.  Its near
-// span [lo, hi] (clipped to the tile and the window) is split analytically into the
-// core segment (|z|^2 < 36, cells [c0, r0)) and the mid-wing cells on either side
-// (nl cells from lo, then the cells from r0 to hi).
-struct alignas(16) NearItem {
-    float ilf, frac, k, a2;      // centre, Doppler factor c/dv_D, a^2 (or -36 K: core cells only)
-    float a, A, Aa6;             // damping, strength, strength x vdW damping
-    int lo, nl, c0, r0;          // span start, mid cells left of the core, core segment [c0, r0)
-    int dlb;                     // local depth | (local line index << 8)
+constexpr int kNearWarps = 8;        // warps per near-core CTA
+constexpr int kNearBatch = 512;      // lines looked at together
+struct NearList {
+    int cnt[kNearBatch / 32];        // lines of each 32 whose near zone reaches the tile
+    int line[kNearBatch];            // their places in the 32 | slabs (of the group) with only the core left << 8
 };
 
-constexpr int kNearBatch = 512;      // lines per shared-memory batch of the backward sums
-constexpr int kNearWarps = 8;        // warps per near-core CTA
-
-// Dense pass over the concatenated cells of one segment kind of the warp's 32 items:
-// cell n of the concatenation belongs to item src with pref[src] <= n < pref[src + 1]
-// (each lane advances its own cursor; consecutive lanes hold consecutive cells, so
-// the items of one iteration form ordered runs).
-//   forward:  cell(item, i, H, dH) adds the cell's term where it belongs;
-//   backward: val(item, i, H, dH) returns the cell's (G A H, G A a6 dH) pair and
-//             done(item, sum) receives the per-run sums of each item.
-template <int T, bool D, bool CORE, class Cell, class Val, class Done>
-__device__ __forceinline__ void near_pass(const LineArgs &g, const NearItem *mine, const int *pref, const float *s_daw,
-                                          Cell &cell, Val &val, Done &done) {
-    const int lane = threadIdx.x & 31;
-    const int total = pref[32];
-    int src = 0;
-    for (int n0 = 0; n0 < total; n0 += 32) {
-        const int n = n0 + lane;
-        int run = -1;
-        float2 v = make_float2(0.0f, 0.0f);
-        if (n < total) {
-            while (pref[src + 1] <= n) ++src;
-            const NearItem &it = mine[src];
-            const int off = n - pref[src];
-            const int i = CORE ? it.c0 + off : (off < it.nl ? it.lo + off : it.r0 + (off - it.nl));
-            const float x = fabsf(offset_u((it.ilf - (float)i) + it.frac, g.lnr) * it.k);
-            run = src;
-            // a mid-wing cell at |z| >= 20 belongs to the far-wing kernels (same test); a core cell
-            // of the series' lines is theirs by U, which only the cells at the boundary need
-            const float x2 = x * x;
-            if (CORE ? (it.a2 >= 0.0f || x2 < 0.999f * kCoreX2 ||
-                        (x2 < 1.001f * kCoreX2 && core_owned<T / 32>(g, it.ilf, it.frac, i, -it.a2)))
-                     : fmaf(x, x, it.a2) < kFar2) {
-                float H, dH;
-                if (CORE)
-                    voigt_core<D>(x, it.a, H, dH, s_daw);
-                else
-                    voigt_mid<D>(x, it.a, H, dH);
-                if (D)
-                    v = val(it, i, H, dH);
-                else
-                    cell(it, i, H, dH);
+// Sweep of the near cells of lines [nlo, nhi) in the tile at the lane's layer: cell(i, A, H, dH)
+// takes each cell that the lane owns, end(l, A, A a6) closes a line (all lanes together).
+template <int T, int ND, bool D, class Cell, class End>
+__device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, int nhi, int dbase, NearList &list,
+                                           const float *s_daw, Cell &&cell, End &&end) {
+    constexpr int NP = 32 / ND;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = dbase + lane % ND, po = lane / ND;
+    const float t0f = (float)t0, tendf = (float)(t0 + T - 1);
+    const int sl0 = dbase / g.tDS, sl1 = (min(dbase + ND, g.nd) - 1) / g.tDS;   // slabs of the group's layers
+    const int dc = min(d, g.nd - 1), slab = dc / g.tDS;
+    for (int b0 = nlo; b0 < nhi; b0 += kNearBatch) {
+        const int nch = (min(kNearBatch, nhi - b0) + 31) / 32;
+        __syncthreads();
+        for (int ch = warp; ch < nch; ch += kNearWarps) {
+            // lane = line: does its near zone reach the tile at any slab of the group
+            const int l = min(b0 + ch * 32 + lane, nhi - 1), sp = g.sp[l];
+            const float il = g.ilf[l], fr = g.frac[l];
+            const float dmin = fmaxf(0.0f, fmaxf(t0f - il - fr, il - tendf + fr));
+            bool need = false;
+            int core = 0;
+            for (int sl = sl0; sl <= sl1; ++sl) {
+                const int gs = sl * g.tDS / g.tDC, ws = sl - gs * (g.tDC / g.tDS);
+                const int m = g.finfo[(int64_t)gs * g.nl + l].amask;
+                const bool series = (m >> ws) & 1;
+                core |= series ? 256 << (sl - sl0) : 0;
+                need = need || (dmin < (series ? kCoreV : 1.0f) * __ldg(g.thr + sp * g.nslab + sl) && !((m >> (8 + ws)) & 1));
             }
+            need = need && b0 + ch * 32 + lane < nhi;
+            const unsigned m = __ballot_sync(0xffffffffu, need);
+            if (need) list.line[ch * 32 + __popc(m & ((1u << lane) - 1u))] = lane | core;
+            if (lane == 0) list.cnt[ch] = __popc(m);
         }
-        if (D) {
-            // segmented sum over the runs of equal items
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float nx = __shfl_up_sync(0xffffffffu, v.x, o);
-                const float ny = __shfl_up_sync(0xffffffffu, v.y, o);
-                const int ns = __shfl_up_sync(0xffffffffu, run, o);
-                if (lane >= o && ns == run) {
-                    v.x += nx;
-                    v.y += ny;
+        __syncthreads();
+        // the warps take the listed lines NP at a time (fewer where the list is short) in turn: lane
+        // (q, layer) forms line q's prefactors and span at its layer, then the lanes sweep the lines
+        // one after the other
+        int total = 0;
+        for (int k = 0; k < nch; ++k) total += list.cnt[k];
+        const int per = max(1, min(NP, (total + kNearWarps - 1) / kNearWarps));
+        int ch = 0, r = warp * per;         // (r counts on from list ch)
+        for (;;) {
+            while (ch < nch && r >= list.cnt[ch]) r -= list.cnt[ch++];
+            if (ch >= nch) break;
+            int mch = ch, mr = r + po;      // this lane's line
+            while (mch < nch && mr >= list.cnt[mch]) mr -= list.cnt[mch++];
+            const bool have = mch < nch && po < per;
+            const int e = have ? list.line[mch * 32 + mr] : 0;
+            const int l = have ? b0 + mch * 32 + (e & 31) : nlo;
+            r += kNearWarps * per;
+            const LineScalars L = load_line(g, l);
+            const float ilf = g.ilf[l], frac = g.frac[l];
+            const bool series = (e >> (8 + slab - sl0)) & 1;
+            float p[16];
+            depth_params<D ? 16 : 8>(g, L, d, p);       // (zero strength and k past the last layer)
+            // the points that may be near [lo, hi], and (series slabs) those that certainly are; |u| <= reach
+            // there, and u = expm1(Delta ln r) differs from Delta ln r by less than 0.6 reach of it
+            const float cut = __ldg(g.cut + L.sp * g.nslab + slab);
+            const float r2 = kFar2 - p[1];
+            const float reach = series ? sqrtf(cut) * (1.0f / kUScale) : sqrtf(fmaxf(r2, 0.0f)) / p[0];
+            int lo = 1 << 30, hi = -(1 << 30), ilo = 0, in = -1;
+            if (have && p[0] > 0.0f && (series || r2 > 0.0f) && pair_kept(g.keep, l, d)) {
+                const float span = reach / g.lnr, m = fmaf(fmaf(0.6f, reach, 1e-3f), span, 0.01f);
+                const int ic = (int)ilf;
+                lo = max(max(t0, ic + (int)ceilf(frac - span - m)), ic - g.W);
+                hi = min(min(t0 + T - 1, ic + (int)floorf(frac + span + m)), ic + g.W);
+                if (series) {
+                    ilo = max(lo, ic + (int)ceilf(frac - span + m));
+                    in = min(hi, ic + (int)floorf(frac + span - m)) - ilo;
                 }
             }
-            const int next = __shfl_down_sync(0xffffffffu, run, 1);
-            if (run >= 0 && (lane == 31 || next != run)) done(mine[run], v);
-        }
-    }
-}
-
-// Backward pass over the mid wing with a blocked assignment: lane l takes the
-// concatenated cells [l P, (l + 1) P), P = ceil(total / 32), so that each lane's cells
-// belong to a few consecutive items; the lane sums an item's cells in registers and
-// hands the sum to done when it moves to the next item (no cross-lane reduction).
-// voigt_mid has no branch on the item's parameters, so lanes of different items do not diverge.
-template <class Val, class Done>
-__device__ __forceinline__ void near_pass_blocked(const LineArgs &g, const NearItem *mine, const int *pref, Val &val,
-                                                  Done &done) {
-    const int lane = threadIdx.x & 31;
-    const int total = pref[32];
-    const int per = (total + 31) >> 5;
-    const int nb = min(lane * per, total), ne = min(nb + per, total);
-    if (nb >= ne) return;
-    int src = 0;
-    while (pref[src + 1] <= nb) ++src;
-    NearItem it = mine[src];
-    int start = pref[src], end = pref[src + 1];
-    float2 acc = make_float2(0.0f, 0.0f);
-    for (int n = nb; n < ne; ++n) {
-        if (n >= end) {
-            done(it, acc);
-            acc = make_float2(0.0f, 0.0f);
-            do {
-                ++src;
-            } while (pref[src + 1] <= n);
-            it = mine[src];
-            start = pref[src];
-            end = pref[src + 1];
-        }
-        const int off = n - start;
-        const int i = off < it.nl ? it.lo + off : it.r0 + (off - it.nl);
-        const float x = fabsf(offset_u((it.ilf - (float)i) + it.frac, g.lnr) * it.k);
-        // a mid-wing cell at |z| >= 20 belongs to the far-wing kernels (same test)
-        if (fmaf(x, x, it.a2) < kFar2) {
-            float H, dH;
-            voigt_mid<true>(x, it.a, H, dH);
-            const float2 v = val(it, i, H, dH);
-            acc.x += v.x;
-            acc.y += v.y;
-        }
-    }
-    done(it, acc);
-}
-
-// Near-core sweep shared by the forward (D = false) and the backward (D = true).
-// Each warp takes rounds of 32 (line, depth) items: every lane sets up one item
-// (coarse span from c/dv_D alone, then the exact prefactors, the clipped span and
-// its core / mid split), a warp scan turns the per-item cell counts into offsets,
-// and the warp then sweeps all mid-wing cells of the round and all core cells of
-// the round, 32 consecutive cells at a time, so the two Voigt forms never diverge
-// within a warp and no lane idles while cells remain.
-template <int T, bool D, class Cell, class Val, class Done>
-__device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int64_t nlo, int64_t nitems, int ndg, int dbase,
-                                           NearItem *s_items, int *s_pref, const float *s_daw, Cell &&cell,
-                                           Val &&val, Done &&done) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    NearItem *mine = s_items + warp * 32;
-    int *pm = s_pref + warp * 66, *pc = pm + 33;      // prefix counts of mid and core cells
-    for (int64_t r0 = (int64_t)warp * 32; r0 < nitems; r0 += (int64_t)nwarp * 32) {
-        const int64_t it = r0 + lane;
-        int nmid = 0, ncore = 0;
-        NearItem item;
-        if (it < nitems) {
-            const int64_t l = nlo + it / ndg;
-            const int dl = (int)(it % ndg), d = dbase + dl;
-            item.ilf = g.ilf[l];
-            item.frac = g.frac[l];
-            item.dlb = dl | ((int)(it / ndg) << 8);
-            const float k = (float)kC * __ldg(g.invdv + g.sp[l] * g.nd + d);
-            const int grp = d / g.tDC;
-            // the far-wing kernels' series take everything but the core of this slab's lines
-            const bool core = (g.finfo[(int64_t)grp * g.nl + l].amask >> ((d - grp * g.tDC) / g.tDS)) & 1;
-            int lo, hi;
-            if (pair_kept(g.keep, l, d) &&
-                near_span(g, item.ilf, item.frac, k, core ? kCoreX2 : kFar2, t0, T, lo, hi)) {
-                float p[16];
-                line_params<D ? 16 : 8>(g, l, d, p);
-                if (core) {
-                    item.k = p[0];
-                    item.a2 = -kCoreX2 * __ldg(g.Ksd + g.sp[l] * g.nd + d);
-                    item.A = p[7];
-                    item.a = D ? p[15] : sqrtf(p[1]);
-                    item.Aa6 = D ? p[14] : 0.0f;
-                    ncore = hi - lo + 1;
-                    item.c0 = lo;
-                } else if (near_span(g, item.ilf, item.frac, p[0], kFar2 - p[1], t0, T, lo, hi)) {
-                    item.k = p[0];
-                    item.a2 = p[1];
-                    item.A = p[7];
-                    item.a = D ? p[15] : sqrtf(p[1]);
-                    item.Aa6 = D ? p[14] : 0.0f;
-                    // core segment: |x| < sqrt(36 - a^2), x = u k, |u| ~ |x_l - i| ln r
-                    int c0 = hi + 1, c1 = hi;
-                    if (p[1] < kMid2) {
-                        const float w = sqrtf(kMid2 - p[1]) / (p[0] * g.lnr);
-                        const float xl = item.ilf + item.frac;
-                        c0 = max(lo, (int)ceilf(xl - w));
-                        c1 = min(hi, (int)floorf(xl + w));
-                        if (c0 > c1) {
-                            c0 = hi + 1;
-                            c1 = hi;
-                        }
+            const float ma = D ? p[15] : sqrtf(p[1]), mcut = series ? cut : -1.0f;
+            for (int q = 0; q < per; ++q) {
+                const int src = q * ND + lane % ND;
+                if (!__shfl_sync(0xffffffffu, (int)have, q * ND)) break;
+                const int lq = __shfl_sync(0xffffffffu, l, q * ND);
+                const float qil = __shfl_sync(0xffffffffu, ilf, q * ND), qfr = __shfl_sync(0xffffffffu, frac, q * ND);
+                const float k = __shfl_sync(0xffffffffu, p[0], src), a = __shfl_sync(0xffffffffu, ma, src);
+                const float a2 = __shfl_sync(0xffffffffu, p[1], src), A = __shfl_sync(0xffffffffu, p[7], src);
+                const float Aa6 = D ? __shfl_sync(0xffffffffu, p[14], src) : 0.0f;
+                const float qcut = __shfl_sync(0xffffffffu, mcut, src);
+                const int qlo = __shfl_sync(0xffffffffu, lo, src), qhi = __shfl_sync(0xffffffffu, hi, src);
+                const int qilo = __shfl_sync(0xffffffffu, ilo, src), qin = __shfl_sync(0xffffffffu, in, src);
+                const int i0 = __reduce_min_sync(0xffffffffu, qlo), i1 = __reduce_max_sync(0xffffffffu, qhi);
+                for (int i = i0 + po; i <= i1; i += NP) {
+                    bool own = qin >= 0 && (unsigned)(i - qilo) <= (unsigned)qin;
+                    const float x = fabsf(offset_u((qil - (float)i) + qfr, g.lnr) * k);
+                    const float z2 = fmaf(x, x, a2);
+                    if (!own && i >= qlo && i <= qhi)
+                        own = qcut >= 0.0f ? far_u2<T / 32>(g, qil, qfr, i) < qcut : z2 < kFar2;
+                    if (own) {
+                        float H, dH;
+                        if (z2 < kMid2)
+                            voigt_core<D>(x, a, H, dH, s_daw);
+                        else
+                            voigt_mid<D>(x, a, H, dH);
+                        cell(i, A, H, dH);
                     }
-                    ncore = c1 - c0 + 1;
-                    nmid = (hi - lo + 1) - ncore;
-                    item.lo = lo;
-                    item.nl = ncore > 0 ? c0 - lo : nmid;
-                    item.c0 = c0;
-                    item.r0 = ncore > 0 ? c1 + 1 : hi + 1;
                 }
+                end(lq, A, Aa6);
             }
-        }
-        // exclusive prefix of the packed counts (mid << 16 | core; a round holds < 2^16 cells)
-        const int own = (nmid << 16) | ncore;
-        int inc = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        __syncwarp();
-        const int exc = inc - own;
-        pm[lane] = exc >> 16;
-        pc[lane] = exc & 0xffff;
-        if (lane == 31) {
-            pm[32] = inc >> 16;
-            pc[32] = inc & 0xffff;
-        }
-        if (own != 0) mine[lane] = item;
-        __syncwarp();
-        if (D) {
-            // mid wing blocked; the core keeps interleaved cells (its damping branches would
-            // diverge across the items of a blocked warp: measured 238 -> 339 ms per batch step)
-            near_pass_blocked(g, mine, pm, val, done);
-            __syncwarp();
-            near_pass<T, D, true>(g, mine, pc, s_daw, cell, val, done);
-        } else {
-            near_pass<T, D, false>(g, mine, pm, s_daw, cell, val, done);
-            __syncwarp();
-            near_pass<T, D, true>(g, mine, pc, s_daw, cell, val, done);
         }
     }
 }
 
-// Forward near-core sums into knear.  Work items: (star, tile, depth group of NDG layers).
-template <int T>
-__global__ void __launch_bounds__(32 * kNearWarps) k_line_near_fwd(LineArgs gq, int NDG) {
+// Forward near-core sums into knear.  Work items: (star, tile, group of ND layers).
+template <int T, int ND>
+__global__ void __launch_bounds__(32 * kNearWarps) k_line_near_fwd(LineArgs gq, bool split) {
     extern __shared__ float4 smem4[];
-    float *s_acc = reinterpret_cast<float *>(smem4);                               // [NDG][T]
-    NearItem *s_items = reinterpret_cast<NearItem *>(s_acc + NDG * T);             // [warps][32]
-    int *s_pref = reinterpret_cast<int *>(s_items + kNearWarps * 32);              // [warps][2][33]
-    float *s_daw = reinterpret_cast<float *>(s_pref + kNearWarps * 66);            // Dawson table
+    float *s_acc = reinterpret_cast<float *>(smem4);                  // [warps][T][ND]
+    float *s_daw = s_acc + kNearWarps * T * ND;                       // Dawson table
+    __shared__ NearList list;
     for (int k = threadIdx.x; k < kDawsonNodes * (kDawsonK + 1); k += blockDim.x) s_daw[k] = g_dawson[k];
     for_each_item(gq, [&](const LineArgs &g, int tile, int group, int nlo, int nhi, int) {
-    const int tid = threadIdx.x;
-    const int t0 = tile * T;
-    const int dbase = group * NDG, ndg = min(NDG, g.nd - dbase);
-    for (int k = tid; k < NDG * T; k += blockDim.x) s_acc[k] = 0.0f;
-    __syncthreads();
-    near_sweep<T, false>(
-        g, t0, nlo, (int64_t)(nhi - nlo) * ndg, ndg, dbase, s_items, s_pref, s_daw,
-        [&](const NearItem &it, int i, float H, float) {
-            atomicAdd(s_acc + (it.dlb & 0xff) * T + (i - t0), it.A * H);
-        },
-        [&](const NearItem &, int, float, float) { return make_float2(0.0f, 0.0f); },
-        [&](const NearItem &, float2) {});
-    __syncthreads();
-    for (int k = tid; k < ndg * T; k += blockDim.x) {
-        const int dl = k / T, q = k - dl * T;
-        g.knear[(int64_t)(dbase + dl) * g.ld + t0 + q] = s_acc[k];
-    }
+        const int t0 = tile * T, dbase = group * ND, ndg = min(ND, g.nd - dbase);
+        for (int k = threadIdx.x; k < kNearWarps * T * ND; k += blockDim.x) s_acc[k] = 0.0f;
+        __syncthreads();
+        float *mine = s_acc + (threadIdx.x >> 5) * T * ND + (threadIdx.x & 31) % ND;
+        near_sweep<T, ND, false>(
+            g, t0, nlo, nhi, dbase, list, s_daw,
+            [&](int i, float A, float H, float) { mine[(i - t0) * ND] += A * H; }, [&](int, float, float) {});
+        __syncthreads();
+        for (int k = threadIdx.x; k < ndg * T; k += blockDim.x) {
+            const int dl = k / T, q = k - dl * T;
+            float v = 0.0f;
+#pragma unroll
+            for (int w = 0; w < kNearWarps; ++w) v += s_acc[(w * T + q) * ND + dl];
+            float *out = g.knear + (int64_t)(dbase + dl) * g.ld + t0 + q;
+            if (split)
+                atomicAdd(out, v);     // one of the pieces of this item's lines (knear starts at zero)
+            else
+                *out = v;
+        }
+        __syncthreads();
     });
 }
 
-// Backward: per-line sums over the near cells of G stim A H and G stim A a6 dH/da.
-// Lines are processed in batches whose per-line sums live in shared memory; one
-// global atomic per (line, tile, depth group) at the end of each batch.
-template <int T, int NDG>
-__global__ void __launch_bounds__(32 * kNearWarps, 5) k_line_near_bwd(LineArgs gq) {
+// Backward: per-line sums over the near cells of G stim A H and G stim A a6 dH/da, one FP64 add
+// per (line, tile, layer group) and sum.
+template <int T, int ND>
+__global__ void __launch_bounds__(32 * kNearWarps) k_line_near_bwd(LineArgs gq) {
     extern __shared__ float4 smem4[];
-    float *s_g = reinterpret_cast<float *>(smem4);                                 // [NDG][T] G * stim
-    float2 *s_sum = reinterpret_cast<float2 *>(s_g + NDG * T);                     // [kNearBatch]
-    NearItem *s_items = reinterpret_cast<NearItem *>(s_sum + kNearBatch);          // [warps][32]
-    int *s_pref = reinterpret_cast<int *>(s_items + kNearWarps * 32);              // [warps][2][33]
-    float *s_daw = reinterpret_cast<float *>(s_pref + kNearWarps * 66);            // Dawson table
+    float *s_g = reinterpret_cast<float *>(smem4);                    // [T][ND] G * stim
+    float *s_daw = s_g + T * ND;                                      // Dawson table
+    __shared__ NearList list;
     for (int k = threadIdx.x; k < kDawsonNodes * (kDawsonK + 1); k += blockDim.x) s_daw[k] = g_dawson[k];
     for_each_item(gq, [&](const LineArgs &g, int tile, int group, int nlo, int nhi, int) {
-    const int tid = threadIdx.x;
-    const int t0 = tile * T;
-    const int dbase = group * NDG, ndg = min(NDG, g.nd - dbase);
-    for (int k = tid; k < ndg * T; k += blockDim.x) {
-        const int dl = k / T, q = k - dl * T;
-        s_g[k] = (t0 + q < g.nlam) ? g.Gt[(int64_t)(dbase + dl) * g.ld + t0 + q] : 0.0f;
-    }
-    for (int b0 = nlo; b0 < nhi; b0 += kNearBatch) {
-        const int nb = min(kNearBatch, nhi - b0);
+        const int t0 = tile * T, dbase = group * ND;
+        for (int k = threadIdx.x; k < ND * T; k += blockDim.x) {
+            const int dl = k / T, q = k - dl * T;
+            s_g[q * ND + dl] = (dbase + dl < g.nd && t0 + q < g.nlam) ? g.Gt[(int64_t)(dbase + dl) * g.ld + t0 + q] : 0.0f;
+        }
         __syncthreads();
-        for (int k = tid; k < nb; k += blockDim.x) s_sum[k] = make_float2(0.0f, 0.0f);
-        __syncthreads();
-        near_sweep<T, true>(
-            g, t0, b0, (int64_t)nb * ndg, ndg, dbase, s_items, s_pref, s_daw,
-            [&](const NearItem &, int, float, float) {},
-            [&](const NearItem &it, int i, float H, float dH) {
-                const float gs = s_g[(it.dlb & 0xff) * T + (i - t0)];
-                return make_float2(gs * it.A * H, gs * it.Aa6 * dH);
+        const float *mine = s_g + (threadIdx.x & 31) % ND;
+        float S1 = 0.0f, S2 = 0.0f;
+        near_sweep<T, ND, true>(
+            g, t0, nlo, nhi, dbase, list, s_daw,
+            [&](int i, float, float H, float dH) {
+                const float gs = mine[(i - t0) * ND];
+                S1 = fmaf(gs, H, S1);
+                S2 = fmaf(gs, dH, S2);
             },
-            [&](const NearItem &it, float2 v) {
-                const int lb = it.dlb >> 8;
-                atomicAdd(&s_sum[lb].x, v.x);
-                atomicAdd(&s_sum[lb].y, v.y);
+            [&](int l, float A, float Aa6) {
+                float v1 = S1 * A, v2 = S2 * Aa6;
+                S1 = S2 = 0.0f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+                    v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+                }
+                if ((threadIdx.x & 31) == 0) {
+                    if (v1 != 0.0f) atomicAdd(g.gacc + l, (double)v1);
+                    if (v2 != 0.0f) atomicAdd(g.gacc + g.nl + l, (double)v2);
+                }
             });
         __syncthreads();
-        for (int k = tid; k < nb; k += blockDim.x) {
-            const float2 v = s_sum[k];
-            if (v.x != 0.0f) atomicAdd(g.gacc + b0 + k, (double)v.x);
-            if (v.y != 0.0f) atomicAdd(g.gacc + g.nl + b0 + k, (double)v.y);
-        }
-    }
-    __syncthreads();
     });
 }
 
-template <int T, bool BWD>
-constexpr size_t near_smem(int ndg) {
-    return (size_t)ndg * T * sizeof(float) + (BWD ? kNearBatch * sizeof(float2) : 0) +
-           (size_t)kNearWarps * 32 * sizeof(NearItem) + (size_t)kNearWarps * 66 * sizeof(int) +
-           (size_t)kDawsonNodes * (kDawsonK + 1) * sizeof(float);
+template <int T, int ND, bool BWD>
+constexpr size_t near_smem() {
+    return ((size_t)(BWD ? 1 : kNearWarps) * ND * T + (size_t)kDawsonNodes * (kDawsonK + 1)) * sizeof(float);
 }
 
 static LineArgs make_args(pz_ctx *c) {
@@ -1922,6 +1775,7 @@ static LineArgs make_args(pz_ctx *c) {
     g.invdv = c->d_invdv;
     g.Ksd = c->d_Ksd;
     g.thr = c->d_thr;
+    g.cut = c->d_cut;
     g.nslab = c->nslab;
     g.beta_hi = c->d_beta_hi;
     g.beta_lo = c->d_beta_lo;
@@ -1969,42 +1823,30 @@ static int persistent_grid(pz_ctx *c, K kernel, int threads, size_t smem, int n_
 
 template <int T, bool BWD>
 static cudaError_t launch_near(pz_ctx *c, LineArgs g, cudaStream_t s) {
-    if (BWD) {
-        if (c->n_nitems_b == 0) return cudaSuccess;
-        g.items = c->d_nitems_b;
-        g.n_items = c->n_nitems_b;
-        g.ngroups = (c->nd + kNearDepthsBwd - 1) / kNearDepthsBwd;
-        g.ctr = c->d_ctr + 3;
-        constexpr size_t smem = near_smem<T, true>(kNearDepthsBwd);
-        static std::atomic<bool> attr_set[kMaxDevices];
-        if (!attr_set[c->device].load(std::memory_order_acquire)) {
-            cudaFuncSetAttribute(k_line_near_bwd<T, kNearDepthsBwd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-            attr_set[c->device].store(true, std::memory_order_release);
-        }
-        int grid = persistent_grid(c, k_line_near_bwd<T, kNearDepthsBwd>, 32 * kNearWarps, smem, g.n_items);
-        cudaEvent_t ev = prof_begin(c, s);
-        k_line_near_bwd<T, kNearDepthsBwd><<<grid, 32 * kNearWarps, smem, s>>>(g);
-        prof_end(c, s, PZ_K_NEAR_BWD, ev);
-    } else {
-        if (c->n_nitems_f == 0) return cudaSuccess;
-        g.items = c->d_nitems_f;
-        g.n_items = c->n_nitems_f;
-        const int ndg = c->near_depths;
-        g.ngroups = (c->nd + ndg - 1) / ndg;
-        g.ctr = c->d_ctr + 0;
-        const size_t smem = near_smem<T, false>(ndg);
-        static std::atomic<bool> attr_set[kMaxDevices];
-        if (!attr_set[c->device].load(std::memory_order_acquire)) {
-            cudaFuncSetAttribute(k_line_near_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)near_smem<T, false>(kNearDepthsFwd));
-            attr_set[c->device].store(true, std::memory_order_release);
-        }
-        int grid = persistent_grid(c, k_line_near_fwd<T>, 32 * kNearWarps, smem, g.n_items);
-        cudaEvent_t ev = prof_begin(c, s);
-        k_line_near_fwd<T><<<grid, 32 * kNearWarps, smem, s>>>(g, ndg);
-        prof_end(c, s, PZ_K_NEAR_FWD, ev);
+    constexpr int ND = kNearDepths;
+    g.items = BWD ? c->d_nitems_b : c->d_nitems_f;
+    g.n_items = BWD ? c->n_nitems_b : c->n_nitems_f;
+    if (g.n_items == 0) return cudaSuccess;
+    g.ngroups = (c->nd + ND - 1) / ND;
+    g.ctr = c->d_ctr + (BWD ? 3 : 0);
+    constexpr size_t smem = near_smem<T, ND, BWD>();
+    static std::atomic<bool> attr_set[kMaxDevices];
+    const void *fn = BWD ? (const void *)k_line_near_bwd<T, ND> : (const void *)k_line_near_fwd<T, ND>;
+    if (!attr_set[c->device].load(std::memory_order_acquire)) {
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        attr_set[c->device].store(true, std::memory_order_release);
     }
+    const int grid = persistent_grid(c, fn, 32 * kNearWarps, smem, g.n_items);
+    if (!BWD && c->near_split) {
+        const cudaError_t e = cudaMemsetAsync(c->d_knear, 0, sizeof(float) * (size_t)c->S * c->nd * c->ld, s);
+        if (e != cudaSuccess) return e;
+    }
+    cudaEvent_t ev = prof_begin(c, s);
+    if (BWD)
+        k_line_near_bwd<T, ND><<<grid, 32 * kNearWarps, smem, s>>>(g);
+    else
+        k_line_near_fwd<T, ND><<<grid, 32 * kNearWarps, smem, s>>>(g, c->near_split);
+    prof_end(c, s, BWD ? PZ_K_NEAR_BWD : PZ_K_NEAR_FWD, ev);
     c->launches++;
     return cudaGetLastError();
 }
