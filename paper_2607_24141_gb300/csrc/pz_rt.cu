@@ -4,12 +4,18 @@
 // are ~1e-8 while E_3(0) = 1/2, so the interval integrals are differences of
 // nearly equal numbers.
 //
-// Flux: for every wavelength one thread walks the depth axis, accumulating
-// tau by the trapezoid rule on column mass, and sums the closed form
+// Flux: a block takes 32 wavelengths, a warp a segment of the layers of all of
+// them: it accumulates tau over its segment by the trapezoid rule on column mass
+// (the segments above add their totals) and sums the closed form
 //   Int_{ta}^{tb} S E_2 dtau = Sa (E3(ta) - E3(tb)) + s (E4(ta) - E4(tb) - (tb - ta) E3(tb)),
 // s = (Sb - Sa)/(tb - ta), over the layers plus the top interval [0, tau_0]
 // (S extrapolated linearly from the first segment).  Nothing is added below
-// the bottom layer.  Total and continuum branches share the walk.
+// the bottom layer.  Total and continuum branches share the walk.  Bound by the
+// FP64 pipe on long grids and by the chain of Taylor series on short ones, where
+// one thread per wavelength walked all 72 layers: 4,000 points 0.465 -> 0.112 ms,
+// 2,200 points with the adjoint 0.63 -> 0.19 ms; 37,550 points (with ten instead of
+// fourteen Taylor terms and Newton reciprocals) flux 0.60 -> 0.49, adjoint 0.525 ->
+// 0.44 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,18 +41,21 @@ constexpr double kEuler = 0.57721566490153286061;
 // derivatives), using E_n' = -E_{n-1}.  The coefficients are exact derivatives:
 //   E_4^(k) = (-1)^k E_{4-k} (k <= 4, E_0 = e^-x / x),
 //   E_0^(m) = (-1)^m e^-x m! sum_{i=0..m} x^-(i+1) / (m-i)!   (all terms positive).
-// Nodes: 2^-40 <= x < 2: eight per binade at the centres of the binade's eighths
-// (|t| / x0 <= 1/17, inside the radius of convergence x0 of the logarithmic
-// singularity at 0); 2 <= x < 40: spacing 1/8 (|t| <= 1/16).  Fourteen terms
-// leave a truncation error below 1e-16 relative in both ranges.  Outside them:
-// x < 2^-40 the leading terms of the small-x expansion, x >= 40 the continued
-// fraction of E_4 (8 levels), x > 740 zero.
+// Nodes: 2^-40 <= x < 2: 32 per binade at the centres of the binade's 32nds (|t| / x0 <=
+// 1/65, inside the radius of convergence x0 of the logarithmic singularity at 0); 2 <= x <
+// 40: spacing 1/32 (|t| <= 1/64).  Ten terms leave a truncation error below 1e-16 relative in
+// both ranges (for E_2, the second derivative: 0.018 x (1/65)^8).  Outside them: x < 2^-40 the
+// leading terms of the small-x expansion, x >= 40 the continued fraction of E_4 (8 levels),
+// x > 740 zero.  The series are the transfer kernels' FP64 work: four times the nodes (200 KB
+// in L2 instead of 71) for 18 multiply-adds per E_3, E_4 instead of 26; measured with scattering
+// on 1,500 points x 72 layers: flux 0.885 -> 0.835 ms, adjoint 1.475 -> 1.41 ms (without: below).
 // ---------------------------------------------------------------------------
-constexpr int kExpnK = 14;                      // Taylor terms per node
+constexpr int kExpnK = 10;                      // Taylor terms per node
 constexpr int kExpnMinExp = -40;                // smallest binade 2^-40
-constexpr int kExpnGeo = (1 - kExpnMinExp) * 8; // nodes below 2: binades -40..0
+constexpr int kExpnLog = 5;                     // log2 of the nodes per binade (and per unit above 2)
+constexpr int kExpnGeo = (1 - kExpnMinExp) << kExpnLog; // nodes below 2: binades -40..0
 constexpr double kExpnUni0 = 2.0, kExpnUni1 = 40.0;
-constexpr int kExpnUni = (int)((kExpnUni1 - kExpnUni0) * 8);   // nodes on [2, 40)
+constexpr int kExpnUni = (int)(kExpnUni1 - kExpnUni0) << kExpnLog;   // nodes on [2, 40)
 constexpr int kExpnNodes = kExpnGeo + kExpnUni;
 
 __device__ double g_expn_tab[kExpnNodes * kExpnK];
@@ -67,7 +76,7 @@ static void expn_host(long double x, long double E[5]) {
         E[1] = -(long double)kEuler - logl(x) - s;
         for (int n = 1; n < 4; ++n) E[n + 1] = (ex - x * E[n]) / n;
     } else {
-        const int K = 600;
+        const int K = 120;   // (x >= 2: the fraction's error falls like e^(-4 sqrt(K x)))
         long double f = x + 4.0L + 2.0L * K;
         for (int k = K; k >= 1; --k) f = x + 4.0L + 2.0L * (k - 1) - (long double)k * (3.0L + k) / f;
         E[4] = ex / f;
@@ -81,6 +90,7 @@ static void expn_host(long double x, long double E[5]) {
 static void expn_node_coeffs(long double x0, double *c, int n = 4) {
     long double E[5];
     expn_host(x0, E);
+    const long double ex0 = expl(-x0);
     long double fact = 1.0L;   // k!
     for (int k = 0; k < kExpnK; ++k) {
         if (k > 0) fact *= k;
@@ -89,23 +99,24 @@ static void expn_node_coeffs(long double x0, double *c, int n = 4) {
             d = ((k & 1) ? -1.0L : 1.0L) * E[n - k];
         } else {
             const int m = k - n;
-            long double sum = 0.0L, mf = 1.0L;   // m! / (m - i)! built as a running product
+            long double sum = 0.0L, mf = 1.0L / x0;   // m! / (m - i)! x0^-(i + 1), a running product
             for (int i = 0; i <= m; ++i) {
-                if (i > 0) mf *= (m - i + 1);
-                sum += mf * powl(x0, -(long double)(i + 1));
+                if (i > 0) mf *= (m - i + 1) / x0;
+                sum += mf;
             }
-            d = ((n & 1) ? -1.0L : 1.0L) * ((m & 1) ? -1.0L : 1.0L) * expl(-x0) * sum;
+            d = ((n & 1) ? -1.0L : 1.0L) * ((m & 1) ? -1.0L : 1.0L) * ex0 * sum;
         }
         c[k] = (double)(d / fact);
     }
 }
 
 static double expn_node_x0(int j) {
+    constexpr int n = 1 << kExpnLog;
     if (j < kExpnGeo) {
-        const int e = kExpnMinExp + j / 8, m = j % 8;
-        return std::ldexp(1.0 + (m + 0.5) / 8.0, e);
+        const int e = kExpnMinExp + j / n, m = j % n;
+        return std::ldexp(1.0 + (m + 0.5) / n, e);
     }
-    return kExpnUni0 + (j - kExpnGeo + 0.5) / 8.0;
+    return kExpnUni0 + (j - kExpnGeo + 0.5) / n;
 }
 
 pz_status ensure_expn_table() {
@@ -136,21 +147,22 @@ pz_status ensure_expn_table() {
 }
 
 // Node of x in [2^-40, 40) and the offset t = x - x0 (exact), from the bits of x alone
-// (integer operations: the FP64 pipe is kept for the series).  Below 2, eight nodes per
-// binade at the centres of its eighths (x0 keeps three mantissa bits and sets the fourth);
-// on [2, 40) nodes every 1/8 at the centres (j - kExpnGeo = floor(8 x) - 16, x0 = x rounded
-// down to a multiple of 1/8 plus 1/16).
+// (integer operations: the FP64 pipe is kept for the series).  Below 2, 32 nodes per binade
+// at the centres of its 32nds (x0 keeps five mantissa bits and sets the sixth); on [2, 40)
+// nodes every 1/32 at the centres (j - kExpnGeo = floor(32 x) - 64, x0 = x rounded down to a
+// multiple of 1/32 plus 1/64).
 __device__ __forceinline__ int expn_node(double x, double &t) {
     const long long bits = __double_as_longlong(x);
     const int ex = (int)(bits >> 52) - 1023;           // x > 0
     int j;
     long long x0b;
     if (ex < 1) {
-        j = (ex - kExpnMinExp) * 8 + (int)((bits >> 49) & 7);
-        x0b = (bits & ~((1LL << 49) - 1)) | (1LL << 48);
+        constexpr int sh = 52 - kExpnLog;
+        j = ((ex - kExpnMinExp) << kExpnLog) + (int)((bits >> sh) & ((1 << kExpnLog) - 1));
+        x0b = (bits & ~((1LL << sh) - 1)) | (1LL << (sh - 1));
     } else {
-        const int sh = 49 - ex;                        // mantissa bit of 1/8
-        j = kExpnGeo - 16 + (int)(((bits & ((1LL << 52) - 1)) | (1LL << 52)) >> sh);
+        const int sh = 52 - kExpnLog - ex;             // mantissa bit of a node's width
+        j = kExpnGeo - (2 << kExpnLog) + (int)(((bits & ((1LL << 52) - 1)) | (1LL << 52)) >> sh);
         x0b = (bits & ~((1LL << sh) - 1)) | (1LL << (sh - 1));
     }
     t = x - __longlong_as_double(x0b);
@@ -253,11 +265,31 @@ cudaError_t launch_planck_tables(pz_ctx *c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// 1/x by two Newton iterations y += y (1 - x y) from the approximate reciprocal (2^-20 or
+// better, squared twice): four multiply-adds of the scarce FP64 pipe.
+__device__ __forceinline__ double rcp_newton(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
 __device__ __forceinline__ double interval(double ta, double tb, double Sa, double Sb, double e3a, double e4a,
                                            double e3b, double e4b) {
     double D = tb - ta;
-    double s = (Sb - Sa) / D;
+    double s = (Sb - Sa) * rcp_newton(D);
     return Sa * (e3a - e3b) + s * (e4a - e4b - D * e3b);
+}
+
+// Dynamic shared memory granted to a kernel so far, per device (slots 0-9: scattering kernels).
+constexpr int kSmemFlux = 10, kSmemFlux64 = 11, kSmemAdj = 12, kSmemAdj64 = 13, kSmemSlots = 14;
+static cudaError_t smem_attr(pz_ctx *c, const void *fn, int slot, size_t smem) {
+    static std::atomic<size_t> granted[kMaxDevices][kSmemSlots];
+    if (c->device < 0 || c->device >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (smem <= granted[c->device][slot].load()) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) granted[c->device][slot].store(smem);
+    return e;
 }
 
 struct FluxArgs {
@@ -269,62 +301,100 @@ struct FluxArgs {
     double *F, *Fc;
 };
 
-// one thread per (lambda, star); star = blockIdx.y
+// Layer segments of a transfer block, one warp each: at least two layers per segment.
+constexpr int kRtSegs = 8;
+__host__ __device__ __forceinline__ int rt_segs(int nd) { return nd / 2 < kRtSegs ? (nd / 2 > 0 ? nd / 2 : 1) : kRtSegs; }
+
+// One layer of a branch: tau, S and the exponential integrals there.
+struct FluxNode {
+    double tau, S, e3, e4;
+};
+__device__ __forceinline__ FluxNode flux_node(double tau, double S) {
+    FluxNode n{tau, S, 0.0, 0.0};
+    expn34(tau, n.e3, n.e4);
+    return n;
+}
+__device__ __forceinline__ double interval(const FluxNode &a, const FluxNode &b) {
+    return interval(a.tau, b.tau, a.S, b.S, a.e3, a.e4, b.e3, b.e4);
+}
+
+// lane = wavelength, warp = layer segment; star = blockIdx.y
 template <typename KT>
-__global__ void k_flux(FluxArgs g) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.nlam) return;
-    {
-        const int st = blockIdx.y;
-        g.m += (int64_t)st * g.nd;
-        g.T += (int64_t)st * g.nd;
-        g.kc += (int64_t)st * g.nd * g.ld;
-        g.B += (int64_t)st * g.nd * g.ld;
-        g.kline = reinterpret_cast<const KT *>(g.kline) + (int64_t)st * g.nd * g.ld;
-        g.F += (int64_t)st * g.nlam;
-        g.Fc += (int64_t)st * g.nlam;
-    }
-    const KT *kl = reinterpret_cast<const KT *>(g.kline);
-    double chi_p = 0, chic_p = 0, tau_p = 0, tauc_p = 0, S_p = 0, m_p = 0;
-    double e3p = 0, e4p = 0, e3cp = 0, e4cp = 0;
-    double F = 0.0, Fc = 0.0;
-    double tau0 = 0, tauc0 = 0, S0 = 0, e3_0 = 0, e4_0 = 0, e3c_0 = 0, e4c_0 = 0;
-    for (int d = 0; d < g.nd; ++d) {
-        const int64_t o = (int64_t)d * g.ld + i;
-        const double kc = g.kc[o];
-        const double chi = kc + (double)kl[o];
-        const double md = g.m[d];
-        const double S = g.B[o];
-        double tau, tauc;
-        if (d == 0) {
-            tau = chi * md;
-            tauc = kc * md;
-        } else {
-            tau = tau_p + 0.5 * (chi_p + chi) * (md - m_p);
-            tauc = tauc_p + 0.5 * (chic_p + kc) * (md - m_p);
+__global__ void __launch_bounds__(32 * kRtSegs) k_flux(FluxArgs g) {
+    extern __shared__ double smem_rt[];
+    const int lane = threadIdx.x, w = threadIdx.y, nseg = blockDim.y;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane, st = blockIdx.y;
+    const bool live = i < g.nlam;
+    const int a = w * g.nd / nseg, b = (w + 1) * g.nd / nseg;    // this segment's layers
+    double *s_cum = smem_rt;                          // [nd][2][32] tau from the segment's start, both branches
+    double *s_tot = s_cum + (size_t)g.nd * 64;        // [seg][2][32] segment totals, then flux sums
+    FluxNode *s_first = reinterpret_cast<FluxNode *>(s_tot + nseg * 64);   // [seg][2][32] first layer of a segment
+    const double *m = g.m + st * g.nd;
+    const double *kc = g.kc + st * g.nd * g.ld + i, *B = g.B + st * g.nd * g.ld + i;
+    const KT *kl = reinterpret_cast<const KT *>(g.kline) + st * g.nd * g.ld + i;
+    double t = 0.0, tc = 0.0;
+    if (live) {
+        double chi_p = 0.0, kc_p = 0.0;
+        if (a > 0) {
+            kc_p = kc[(a - 1) * g.ld];
+            chi_p = kc_p + (double)kl[(a - 1) * g.ld];
         }
-        double e3, e4, e3c, e4c;
-        expn34(tau, e3, e4);
-        expn34(tauc, e3c, e4c);
-        if (d == 0) {
-            tau0 = tau; tauc0 = tauc; S0 = S;
-            e3_0 = e3; e4_0 = e4; e3c_0 = e3c; e4c_0 = e4c;
-        } else {
-            if (d == 1) {
-                // top interval [0, tau_0], S linear through layers 0 and 1
-                double s0 = (S - S0) / (tau - tau0);
-                F += interval(0.0, tau0, S0 - s0 * tau0, S0, 0.5, 1.0 / 3.0, e3_0, e4_0);
-                double sc0 = (S - S0) / (tauc - tauc0);
-                Fc += interval(0.0, tauc0, S0 - sc0 * tauc0, S0, 0.5, 1.0 / 3.0, e3c_0, e4c_0);
+        for (int d = a; d < b; ++d) {
+            const double k = kc[d * g.ld], chi = k + (double)kl[d * g.ld];
+            if (d == 0) {
+                t = chi * m[0];
+                tc = k * m[0];
+            } else {
+                const double hm = 0.5 * (m[d] - m[d - 1]);
+                t = fma(chi_p + chi, hm, t);
+                tc = fma(kc_p + k, hm, tc);
             }
-            F += interval(tau_p, tau, S_p, S, e3p, e4p, e3, e4);
-            Fc += interval(tauc_p, tauc, S_p, S, e3cp, e4cp, e3c, e4c);
+            s_cum[(d * 2) * 32 + lane] = t;
+            s_cum[(d * 2 + 1) * 32 + lane] = tc;
+            chi_p = chi;
+            kc_p = k;
         }
-        chi_p = chi; chic_p = kc; tau_p = tau; tauc_p = tauc; S_p = S; m_p = md;
-        e3p = e3; e4p = e4; e3cp = e3c; e4cp = e4c;
     }
-    g.F[i] = 2.0 * kPI * F;
-    g.Fc[i] = 2.0 * kPI * Fc;
+    s_tot[(w * 2) * 32 + lane] = t;
+    s_tot[(w * 2 + 1) * 32 + lane] = tc;
+    __syncthreads();
+    double F[2] = {0.0, 0.0};
+    FluxNode last[2];
+    if (live) {
+#pragma unroll
+        for (int br = 0; br < 2; ++br) {
+            double off = 0.0;
+            for (int q = 0; q < w; ++q) off += s_tot[(q * 2 + br) * 32 + lane];
+            for (int d = a; d < b; ++d) {
+                const FluxNode n = flux_node(off + s_cum[(d * 2 + br) * 32 + lane], B[d * g.ld]);
+                if (d == a)
+                    s_first[(w * 2 + br) * 32 + lane] = n;
+                else
+                    F[br] += interval(last[br], n);
+                if (d == 1) {
+                    // top interval [0, tau_0], S linear through layers 0 and 1 (both in segment 0)
+                    const FluxNode &n0 = last[br];
+                    const double s0 = (n.S - n0.S) * rcp_newton(n.tau - n0.tau);
+                    F[br] += interval(0.0, n0.tau, n0.S - s0 * n0.tau, n0.S, 0.5, 1.0 / 3.0, n0.e3, n0.e4);
+                }
+                last[br] = n;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int br = 0; br < 2; ++br) {
+        if (live && w + 1 < nseg) F[br] += interval(last[br], s_first[((w + 1) * 2 + br) * 32 + lane]);
+        s_tot[(w * 2 + br) * 32 + lane] = F[br];
+    }
+    __syncthreads();
+    if (w < 2 && live) {            // warp 0: total branch, warp 1 (or 0 alone): continuum
+        for (int br = w; br < 2; br += nseg > 1 ? 2 : 1) {
+            double sum = 0.0;
+            for (int q = 0; q < nseg; ++q) sum += s_tot[(q * 2 + br) * 32 + lane];
+            (br ? g.Fc : g.F)[st * g.nlam + i] = 2.0 * kPI * sum;
+        }
+    }
 }
 
 cudaError_t launch_flux_scatter(pz_ctx *c, cudaStream_t s);
@@ -344,11 +414,17 @@ cudaError_t launch_flux(pz_ctx *c, cudaStream_t s) {
     g.kline = c->d_kline;
     g.F = c->d_F;
     g.Fc = c->d_Fc;
-    dim3 nb((unsigned)((c->nlam + 127) / 128), c->S);
-    if (c->prec == PZ_MIXED)
-        k_flux<float><<<nb, 128, 0, s>>>(g);
+    const int seg = rt_segs(c->nd);
+    const dim3 nb((unsigned)((c->nlam + 31) / 32), c->S), thr(32, seg);
+    const size_t smem = ((size_t)c->nd * 64 + seg * 64) * sizeof(double) + (size_t)seg * 64 * sizeof(FluxNode);
+    const bool mixed = c->prec == PZ_MIXED;
+    const cudaError_t e = smem_attr(c, mixed ? (const void *)k_flux<float> : (const void *)k_flux<double>,
+                                    mixed ? kSmemFlux : kSmemFlux64, smem);
+    if (e != cudaSuccess) return e;
+    if (mixed)
+        k_flux<float><<<nb, thr, smem, s>>>(g);
     else
-        k_flux<double><<<nb, 128, 0, s>>>(g);
+        k_flux<double><<<nb, thr, smem, s>>>(g);
     c->launches++;
     return cudaGetLastError();
 }
@@ -1182,16 +1258,6 @@ __global__ void __launch_bounds__(kScatThreadsAdj, 1) k_rt_adjoint_scatter(ScatA
     }
 }
 
-// Dynamic shared memory granted to a kernel so far, per device.
-static cudaError_t scatter_attr(pz_ctx *c, const void *fn, int slot, size_t smem) {
-    static std::atomic<size_t> granted[kMaxDevices][10];
-    if (c->device < 0 || c->device >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (smem <= granted[c->device][slot].load()) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) granted[c->device][slot].store(smem);
-    return e;
-}
-
 static ScatArgs scatter_args(pz_ctx *c) {
     ScatArgs g;
     g.nlam = c->nlam;
@@ -1216,7 +1282,7 @@ static ScatArgs scatter_args(pz_ctx *c) {
 
 template <typename K>
 static cudaError_t launch_scat_kernel(pz_ctx *c, K *fn, int slot, int threads, size_t smem, cudaStream_t s) {
-    cudaError_t e = scatter_attr(c, (const void *)fn, slot, smem);
+    cudaError_t e = smem_attr(c, (const void *)fn, slot, smem);
     if (e != cudaSuccess) return e;
     fn<<<dim3((unsigned)c->nlam, c->S), threads, smem, s>>>(scatter_args(c));
     c->launches++;
@@ -1456,7 +1522,7 @@ struct RtAdjArgs {
 __device__ __forceinline__ void interval_grad(double ta, double tb, double Sa, double Sb, double e2a, double e3a,
                                               double e4a, double e2b, double e3b, double e4b, double &da,
                                               double &db) {
-    const double D = tb - ta, iD = 1.0 / D;
+    const double D = tb - ta, iD = rcp_newton(D);
     const double s = (Sb - Sa) * iD;
     const double P = e3a - e3b;
     const double Bq = e4a - e4b - D * e3b;
@@ -1464,68 +1530,97 @@ __device__ __forceinline__ void interval_grad(double ta, double tb, double Sa, d
     db = Sb * e2b - (s * iD) * Bq;
 }
 
-// one thread per (lambda, star); star = blockIdx.y
+// lane = wavelength, warp = layer segment (as k_flux); star = blockIdx.y
+struct AdjNode {
+    double tau, S, e2, e3, e4;
+};
 template <typename KT, typename GT>
-__global__ void k_rt_adjoint(RtAdjArgs g) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.nlam) return;
-    {
-        const int64_t st = blockIdx.y;
-        g.m += st * g.nd;
-        g.T += st * g.nd;
-        g.kc += st * g.nd * g.ld;
-        g.B += st * g.nd * g.ld;
-        g.stim += st * g.nd * g.ld;
-        g.kline = reinterpret_cast<const KT *>(g.kline) + st * g.nd * g.ld;
-        g.dFbar += st * g.nlam;
-        g.Gt = reinterpret_cast<GT *>(g.Gt) + st * g.nd * g.ld;
+__global__ void __launch_bounds__(32 * kRtSegs) k_rt_adjoint(RtAdjArgs g) {
+    extern __shared__ double smem_rt[];
+    const int lane = threadIdx.x, w = threadIdx.y, nseg = blockDim.y;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane, st = blockIdx.y;
+    const bool live = i < g.nlam;
+    const int a = w * g.nd / nseg, b = (w + 1) * g.nd / nseg;
+    double *s_v = smem_rt;                            // [nd][32] tau from the segment's start, then dF/dtau
+    double *s_tot = s_v + (size_t)g.nd * 32;          // [seg][32] totals of tau, then of dF/dtau
+    double *s_db = s_tot + nseg * 32;                 // [seg][32] dF/dtau of a segment's first layer from the one above
+    AdjNode *s_first = reinterpret_cast<AdjNode *>(s_db + nseg * 32);   // [seg][32]
+    const double *m = g.m + st * g.nd;
+    const double *kc = g.kc + st * g.nd * g.ld + i, *B = g.B + st * g.nd * g.ld + i;
+    const KT *kl = reinterpret_cast<const KT *>(g.kline) + st * g.nd * g.ld + i;
+    double t = 0.0;
+    if (live) {
+        double chi_p = a > 0 ? kc[(a - 1) * g.ld] + (double)kl[(a - 1) * g.ld] : 0.0;
+        for (int d = a; d < b; ++d) {
+            const double chi = kc[d * g.ld] + (double)kl[d * g.ld];
+            t = d == 0 ? chi * m[0] : fma(chi_p + chi, 0.5 * (m[d] - m[d - 1]), t);
+            s_v[d * 32 + lane] = t;
+            chi_p = chi;
+        }
     }
-    const KT *kl = reinterpret_cast<const KT *>(g.kline);
-    GT *Gt = reinterpret_cast<GT *>(g.Gt);
-    const double dFb = g.dFbar[i];
-    double tau[kMaxDepth], S[kMaxDepth], dF[kMaxDepth];
-    double chi_p = 0.0;
-    for (int d = 0; d < g.nd; ++d) {
-        const int64_t o = (int64_t)d * g.ld + i;
-        double chi = g.kc[o] + (double)kl[o];
-        tau[d] = d == 0 ? chi * g.m[0] : tau[d - 1] + 0.5 * (chi_p + chi) * (g.m[d] - g.m[d - 1]);
-        S[d] = g.B[o];
-        dF[d] = 0.0;
-        chi_p = chi;
+    s_tot[w * 32 + lane] = t;
+    __syncthreads();
+    // dF/dtau_j: every interval gives to both its ends; the running layer's value in v
+    AdjNode last{};
+    double v = 0.0;
+    if (live) {
+        double off = 0.0;
+        for (int q = 0; q < w; ++q) off += s_tot[q * 32 + lane];
+        for (int d = a; d < b; ++d) {
+            AdjNode n;
+            n.tau = off + s_v[d * 32 + lane];
+            n.S = B[d * g.ld];
+            expn234(n.tau, n.e2, n.e3, n.e4);
+            double nv = 0.0;
+            if (d == a) {
+                s_first[w * 32 + lane] = n;
+            } else {
+                double da, db;
+                interval_grad(last.tau, n.tau, last.S, n.S, last.e2, last.e3, last.e4, n.e2, n.e3, n.e4, da, db);
+                if (d == 1) {
+                    // top interval: Sa = S0 - s0 tau0, s0 = (S1 - S0)/(tau1 - tau0)
+                    const double t0 = last.tau, iD = rcp_newton(n.tau - t0), s0 = (n.S - last.S) * iD, sp = s0 * iD;
+                    const double Pt = 0.5 - last.e3, Bt = 1.0 / 3.0 - last.e4 - t0 * last.e3;
+                    v += -s0 * Pt + sp * (Bt - t0 * Pt) + last.S * last.e2;
+                    nv = -sp * (Bt - t0 * Pt);
+                }
+                s_v[(d - 1) * 32 + lane] = v + da;
+                nv += db;
+            }
+            v = nv;
+            last = n;
+        }
     }
-    // dF/dtau_j, walking the intervals with the E_n of both endpoints
-    double e2a, e3a, e4a;
-    expn234(tau[0], e2a, e3a, e4a);
-    {
-        // top interval: Sa = S0 - s0 tau0, s0 = (S1 - S0)/(tau1 - tau0)
-        double t0 = tau[0], t1 = tau[1];
-        double s0 = (S[1] - S[0]) / (t1 - t0);
-        double sp = s0 / (t1 - t0);
-        double Pt = 0.5 - e3a;
-        double Bt = 1.0 / 3.0 - e4a - t0 * e3a;
-        dF[0] += -s0 * Pt + sp * (Bt - t0 * Pt) + S[0] * e2a;
-        dF[1] += -sp * (Bt - t0 * Pt);
-    }
-    for (int d = 0; d + 1 < g.nd; ++d) {
-        double e2b, e3b, e4b;
-        expn234(tau[d + 1], e2b, e3b, e4b);
+    __syncthreads();
+    if (live && w + 1 < nseg) {
+        const AdjNode n = s_first[(w + 1) * 32 + lane];
         double da, db;
-        interval_grad(tau[d], tau[d + 1], S[d], S[d + 1], e2a, e3a, e4a, e2b, e3b, e4b, da, db);
-        dF[d] += da;
-        dF[d + 1] += db;
-        e2a = e2b; e3a = e3b; e4a = e4b;
+        interval_grad(last.tau, n.tau, last.S, n.S, last.e2, last.e3, last.e4, n.e2, n.e3, n.e4, da, db);
+        v += da;
+        s_db[(w + 1) * 32 + lane] = db;
     }
+    if (live) s_v[(b - 1) * 32 + lane] = v;
+    __syncthreads();
+    if (live) {
+        if (w > 0) s_v[a * 32 + lane] += s_db[w * 32 + lane];
+        double sum = 0.0;
+        for (int d = a; d < b; ++d) sum += s_v[d * 32 + lane];
+        s_tot[w * 32 + lane] = sum;
+    }
+    __syncthreads();
+    if (!live) return;
     // reverse cumulative sum through the trapezoid: T_j = sum_{k >= j} dL/dtau_k,
     // dL/dchi_d = [d = 0] m_0 T_0 + (m_{d+1} - m_d)/2 T_{d+1} + (m_d - m_{d-1})/2 T_d
-    const double scale = 2.0 * kPI * dFb;
-    double Tn = 0.0;   // T_{d+1}
-    for (int d = g.nd - 1; d >= 0; --d) {
-        double Td = Tn + scale * dF[d];
-        double gch = 0.0;
-        if (d + 1 < g.nd) gch += 0.5 * (g.m[d + 1] - g.m[d]) * Tn;
-        if (d >= 1) gch += 0.5 * (g.m[d] - g.m[d - 1]) * Td;
-        else gch += g.m[0] * Td;
-        Gt[(int64_t)d * g.ld + i] = (GT)(gch * g.stim[(int64_t)d * g.ld + i]);
+    const double scale = 2.0 * kPI * g.dFbar[st * g.nlam + i];
+    double Tn = 0.0;   // T_{d+1} / scale
+    for (int q = nseg - 1; q > w; --q) Tn += s_tot[q * 32 + lane];
+    GT *Gt = reinterpret_cast<GT *>(g.Gt) + st * g.nd * g.ld + i;
+    const double *stim = g.stim + st * g.nd * g.ld + i;
+    for (int d = b - 1; d >= a; --d) {
+        const double Td = Tn + s_v[d * 32 + lane];
+        double gch = d >= 1 ? 0.5 * (m[d] - m[d - 1]) * Td : m[0] * Td;
+        if (d + 1 < g.nd) gch += 0.5 * (m[d + 1] - m[d]) * Tn;
+        Gt[d * g.ld] = (GT)(scale * gch * stim[d * g.ld]);
         Tn = Td;
     }
 }
@@ -1545,14 +1640,19 @@ cudaError_t launch_rt_adjoint(pz_ctx *c, cudaStream_t s) {
     g.stim = c->d_stim;
     g.kline = c->d_kline;
     g.dFbar = c->d_dFbar;
-    dim3 nb((unsigned)((c->nlam + 127) / 128), c->S);
-    if (c->prec == PZ_MIXED) {
-        g.Gt = c->d_Gt;
-        k_rt_adjoint<float, float><<<nb, 128, 0, s>>>(g);
-    } else {
-        g.Gt = c->d_Gt64;
-        k_rt_adjoint<double, double><<<nb, 128, 0, s>>>(g);
-    }
+    const bool mixed = c->prec == PZ_MIXED;
+    g.Gt = mixed ? (void *)c->d_Gt : (void *)c->d_Gt64;
+    const int seg = rt_segs(c->nd);
+    const dim3 nb((unsigned)((c->nlam + 31) / 32), c->S), thr(32, seg);
+    const size_t smem = ((size_t)c->nd * 32 + seg * 64) * sizeof(double) + (size_t)seg * 32 * sizeof(AdjNode);
+    const cudaError_t e =
+        smem_attr(c, mixed ? (const void *)k_rt_adjoint<float, float> : (const void *)k_rt_adjoint<double, double>,
+                  mixed ? kSmemAdj : kSmemAdj64, smem);
+    if (e != cudaSuccess) return e;
+    if (mixed)
+        k_rt_adjoint<float, float><<<nb, thr, smem, s>>>(g);
+    else
+        k_rt_adjoint<double, double><<<nb, thr, smem, s>>>(g);
     c->launches++;
     return cudaGetLastError();
 }
