@@ -261,6 +261,17 @@ namespace pz {
 cudaEvent_t prof_begin(pz_ctx *c, cudaStream_t s);
 void prof_end(pz_ctx *c, cudaStream_t s, int kid, cudaEvent_t begin);
 
+#ifdef __CUDACC__
+// 1/x by two Newton iterations y += y (1 - x y) from the approximate reciprocal (2^-20 or
+// better, squared twice): four multiply-adds of the scarce FP64 pipe.
+__device__ __forceinline__ double rcp_newton(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+#endif
+
 // error reporting (pz_api.cu)
 pz_status fail(pz_status st, const std::string &msg);
 pz_status cuda_check(cudaError_t e, const char *what);

@@ -265,15 +265,6 @@ cudaError_t launch_planck_tables(pz_ctx *c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// 1/x by two Newton iterations y += y (1 - x y) from the approximate reciprocal (2^-20 or
-// better, squared twice): four multiply-adds of the scarce FP64 pipe.
-__device__ __forceinline__ double rcp_newton(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
 __device__ __forceinline__ double interval(double ta, double tb, double Sa, double Sb, double e3a, double e4a,
                                            double e3b, double e4b) {
     double D = tb - ta;
