@@ -440,11 +440,19 @@ constexpr float kFast2V = 5.0f;      // distance threshold factor: |v| >= 5 x 20
 constexpr float kCoreV = 0.3f;       // distance threshold factor: |v| >= 0.3 x 20 = 6
 constexpr float kFast3V = 1.5f;      // distance threshold factor: |v| >= 1.5 x 20
 constexpr float kFast2A2 = 1.5f;     // a^2 bound
+// Larger damping, a^2 <= 44 (a <= 20/3): the eight terms hold where |v| >= 20, so |v| >= 3a (H below
+// 3.5e-9, dH/da below 7e-8 of its scale); those lines keep the whole near zone, U < 400 K of the slab's
+// widest layer, in the near-core kernels.  They are few in giants but a third of the deepest layers'
+// lines in dwarfs, where the polynomial in t (two reciprocals per depth pair and cell, and a mask)
+// took most of the far-wing time: two-star fit on 10^5 lines, far
+// forward 2.45 -> 2.2 ms, reverse 3.8 -> 3.3 ms (the fill by all lanes included).
+constexpr float kWideA2 = 44.0f;
+constexpr float kWideCut = 400.0f / 36.0f;   // its cut over the core's
 
 // The line record of every (depth group, line), whose amask has bit w set when
 // a^2 <= kFast2A2 at every layer of slab w (DS layers) of the group, and bit 8 + w when
 // the centre test rejects every layer of slab w (its warp skips the line).
-// Bits 16 + 3w..: the line's box separation class at slab w: the smallest c whose nearest
+// Bit 4 + w: a^2 <= kWideA2 at every layer of slab w.  Bits 16 + 3w..: the line's box separation class at slab w: the smallest c whose nearest
 // distance (n_c - 1) B has |v| >= 9 a at every layer (thresholds of |v| >= 20 are in n_c), or
 // kBoxClasses.  Lines of class >= 1 that keep a layer are also marked in the words of wide.
 // Depth group = blockIdx.y; warp w of each half of the block takes slab w (of at most 4) of 32
@@ -460,7 +468,7 @@ __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, L
     const LineArgs g = star_view(gq, st);
     int amask = 0;
     if (w < DC / DS) {
-        bool ok = true, none = true;
+        bool ok = true, wide = true, none = true;
         float need = 0.0f;
         if (in) {
             const LineScalars L = load_line(g, l);
@@ -469,11 +477,12 @@ __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, L
                 float q[8];
                 depth_params<8>(g, L, dd, q);
                 ok = ok && q[1] <= kFast2A2;
+                wide = wide && q[1] <= kWideA2;
                 none = none && !pair_kept(g.keep, l, dd);
                 need = fmaxf(need, sqrtf(q[1]) / q[0]);
             }
         }
-        amask = (ok ? 1 << w : 0) | (none ? 1 << (8 + w) : 0);
+        amask = (ok ? 1 << w : 0) | (wide ? 16 << w : 0) | (none ? 256 << w : 0);
         int cls = kBoxClasses;
         if (gq.boxB) {
             if (in) {
@@ -526,7 +535,8 @@ __device__ __forceinline__ void poly_coeffs(float x, float K, float s, float (&c
                                             PZ_Q(3, -3217.5f)), PZ_Q(2, 8445.9375f)), PZ_Q(1, -8445.9375f)),
                     PZ_Q(0, 2111.484375f));
     x *= K;
-    c[7] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(6, 52.5f), PZ_Q(5, -1023.75f)), PZ_Q(4, 9384.375f)),
+    c[7] = x * fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, fmaf(s, PZ_Q(7, -1.0f), PZ_Q(6, 52.5f)),
+                                                            PZ_Q(5, -1023.75f)), PZ_Q(4, 9384.375f)),
                                             PZ_Q(3, -42229.6875f)), PZ_Q(2, 88682.34375f)), PZ_Q(1, -73901.953125f)),
                     PZ_Q(0, 15836.1328125f));
 #undef PZ_Q
@@ -574,7 +584,7 @@ namespace pz {
 // Per-warp staging of a chunk of lines.  Each warp keeps, in its own part of shared
 // memory, the layer constants of its slab (dc: DS x {beta_hi, beta_lo, n_e, n_pert}),
 // and for the chunk's lines their records and the prefactor quads of its DP depth pairs
-// (par: [LC][DP][NQ]).  Lane li fills line li (li + 32, ... for chunks over 32 lines); a
+// (par: [LC][DP][NQ]).  Lanes li and li + 16 fill line li (li + 16, ...); a
 // warp barrier publishes the chunk, and the next fill waits on a warp barrier so that
 // no lane still reads the previous chunk.  No CTA-wide barrier is involved.
 struct WarpStage {
@@ -708,21 +718,25 @@ __device__ __forceinline__ void warp_fill(const LineArgs &g, const WarpStage &ws
                                           int64_t first, int nl, int dfirst, int lane, bool listed = false) {
     constexpr int DP = DS / 2;
     __syncwarp();
-    for (int li = lane; li < nl; li += 32) {
+    // lane = (line, half of the slab's layers): a chunk of 16 lines occupies the whole warp
+    const int half = lane >> 4;
+    for (int li = lane & 15; li < nl; li += 16) {
         const int64_t l = listed ? (int64_t)ws.idx[li] : first + li;
-        ws.info[li] = ginfo[l];
+        if (half == 0) ws.info[li] = ginfo[l];
         const LineScalars L = load_line(g, l);
-        float4 *dst = ws.par + (size_t)li * DP * NQ;
+        float *dst = reinterpret_cast<float *>(ws.par + (size_t)li * DP * NQ);
 #pragma unroll
-        for (int dp = 0; dp < DP; ++dp) {
-            float K0, K1, a0, a1, c0[kPolyN], c1[kPolyN], e0[kPolyN], e1[kPolyN];
-            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp, ws.dc[2 * dp], K0, a0, c0, e0);
-            far_depth_prefactors<NQ>(g, L, l, dfirst + 2 * dp + 1, ws.dc[2 * dp + 1], K1, a1, c1, e1);
-            dst[NQ * dp] = make_float4(K0, K1, a0, a1);
+        for (int q = 0; q < DP; ++q) {
+            const int dd = half * DP + q;                 // layer of the slab
+            float K, a2, c[kPolyN], e[kPolyN];
+            far_depth_prefactors<NQ>(g, L, l, dfirst + dd, ws.dc[dd], K, a2, c, e);
+            float *o = dst + (dd >> 1) * NQ * 4 + (dd & 1);
+            o[0] = K;
+            o[2] = a2;
 #pragma unroll
-            for (int n = 0; n < kPolyN; n += 2) {
-                dst[NQ * dp + 1 + n / 2] = make_float4(c0[n], c1[n], c0[n + 1], c1[n + 1]);
-                if (NQ == kNQB) dst[NQ * dp + 1 + (kPolyN + n) / 2] = make_float4(e0[n], e1[n], e0[n + 1], e1[n + 1]);
+            for (int n = 0; n < kPolyN; ++n) {
+                o[4 + 2 * n] = c[n];
+                if (NQ == kNQB) o[4 + 2 * (kPolyN + n)] = e[n];
             }
         }
     }
@@ -771,8 +785,10 @@ enum FarForm {
     kFormFour,          // |v| >= 20: four
     kFormEight,         // eight, the points with U < cut (x^2 < 36 at the slab's widest layer) left to the
                         // near-core kernels at every layer of the slab
-    kFormLarge,         // a^2 > kFast2A2 somewhere in the slab, |v| >= 20, the window covers the tile: polynomial in t
-    kFormLargeMask,     // a^2 > kFast2A2: the cells with |z| >= 20 inside the window, the others left to the
+    kFormWide,          // kFast2A2 < a^2 <= kWideA2 somewhere in the slab: eight, the points with U < kWideCut cut
+                        // left to the near-core kernels
+    kFormLarge,         // a^2 > kWideA2 somewhere in the slab, |v| >= 20, the window covers the tile: polynomial in t
+    kFormLargeMask,     // a^2 > kWideA2: the cells with |z| >= 20 inside the window, the others left to the
                         // near-core kernels
     kFormFull = 8       // bit: the window covers the tile
 };
@@ -786,12 +802,22 @@ __device__ __forceinline__ int far_form(const LineArgs &g, const LineInfo &info,
     const int sbox = (int)info.ilf >> g.boxsh, nb = box_nmin(bv, box_class(info.amask, w));
     if (sbox <= bv.ta - nb || sbox >= bv.tb + nb) return kFormSkip;
     const float thr = __ldg(g.thr + info.sp * g.nslab + slab);   // 20 Doppler widths of the slab's widest layer
-    if (!((info.amask >> w) & 1)) return full && dmin >= thr ? kFormLarge : kFormLargeMask;
+    if (!((info.amask >> w) & 1)) {
+        if ((info.amask >> (4 + w)) & 1) return kFormWide | (full ? kFormFull : 0);
+        return full && dmin >= thr ? kFormLarge : kFormLargeMask;
+    }
     const int f = dmin >= kFast2V * thr ? kFormTwo
                   : dmin >= kFast3V * thr ? kFormThree
                   : dmin >= thr ? kFormFour
                                 : kFormEight;
     return f | (full ? kFormFull : 0);
+}
+
+// Points with U below it belong to the near-core kernels (series forms).
+__device__ __forceinline__ float far_cut(const LineArgs &g, int form, int sp, int slab) {
+    if ((form & 7) < kFormEight) return 0.0f;
+    const float cut = __ldg(g.cut + sp * g.nslab + slab);
+    return (form & 7) == kFormWide ? kWideCut * cut : cut;
 }
 
 // k = c/dv_D of the warp's depth pairs, rounded exactly as depth_params forms it, for the
@@ -1026,11 +1052,11 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
             const LineInfo info = s_line[li];
             const ulonglong2 *par = s_par + (size_t)li * DP * NQ;
             const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-            if ((fl & 7) <= kFormEight) {
+            if ((fl & 7) <= kFormWide) {
                 f2_t sp[J];
                 far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
-                                (fl & 7) == kFormEight ? __ldg(g.cut + info.sp * g.nslab + slab) : 0.0f, sp);
-                if ((fl & 7) == kFormEight)
+                                far_cut(g, fl, info.sp, slab), sp);
+                if ((fl & 7) >= kFormEight)
                     far_fwd_series<J, DP, 8>(par, sp, acc);
                 else if ((fl & 7) == kFormFour)
                     far_fwd_series<J, DP, 4>(par, sp, acc);
@@ -1408,11 +1434,11 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
                 // (a slab whose every layer the centre test rejects keeps zero sums)
                 if ((fl & 7) != kFormSkip) {
                     const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
-                    if ((fl & 7) <= kFormEight) {
+                    if ((fl & 7) <= kFormWide) {
                         f2_t sp[J];
                         far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
-                                        (fl & 7) == kFormEight ? __ldg(g.cut + info.sp * g.nslab + slab) : 0.0f, sp);
-                        if ((fl & 7) == kFormEight)
+                                        far_cut(g, fl, info.sp, slab), sp);
+                        if ((fl & 7) >= kFormEight)
                             far_bwd_series<J, DP, 8>(par, sp, gv, S1, S2);
                         else if ((fl & 7) == kFormFour)
                             far_bwd_series<J, DP, 4>(par, sp, gv, S1, S2);
@@ -1523,8 +1549,8 @@ __global__ void __launch_bounds__(128, MINB) k_line_bwd(LineArgs g, int GW, int 
 
 // ---------------------------------------------------------------------------
 // Near-core kernels: the cells that the far-wing kernels leave.  At a slab whose damping the
-// series forms take (a^2 <= kFast2A2 at every layer) those are the points with U < cut (the core
-// x^2 < 36 of the slab's widest layer) by the far kernels' own U; otherwise the mid wing and
+// series forms take those are the points with U < cut by the far kernels' own U (a^2 <= kFast2A2 at
+// every layer: the core x^2 < 36 of the slab's widest layer; a^2 <= kWideA2: x^2 < 400); otherwise the mid wing and
 // core, |v|^2 + a^2 < 400, classified with the same prefactors, offset and test as the masked far
 // form.  Every cell is counted exactly once across the two kernels.
 //
@@ -1556,6 +1582,7 @@ constexpr int kNearBatch = 512;      // lines looked at together
 struct NearList {
     int cnt[kNearBatch / 32];        // lines of each 32 whose near zone reaches the tile
     int line[kNearBatch];            // their places in the 32 | slabs (of the group) with only the core left << 8
+                                     // | slabs cut at x^2 = 400 << 12
 };
 
 // Sweep of the near cells of lines [nlo, nhi) in the tile at the lane's layer: cell(i, A, H, dH)
@@ -1583,7 +1610,7 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
                 const int gs = sl * g.tDS / g.tDC, ws = sl - gs * (g.tDC / g.tDS);
                 const int m = g.finfo[(int64_t)gs * g.nl + l].amask;
                 const bool series = (m >> ws) & 1;
-                core |= series ? 256 << (sl - sl0) : 0;
+                core |= series ? 256 << (sl - sl0) : (m >> (4 + ws)) & 1 ? 4096 << (sl - sl0) : 0;
                 need = need || (dmin < (series ? kCoreV : 1.0f) * __ldg(g.thr + sp * g.nslab + sl) && !((m >> (8 + ws)) & 1));
             }
             need = need && b0 + ch * 32 + lane < nhi;
@@ -1610,12 +1637,12 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
             r += kNearWarps * per;
             const LineScalars L = load_line(g, l);
             const float ilf = g.ilf[l], frac = g.frac[l];
-            const bool series = (e >> (8 + slab - sl0)) & 1;
+            const bool wide = (e >> (12 + slab - sl0)) & 1, series = wide || ((e >> (8 + slab - sl0)) & 1);
             float p[16];
             depth_params<D ? 16 : 8>(g, L, d, p);       // (zero strength and k past the last layer)
             // the points that may be near [lo, hi], and (series slabs) those that certainly are; |u| <= reach
             // there, and u = expm1(Delta ln r) differs from Delta ln r by less than 0.6 reach of it
-            const float cut = __ldg(g.cut + L.sp * g.nslab + slab);
+            const float cut = (wide ? kWideCut : 1.0f) * __ldg(g.cut + L.sp * g.nslab + slab);
             const float r2 = kFar2 - p[1];
             const float reach = series ? sqrtf(cut) * (1.0f / kUScale) : sqrtf(fmaxf(r2, 0.0f)) / p[0];
             int lo = 1 << 30, hi = -(1 << 30), ilo = 0, in = -1;
