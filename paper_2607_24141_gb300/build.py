@@ -14,8 +14,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpz.so")
-SOURCES = ["pz_api.cu", "pz_line.cu", "pz_rt.cu", "pz_noalloc.cu"]
-HEADERS = ["pz_internal.h", "pz_voigt.cuh", "pz_box.cuh"]
+SOURCES = ["pz_line.cu", "pz_line_bwd.cu", "pz_line_bwd4.cu", "pz_rt.cu", "pz_api.cu", "pz_noalloc.cu"]
+HEADERS = ["pz_internal.h", "pz_voigt.cuh", "pz_far.cuh", "pz_box.cuh"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-O2", "--expt-relaxed-constexpr"]
 _lock = threading.Lock()

@@ -821,18 +821,21 @@ static pz_status enqueue_backward(pz_ctx *c, const float *dLdf, float *g_gf, flo
     const int64_t nl1 = std::max<int64_t>(c->L.n, 1);
     PZ_CUDA(cudaMemsetAsync(c->d_gacc, 0, sizeof(double) * (four ? 6 : 2) * nl1, s), "backward");
     if (c->L.n > 0) {
-        // one line pass per damping family: the first gives the gf and van der Waals sums,
-        // the radiative and Stark passes their second sums (rows 3 and 5)
-        const int passes = four ? 3 : 1;
-        for (int p = 0; p < passes; ++p) {
-            c->bwd_dsel = p;
-            c->gacc_off = 2 * p * c->L.n;
-            cudaError_t e = timed(c, s, PZ_K_LINE_BWD, [&] {
-                return c->prec == PZ_MIXED ? launch_line_bwd_mixed(c, s) : launch_line_bwd_fp64(c, s);
-            });
-            c->bwd_dsel = 0;
-            c->gacc_off = 0;
-            PZ_CUDA(e, "line gradient kernel");
+        if (c->prec == PZ_MIXED) {
+            PZ_CUDA(timed(c, s, PZ_K_LINE_BWD, [&] { return launch_line_bwd_mixed(c, s, four); }),
+                    "line gradient kernel");
+        } else {
+            // plain FP64 form: one line pass per damping family, the first with the gf and van der Waals
+            // sums, the radiative and Stark passes with their second sums (rows 3 and 5)
+            const int passes = four ? 3 : 1;
+            for (int p = 0; p < passes; ++p) {
+                c->bwd_dsel = p;
+                c->gacc_off = 2 * p * c->L.n;
+                cudaError_t e = timed(c, s, PZ_K_LINE_BWD, [&] { return launch_line_bwd_fp64(c, s); });
+                c->bwd_dsel = 0;
+                c->gacc_off = 0;
+                PZ_CUDA(e, "line gradient kernel");
+            }
         }
     }
     PZ_CUDA(timed(c, s, PZ_K_OTHER, [&] { return launch_grad_finalize(c, g_gf, g_g6, g_ab, s, four, g_rad, g_g4); }),
@@ -939,7 +942,7 @@ pz_status pz_autotune(pz_ctx *c, int32_t with_backward, int32_t reps, int32_t *b
         PZ_TRY(apply_tiling(c, t, "pz_autotune"));
         auto bwd = [&]() -> cudaError_t {
             cudaError_t e = cudaMemsetAsync(c->d_gacc, 0, gbytes, s);
-            return e != cudaSuccess ? e : launch_line_bwd_mixed(c, s);
+            return e != cudaSuccess ? e : launch_line_bwd_mixed(c, s, false);
         };
         PZ_CUDA(launch_line_fwd_mixed(c, s), "pz_autotune: forward");
         if (with_backward) PZ_CUDA(bwd(), "pz_autotune: backward");

@@ -141,11 +141,12 @@ __device__ __forceinline__ void box_weights(const BoxArgs &b, float x, float4 *w
     }
 }
 
-// Series weights of a (line, layer): A a/sqrt(pi) beta_n kap^(n+1) and, with D, A a6/sqrt(pi)
-// gamma_n kap^(n+1), with the prefactors of depth_params; dc = {beta_hi, beta_lo, n_e, n_pert}.
+// Series weights of a (line, layer): A a/sqrt(pi) beta_n kap^(n+1) and, with D, A/sqrt(pi) gamma_n
+// kap^(n+1)/(4 pi dnu_D) without the families' factors gb (van der Waals, radiative, Stark), with the
+// prefactors of depth_params; dc = {beta_hi, beta_lo, n_e, n_pert}.
 template <bool D>
 __device__ __forceinline__ void box_series(const LineArgs &g, const BoxArgs &b, const LineScalars &L, int64_t l, int d,
-                                           const float4 dc, float4 &w, float4 &c) {
+                                           const float4 dc, float4 &w, float4 &c, float3 &gb) {
     const int id = L.sp * g.nd + d;
     const float invdv = __ldg(g.invdv + id);
     const float p = L.E * dc.x;
@@ -163,8 +164,8 @@ __device__ __forceinline__ void box_series(const LineArgs &g, const BoxArgs &b, 
     w.z = B1 * k2 * fmaf(a2, a2 - 5.0f, 3.75f);
     w.w = B1 * k3 * fmaf(a2, fmaf(a2, 10.5f - a2, -26.25f), 13.125f);
     if (D) {
-        const float gb = g.dsel == 0 ? g6n : (g.dsel == 1 ? L.grad : L.g4 * dc.z);
-        const float C1 = A * gb * lw * kInvSqrtPiF * kap;
+        gb = make_float3(g6n, L.grad, L.g4 * dc.z);
+        const float C1 = A * lw * kInvSqrtPiF * kap;
         c.x = C1;
         c.y = C1 * kap * fmaf(-3.0f, a2, 1.5f);
         c.z = C1 * k2 * fmaf(a2, fmaf(5.0f, a2, -15.0f), 3.75f);
@@ -231,7 +232,8 @@ __global__ void __launch_bounds__(128) k_box_moments(LineArgs gq, BoxArgs b) {
             for (int m = 0; m < kBoxBatch; ++m) {
                 const int li = min(lb + m, n - 1);
                 float4 c;
-                if (live) box_series<false>(g, b, s_l[li], c0 + li, d, dc, w[m], c);
+                float3 gb;
+                if (live) box_series<false>(g, b, s_l[li], c0 + li, d, dc, w[m], c, gb);
             }
 #pragma unroll
             for (int m = 0; m < kBoxBatch; ++m) {
@@ -473,8 +475,9 @@ static size_t box_grad_smem(int B, int KE, int nd) {
     return sizeof(float) * ((size_t)kBoxClasses * kBoxK * nd + (ends > copies ? ends : copies));
 }
 
-// Per-line sums of one source box over the boxes of its window: S1 (strength) and S2 (damping).
-template <int KE>
+// Per-line sums of one source box over the boxes of its window: strength and van der Waals damping,
+// FOUR: the radiative and Stark damping too.
+template <int KE, bool FOUR>
 __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -564,7 +567,7 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
         const int q = (int)il - i0;
         float4 W[kBoxK];
         box_weights(b, ((il - (float)i0) + g.frac[l] - b.ctr) * b.invh, W);
-        float S1 = 0.0f, S2 = 0.0f;
+        float S1 = 0.0f, S2 = 0.0f, S3 = 0.0f, S4 = 0.0f;
         const int d1 = (part + 1) * nd / kBoxGradSplit;
         for (int dd = part * nd / kBoxGradSplit; dd < d1; ++dd) {
             const int grp = dd / b.DC;
@@ -582,14 +585,24 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
                 F.w = fmaf(W[k].w, v, F.w);
             }
             float4 w, c;
+            float3 gb;
             box_series<true>(g, b, L, l, dd,
                              make_float4(__ldg(g.beta_hi + dd), __ldg(g.beta_lo + dd), __ldg(g.ne + dd), __ldg(g.npert + dd)),
-                             w, c);
+                             w, c, gb);
             S1 += fmaf(w.w, F.w, fmaf(w.z, F.z, fmaf(w.y, F.y, w.x * F.x)));
-            S2 += fmaf(c.w, F.w, fmaf(c.z, F.z, fmaf(c.y, F.y, c.x * F.x)));
+            const float Y = fmaf(c.w, F.w, fmaf(c.z, F.z, fmaf(c.y, F.y, c.x * F.x)));
+            S2 = fmaf(gb.x, Y, S2);
+            if (FOUR) {
+                S3 = fmaf(gb.y, Y, S3);
+                S4 = fmaf(gb.z, Y, S4);
+            }
         }
         atomicAdd(gq.gacc + l, (double)S1);
         atomicAdd(gq.gacc + gq.nl + l, (double)S2);
+        if (FOUR) {
+            atomicAdd(gq.gacc + far_row(2) * gq.nl + l, (double)S3);
+            atomicAdd(gq.gacc + far_row(3) * gq.nl + l, (double)S4);
+        }
     }
 }
 

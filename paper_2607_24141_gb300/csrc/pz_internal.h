@@ -226,7 +226,7 @@ struct pz_ctx {
     double *d_gacc = nullptr;       // [6][L.n] per table line: (gf, vdW) of the first pass, then
                                     // (unused, rad) and (unused, Stark) of the four-family passes
     double *d_gline = nullptr;      // [4][nl_caller] summed over stars, caller order: gf, vdW, rad, Stark
-    int bwd_dsel = 0;               // damping family of the line backward pass (0 vdW, 1 rad, 2 Stark)
+    int bwd_dsel = 0;               // plain FP64 form: damping family of the line backward pass (0 vdW, 1 rad, 2 Stark)
     int64_t gacc_off = 0;           // its offset into d_gacc
     double *d_gab = nullptr;        // [n_elem]
     float *d_dLdf = nullptr;        // [S][n_out] seed of the captured step
@@ -262,6 +262,14 @@ cudaEvent_t prof_begin(pz_ctx *c, cudaStream_t s);
 void prof_end(pz_ctx *c, cudaStream_t s, int kid, cudaEvent_t begin);
 
 #ifdef __CUDACC__
+constexpr float kInvSqrtPiF = 0.564189583547756287f;
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // 1/x by two Newton iterations y += y (1 - x y) from the approximate reciprocal (2^-20 or
 // better, squared twice): four multiply-adds of the scarce FP64 pipe.
 __device__ __forceinline__ double rcp_newton(double x) {
@@ -282,7 +290,7 @@ pz_status ensure_expn_table();
 
 // launches (return cudaGetLastError() of the launch)
 cudaError_t launch_line_fwd_mixed(pz_ctx *c, cudaStream_t s);
-cudaError_t launch_line_bwd_mixed(pz_ctx *c, cudaStream_t s);
+cudaError_t launch_line_bwd_mixed(pz_ctx *c, cudaStream_t s, bool four);
 cudaError_t launch_line_fwd_fp64(pz_ctx *c, cudaStream_t s);
 cudaError_t launch_line_bwd_fp64(pz_ctx *c, cudaStream_t s);
 cudaError_t launch_apply_corrections(pz_ctx *c, cudaStream_t s);

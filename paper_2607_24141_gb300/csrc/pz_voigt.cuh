@@ -45,14 +45,7 @@ __constant__ double c_weidL64;
 // Lanes evaluating nearby x read adjacent words of each coefficient row.
 __device__ float g_dawson[kDawsonNodes * (kDawsonK + 1)];
 
-constexpr float kInvSqrtPiF = 0.564189583547756287f;
 constexpr float kTwoInvSqrtPiF = 1.12837916709551257f;
-
-__device__ __forceinline__ float rcp_approx(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 
 // Asymptotic series with NC corrections in real arithmetic.  H and (if D) dH/da.
 template <int NC, bool D>
