@@ -676,8 +676,11 @@ def _torch_function4():
 
 
 def __getattr__(name):
+    # made on first use (torch is imported there) and kept: a class per access cost a fit 50 us a call
     if name == "SynthesisFunction":
-        return _torch_function()
-    if name == "SynthesisFunction4":
-        return _torch_function4()
-    raise AttributeError(name)
+        globals()[name] = _torch_function()
+    elif name == "SynthesisFunction4":
+        globals()[name] = _torch_function4()
+    else:
+        raise AttributeError(name)
+    return globals()[name]

@@ -710,6 +710,7 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         upload(&c->d_mass64, mass64, "species") || upload(&c->d_xi64, xi64, "species") || build_thresholds(c) ||
         upload(&c->d_dab, dab, "abund") || upload(&c->d_eos, eos, "abund"))
         return bail(PZ_ENOMEM);
+    c->h_eos = eos;
 
     // ---- continuum opacity [S][nd][ld] ----
     if (dalloc(&c->d_kc, SD * c->ld, "kappa_c")) return bail(PZ_ENOMEM);
@@ -1094,6 +1095,16 @@ pz_status pz_set_corrections(pz_ctx *c, const float *dgf, const float *dg6, cons
         PZ_CUDA(cudaStreamSynchronize(s), what);
         return cuda_check(cudaMemcpy(dst, src, sizeof(float) * n, cudaMemcpyHostToDevice), what);
     };
+    // the species' elements seldom change between calls: an unchanged map is not sent again, and the
+    // call then waits for nothing (a fit sets corrections before every evaluation)
+    auto set_eos = [&](const std::vector<int32_t> &v) -> pz_status {
+        if (v == c->h_eos) return PZ_OK;
+        c->h_eos.clear();
+        PZ_CUDA(cudaStreamSynchronize(s), "elem_of_species");
+        PZ_CUDA(cudaMemcpy(c->d_eos, v.data(), sizeof(int32_t) * c->ns, cudaMemcpyHostToDevice), "elem_of_species");
+        c->h_eos = v;
+        return PZ_OK;
+    };
     PZ_TRY(set_master(dgf, c->d_mdgf, "dlog_gf"));
     PZ_TRY(set_master(dg6, c->d_mdg6, "dlog_gamma6"));
     if (dab) {
@@ -1106,9 +1117,7 @@ pz_status pz_set_corrections(pz_ctx *c, const float *dgf, const float *dg6, cons
             c->d_gab = nullptr;
             PZ_TRY(dalloc(&c->d_dab, n_elem, "dabund"));
         }
-        std::vector<int32_t> heos(eos, eos + c->ns);
-        PZ_CUDA(cudaStreamSynchronize(s), "elem_of_species");
-        PZ_CUDA(cudaMemcpy(c->d_eos, heos.data(), sizeof(int32_t) * c->ns, cudaMemcpyHostToDevice), "elem_of_species");
+        PZ_TRY(set_eos(std::vector<int32_t>(eos, eos + c->ns)));
         if (is_device_ptr(dab)) {
             PZ_CUDA(timed(c, s, PZ_K_OTHER, [&] {
                         k_f32_to_f64<<<(n_elem + 255) / 256, 256, 0, s>>>(n_elem, dab, c->d_dab);
@@ -1118,15 +1127,14 @@ pz_status pz_set_corrections(pz_ctx *c, const float *dgf, const float *dg6, cons
             c->launches++;
         } else {
             std::vector<double> h(dab, dab + n_elem);
+            PZ_CUDA(cudaStreamSynchronize(s), "dabund");   // earlier work on the stream may still read d_dab
             PZ_CUDA(cudaMemcpy(c->d_dab, h.data(), sizeof(double) * n_elem, cudaMemcpyHostToDevice), "dabund");
         }
         c->n_elem = n_elem;
     } else {
         if (c->n_elem != 0) drop_graph(c);
         c->n_elem = 0;
-        std::vector<int32_t> heos(c->ns, -1);
-        PZ_CUDA(cudaStreamSynchronize(s), "elem_of_species");
-        PZ_CUDA(cudaMemcpy(c->d_eos, heos.data(), sizeof(int32_t) * c->ns, cudaMemcpyHostToDevice), "elem_of_species");
+        PZ_TRY(set_eos(std::vector<int32_t>(c->ns, -1)));
     }
     PZ_CUDA(timed(c, s, PZ_K_OTHER, [&] { return launch_apply_corrections(c, s); }), "apply corrections");
     c->have_kline = c->have_flux = c->have_inst = false;

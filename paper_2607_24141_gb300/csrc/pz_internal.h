@@ -181,6 +181,7 @@ struct pz_ctx {
     int32_t *d_grp_mem = nullptr;   // [members]
     int64_t n_groups = 0;
     int32_t *d_eos = nullptr;       // [ns] element of species (or -1)
+    std::vector<int32_t> h_eos;     // what d_eos holds
     int n_elem = 0;
 
     pz::LineTable L;
