@@ -449,7 +449,7 @@ static pz_status build_boxes(pz_ctx *c) {
     PZ_TRY(dalloc(&b.d_C, (size_t)2 * (b.omax + 3) * K * row, "box tables"));
     PZ_TRY(dalloc(&b.d_E, (size_t)4 * b.B * b.KE, "box tables"));
     PZ_TRY(dalloc(&b.d_A, 3 * K * K, "box tables"));
-    PZ_TRY(dalloc(&b.d_start, (size_t)c->S * (b.nbox + 1), "box tables"));
+    PZ_TRY(dalloc(&b.d_start, (size_t)c->S * (kBoxQuarters * b.nbox + 1), "box tables"));
     PZ_TRY(dalloc(&b.d_ws, box_workspace_floats(c, b.chunk), "box workspace"));
     return cuda_check(launch_box_tables(c), "box tables");
 }

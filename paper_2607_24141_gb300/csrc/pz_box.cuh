@@ -42,6 +42,7 @@ namespace pz {
 constexpr int kBoxP = 13;                 // largest order: k + j <= 13 at the nearest box pair
 constexpr int kBoxK = kBoxP + 1;          // moments per box
 constexpr int kBoxRow = 16;               // row stride of the C tables (floats)
+constexpr int kBoxSplit = kBoxQuarters;   // threads that share a (box, layer)
 
 // Order of the expansion at box offset |o|: the worst error over the two boxes, relative to
 // the pair's largest term, stays below 1e-7 at |o| = 3 and 4e-8 beyond (the corners; the mean
@@ -89,17 +90,17 @@ __global__ void k_box_edges(int B, int omax, int KE, const float *C, float *E) {
     E[(((size_t)side * 2 + e) * B + r) * KE + k] = s;
 }
 
-// First line of every box: start[star][box] = first line of the star with i_l >= (s_lo + box) B.
-__global__ void k_box_start(int nbox, int s_lo, int B, const int32_t *il, const int64_t *off, int32_t *start) {
+// First line of every quarter of a box: start[star][q] = first line of the star with i_l >= s_lo B + q B/4.
+__global__ void k_box_start(int nq, int s_lo, int B, const int32_t *il, const int64_t *off, int32_t *start) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x, st = blockIdx.y;
-    if (b > nbox) return;
+    if (b > nq) return;
     int64_t lo = off[st], hi = off[st + 1];
-    const int64_t key = (int64_t)(s_lo + b) * B;
+    const int64_t key = (int64_t)s_lo * B + (int64_t)b * (B / kBoxSplit);
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
         if (il[mid] < key) lo = mid + 1; else hi = mid;
     }
-    start[(int64_t)st * (nbox + 1) + b] = (int32_t)lo;
+    start[(int64_t)st * (nq + 1) + b] = (int32_t)lo;
 }
 
 struct BoxArgs {
@@ -180,107 +181,161 @@ __device__ __forceinline__ void two_sum(float &hi, float &lo, float p) {
     hi = s;
 }
 
-constexpr int kBoxChunk = 32;     // lines staged at a time
-constexpr int kBoxBatch = 4;      // lines whose weights are formed together
+// Running sum of an expansion: the leading coefficients, which hold nearly all of the sum, are
+// compensated.
+constexpr int kBoxComp = 4;
+struct BoxSum {
+    float acc[kBoxK], hi[kBoxComp], lo[kBoxComp];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int k = 0; k < kBoxK; ++k) acc[k] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kBoxComp; ++k) hi[k] = lo[k] = 0.0f;
+    }
+    __device__ __forceinline__ void fold() {
+#pragma unroll
+        for (int k = 0; k < kBoxComp; ++k) {
+            two_sum(hi[k], lo[k], acc[k]);
+            acc[k] = 0.0f;
+        }
+    }
+    __device__ __forceinline__ float get(int k) const { return k < kBoxComp ? hi[k] + (lo[k] + acc[k]) : acc[k]; }
+};
 
-// Moments of one source box: thread = layer, block = box (x) and star (y).
-template <int KE>
-__global__ void __launch_bounds__(128) k_box_moments(LineArgs gq, BoxArgs b) {
-    __shared__ float4 s_w[kBoxChunk][kBoxK];
-    __shared__ LineScalars s_l[kBoxChunk];
-    __shared__ int s_q[kBoxChunk];
-    extern __shared__ float s_cls[];          // [3][kBoxK][threads]: sums of the lines of classes 1..3
-    const int tid = threadIdx.x, nthr = blockDim.x, d = tid;
-    const int box = blockIdx.x, sl = blockIdx.y, st = b.star0 + sl;
+__host__ __device__ constexpr int box_chunk(int NP) { return NP == 1 ? 32 : 16; }   // lines staged at a time and part
+constexpr int kBoxBatch = 4;      // lines whose weights are formed together
+template <int NP>
+struct BoxStage {
+    float4 w[NP][box_chunk(NP)][kBoxK];
+    LineScalars l[NP][box_chunk(NP)];
+    int q[NP][box_chunk(NP)];
+};
+template <int NP>
+static size_t box_moment_smem(int KE, int nd) {
+    return sizeof(BoxStage<NP>) + sizeof(float) * (size_t)NP * nd * (4 * kBoxK + KE);
+}
+
+// Moments of one source box: thread = (part of the box's indices, layer), block = box (x) and star
+// (y).  NP = 4 parts where the grid has few boxes: with one, the lines' chain of loads and sums leaves
+// the chip waiting (5,300 lines in 163 boxes: forward lines 0.485 -> 0.421 ms); NP = 1 on longer grids,
+// where the parts' shared memory leaves two boxes per SM (two stars on 10^5 lines: 2.50 ms, one part 2.40).
+template <int KE, int NP>
+__global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b) {
+    constexpr int QP = kBoxSplit / NP, CH = box_chunk(NP);   // quarters per part, lines per chunk
+    extern __shared__ float4 smem4[];
+    BoxStage<NP> &sg = *reinterpret_cast<BoxStage<NP> *>(smem4);
+    const int tid = threadIdx.x, box = blockIdx.x, sl = blockIdx.y, st = b.star0 + sl;
     const LineArgs g = star_view(gq, st);
-    const int lo = gq.bstart[(int64_t)st * (b.nbox + 1) + box], hi = gq.bstart[(int64_t)st * (b.nbox + 1) + box + 1];
+    const int nd = g.nd, part = tid / nd, d = tid - part * nd;
+    const bool live = part < NP;
+    float *s_cls = reinterpret_cast<float *>(&sg + 1);          // [part][3][kBoxK][nd]: lines of classes 1..3
+    float *s_m = s_cls + NP * 3 * kBoxK * nd;            // [part][kBoxK][nd]: class 0
+    float *s_pm = s_m + NP * kBoxK * nd;                 // [part][KE][nd]: totals of the prefixes
+    const int32_t *start = gq.bstart + (int64_t)st * (kBoxSplit * b.nbox + 1) + kBoxSplit * box;
     const int i0 = (b.s_lo + box) * b.B;
-    const bool live = d < g.nd;
+    int most = 0;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) most = max(most, start[(q + 1) * QP] - start[q * QP]);
+    const int lo = live ? start[part * QP] : 0, hi = live ? start[(part + 1) * QP] : 0;
     const float4 dc = live ? make_float4(__ldg(g.beta_hi + d), __ldg(g.beta_lo + d), __ldg(g.ne + d), __ldg(g.npert + d))
                            : make_float4(0.f, 0.f, 0.f, 0.f);
     const int grp = live ? d / b.DC : 0, shift = 16 + 3 * (live ? (d % b.DC) / b.DS : 0);
     const LineInfo *info = gq.finfo + (int64_t)grp * gq.nl;
-    float acc[kBoxK], hs[kBoxK], ls[kBoxK], pm[KE];
-#pragma unroll
-    for (int k = 0; k < kBoxK; ++k) acc[k] = hs[k] = ls[k] = 0.0f;
+    BoxSum S;
+    S.clear();
+    float pm[KE];
 #pragma unroll
     for (int k = 0; k < KE; ++k) pm[k] = 0.0f;
-    for (int k = 0; k < 3 * kBoxK; ++k) s_cls[k * nthr + tid] = 0.0f;
-    float *PM = b.PM + (((int64_t)sl * b.nbox + box) * b.B * KE) * g.nd + d;
-    int qcur = 0;
-    for (int c0 = lo; c0 < hi; c0 += kBoxChunk) {
-        const int n = min(kBoxChunk, hi - c0);
+    for (int k = tid; k < NP * 3 * kBoxK * nd; k += blockDim.x) s_cls[k] = 0.0f;
+    float *PM = b.PM + (((int64_t)sl * b.nbox + box) * b.B * KE) * nd + d;
+    const int q0 = part * (b.B / NP), q1 = q0 + b.B / NP;
+    int qcur = q0;
+    for (int c = 0; c < most; c += CH) {
         __syncthreads();
-        if (tid < n) {
-            const int l = c0 + tid;
-            s_l[tid] = load_line(g, l);
-            const float il = g.ilf[l];
-            s_q[tid] = (int)il - i0;
-            box_weights(b, ((il - (float)i0) + g.frac[l] - b.ctr) * b.invh, s_w[tid]);
+        for (int k = tid; k < NP * CH; k += blockDim.x) {
+            const int pt = k / CH, li = k % CH, l = start[pt * QP] + c + li;
+            if (l < start[(pt + 1) * QP]) {
+                sg.l[pt][li] = load_line(g, l);
+                const float il = g.ilf[l];
+                sg.q[pt][li] = (int)il - i0;
+                box_weights(b, ((il - (float)i0) + g.frac[l] - b.ctr) * b.invh, sg.w[pt][li]);
+            }
         }
         __syncthreads();
+        const int c0 = lo + c, n = live ? min(CH, hi - c0) : 0;
         for (int lb = 0; lb < n; lb += kBoxBatch) {
             // the batch's weights first: their table loads are independent and overlap
             float4 w[kBoxBatch];
             int cls[kBoxBatch];
 #pragma unroll
-            for (int m = 0; m < kBoxBatch; ++m) {
-                const int li = min(lb + m, n - 1);
-                cls[m] = live && lb + m < n ? (info[c0 + li].amask >> shift) & 7 : kBoxClasses;
-            }
+            for (int m = 0; m < kBoxBatch; ++m)
+                cls[m] = lb + m < n ? (info[c0 + lb + m].amask >> shift) & 7 : kBoxClasses;
 #pragma unroll
             for (int m = 0; m < kBoxBatch; ++m) {
                 const int li = min(lb + m, n - 1);
-                float4 c;
+                float4 cw;
                 float3 gb;
-                if (live) box_series<false>(g, b, s_l[li], c0 + li, d, dc, w[m], c, gb);
+                box_series<false>(g, b, sg.l[part][li], c0 + li, d, dc, w[m], cw, gb);
             }
 #pragma unroll
             for (int m = 0; m < kBoxBatch; ++m) {
                 if (lb + m >= n) break;
                 // prefixes up to the grid index before this line's
-                const int q = s_q[lb + m];
+                const int q = sg.q[part][lb + m];
                 for (; qcur < q; ++qcur)
-                    if (live)
 #pragma unroll
-                        for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * g.nd] = pm[k];
+                    for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * nd] = pm[k];
                 if (cls[m] >= kBoxClasses) continue;
                 float v[kBoxK];
 #pragma unroll
                 for (int k = 0; k < kBoxK; ++k) {
-                    const float4 W = s_w[lb + m][k];
+                    const float4 W = sg.w[part][lb + m][k];
                     v[k] = fmaf(w[m].w, W.w, fmaf(w[m].z, W.z, fmaf(w[m].y, W.y, w[m].x * W.x)));
                     if (k < KE) pm[k] += v[k];
                 }
                 if (cls[m] == 0) {
 #pragma unroll
-                    for (int k = 0; k < kBoxK; ++k) acc[k] += v[k];
+                    for (int k = 0; k < kBoxK; ++k) S.acc[k] += v[k];
                 } else {
-                    float *sc = s_cls + (cls[m] - 1) * kBoxK * nthr + tid;
+                    float *sc = s_cls + ((part * 3 + cls[m] - 1) * kBoxK) * nd + d;
 #pragma unroll
-                    for (int k = 0; k < kBoxK; ++k) sc[k * nthr] += v[k];
+                    for (int k = 0; k < kBoxK; ++k) sc[k * nd] += v[k];
                 }
             }
         }
+        S.fold();
+    }
+    if (live) {
+        for (; qcur < q1; ++qcur)
 #pragma unroll
-        for (int k = 0; k < kBoxK; ++k) {
-            two_sum(hs[k], ls[k], acc[k]);
-            acc[k] = 0.0f;
+            for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * nd] = pm[k];
+#pragma unroll
+        for (int k = 0; k < kBoxK; ++k) s_m[(part * kBoxK + k) * nd + d] = S.get(k);
+#pragma unroll
+        for (int k = 0; k < KE; ++k) s_pm[(part * KE + k) * nd + d] = pm[k];
+    }
+    __syncthreads();
+    if (!live) return;
+    if (part > 0) {
+        // the prefixes of this part, from the start of the box
+#pragma unroll
+        for (int k = 0; k < KE; ++k) {
+            float off = 0.0f;
+            for (int q = 0; q < part; ++q) off += s_pm[(q * KE + k) * nd + d];
+            for (int q = q0; q < q1; ++q) PM[((int64_t)q * KE + k) * nd] += off;
         }
     }
-    if (!live) return;
-    for (; qcur < b.B; ++qcur)
-#pragma unroll
-        for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * g.nd] = pm[k];
     // sets by class, each with the classes below it
-    float *M = b.M + ((int64_t)sl * b.nbox + box) * kBoxClasses * kBoxK * g.nd + d;
+    float *M = b.M + ((int64_t)sl * b.nbox + box) * kBoxClasses * kBoxK * nd + d;
+    for (int k = part; k < kBoxK; k += NP) {
+        float m = 0.0f;
 #pragma unroll
-    for (int k = 0; k < kBoxK; ++k) {
-        float m = hs[k] + ls[k];
-        M[(int64_t)k * g.nd] = m;
+        for (int q = 0; q < NP; ++q) m += s_m[(q * kBoxK + k) * nd + d];
+        M[(int64_t)k * nd] = m;
         for (int c = 1; c < kBoxClasses; ++c) {
-            m += s_cls[((c - 1) * kBoxK + k) * nthr + tid];
-            M[((int64_t)c * kBoxK + k) * g.nd] = m;
+#pragma unroll
+            for (int q = 0; q < NP; ++q) m += s_cls[((q * 3 + c - 1) * kBoxK + k) * nd + d];
+            M[((int64_t)c * kBoxK + k) * nd] = m;
         }
     }
 }
@@ -332,31 +387,9 @@ __device__ __forceinline__ void box_translate_at(int P, const float *C, const fl
     }
 }
 
-// Running sum of an expansion over the offsets: the leading coefficients, which hold nearly all
-// of the sum, are compensated.
-constexpr int kBoxComp = 4;
-struct BoxSum {
-    float acc[kBoxK], hi[kBoxComp], lo[kBoxComp];
-    __device__ __forceinline__ void clear() {
-#pragma unroll
-        for (int k = 0; k < kBoxK; ++k) acc[k] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < kBoxComp; ++k) hi[k] = lo[k] = 0.0f;
-    }
-    __device__ __forceinline__ void fold() {
-#pragma unroll
-        for (int k = 0; k < kBoxComp; ++k) {
-            two_sum(hi[k], lo[k], acc[k]);
-            acc[k] = 0.0f;
-        }
-    }
-    __device__ __forceinline__ float get(int k) const { return k < kBoxComp ? hi[k] + (lo[k] + acc[k]) : acc[k]; }
-};
-
 // Far field of a target box, added to the near-core sums.  kBoxSplit threads share a layer: each
 // takes every kBoxSplit-th offset, then every kBoxSplit-th point (one thread per layer left a
 // single spectrum's few boxes waiting on the chain of table and moment loads).
-constexpr int kBoxSplit = 4;
 template <int KE>
 __global__ void __launch_bounds__(kBoxSplit * 128) k_box_field(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [B][nd + 1]
@@ -470,11 +503,13 @@ constexpr int kBoxGradSplit = 4;          // a warp's unit: 32 lines x a quarter
 
 // row of the window-end sums of one layer: [KE][B + 1] floats, odd length
 __host__ __device__ __forceinline__ int box_zrow(int B, int KE) { return (KE * (B + 1)) | 1; }
+// nd: layers of the block
 static size_t box_grad_smem(int B, int KE, int nd) {
     const size_t ends = (size_t)nd * box_zrow(B, KE) + (size_t)2 * nd * (B + 1), copies = (size_t)2 * kBoxClasses * kBoxK * nd;
     return sizeof(float) * ((size_t)kBoxClasses * kBoxK * nd + (ends > copies ? ends : copies));
 }
 
+// Block = box (x), star (y) and part of the layers (z; one part where the grid has boxes enough).
 // Per-line sums of one source box over the boxes of its window: strength and van der Waals damping,
 // FOUR: the radiative and Stark damping too.
 template <int KE, bool FOUR>
@@ -483,9 +518,13 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int box = blockIdx.x, sl = blockIdx.y, st = b.star0 + sl;
     const LineArgs g = star_view(gq, st);
-    const int lo = gq.bstart[(int64_t)st * (b.nbox + 1) + box], hi = gq.bstart[(int64_t)st * (b.nbox + 1) + box + 1];
+    const int32_t *start = gq.bstart + (int64_t)st * (kBoxSplit * b.nbox + 1) + kBoxSplit * box;
+    const int lo = start[0], hi = start[kBoxSplit];
     if (lo >= hi) return;
-    const int nd = g.nd, zrow = box_zrow(b.B, KE);
+    // the block's layers dz .. dz + nd
+    const int nz = gridDim.z, dz = (int)blockIdx.z * g.nd / nz, nd = ((int)blockIdx.z + 1) * g.nd / nz - dz;
+    const int64_t gnd = g.nd;
+    const int zrow = box_zrow(b.B, KE);
     float *s_psi = smem;                                   // [class][k][nd]
     float *s_z = s_psi + (size_t)kBoxClasses * kBoxK * nd; // [nd][zrow]: [k][q]
     float *s_g = s_z + (size_t)nd * zrow;                  // [2][nd][B + 1]: G of two target boxes
@@ -494,8 +533,8 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
     // each taking every np-th offset, their copies added in order afterwards
     const int np = min(3, 32 * kBoxGradWarps / nd), part = tid / nd, d = tid - part * nd;
     if (part < np) {
-        const int4 nm = *reinterpret_cast<const int4 *>(b.nmin + ((int64_t)st * gq.nslab + d / b.DS) * 4);
-        const float *Nst = b.N + (int64_t)sl * b.ntb * kBoxK * nd + d;
+        const int4 nm = *reinterpret_cast<const int4 *>(b.nmin + ((int64_t)st * gq.nslab + (dz + d) / b.DS) * 4);
+        const float *Nst = b.N + (int64_t)sl * b.ntb * kBoxK * gnd + dz + d;
         float *mine = part == 0 ? s_psi : s_z + (size_t)(part - 1) * kBoxClasses * kBoxK * nd;
         BoxSum S;
         S.clear();
@@ -509,7 +548,7 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
                     const int t = s + (side ? o : -o);
                     if (t >= 0 && t < b.ntb)
                         box_translate_at<true>(box_order(o), b.C + ((size_t)side * (b.omax + 3) + o) * kBoxK * kBoxRow,
-                                               Nst + (int64_t)t * kBoxK * nd, nd, S.acc);
+                                               Nst + (int64_t)t * kBoxK * gnd, gnd, S.acc);
                 }
                 if ((n & 3) == 3 || o < 12) S.fold();
             }
@@ -527,15 +566,15 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
             const int e = k / (nd * b.B), kk = k - e * nd * b.B, row = kk / b.B, col = kk - row * b.B;
             const int t = side ? s + b.omax + 1 + e : s - b.omax - 1 - e;
             const int64_t i = (int64_t)t * b.B + col;
-            s_g[(e * nd + row) * (b.B + 1) + col] = (t >= 0 && i < g.nlam) ? g.Gt[(int64_t)row * g.ld + i] : 0.0f;
+            s_g[(e * nd + row) * (b.B + 1) + col] = (t >= 0 && i < g.nlam) ? g.Gt[(int64_t)(dz + row) * g.ld + i] : 0.0f;
         }
         __syncthreads();
         // thread = (layer, moment): the points' G times E_k, running over the lines' indices q
         for (int u = tid; u < nd * KE; u += blockDim.x) {
-            const int k = u / nd, dz = u - k * nd;
+            const int k = u / nd, dl = u - k * nd;
             const float *E0 = b.E + (size_t)side * 2 * b.B * KE + k, *E1 = E0 + (size_t)b.B * KE;
-            const float *g0 = s_g + dz * (b.B + 1), *g1 = s_g + (nd + dz) * (b.B + 1);
-            float *zr = s_z + dz * zrow + k * (b.B + 1);
+            const float *g0 = s_g + dl * (b.B + 1), *g1 = s_g + (nd + dl) * (b.B + 1);
+            float *zr = s_z + dl * zrow + k * (b.B + 1);
             float z = 0.0f;
             if (side == 0) {
                 // points left of the line, box s - omax - 1 - e: r >= q - rem + 1 + e B, q downwards
@@ -570,8 +609,8 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
         float S1 = 0.0f, S2 = 0.0f, S3 = 0.0f, S4 = 0.0f;
         const int d1 = (part + 1) * nd / kBoxGradSplit;
         for (int dd = part * nd / kBoxGradSplit; dd < d1; ++dd) {
-            const int grp = dd / b.DC;
-            const int cls = (gq.finfo[(int64_t)grp * gq.nl + l].amask >> (16 + 3 * ((dd - grp * b.DC) / b.DS))) & 7;
+            const int da = dz + dd, grp = da / b.DC;
+            const int cls = (gq.finfo[(int64_t)grp * gq.nl + l].amask >> (16 + 3 * ((da - grp * b.DC) / b.DS))) & 7;
             if (cls >= kBoxClasses) continue;
             float4 F = make_float4(0.f, 0.f, 0.f, 0.f);
             const float *psi = s_psi + cls * kBoxK * nd + dd, *z = s_z + dd * zrow + q;
@@ -586,8 +625,8 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
             }
             float4 w, c;
             float3 gb;
-            box_series<true>(g, b, L, l, dd,
-                             make_float4(__ldg(g.beta_hi + dd), __ldg(g.beta_lo + dd), __ldg(g.ne + dd), __ldg(g.npert + dd)),
+            box_series<true>(g, b, L, l, da,
+                             make_float4(__ldg(g.beta_hi + da), __ldg(g.beta_lo + da), __ldg(g.ne + da), __ldg(g.npert + da)),
                              w, c, gb);
             S1 += fmaf(w.w, F.w, fmaf(w.z, F.z, fmaf(w.y, F.y, w.x * F.x)));
             const float Y = fmaf(c.w, F.w, fmaf(c.z, F.z, fmaf(c.y, F.y, c.x * F.x)));

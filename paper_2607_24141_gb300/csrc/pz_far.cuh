@@ -56,7 +56,7 @@ struct LineArgs {
     int boxB, boxsh, s_lo, nbox;                    // box points (0: off) and log2, first source box, boxes
     float shrink;                                   // |v| >= |Delta| ln r shrink k over a window
     const int *nmin;                                // [S][nslab][4] nearest offset of each class
-    const int32_t *bstart;                          // [S][nbox + 1] first line of each box
+    const int32_t *bstart;                          // [S][4 nbox + 1] first line of each quarter of a box
     uint32_t *wide;                                 // [4][nslab][wwords] lines of class >= 1..4
     int64_t wwords;
 };
@@ -509,7 +509,7 @@ template <class F>
 __device__ __forceinline__ void box_rings(const LineArgs &g, const BoxView &v, int st, int slab, int n0g, int t0, int T,
                                           int q, int P, const WarpStage &ws, int LC, int lane, F &&f) {
     if (!g.boxB || n0g >= kBoxNever) return;
-    const int32_t *bs = g.bstart + (int64_t)st * (g.nbox + 1);
+    const int32_t *bs = g.bstart + (int64_t)st * (kBoxQuarters * g.nbox + 1);
     int below = n0g;
     for (int c = 1; c <= kBoxClasses; ++c) {
         const int n = box_nmin(v, c);
@@ -522,7 +522,7 @@ __device__ __forceinline__ void box_rings(const LineArgs &g, const BoxView &v, i
             s0 = max(max(s0, (t0 - g.W) >> g.boxsh), g.s_lo);
             s1 = min(min(s1, (t0 + T - 1 + g.W) >> g.boxsh), g.s_lo + g.nbox - 1);
             if (s0 > s1) continue;
-            const int a = bs[s0 - g.s_lo], b = bs[s1 - g.s_lo + 1];
+            const int a = bs[kBoxQuarters * (s0 - g.s_lo)], b = bs[kBoxQuarters * (s1 - g.s_lo + 1)];
             int cur = a + (int)((int64_t)(b - a) * q / P);
             const int hi = a + (int)((int64_t)(b - a) * (q + 1) / P);
             while (cur < hi) {

@@ -102,13 +102,14 @@ struct BoxPlan {
     int KE = 0;                 // moments kept per grid index for the window ends
     int chunk = 0;              // stars per launch (bounds the workspace)
     int *d_nmin = nullptr;      // [S][nslab][4] nearest offset of each separation class
-    int32_t *d_start = nullptr; // [S][nbox + 1] first line of each box
+    int32_t *d_start = nullptr; // [S][4 nbox + 1] first line of each quarter of a box
     float *d_A = nullptr, *d_C = nullptr, *d_E = nullptr;
     float *d_ws = nullptr;      // moments and prefixes, or the moments of G
     uint32_t *d_wide = nullptr; // [4][nslab][words] lines of class >= 1..4, one bit per line
     size_t wide_cap = 0;
     std::vector<int> h_nmin;
 };
+constexpr int kBoxQuarters = 4;      // parts of a box with a first line of their own
 constexpr int kBoxNever = 1 << 28;   // offset of a class that does not exist
 
 // A pair of profiler events around one launch and the kernel family it times.

@@ -649,7 +649,8 @@ cudaError_t launch_box_tables(pz_ctx *c) {
     const BoxPlan &b = c->box;
     k_box_tables<<<dim3(b.omax + 2, 2), 256>>>(b.B, c->lnr, b.omax, b.d_C);
     k_box_edges<<<dim3(b.B, 2, 2), 32>>>(b.B, b.omax, b.KE, b.d_C, b.d_E);
-    k_box_start<<<dim3(b.nbox / 256 + 1, c->S), 256>>>(b.nbox, b.s_lo, b.B, c->L.il32, c->d_line_off, b.d_start);
+    k_box_start<<<dim3(kBoxSplit * b.nbox / 256 + 1, c->S), 256>>>(kBoxSplit * b.nbox, b.s_lo, b.B, c->L.il32,
+                                                                 c->d_line_off, b.d_start);
     // operators of f^2, f^3, f^4 on the Chebyshev basis: column k of (1/m)(d + p eps)(d + q eps)
     const double eps = 0.5 * b.B * c->lnr;
     std::vector<double> cur((size_t)kBoxK * kBoxK, 0.0);   // [k][j]: image of T_k as coefficients of T_j
@@ -702,26 +703,44 @@ static BoxArgs box_args(const pz_ctx *c, int star0) {
     return b;
 }
 
+// Fewer than two boxes per SM: the boxes' blocks are cut further (by indices of the box or layers).
+static bool box_few(const pz_ctx *c) {
+    return (int64_t)c->box.nbox * std::min(c->box.chunk, c->S) < 2 * (int64_t)c->n_sm;
+}
+
 // Forward: moments of the lines, then the far field of every point into knear.
-template <int KE>
-static cudaError_t launch_box_fwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
-    const int thr = (c->nd + 31) / 32 * 32;
+template <int KE, int NP>
+static cudaError_t launch_box_fwd_parts(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+    static std::atomic<bool> attr_set[kMaxDevices];
+    if (!attr_set[c->device].load(std::memory_order_acquire)) {
+        const cudaError_t e = cudaFuncSetAttribute(k_box_moments<KE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)box_moment_smem<NP>(KE, kMaxDepth));
+        if (e != cudaSuccess) return e;
+        attr_set[c->device].store(true, std::memory_order_release);
+    }
+    const int thr_m = (NP * c->nd + 31) / 32 * 32, thr_f = (kBoxSplit * c->nd + 31) / 32 * 32;
     for (int st = 0; st < c->S; st += c->box.chunk) {
         const int n = std::min(c->box.chunk, c->S - st);
         const BoxArgs b = box_args(c, st);
-        k_box_moments<KE><<<dim3(b.nbox, n), thr, sizeof(float) * 3 * kBoxK * thr, s>>>(g, b);
-        k_box_field<KE><<<dim3(b.ntb, n), (kBoxSplit * c->nd + 31) / 32 * 32,
-                          sizeof(float) * (kBoxSplit * kBoxK * c->nd + b.B * (c->nd + 1)), s>>>(g, b);
+        k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(KE, c->nd), s>>>(g, b);
+        k_box_field<KE><<<dim3(b.ntb, n), thr_f, sizeof(float) * (kBoxSplit * kBoxK * c->nd + b.B * (c->nd + 1)), s>>>(
+            g, b);
         c->launches += 2;
     }
     return cudaGetLastError();
+}
+template <int KE>
+static cudaError_t launch_box_fwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+    return box_few(c) ? launch_box_fwd_parts<KE, kBoxSplit>(c, g, s) : launch_box_fwd_parts<KE, 1>(c, g, s);
 }
 
 // Backward: moments of G, then every line's sums over the points its boxes reach, into gacc.
 template <int KE, bool FOUR>
 static cudaError_t launch_box_bwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
     const int thr = (c->nd + 31) / 32 * 32;
-    const size_t smem = box_grad_smem(c->box.B, KE, c->nd);
+    // several blocks per box, each with part of the layers, where the lines fill few boxes
+    const int nz = box_few(c) ? std::min(3, c->nd) : 1;
+    const size_t smem = box_grad_smem(c->box.B, KE, (c->nd + nz - 1) / nz);
     static std::atomic<bool> attr_set[kMaxDevices];
     if (!attr_set[c->device].load(std::memory_order_acquire)) {
         const cudaError_t e = cudaFuncSetAttribute(k_box_grad<KE, FOUR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -733,7 +752,7 @@ static cudaError_t launch_box_bwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) 
         const int n = std::min(c->box.chunk, c->S - st);
         const BoxArgs b = box_args(c, st);
         k_box_gmoments<<<dim3(b.ntb, n), thr, sizeof(float) * c->nd * (b.B + 1), s>>>(g, b);
-        k_box_grad<KE, FOUR><<<dim3(b.nbox, n), 32 * kBoxGradWarps, smem, s>>>(g, b);
+        k_box_grad<KE, FOUR><<<dim3(b.nbox, n, nz), 32 * kBoxGradWarps, smem, s>>>(g, b);
         c->launches += 2;
     }
     return cudaGetLastError();
