@@ -300,10 +300,10 @@ pz_status pz_get_damping_corrections(pz_ctx *ctx, float *dlog_gamma_rad, float *
  *   dL/dDelta log gamma_beta,l = ln10 sum_{i in window, d} G stim A_ld (dH/da) a_beta,ld
  * with a_beta the part of the damping parameter a that family beta contributes
  * (radiative gamma_rad, Stark gamma_4 n_e, van der Waals gamma_6 n_pert, each over
- * 4 pi dnu_D).  The line stage runs once per family (the van der Waals pass also
- * gives the gf sums), so it costs three pz_backward line passes.  Outputs as
- * pz_backward (device FP32, caller order, each may be NULL).  Requirements and
- * errors as pz_backward. */
+ * 4 pi dnu_D).  The mixed form sums all four in one line pass (the families
+ * share everything but one factor per layer); the plain FP64 form runs one pass
+ * per family.  Outputs as pz_backward (device FP32, caller order, each may be
+ * NULL).  Requirements and errors as pz_backward. */
 pz_status pz_backward4(pz_ctx *ctx, const float *dL_df, float *g_dlog_gf, float *g_dlog_gamma_rad,
                        float *g_dlog_gamma4, float *g_dlog_gamma6, float *g_dabund, void *stream);
 

@@ -217,7 +217,7 @@ static size_t box_moment_smem(int KE, int nd) {
 
 // Moments of one source box: thread = (part of the box's indices, layer), block = box (x) and star
 // (y).  NP = 4 parts where the grid has few boxes: with one, the lines' chain of loads and sums leaves
-// the chip waiting (5,300 lines in 163 boxes: forward lines 0.485 -> 0.421 ms); NP = 1 on longer grids,
+// the chip waiting (12,000 lines in 165 boxes: forward lines 0.485 -> 0.420 ms); NP = 1 on longer grids,
 // where the parts' shared memory leaves two boxes per SM (two stars on 10^5 lines: 2.50 ms, one part 2.40).
 template <int KE, int NP>
 __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b) {

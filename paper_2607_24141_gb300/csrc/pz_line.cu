@@ -1,26 +1,31 @@
 // pz_line.cu -- windowed Voigt line-opacity sum (Eqs. 4-5) and its adjoint
 // (Sec. 6), FP32-mixed and plain FP64 forms, plus the per-device Voigt tables.
 //
-// Mixed-precision kernels.  The work is a queue of items (star, lambda tile,
-// depth group, line range) built on the host: lines are sorted by centre
-// within each star, and an item's range [lo, hi) holds the star's lines whose
-// window |i - i_l| <= W touches the tile (binary search).  The kernels are
-// persistent: every CTA takes the next item from an atomic counter until the
-// queue is empty, and the items are ordered longest first, so stars and tiles
-// of very different line counts share one launch.  A far-wing item covers a
+// Mixed-precision kernels.  A windowed sum is shared by three families, which own
+// every (line, point, layer) exactly once between them:
+//   box expansions (pz_box.cuh)  pairs of boxes of B points at least n_c boxes apart, inside
+//                                the window of every line of the source box;
+//   far wings (pz_far.cuh)       the nearer boxes down to the core: series in 1/v^2;
+//   near cores (below)           the points of the core, the full Voigt function.
+//
+// The far-wing work is a queue of items (star, lambda tile, depth group, line
+// range) built on the host: lines are sorted by centre within each star, and an
+// item's range [lo, hi) holds the star's lines whose window |i - i_l| <= W
+// touches the tile (with boxes: whose box is near the tile; the lines further
+// out that the expansions leave are gathered from one bit per line).  The
+// kernels are persistent: every CTA takes the next item from an atomic counter
+// until the queue is empty, and the items are ordered longest first, so stars
+// and tiles of very different line counts share one launch.  An item covers a
 // tile of T = 32 J grid points and GW x DS layers; warp w sweeps layers
 // [d0 + w DS, d0 + (w+1) DS) and lane l owns the J contiguous points
-// t0 + l J + [0, J).  Lines are staged into shared memory LC at a time: the
-// CTA first computes the per-(line, depth) prefactors of Eqs. 4-5 (strength A,
-// damping a, Doppler factor c/dv_D and the pre-scaled far-wing polynomial
-// coefficients) once for the whole tile, then every thread accumulates its
-// J x DS (lambda, depth) sums in registers.  Whether a line is entirely inside
-// its window and in the far wing (|v| >= 20 at every depth of the warp's slab)
-// over the whole tile is decided once per line and warp.  Per-chunk FP32
-// partial sums are folded into a compensated (hi, lo) pair (2Sum).  The
-// frequency offset is formed in index space: v = expm1((x_l - i) ln r) c/dv_D
-// with x_l - i = (i_l - i) + frac_l, the integer part exact, avoiding the
-// cancellation of lambda_l/lambda_i - 1.
+// t0 + l J + [0, J).  Each warp stages LC lines at a time in its own part of
+// shared memory (the prefactors of Eqs. 4-5 and the series coefficients, formed
+// by all lanes), then every thread accumulates its J x DS (lambda, depth) sums
+// in registers.  How a line is summed over the tile and slab (far_form) is
+// decided once per line and warp.  Per-chunk FP32 partial sums are folded into a
+// compensated (hi, lo) pair (2Sum).  The frequency offset is formed in index
+// space: v = expm1((x_l - i) ln r) c/dv_D with x_l - i = (i_l - i) + frac_l, the
+// integer part exact, avoiding the cancellation of lambda_l/lambda_i - 1.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -135,9 +140,9 @@ pz_status ensure_device_tables() {
 // The line record of every (depth group, line), whose amask has bit w set when
 // a^2 <= kFast2A2 at every layer of slab w (DS layers) of the group, and bit 8 + w when
 // the centre test rejects every layer of slab w (its warp skips the line).
-// Bit 4 + w: a^2 <= kWideA2 at every layer of slab w.  Bits 16 + 3w..: the line's box separation class at slab w: the smallest c whose nearest
-// distance (n_c - 1) B has |v| >= 9 a at every layer (thresholds of |v| >= 20 are in n_c), or
-// kBoxClasses.  Lines of class >= 1 that keep a layer are also marked in the words of wide.
+// Bit 4 + w: a^2 <= kWideA2 at every layer of slab w.  Bits 16 + 3w..: the line's box separation
+// class at slab w: the smallest c whose nearest distance (n_c - 1) B has |v| >= 9 a at every layer
+// (thresholds of |v| >= 20 are in n_c), or kBoxClasses.  Lines of class >= 1 that keep a layer are also marked in the words of wide.
 // Depth group = blockIdx.y; warp w of each half of the block takes slab w (of at most 4) of 32
 // consecutive lines, one word of wide (with one thread per line over all slabs a short list
 // waited on the chain of table loads: 11 -> 6 us at 5,300 lines; 50 us at 2 10^5 either way).

@@ -13,8 +13,11 @@
 //                      dH/da sqrt(pi) = t (1 + (1.5 - 2a^2) t + (3.75 - 12 a^2) t^2
 //                                       + (12 a^4 - 67.5 a^2) t^3 + 180 a^4 t^4 - 120 a^6 t^5)
 //                    (relative truncation error < 3e-7).
+//                    Lines of damping a^2 <= 44 take series in 1/v^2 instead, down to
+//                    |v| = 6 (a^2 <= 1.5) or 20 (pz_far.cuh).
 //   6 <= |z| < 20    the same series to six corrections in real arithmetic
-//                    through the Chebyshev recurrences of sin/cos((2n+1) arg z).
+//                    through the Chebyshev recurrences of sin/cos((2n+1) arg z)
+//                    (a^2 > 1.5; below that only next to the core's cut).
 //   |z| < 6, a < 0.5 w = exp(-z^2) + (2i/sqrt(pi)) D(z), D Dawson's integral.
 //                    Re/Im D(x + i a) from a Taylor expansion of D about the
 //                    nearest table node x_j = j/16 in the complex offset
