@@ -55,7 +55,10 @@ constexpr float kKScale = 68719476736.0f;
 struct Tiling {
     int J = 4;       // lambda points per thread (contiguous)
     int DS = 6;      // depths per warp (even: the far-wing kernels work on depth pairs)
-    int GW = 4;      // warps per CTA (each a depth slab)
+    // two warps per CTA (each a depth slab): the reverse pass's barrier per chunk holds up two warps
+    // instead of four (2e5 lines, forward + reverse 10.46 -> 10.30 ms; two stars on 1e5 lines
+    // 12.68 -> 12.61; one warp 10.71 and three, which leave 18 layers for the last group, 10.80)
+    int GW = 2;
     // 16 lines per chunk: with the series' nine quads per depth pair of the reverse pass 32 lines
     // would take 77 KB per CTA (2 resident per SM against 4)
     int LC = 16;     // lines per shared-memory chunk (forward)
