@@ -368,7 +368,7 @@ static pz_status build_items(pz_ctx *c) {
     PZ_TRY(upload(&c->d_fitems, hf, "work items"));
     PZ_TRY(upload(&c->d_fext, hx, "work items"));
     PZ_TRY(upload(&c->d_bitems, hbf, "work items"));
-    PZ_TRY(upload(&c->d_bext, hbx, "work items"));
+    if (c->prec == PZ_MIXED) PZ_TRY(upload(&c->d_bext, hbx, "work items"));
     PZ_TRY(upload(&c->d_nitems_f, hn, "work items"));
     PZ_TRY(upload(&c->d_nitems_b, hb, "work items"));
     PZ_TRY(dalloc(&c->d_fcnt, (size_t)nsplit, "work items"));
@@ -418,8 +418,9 @@ static pz_status build_thresholds(pz_ctx *c) {
     dfree(c->d_cut);
     c->d_thr = c->d_cut = nullptr;
     PZ_TRY(upload(&c->d_thr, thr, "thresholds"));
-    PZ_TRY(upload(&c->d_cut, cut, "thresholds"));
     c->nslab = nslab;
+    if (c->prec != PZ_MIXED) return PZ_OK;   // the rest serves the mixed form's kernels
+    PZ_TRY(upload(&c->d_cut, cut, "thresholds"));
     // box expansions: nearest offset n_c of class c at each (star, slab): the points of boxes n_c
     // apart lie beyond 2^c times the widest species' threshold; kBoxNever if no whole box or
     // window end is that far.  Layers past the last one take the bounds of no line.
