@@ -389,9 +389,12 @@ __device__ __forceinline__ void box_translate_at(int P, const float *C, const fl
 
 // Far field of a target box, added to the near-core sums.  kBoxSplit threads share a layer: each
 // takes every kBoxSplit-th offset, then every kBoxSplit-th point (one thread per layer left a
-// single spectrum's few boxes waiting on the chain of table and moment loads).
+// single spectrum's few boxes waiting on the chain of table and moment loads).  Bound by the latency
+// of those loads: 96 registers let two blocks of nine warps (72 layers) share an SM, where the 102
+// of the free choice left one (two stars on 43,000 lines: forward lines 2.38 -> 2.19 ms; 72
+// registers and three blocks spill and slow short grids, 0.419 -> 0.429 ms on 2,200 points).
 template <int KE>
-__global__ void __launch_bounds__(kBoxSplit * 128) k_box_field(LineArgs gq, BoxArgs b) {
+__global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [B][nd + 1]
     const int sl = blockIdx.y, st = b.star0 + sl, t = blockIdx.x;
     const LineArgs g = star_view(gq, st);
