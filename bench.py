@@ -49,33 +49,30 @@ GOLDEN = os.path.join(ROOT, "tests", "golden")
 # the dominant kernel, from one ncu capture per (kernel, workload) written up under profiles/;
 # each entry is valid only while the library sources hash to the recorded value, and is
 # reported as null otherwise.
-TRAFFIC = {
-    # 8-star batch launch: 162.6 MB read + 9.8 MB written, scaled to the 64-star launch by its
-    # evaluations (1.6398e12 / 1.6699e11 = 9.82; the traffic is line records per tile plus the
-    # G stim rows, both in proportion to the stars' lines and tiles)
-    ("k_line_bwd", "batch64"): (1.693e9, "de30e54c2e5da9e3"),
-}
-NCU_PIPES = {
-    ("k_line_bwd", "batch64"): ({"fma_pipe_pct": 58.2, "alu_pipe_pct": 27.8, "xu_pipe_pct": 9.3,
-                                 "issue_active_pct": 66.4, "warps_active_pct": 31.0, "registers": 96,
-                                 "capture": "8-star batch, one launch, --set full"}, "de30e54c2e5da9e3"),
-}
-KERNEL_SOURCES = ("pz_line.cu", "pz_voigt.cuh", "pz_internal.h", "pz_api.cu")
-FMA_PER_EN = 39      # FP64 FMAs of one E_2/E_3/E_4 Taylor step (13 rounds of value + two derivatives)
+TRAFFIC = {}
+NCU_PIPES = {}
+KERNEL_SOURCES = ("pz_line.cu", "pz_far.cuh", "pz_box.cuh", "pz_line_bwd.cu", "pz_line_bwd4.cu", "pz_voigt.cuh",
+                  "pz_internal.h", "pz_api.cu")
+FMA_PER_EN = 27      # FP64 FMAs of one E_2/E_3/E_4 Taylor step (9 rounds of value + two derivatives)
 
 
-# Per-evaluation pipe work of the far-wing kernels, which evaluate every in-window cell.
-# Reduced form (lines >= 100 Doppler widths from the whole tile, most cells of these
-# workloads), with s = 1/U shared by the depths of a warp and the table's coefficients
-# (B1 K, B2' K^2, C1 K, C2' K^2): forward 2 FP32-pipe lane operations per cell (two
-# products accumulated); backward, per depth and thread, X1 = sum_j G s_j and
-# X2 = sum_j G s_j^2 over the thread's J points (2 per cell) and four products into
-# the two sums, 2 + 4/J per cell; one MUFU reciprocal per line and point shared by the
-# DS = 6 depths of a warp.  Full far form: 7 / 13 FP32-pipe operations and 1 MUFU
-# reciprocal.  With 128 FP32 lanes and 16 MUFU lanes per SM the FP32 pipe binds.
+# Pipe work of the direct far-wing kernels.  Box expansions take every pair of a line and a point at
+# least three boxes of 32 points apart (on grids of R = 3e5), so the direct kernels evaluate about five
+# boxes, 160 points, of every line and layer; most are within 20 Doppler widths and take eight terms:
+# forward 8 FP32-pipe lane operations per cell; reverse 8 for the sums of G s^n over the thread's J points
+# and 2 x 8 per depth and thread, 8 + 16/J per cell.  Set-up of the lines, offsets, reciprocals and the
+# points of further rings are not counted.  One MUFU reciprocal per line and point serves the DS = 6
+# depths of a warp.  With 128 FP32 lanes and 16 MUFU lanes per SM the FP32 pipe binds.
+NEAR_POINTS = 160
+
+
 def far_ops(J):
-    return {"line_fwd": {"fp32_reduced": 2, "fp32_full": 7, "mufu_reduced": 1.0 / 6, "mufu_full": 1},
-            "line_bwd": {"fp32_reduced": 2 + 4.0 / J, "fp32_full": 13, "mufu_reduced": 1.0 / 6, "mufu_full": 1}}
+    return {"line_fwd": {"fp32": 8, "mufu": 1.0 / 6}, "line_bwd": {"fp32": 8 + 16.0 / J, "mufu": 1.0 / 6}}
+
+
+def direct_cells(evals, half_window):
+    """(line, point, layer) terms left to the direct far-wing kernels, about: NEAR_POINTS of the window."""
+    return evals * min(1.0, NEAR_POINTS / (2.0 * half_window + 1.0))
 
 
 def parse():
@@ -178,11 +175,11 @@ def grad_rel(g, ref):
     return np.abs(g - ref) / np.maximum(np.abs(ref), floor)
 
 
-def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key):
+def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key, half_window=1500):
     """Roofline of the dominant far-wing line kernel from the profiler's kernel times
-    {family: (ms, launches)}: achieved FP32-pipe lane operations per second at the
-    two-term reduced form's count (a lower bound of the work) against the measured
-    FP32 pipe peak."""
+    {family: (ms, launches)}: FP32-pipe lane operations per second on the cells summed
+    directly (direct_cells) at the eight-term form's count against the measured FP32 pipe
+    peak.  The family's time includes the box expansions' kernels."""
     far = {"line_fwd": kt["line_fwd"][0] - kt["near_fwd"][0], "line_bwd": kt["line_bwd"][0] - kt["near_bwd"][0]}
     dom = max(far, key=far.get)
     t_dom = far[dom] * 1e-3 / max(kt[dom][1], 1)
@@ -190,7 +187,8 @@ def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key):
     peak_fp32_lanes = n_sm * 128 * clk_max * 1e6
     peak_mufu = pipe_peaks.get("mufu") or n_sm * 16 * clk_max * 1e6
     peak_fp32 = pipe_peaks.get("fp32") or peak_fp32_lanes
-    achieved = evals * ops["fp32_reduced"] / t_dom
+    cells = direct_cells(evals, half_window)
+    achieved = cells * ops["fp32"] / t_dom
     kname = "k_line_bwd" if dom == "line_bwd" else "k_line_fwd"
     hsh = source_hash()
     tr = TRAFFIC.get((kname, workload_key))
@@ -206,9 +204,8 @@ def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key):
                         % (n_sm, peak_fp32_lanes * 1e-9)) if pipe_peaks.get("fp32") else
                        "derived: %d SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % (n_sm, clk_max),
         "evals_per_launch": evals, "ms_per_launch": t_dom * 1e3, "evals_per_s": evals / t_dom,
-        "ops_per_eval": ops,
-        "fp32_pipe_frac_full_form": evals * ops["fp32_full"] / t_dom / peak_fp32,
-        "mufu_pipe_frac_reduced_form": evals * ops["mufu_reduced"] / t_dom / peak_mufu,
+        "direct_cells_per_launch": cells, "ops_per_direct_cell": ops,
+        "mufu_pipe_frac": cells * ops["mufu"] / t_dom / peak_mufu,
         "kernel_share": {k: round(v / tot, 4) for k, v in share.items() if tot > 0},
         "far_ms_per_launch": {k: v / max(kt[k][1], 1) for k, v in far.items()},
         "near_ms_per_launch": {k: kt[k][0] / max(kt[k][1], 1) for k in ("near_fwd", "near_bwd")},
@@ -463,7 +460,8 @@ def run_broad(args, dev, barrier, max_over_ranks, ws, tiling=None, pipe_peaks=No
            "create_s": t_create,
            "kernel_ms_per_step": {k: v[0] / args.broad_steps for k, v in kt.items() if v[1] > 0},
            "far_fwd_ms": far_ms,
-           "far_fwd_fp32_ops_per_s": evals * far_ops(4)["line_fwd"]["fp32_reduced"] / (far_ms * 1e-3),
+           "far_fwd_fp32_ops_per_s": direct_cells(evals, prob.lines.half_window) * far_ops(4)["line_fwd"]["fp32"]
+                                     / (far_ms * 1e-3),
            "scattering": scat}
     # plain FP64 GPU form on a slice of the same line list
     if not args.no_fp64:
