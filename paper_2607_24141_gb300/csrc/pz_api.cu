@@ -410,8 +410,8 @@ static pz_status build_thresholds(pz_ctx *c) {
                 if (mn < 1e300) {
                     thr[((size_t)st * c->ns + s) * nslab + b] =
                         (float)(20.0 / (kC * mn * c->lnr * shrink) * (1.0 + 1e-4) + 1e-3);
-                    // U = 2^36 u^2 at x = u k = 6, k = c/dv_D of the widest layer
-                    cut[((size_t)st * c->ns + s) * nslab + b] = (float)(36.0 * (double)kKScale / (kC * mn * kC * mn));
+                    // U = 4^uexp u^2 at x = u k = 6, k = c/dv_D of the widest layer
+                    cut[((size_t)st * c->ns + s) * nslab + b] = (float)(std::ldexp(36.0, 2 * c->uexp) / (kC * mn * kC * mn));
                 }
             }
     dfree(c->d_thr);
@@ -688,9 +688,6 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
                 double dv = std::sqrt(2.0 * kKB * at->T[d] / (at->mass_amu[s] * kAMU) + at->xi_cms * at->xi_cms);
                 const size_t id = (size_t)s * nd + d, o = (size_t)st * ns * nd + id;
                 invdv[o] = (float)(1.0 / dv);
-                // K = 2^36/k^2 of the far-wing prefactors, k = c/dv_D rounded as the kernels form it
-                const float kf = (float)kC * invdv[o];
-                Ksd[o] = kKScale / (kf * kf);
                 pop64[o] = at->pop[id];
                 Rb[o] = (1.0 / dv) * at->pop[id] / at->rho[d];
                 Rf[o] = (float)Rb[o];
@@ -698,6 +695,14 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         }
     }
     c->h_invdv = invdv;
+    // K = 4^uexp/k^2 of the far-wing prefactors, k = c/dv_D rounded as the kernels form it.  The series' last
+    // coefficient holds K^8, so K stays at 1 or below (a fixed 2^36/k^2 left FP32 for lines a few times 10 km/s wide)
+    const float kmin = (float)kC * *std::min_element(invdv.begin(), invdv.end());
+    c->uexp = kmin >= 1.0f ? std::ilogb(kmin) : 0;
+    for (size_t o = 0; o < SSD; ++o) {
+        const float kf = (float)kC * invdv[o];
+        Ksd[o] = std::ldexp(1.0f, 2 * c->uexp) / (kf * kf);
+    }
     // widest near zone (20 Doppler widths, in grid points) over stars, species and layers
     box_choose(c, 20.0 / (kC * (double)*std::min_element(invdv.begin(), invdv.end()) * c->lnr));
     std::vector<double> dab(1, 0.0);

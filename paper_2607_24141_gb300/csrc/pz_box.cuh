@@ -109,7 +109,7 @@ struct BoxArgs {
     int DC, DS;                   // tiling of the line records (class bits)
     int star0;                    // first star of this launch
     float invh, ctr;              // 2/B, (B - 1)/2
-    float kapscale;               // kap = K kapscale (K = 2^36/k^2)
+    float kapscale;               // kap = K kapscale (K = 4^uexp/k^2)
     const float *A;               // [3][kBoxK][kBoxK]: W_qk = sum_j A[q - 2][k][j] T_j, q = 2..4
     const float *C, *E;           // expansion and window-end tables
     const int *nmin;              // [S][nslab][4]

@@ -30,7 +30,7 @@ struct LineArgs {
     const int32_t *sp;
     const float *R, *invdv, *thr;                   // [ns][nd], [ns][nd], [ns][nslab] of the star
     const float *cut;                               // [ns][nslab] 36 K of the slab's widest layer
-    const float *Ksd;                               // [ns][nd] K = 2^36/k^2 of the star
+    const float *Ksd;                               // [ns][nd] K = 4^uexp/k^2 of the star
     int nslab;
     const float *beta_hi, *beta_lo, *ne, *npert, *c2T;   // [nd] of the star
     float *kline;                                   // forward output [nd][ld] of the star
@@ -46,7 +46,8 @@ struct LineArgs {
     int n_items, ngroups;
     int *ctr;
     int64_t sstride, dstride, bstride, tstride;     // per-star strides of the tables above
-    float rj[4], rm1j[4];                           // r^-j and r^-j - 1, j = 0..3 (r = 1 + 1/R)
+    float uscale, kunscale;                         // 2^uexp and 4^-uexp: scaled offset u 2^uexp, 1/k^2 = K 4^-uexp
+    float rj[4], rm1j[4];                           // r^-j and (r^-j - 1) 2^uexp, j = 0..3 (r = 1 + 1/R)
     const int32_t *star;                            // [nl] star of each line
     const LineInfo *finfo;                          // far-wing line records [ngroups][nl] (k_far_info)
     int *status;                                    // device status word (bounded-wait failures)
@@ -280,13 +281,13 @@ __device__ __forceinline__ float f2_hi(f2_t v) {
 //   backward (NQ = 9): the same, then (C1 K, C2' K^2) .. (C7' K^7, C8' K^8)
 //   backward, all damping families (NQ = 11): C without its family factor gamma n, then the three
 //   families' factors (van der Waals, radiative) (Stark, -)
-// with k = c/dv_D, K = 2^36/k^2 (the power of two keeps every product of the
-// prefactors and of the offsets far from the FP32 exponent limits), B2' = B2 - B1 a^2
+// with k = c/dv_D, K = 4^uexp/k^2 (the power of four brings the largest K of the context to 1/4..1
+// and keeps every product of the prefactors, K^8 among them, and of the offsets inside FP32), B2' = B2 - B1 a^2
 // = B1 (1.5 - a^2) and C2' = C2 - C1 a^2 = C1 (1.5 - 3a^2).  The far kernels take the
-// squared offsets scaled alike, U = 2^36 u^2, so that with s = 1/U
+// squared offsets scaled alike, U = 4^uexp u^2, so that with s = 1/U
 //   reduced form:  H sqrt(pi)/A = (B1 K) s + (B2' K^2) s^2   (p = K s exactly, see below)
 //   full form:     r = 1/(U + a^2 K) and t = 1/|z|^2 = K r, so B1 t (...) = (B1 K) r (...)
-// and the masked lines recover B1 = (B1 K) k^2 2^-36 (and C1 alike) per depth pair.
+// and the masked lines recover B1 = (B1 K) k^2 4^-uexp (and C1 alike) per depth pair.
 // Each warp stages the quads of its own slab, par[li][pair][q] in its part of shared
 // memory; the polynomial in t of the large-damping lines (B3..B5, C3..C6) follows from a^2
 // and B1 K (C1 K) in registers.  Lane li computes line li's quads from the line data and the
@@ -297,8 +298,6 @@ __device__ __forceinline__ float f2_hi(f2_t v) {
 constexpr int kPolyN = 8;          // terms of the series in p = K s
 constexpr int kNQF = 1 + kPolyN / 2, kNQB = 1 + kPolyN, kNQB4 = kNQB + 2;
 constexpr int kBwdBatch = 16;   // lines per transposed partial-sum batch of the far-wing backward (2 lanes per line)
-constexpr float kUScale = 262144.0f;              // 2^18: scaled offset u 2^18
-constexpr float kKUnscale = 1.4551915228366852e-11f;   // 2^-36
 
 // Reduced far-wing form.  Far from the core the polynomial in t = 1/|z|^2 is cut
 // after its t^2 term: H sqrt(pi)/(A a) = t (1 + 1.5 t) and, for dH/da, C1 t (1 +
@@ -372,7 +371,7 @@ __device__ __forceinline__ void poly_coeffs(float x, float K, float s, float (&c
 
 // Prefactors of line l at layer d (one half of a depth pair), with the roundings of
 // depth_params for k and a^2 (the cells' near / far classification depends on them):
-// K = 2^36/k^2, a^2, the series coefficients c (B1 K, B2' K^2, ..) and (NQ = kNQB) e (C1 K, C2' K^2, ..).  dc holds the layer's
+// K = 4^uexp/k^2, a^2, the series coefficients c (B1 K, B2' K^2, ..) and (NQ = kNQB) e (C1 K, C2' K^2, ..).  dc holds the layer's
 // {beta_hi, beta_lo, n_e, n_pert}.  Layers past the last one get K = 0, a^2 = 1 and zero
 // coefficients, pairs rejected by the centre test zero coefficients.
 template <int NQ>
@@ -662,17 +661,17 @@ __device__ __forceinline__ void far_c3456(f2_t a2, f2_t C1, f2_t &C3, f2_t &C4, 
 
 // Reciprocals s_j = 1/U_j of the squared scaled offsets of one line at the thread's J
 // points (and their squares), for the reduced forms: offsets from the first point's,
-// u_j = u_0 r^-j + (r^-j - 1) scaled by 2^18; points outside the line's window get
+// u_j = u_0 r^-j + (r^-j - 1) scaled by 2^uexp; points outside the line's window get
 // s = 0 unless the window covers the tile (full), points of a lane whose box is left to the
 // box expansions (not near) too.
 template <int J>
 __device__ __forceinline__ void far_scaled_u2(const LineArgs &g, const LineInfo &info, float lamf, float (&U)[J]) {
     // scalar chain: the offsets depend on the line and the point only, not on the depth
-    const float u0 = offset_u((info.ilf - lamf) + info.frac, g.lnr) * kUScale;
+    const float u0 = offset_u((info.ilf - lamf) + info.frac, g.lnr) * g.uscale;
     U[0] = u0 * u0;
 #pragma unroll
     for (int j = 1; j < J; ++j) {
-        const float u = fmaf(u0, g.rj[j], g.rm1j[j] * kUScale);
+        const float u = fmaf(u0, g.rj[j], g.rm1j[j]);
         U[j] = u * u;
     }
 }
@@ -910,7 +909,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
                     const f2_t ak = f2_mul(q0.y, q0.x);          // a^2 K
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
-                        // r = 1/(U + a^2 K) = 2^-36/(u^2 + a^2/k^2), t = 1/(u^2 k^2 + a^2) = K r
+                        // r = 1/(U + a^2 K) = 4^-uexp/(u^2 + a^2/k^2), t = 1/(u^2 k^2 + a^2) = K r
                         const f2_t rr = f2_rcp(f2_fma(u2[j], f2_splat(1.0f), ak));
                         const f2_t r = near ? rr : 0ull;
                         const f2_t t = f2_mul(q0.x, r);
@@ -939,8 +938,8 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
 #pragma unroll
                 for (int dp = 0; dp < DP; ++dp) {
                     const ulonglong2 q0 = par[NQ * dp], q1 = par[NQ * dp + 1];
-                    // B1 = (B1 K) k^2 2^-36
-                    const f2_t B1 = f2_mul(q1.x, f2_mul(f2_mul(kp[dp], kp[dp]), f2_splat(kKUnscale)));
+                    // B1 = (B1 K) k^2 4^-uexp
+                    const f2_t B1 = f2_mul(q1.x, f2_mul(f2_mul(kp[dp], kp[dp]), f2_splat(g.kunscale)));
                     f2_t B3, B4, B5;
                     far_b345(q0.y, B1, B3, B4, B5);
                     const f2_t B2 = f2_mul(B1, f2_splat(1.5f));
@@ -1106,11 +1105,12 @@ __global__ void __launch_bounds__(128, MINB) k_line_fwd(LineArgs g, int GW, int 
 
 // One line's far-wing backward sums over a warp's J x DS cells (depth pairs):
 // S[0] += G stim A H, Y += G stim A a6 dH/da.  Without MASK, w holds the scaled squared
-// offsets U = 2^36 u^2; with MASK, w holds the offsets u and kp the depth pairs' k, and
+// offsets U = 4^uexp u^2; with MASK, w holds the offsets u and kp the depth pairs' k, and
 // only the far cells inside the window (inwin per lambda point) are kept.
 template <int J, int DP, bool MASK, bool FOUR>
-__device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (&w)[J], const f2_t (&gv)[DP][J],
-                                             const bool near, const bool *inwin, const f2_t *kp, FarSums<FOUR> &R) {
+__device__ __forceinline__ void far_bwd_line(const LineArgs &g, const ulonglong2 *par, const f2_t (&w)[J],
+                                             const f2_t (&gv)[DP][J], const bool near, const bool *inwin, const f2_t *kp,
+                                             FarSums<FOUR> &R) {
     constexpr int NQ = far_nqb<FOUR>();
 #pragma unroll
     for (int dp = 0; dp < DP; ++dp) {
@@ -1119,8 +1119,8 @@ __device__ __forceinline__ void far_bwd_line(const ulonglong2 *par, const f2_t (
         f2_t Y = R.open();
         f2_t B1 = q1.x, C1 = q2.x;
         if (MASK) {
-            // the masked cells use t = 1/|z|^2 itself: B1 = (B1 K) k^2 2^-36, C1 alike
-            const f2_t kk = f2_mul(f2_mul(kp[dp], kp[dp]), f2_splat(kKUnscale));
+            // the masked cells use t = 1/|z|^2 itself: B1 = (B1 K) k^2 4^-uexp, C1 alike
+            const f2_t kk = f2_mul(f2_mul(kp[dp], kp[dp]), f2_splat(g.kunscale));
             B1 = f2_mul(B1, kk);
             C1 = f2_mul(C1, kk);
         }
@@ -1277,7 +1277,7 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
                         f2_t u2[J];
 #pragma unroll
                         for (int j = 0; j < J; ++j) u2[j] = f2_splat(U[j]);
-                        far_bwd_line<J, DP, false, FOUR>(par, u2, gv, near, nullptr, nullptr, R);
+                        far_bwd_line<J, DP, false, FOUR>(g, par, u2, gv, near, nullptr, nullptr, R);
                     } else {
                         // line near the tile or partly outside its window: far cells inside the window only
                         f2_t u2[J];
@@ -1293,7 +1293,7 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
                         }
                         f2_t kp[DP];
                         far_kpairs<DP>(g, info.sp, d0 + warp * DS, kp);
-                        far_bwd_line<J, DP, true, FOUR>(par, u2, gv, near, inwin, kp, R);
+                        far_bwd_line<J, DP, true, FOUR>(g, par, u2, gv, near, inwin, kp, R);
                     }
                 }
                 const int r = b & (kBwdBatch - 1);

@@ -48,9 +48,6 @@ constexpr int kWeidN64 = 32;      // Weideman rational order (FP64 plain form)
 constexpr int kStatusWaitGaveUp = 1;      // a bounded device-side wait gave up
 constexpr int kStatusScatNoConverge = 2;  // the scattering-source refinement hit its round limit
 
-// Scale of the far-wing prefactors and offsets: K = 2^36/k^2 with k = c/dv_D, U = 2^36 u^2.
-constexpr float kKScale = 68719476736.0f;
-
 // Mixed-precision line-kernel tiling.
 struct Tiling {
     int J = 4;       // lambda points per thread (contiguous)
@@ -164,7 +161,9 @@ struct pz_ctx {
     float *d_R = nullptr;           // [S][ns][nd] (1/dv_D) (pop/rho) 10^dabund
     double *d_Rbase = nullptr;      // [S][ns][nd] (1/dv_D)(pop/rho), FP64
     float *d_invdv = nullptr;       // [S][ns][nd] 1/dv_D (s/cm)
-    float *d_Ksd = nullptr;         // [S][ns][nd] K = 2^36/k^2, k = c/dv_D (far-wing prefactors)
+    float *d_Ksd = nullptr;         // [S][ns][nd] K = 4^uexp/k^2, k = c/dv_D (far-wing prefactors)
+    int uexp = 0;                   // scale of the far-wing prefactors and offsets, U = 4^uexp u^2: 2^uexp <= the
+                                    // smallest k (the widest line), so that 1/4 < max K <= 1
     double *d_pop64 = nullptr;      // [S][ns][nd]
     double *d_mass64 = nullptr;     // [S][ns]
     double *d_xi64 = nullptr;       // [S]

@@ -253,13 +253,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
 // lines x 1,500 points, forward items cut by lines: 0.090 -> 0.086, reverse 0.146 -> 0.086 ms).
 // ---------------------------------------------------------------------------
 
-// U = 2^36 u^2 of point i as the far kernels form it, from their lane's first point (far_scaled_u2).
+// U = 4^uexp u^2 of point i as the far kernels form it, from their lane's first point (far_scaled_u2).
 template <int J>
 __device__ __forceinline__ float far_u2(const LineArgs &g, float ilf, float frac, int i) {
     const int j = i & (J - 1);
-    const float u0 = offset_u((ilf - (float)(i - j)) + frac, g.lnr) * kUScale;
+    const float u0 = offset_u((ilf - (float)(i - j)) + frac, g.lnr) * g.uscale;
     const float rj = j == 1 ? g.rj[1] : j == 2 ? g.rj[2] : g.rj[3], rm = j == 1 ? g.rm1j[1] : j == 2 ? g.rm1j[2] : g.rm1j[3];
-    const float u = j == 0 ? u0 : fmaf(u0, rj, rm * kUScale);
+    const float u = j == 0 ? u0 : fmaf(u0, rj, rm);
     return u * u;
 }
 
@@ -332,7 +332,7 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
             // there, and u = expm1(Delta ln r) differs from Delta ln r by less than 0.6 reach of it
             const float cut = (wide ? kWideCut : 1.0f) * __ldg(g.cut + L.sp * g.nslab + slab);
             const float r2 = kFar2 - p[1];
-            const float reach = series ? sqrtf(cut) * (1.0f / kUScale) : sqrtf(fmaxf(r2, 0.0f)) / p[0];
+            const float reach = series ? sqrtf(cut * g.kunscale) : sqrtf(fmaxf(r2, 0.0f)) / p[0];
             int lo = 1 << 30, hi = -(1 << 30), ilo = 0, in = -1;
             if (have && p[0] > 0.0f && (series || r2 > 0.0f) && pair_kept(g.keep, l, d)) {
                 const float span = reach / g.lnr, m = fmaf(fmaf(0.6f, reach, 1e-3f), span, 0.01f);
@@ -471,8 +471,10 @@ static LineArgs make_args(pz_ctx *c) {
     g.lnr = (float)c->lnr;
     for (int j = 0; j < 4; ++j) {
         g.rj[j] = (float)std::exp(-j * c->lnr);
-        g.rm1j[j] = (float)std::expm1(-j * c->lnr);
+        g.rm1j[j] = std::ldexp((float)std::expm1(-j * c->lnr), c->uexp);
     }
+    g.uscale = std::ldexp(1.0f, c->uexp);
+    g.kunscale = std::ldexp(1.0f, -2 * c->uexp);
     g.star = c->L.star;
     g.fext = nullptr;
     g.fpart = c->d_fpart;
@@ -697,7 +699,7 @@ static BoxArgs box_args(const pz_ctx *c, int star0) {
     b.invh = 2.0f / p.B;
     b.ctr = 0.5f * (p.B - 1);
     const double eps = 0.5 * p.B * c->lnr;
-    b.kapscale = (float)(1.0 / ((double)kKScale * eps * eps));
+    b.kapscale = (float)(1.0 / (std::ldexp(eps, c->uexp) * std::ldexp(eps, c->uexp)));
     b.A = p.d_A;
     b.C = p.d_C;
     b.E = p.d_E;
