@@ -122,7 +122,7 @@ __device__ __forceinline__ void dawson_taylor(float d, float a, const float *T, 
 // Core, small a: Dawson-derivative table (coefficient-major, in global or shared
 // memory).  x >= 0, x*x + a*a < 36, a < 0.5.  The Taylor order follows a (|d| <= 1/32):
 // measured in FP64 against the Faddeeva function over 0 <= x <= 6, the truncation stays
-// below 2.1e-8 with order 5 for a < 0.05, 3e-8 with order 6 for a < 0.1, 1.1e-8 with order 10 for a < 0.3 and 4e-9 with
+// below 3e-8 with order 6 for a < 0.1, 1.1e-8 with order 10 for a < 0.3 and 4e-9 with
 // order 14 for a < 0.5.  sin/cos of 2xa (< 6) use the MUFU forms (absolute error below
 // 5e-7, scaled by exp(a^2 - x^2) <= H in H and L).
 __device__ __forceinline__ void voigt_core_table(float x, float a, float &H, float &L, const float *tab) {
@@ -131,9 +131,7 @@ __device__ __forceinline__ void voigt_core_table(float x, float a, float &H, flo
     float d = x - (float)j * (1.0f / kDawsonPerUnit);
     const float *T = tab + j;
     float pr, pi;
-    if (a < 0.05f)
-        dawson_taylor<5>(d, a, T, pr, pi);
-    else if (a < 0.1f)
+    if (a < 0.1f)
         dawson_taylor<6>(d, a, T, pr, pi);
     else if (a < 0.3f)
         dawson_taylor<10>(d, a, T, pr, pi);

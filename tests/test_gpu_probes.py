@@ -38,6 +38,33 @@ def test_fp32_voigt_accuracy(oracle):
     assert derr.max() < 3e-5, (float(derr.max()), A[np.argmax(derr)], V[np.argmax(derr)])
 
 
+def test_core_table_keeps_the_sixth_order():
+    """Below a = 0.1 the core's Taylor sum of Dawson's integral runs to order 6.  The order-6 term of Im D is odd in
+    the distance d from the node, so the errors at +d and -d are subtracted (the table's own FP32 rounding is even
+    to leading order) and projected on it: 0 if the term is summed, 1 if it is dropped."""
+    special = pytest.importorskip("scipy.special")
+    rng = np.random.default_rng(6)
+    n = 100000
+    j = rng.integers(4, 92, n)
+    x = j / 16.0
+    a = rng.uniform(0.046, 0.0499, n).astype(np.float32)
+    d = a * rng.uniform(0.22, 0.32, n)             # arg(d + i a) near 75 degrees, where Im (d + i a)^6 is largest
+    D = [special.dawsn(x)]
+    D.append(1.0 - 2.0 * x * D[0])
+    for k in range(1, 6):
+        D.append(-2.0 * x * D[k] - 2.0 * k * D[k - 1])
+    A = a.astype(np.float64)
+    err, term = 0.0, 0.0
+    for sign in (1, -1):
+        v = (x + sign * d).astype(np.float32)
+        V = v.astype(np.float64)
+        err = err + sign * (voigt_gpu(a, v)[0] - special.wofz(V + 1j * A).real)
+        term = term + sign * 2.0 / np.sqrt(np.pi) * (D[6] / 720.0 * (V - x + 1j * A) ** 6).imag
+    w = 1.0 / special.wofz(x + 1j * A).real ** 2   # FP32 rounds in proportion to H
+    coef = np.sum(w * err * term) / np.sum(w * term * term)
+    assert abs(coef) < 0.2, coef
+
+
 def test_fp64_expn(oracle):
     import torch
     edges = np.array([2.0 ** -40, 2.0, 40.0, 0.5, 1.0, 0.25])
