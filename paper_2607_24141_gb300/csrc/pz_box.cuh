@@ -28,7 +28,8 @@
 // too.  Lines whose damping needs more than the widest class keep class 4 and are summed
 // directly over their whole window.  A window ends inside at most two further boxes on each
 // side; there f is almost constant over a box, a few k suffice, and the sharp end is kept by
-// prefix sums of the moments over the boxes' grid indices (one per index and layer).
+// moments of every grid index of the boxes by itself, which the points add up in the order in
+// which their windows reach the indices.
 // Pairs nearer than n_c stay with the far-wing kernels, which skip exactly the pairs that
 // are summed here (box_near).
 //
@@ -113,7 +114,7 @@ struct BoxArgs {
     const float *A;               // [3][kBoxK][kBoxK]: W_qk = sum_j A[q - 2][k][j] T_j, q = 2..4
     const float *C, *E;           // expansion and window-end tables
     const int *nmin;              // [S][nslab][4]
-    float *M, *PM, *N;            // moments [star][box][class][k][nd], prefixes [star][box][B][KE][nd],
+    float *M, *PM, *N;            // moments [star][box][class][k][nd], those of each grid index [star][box][B][KE][nd],
                                   // moments of G [star][target box][k][nd]
 };
 
@@ -211,8 +212,8 @@ struct BoxStage {
     int q[NP][box_chunk(NP)];
 };
 template <int NP>
-static size_t box_moment_smem(int KE, int nd) {
-    return sizeof(BoxStage<NP>) + sizeof(float) * (size_t)NP * nd * (4 * kBoxK + KE);
+static size_t box_moment_smem(int nd) {
+    return sizeof(BoxStage<NP>) + sizeof(float) * (size_t)NP * nd * 4 * kBoxK;
 }
 
 // Moments of one source box: thread = (part of the box's indices, layer), block = box (x) and star
@@ -230,7 +231,6 @@ __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b
     const bool live = part < NP;
     float *s_cls = reinterpret_cast<float *>(&sg + 1);          // [part][3][kBoxK][nd]: lines of classes 1..3
     float *s_m = s_cls + NP * 3 * kBoxK * nd;            // [part][kBoxK][nd]: class 0
-    float *s_pm = s_m + NP * kBoxK * nd;                 // [part][KE][nd]: totals of the prefixes
     const int32_t *start = gq.bstart + (int64_t)st * (kBoxSplit * b.nbox + 1) + kBoxSplit * box;
     const int i0 = (b.s_lo + box) * b.B;
     int most = 0;
@@ -280,11 +280,14 @@ __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b
 #pragma unroll
             for (int m = 0; m < kBoxBatch; ++m) {
                 if (lb + m >= n) break;
-                // prefixes up to the grid index before this line's
+                // the sums of the grid indices before this line's are complete
                 const int q = sg.q[part][lb + m];
                 for (; qcur < q; ++qcur)
 #pragma unroll
-                    for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * nd] = pm[k];
+                    for (int k = 0; k < KE; ++k) {
+                        PM[((int64_t)qcur * KE + k) * nd] = pm[k];
+                        pm[k] = 0.0f;
+                    }
                 if (cls[m] >= kBoxClasses) continue;
                 float v[kBoxK];
 #pragma unroll
@@ -308,23 +311,15 @@ __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b
     if (live) {
         for (; qcur < q1; ++qcur)
 #pragma unroll
-            for (int k = 0; k < KE; ++k) PM[((int64_t)qcur * KE + k) * nd] = pm[k];
+            for (int k = 0; k < KE; ++k) {
+                PM[((int64_t)qcur * KE + k) * nd] = pm[k];
+                pm[k] = 0.0f;
+            }
 #pragma unroll
         for (int k = 0; k < kBoxK; ++k) s_m[(part * kBoxK + k) * nd + d] = S.get(k);
-#pragma unroll
-        for (int k = 0; k < KE; ++k) s_pm[(part * KE + k) * nd + d] = pm[k];
     }
     __syncthreads();
     if (!live) return;
-    if (part > 0) {
-        // the prefixes of this part, from the start of the box
-#pragma unroll
-        for (int k = 0; k < KE; ++k) {
-            float off = 0.0f;
-            for (int q = 0; q < part; ++q) off += s_pm[(q * KE + k) * nd + d];
-            for (int q = q0; q < q1; ++q) PM[((int64_t)q * KE + k) * nd] += off;
-        }
-    }
     // sets by class, each with the classes below it
     float *M = b.M + ((int64_t)sl * b.nbox + box) * kBoxClasses * kBoxK * nd + d;
     for (int k = part; k < kBoxK; k += NP) {
@@ -387,20 +382,63 @@ __device__ __forceinline__ void box_translate_at(int P, const float *C, const fl
     }
 }
 
+// Window ends of target box t at one layer: the part of one of the boxes omax + 1 and omax + 2 on either
+// side (end: side and box) that the windows of the target's points reach, into out[r row].  The
+// indices are added in the order in which the windows reach them, so a line beyond a point's window
+// leaves no rounding there however strong it is (a difference of prefixes left 6e-8 of the line).
+template <int KE>
+__device__ __forceinline__ void box_ends(const BoxArgs &b, const float *PM, int nd, int t, int end, float *out, int row) {
+    const bool left = end >> 1;                // lines left of the points
+    const int e = end & 1, B = b.B;
+    const int s = t + (left ? -1 : 1) * (b.omax + 1 + e) - b.s_lo;
+    for (int r = 0; r < B; ++r) out[r * row] = 0.0f;
+    if (s < 0 || s >= b.nbox) return;
+    const float *m = PM + (int64_t)s * B * KE * nd, *E = b.E + (size_t)end * B * KE;
+    float P[KE];
+#pragma unroll
+    for (int k = 0; k < KE; ++k) P[k] = 0.0f;
+    auto put = [&](int r) {
+        float v = 0.0f;
+#pragma unroll
+        for (int k = 0; k < KE; ++k) v = fmaf(__ldg(E + r * KE + k), P[k], v);
+        out[r * row] = v;
+    };
+    // point r reaches the indices q <= r + rem - 1 - e B of a box to its right, q >= r - rem + 1 + e B to its left
+    const int off = e * B + 1 - b.rem;
+#pragma unroll 4
+    for (int j = 0; j < B; ++j) {
+        const int q = left ? B - 1 - j : j;
+#pragma unroll
+        for (int k = 0; k < KE; ++k) P[k] += m[((int64_t)q * KE + k) * nd];
+        const int r = left ? q - off : q + off;
+        if (r >= 0 && r < B) put(r);
+    }
+    // points whose window holds the whole box
+    if (left)
+        for (int r = min(B - 1, -off - 1); r >= 0; --r) put(r);
+    else
+        for (int r = max(0, B + off); r < B; ++r) put(r);
+}
+
 // Far field of a target box, added to the near-core sums.  kBoxSplit threads share a layer: each
 // takes every kBoxSplit-th offset, then every kBoxSplit-th point (one thread per layer left a
 // single spectrum's few boxes waiting on the chain of table and moment loads).  Bound by the latency
 // of those loads: 96 registers let two blocks of nine warps (72 layers) share an SM, where the 102
 // of the free choice left one (two stars on 43,000 lines: forward lines 2.38 -> 2.19 ms; 72
 // registers and three blocks spill and slow short grids, 0.419 -> 0.429 ms on 2,200 points).
+static size_t box_field_smem(int B, int nd) {
+    return sizeof(float) * kBoxSplit * ((size_t)kBoxK * nd + (size_t)B * (nd + 1));
+}
 template <int KE>
 __global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
-    extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [B][nd + 1]
+    extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [kBoxSplit][B][nd + 1]
     const int sl = blockIdx.y, st = b.star0 + sl, t = blockIdx.x;
     const LineArgs g = star_view(gq, st);
     const int nd = g.nd, part = threadIdx.x / nd, d = threadIdx.x - part * nd;
     const bool live = part < kBoxSplit;
-    float *s_phi = smem_f, *s_out = smem_f + kBoxSplit * kBoxK * nd;
+    const int row = nd + 1, pts = b.B * row;
+    float *s_phi = smem_f, *s_out = smem_f + kBoxSplit * kBoxK * nd;   // s_out: window ends, then the field
+    if (live) box_ends<KE>(b, b.PM + (int64_t)sl * b.nbox * b.B * KE * nd + d, nd, t, part, s_out + part * pts + d, row);
     if (live) {
         const int4 nm = *reinterpret_cast<const int4 *>(b.nmin + ((int64_t)st * gq.nslab + d / b.DS) * 4);
         const float *Mst = b.M + (int64_t)sl * b.nbox * kBoxClasses * kBoxK * nd + d;
@@ -431,46 +469,22 @@ __global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
 #pragma unroll
             for (int q = 1; q < kBoxSplit; ++q) phi[j] += s_phi[(q * kBoxK + j) * nd + d];
         }
-        const float *PMst = b.PM + (int64_t)sl * b.nbox * b.B * KE * nd + d;
-        const int64_t pbox = (int64_t)b.B * KE * nd;   // prefix stride of a box
         for (int r = part; r < b.B; r += kBoxSplit) {
             const float x = ((float)r - b.ctr) * b.invh;
-            float v = 0.0f;
-            // window ends: the part of the boxes omax + 1 and omax + 2 on each side that the
-            // window of point r reaches
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int s1 = t + b.omax + 1 + e - b.s_lo;          // lines right of the point: index <= q1
-                const int q1 = r + b.rem - 1 - e * b.B;
-                if (q1 >= 0 && s1 >= 0 && s1 < b.nbox) {
-                    const float *pm = PMst + s1 * pbox + (int64_t)min(q1, b.B - 1) * KE * nd;
-                    const float *E = b.E + ((size_t)e * b.B + r) * KE;
-#pragma unroll
-                    for (int k = 0; k < KE; ++k) v = fmaf(__ldg(E + k), pm[k * nd], v);
-                }
-                const int s2 = t - b.omax - 1 - e - b.s_lo;          // lines left of it: index >= q2
-                const int q2 = r - b.rem + 1 + e * b.B;
-                if (q2 < b.B && s2 >= 0 && s2 < b.nbox) {
-                    const float *pt = PMst + s2 * pbox + (int64_t)(b.B - 1) * KE * nd;
-                    const float *pq = PMst + s2 * pbox + (int64_t)max(q2 - 1, 0) * KE * nd;
-                    const float *E = b.E + ((size_t)(2 + e) * b.B + r) * KE;
-#pragma unroll
-                    for (int k = 0; k < KE; ++k)
-                        v = fmaf(__ldg(E + k), pt[k * nd] - (q2 > 0 ? pq[k * nd] : 0.0f), v);
-                }
-            }
+            float *out = s_out + r * row + d;
+            const float v = (out[0] + out[pts]) + (out[2 * pts] + out[3 * pts]);
             float T[kBoxK], s = 0.0f;
             box_cheb(x, T);
 #pragma unroll
             for (int j = kBoxK - 1; j >= 0; --j) s = fmaf(phi[j], T[j], s);
-            s_out[r * (nd + 1) + d] = v + s;
+            out[0] = v + s;
         }
     }
     __syncthreads();
     for (int k = threadIdx.x; k < b.B * nd; k += blockDim.x) {
-        const int row = k / b.B, col = k - row * b.B;
+        const int dl = k / b.B, col = k - dl * b.B;
         const int64_t i = (int64_t)t * b.B + col;
-        if (i < g.ld) g.knear[(int64_t)row * g.ld + i] += s_out[col * (nd + 1) + row];
+        if (i < g.ld) g.knear[(int64_t)dl * g.ld + i] += s_out[col * row + dl];
     }
 }
 

@@ -721,17 +721,19 @@ static cudaError_t launch_box_fwd_parts(pz_ctx *c, const LineArgs &g, cudaStream
     static std::atomic<bool> attr_set[kMaxDevices];
     if (!attr_set[c->device].load(std::memory_order_acquire)) {
         const cudaError_t e = cudaFuncSetAttribute(k_box_moments<KE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)box_moment_smem<NP>(KE, kMaxDepth));
+                                                   (int)box_moment_smem<NP>(kMaxDepth));
         if (e != cudaSuccess) return e;
+        const cudaError_t ef = cudaFuncSetAttribute(k_box_field<KE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)box_field_smem(32, kMaxDepth));
+        if (ef != cudaSuccess) return ef;
         attr_set[c->device].store(true, std::memory_order_release);
     }
     const int thr_m = (NP * c->nd + 31) / 32 * 32, thr_f = (kBoxSplit * c->nd + 31) / 32 * 32;
     for (int st = 0; st < c->S; st += c->box.chunk) {
         const int n = std::min(c->box.chunk, c->S - st);
         const BoxArgs b = box_args(c, st);
-        k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(KE, c->nd), s>>>(g, b);
-        k_box_field<KE><<<dim3(b.ntb, n), thr_f, sizeof(float) * (kBoxSplit * kBoxK * c->nd + b.B * (c->nd + 1)), s>>>(
-            g, b);
+        k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(c->nd), s>>>(g, b);
+        k_box_field<KE><<<dim3(b.ntb, n), thr_f, box_field_smem(b.B, c->nd), s>>>(g, b);
         c->launches += 2;
     }
     return cudaGetLastError();

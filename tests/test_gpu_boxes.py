@@ -69,3 +69,35 @@ def test_boxes_against_the_term_by_term_sum(name):
     for a, b in zip(got, ref):
         # FP32 sums: kappa 2e-7 and gradients up to 6e-7 measured with every pair summed directly
         assert np.linalg.norm(a - b) < 2e-6 * np.linalg.norm(b)
+
+
+def dominant_line_problem(W=511, n=3000, lines=4000, ratio=1e8):
+    """Weak lines in one box of 32 indices and one line 10^8 times stronger among them."""
+    at = I.make_atmosphere(5000.0, 4.0, 4, 3, log_abund_mean=-10.0)
+    grid = I.Grid(1600.0, 3e5, n)
+    rng = np.random.default_rng(3)
+    x = rng.uniform(1504.5, 1535.0, lines)       # indices 1505 .. 1535
+    x[0] = 1516.2
+    gf = rng.normal(-3.0, 0.3, lines)
+    gf[0] = -3.0 + np.log10(ratio)
+    const = lambda v: np.full(lines, v)          # noqa: E731
+    species = rng.integers(0, 4, lines)
+    species[0] = np.argmax(at.pop[:, 36])
+    parts = (1600.0 * np.exp(x * np.log1p(1 / 3e5)), gf, const(1.0), species, const(8.0), const(-5.5), const(-7.5))
+    return I.Problem("dominant", at, grid, I._pack([parts], W), I.make_kappa_c(at, grid))
+
+
+@pytest.mark.parametrize("W", [511, 500, 495])
+def test_points_past_a_dominant_lines_window(W):
+    """Where the window of a line that dwarfs its neighbours has ended the opacity is that of the others, to
+    FP32 rounding of their own sum."""
+    prob = dominant_line_problem(W)
+    got, launches = outputs(prob, pz.PZ_MIXED, 0.0, None)
+    ref, _ = outputs(prob, pz.PZ_FP64, 0.0, None)
+    assert launches == 5
+    err = np.abs(got[0] / np.where(ref[0] > 0, ref[0], 1.0) - 1)
+    for side in (np.arange(1516 + W + 1, 1530 + W), np.arange(1510 - W, 1516 - W)):
+        assert np.all(ref[0][:, side] > 0) and np.all(ref[0][:, side] < 1e-2 * ref[0][:, [1516 + W]])
+        assert err[:, side].max() < 2e-6
+    # beyond every window: nothing at all
+    assert np.all(got[0][:, 1536 + W:] == 0.0) and np.all(got[0][:, :1504 - W] == 0.0)
