@@ -243,18 +243,19 @@ static pz_status build_items(pz_ctx *c) {
         for (int k = 0; k < c->ns * c->nd; ++k)
             kmin = std::min(kmin, kC * (double)c->h_invdv[(size_t)st * c->ns * c->nd + k]);
         const double hw = 20.0 / (kmin * c->lnr) * 1.02 + 4.0;
+        const BoxGroup *gb = c->box.on(st) ? &c->box.groups[c->box.of[st]] : nullptr;
         for (int t = 0; t < nt; ++t) {
             for (int g = 0; g < ngf; ++g) {
                 // lines whose window touches the tile; with the box expansions those in the boxes
                 // nearer than every class of the group's slabs (the kernels gather the few others)
                 int64_t a = (int64_t)t * T - c->W, b = (int64_t)t * T + T - 1 + c->W;
-                if (c->box.B) {
+                if (gb) {
                     int n0 = 0;
                     for (int w = 0; w < c->tiling.GW; ++w)
                         n0 = std::max(n0, c->box.h_nmin[((size_t)st * c->nslab + g * c->tiling.GW + w) * 4]);
                     if (n0 < kBoxNever) {
-                        a = std::max(a, (int64_t)t * T - (int64_t)(n0 - 1) * c->box.B);
-                        b = std::min(b, (int64_t)t * T + T - 1 + (int64_t)(n0 - 1) * c->box.B);
+                        a = std::max(a, (int64_t)t * T - (int64_t)(n0 - 1) * gb->B);
+                        b = std::min(b, (int64_t)t * T + T - 1 + (int64_t)(n0 - 1) * gb->B);
                     }
                 }
                 const int lo =
@@ -307,7 +308,7 @@ static pz_status build_items(pz_ctx *c) {
             const int4 v = make_int4(it.v.x, it.v.y, lo, hi);
             const int4 ext = P > 1 ? make_int4(nslot, P, nsplit, q) : make_int4(-1, 1, -1, 0);
             fp.push_back({v, ext, it.cost / P});
-            if (hi > lo || c->box.B) bp.push_back({v, make_int4(0, P, 0, q), it.cost / P});
+            if (hi > lo || c->box.on(it.v.x)) bp.push_back({v, make_int4(0, P, 0, q), it.cost / P});
         }
         if (P > 1) {
             nslot += P;
@@ -426,16 +427,18 @@ static pz_status build_thresholds(pz_ctx *c) {
     // window end is that far.  Layers past the last one take the bounds of no line.
     BoxPlan &bx = c->box;
     bx.h_nmin.assign((size_t)c->S * nslab * 4, kBoxNever);
-    if (bx.B)
-        for (int st = 0; st < c->S; ++st)
-            for (int b = 0; b < nslab; ++b) {
-                float w = 0.0f;
-                for (int s = 0; s < c->ns; ++s) w = std::max(w, thr[((size_t)st * c->ns + s) * nslab + b]);
-                for (int k = 0; k < 4; ++k) {
-                    const int n = std::max(3, 1 + (int)std::ceil(std::ldexp((double)w, k) / bx.B));
-                    if (n <= bx.omax + 1) bx.h_nmin[((size_t)st * nslab + b) * 4 + k] = n;
-                }
+    for (int st = 0; st < c->S; ++st) {
+        if (!bx.on(st)) continue;
+        const BoxGroup &gb = bx.groups[bx.of[st]];
+        for (int b = 0; b < nslab; ++b) {
+            float w = 0.0f;
+            for (int s = 0; s < c->ns; ++s) w = std::max(w, thr[((size_t)st * c->ns + s) * nslab + b]);
+            for (int k = 0; k < 4; ++k) {
+                const int n = std::max(3, 1 + (int)std::ceil(std::ldexp((double)w, k) / gb.B));
+                if (n <= gb.omax + 1) bx.h_nmin[((size_t)st * nslab + b) * 4 + k] = n;
             }
+        }
+    }
     dfree(bx.d_nmin);
     bx.d_nmin = nullptr;
     PZ_TRY(upload(&bx.d_nmin, bx.h_nmin, "box offsets"));
@@ -444,14 +447,22 @@ static pz_status build_thresholds(pz_ctx *c) {
 
 // Device tables and workspace of the box expansions (once per context).
 static pz_status build_boxes(pz_ctx *c) {
-    BoxPlan &b = c->box;
-    if (!b.B) return PZ_OK;
+    BoxPlan &p = c->box;
+    if (p.groups.empty()) return PZ_OK;
     const size_t K = 14, row = 16;   // moments per box, row of the tables
-    PZ_TRY(dalloc(&b.d_C, (size_t)2 * (b.omax + 3) * K * row, "box tables"));
-    PZ_TRY(dalloc(&b.d_E, (size_t)4 * b.B * b.KE, "box tables"));
-    PZ_TRY(dalloc(&b.d_A, 3 * K * K, "box tables"));
-    PZ_TRY(dalloc(&b.d_start, (size_t)c->S * (kBoxQuarters * b.nbox + 1), "box tables"));
-    PZ_TRY(dalloc(&b.d_ws, box_workspace_floats(c, b.chunk), "box workspace"));
+    std::vector<int4> geo(c->S, make_int4(0, 0, 0, 0));
+    size_t ws = 0;
+    for (BoxGroup &b : p.groups) {
+        PZ_TRY(dalloc(&b.d_C, (size_t)2 * (b.omax + 3) * K * row, "box tables"));
+        PZ_TRY(dalloc(&b.d_E, (size_t)4 * b.B * b.KE, "box tables"));
+        PZ_TRY(dalloc(&b.d_A, 3 * K * K, "box tables"));
+        for (int k = 0; k < b.count; ++k) geo[p.stars[b.first + k]] = make_int4(b.B, b.sh, b.s_lo, b.nbox);
+        ws = std::max(ws, box_workspace_floats(c, b, b.chunk));
+    }
+    PZ_TRY(upload(&p.d_geo, geo, "box tables"));
+    PZ_TRY(upload(&p.d_stars, p.stars, "box tables"));
+    PZ_TRY(dalloc(&p.d_start, (size_t)c->S * p.stride, "box tables"));
+    PZ_TRY(dalloc(&p.d_ws, ws, "box workspace"));
     return cuda_check(launch_box_tables(c), "box tables");
 }
 
@@ -478,8 +489,13 @@ static void destroy_ctx(pz_ctx *c) {
                     c->d_Gt64, c->d_gacc, c->d_gline, c->d_gab, c->d_dLdf, c->d_finfo, c->d_status,
                     c->d_keep, c->L.gradbase, c->L.g4base, c->L.dgrad, c->L.dg4, c->d_mdgrad, c->d_mdg4,
                     c->d_grp_of, c->d_grp_off, c->d_grp_mem, c->d_sigma,
-                    c->box.d_nmin, c->box.d_start, c->box.d_A, c->box.d_C, c->box.d_E, c->box.d_ws, c->box.d_wide};
+                    c->box.d_nmin, c->box.d_start, c->box.d_stars, c->box.d_geo, c->box.d_ws, c->box.d_wide};
     for (void *p : ptrs) dfree(p);
+    for (BoxGroup &b : c->box.groups) {
+        dfree(b.d_A);
+        dfree(b.d_C);
+        dfree(b.d_E);
+    }
     destroy_marks(c->marks);
     destroy_marks(c->cap_marks);
     for (auto e : c->ev_pool) cudaEventDestroy(e);
@@ -617,7 +633,7 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         lg_6(n), zeros(n, 0.0f);
     std::vector<double> Qb(n), x64(n);
     const double C0 = kPI * kE * kE / (kME * kC) / kSQRTPI;
-    int64_t evals = 0;
+    std::vector<int64_t> evals(S, 0);    // (line, point, layer) terms of each star
     for (int64_t k = 0; k < n; ++k) {
         int64_t l = keep[k];
         double il = std::floor(x[l] + 0.5);
@@ -640,9 +656,9 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         lg_4[k] = ll->log_gamma4[l];
         lg_6[k] = ll->log_gamma6[l];
         int64_t i0 = std::max<int64_t>(0, (int64_t)il - c->W), i1 = std::min<int64_t>(nlam - 1, (int64_t)il + c->W);
-        evals += (i1 - i0 + 1);
+        evals[kstar[k]] += (i1 - i0 + 1) * nd;
     }
-    c->n_evals = evals * nd;
+    c->n_evals = std::accumulate(evals.begin(), evals.end(), (int64_t)0);
     c->h_il = il32;
     std::vector<float> mzeros(std::max<int64_t>(nl, 1), 0.0f);
     if (upload(&c->L.orig, orig, "lines") || upload(&c->L.star, kstar, "lines") || upload(&c->L.il32, il32, "lines") ||
@@ -703,8 +719,7 @@ static pz_status create_impl(int S, const pz_atmos *atv, const pz_linelist *ll, 
         const float kf = (float)kC * invdv[o];
         Ksd[o] = std::ldexp(1.0f, 2 * c->uexp) / (kf * kf);
     }
-    // widest near zone (20 Doppler widths, in grid points) over stars, species and layers
-    box_choose(c, 20.0 / (kC * (double)*std::min_element(invdv.begin(), invdv.end()) * c->lnr));
+    box_choose(c, evals);
     std::vector<double> dab(1, 0.0);
     std::vector<int32_t> eos(ns, -1);
     if (upload(&c->d_m, c->h_m, "depth") || upload(&c->d_T, c->h_T, "depth") || upload(&c->d_beta_hi, bh, "depth") ||
@@ -789,7 +804,7 @@ static pz_status ensure_far_tables(pz_ctx *c) {
         }
         c->finfo_cap = ib;
     }
-    const size_t wb = c->box.B ? box_wide_bytes(c) : 0;
+    const size_t wb = c->box.groups.empty() ? 0 : box_wide_bytes(c);
     if (c->box.wide_cap < wb) {
         dfree(c->box.d_wide);
         c->box.d_wide = nullptr;

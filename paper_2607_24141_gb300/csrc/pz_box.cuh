@@ -92,8 +92,9 @@ __global__ void k_box_edges(int B, int omax, int KE, const float *C, float *E) {
 }
 
 // First line of every quarter of a box: start[star][q] = first line of the star with i_l >= s_lo B + q B/4.
-__global__ void k_box_start(int nq, int s_lo, int B, const int32_t *il, const int64_t *off, int32_t *start) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x, st = blockIdx.y;
+__global__ void k_box_start(int nq, int s_lo, int B, const int32_t *stars, const int32_t *il, const int64_t *off,
+                            int64_t row, int32_t *start) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, st = stars[blockIdx.y];
     if (b > nq) return;
     int64_t lo = off[st], hi = off[st + 1];
     const int64_t key = (int64_t)s_lo * B + (int64_t)b * (B / kBoxSplit);
@@ -101,14 +102,14 @@ __global__ void k_box_start(int nq, int s_lo, int B, const int32_t *il, const in
         const int64_t mid = (lo + hi) >> 1;
         if (il[mid] < key) lo = mid + 1; else hi = mid;
     }
-    start[(int64_t)st * (nq + 1) + b] = (int32_t)lo;
+    start[(int64_t)st * row + b] = (int32_t)lo;
 }
 
 struct BoxArgs {
     int B, omax, rem;             // box, widest whole offset, (W + 1) - (omax + 1) B
     int s_lo, nbox, ntb;          // first source box, source boxes, target boxes
     int DC, DS;                   // tiling of the line records (class bits)
-    int star0;                    // first star of this launch
+    const int32_t *stars;         // stars of this launch
     float invh, ctr;              // 2/B, (B - 1)/2
     float kapscale;               // kap = K kapscale (K = 4^uexp/k^2)
     const float *A;               // [3][kBoxK][kBoxK]: W_qk = sum_j A[q - 2][k][j] T_j, q = 2..4
@@ -225,13 +226,13 @@ __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b
     constexpr int QP = kBoxSplit / NP, CH = box_chunk(NP);   // quarters per part, lines per chunk
     extern __shared__ float4 smem4[];
     BoxStage<NP> &sg = *reinterpret_cast<BoxStage<NP> *>(smem4);
-    const int tid = threadIdx.x, box = blockIdx.x, sl = blockIdx.y, st = b.star0 + sl;
+    const int tid = threadIdx.x, box = blockIdx.x, sl = blockIdx.y, st = b.stars[sl];
     const LineArgs g = star_view(gq, st);
     const int nd = g.nd, part = tid / nd, d = tid - part * nd;
     const bool live = part < NP;
     float *s_cls = reinterpret_cast<float *>(&sg + 1);          // [part][3][kBoxK][nd]: lines of classes 1..3
     float *s_m = s_cls + NP * 3 * kBoxK * nd;            // [part][kBoxK][nd]: class 0
-    const int32_t *start = gq.bstart + (int64_t)st * (kBoxSplit * b.nbox + 1) + kBoxSplit * box;
+    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * box;
     const int i0 = (b.s_lo + box) * b.B;
     int most = 0;
 #pragma unroll
@@ -432,7 +433,7 @@ static size_t box_field_smem(int B, int nd) {
 template <int KE>
 __global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [kBoxSplit][B][nd + 1]
-    const int sl = blockIdx.y, st = b.star0 + sl, t = blockIdx.x;
+    const int sl = blockIdx.y, st = b.stars[sl], t = blockIdx.x;
     const LineArgs g = star_view(gq, st);
     const int nd = g.nd, part = threadIdx.x / nd, d = threadIdx.x - part * nd;
     const bool live = part < kBoxSplit;
@@ -491,7 +492,7 @@ __global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
 // Chebyshev moments of G stim over the points of a target box: thread = layer.
 __global__ void __launch_bounds__(128) k_box_gmoments(LineArgs gq, BoxArgs b) {
     extern __shared__ float s_g[];            // [nd][B + 1]
-    const int d = threadIdx.x, sl = blockIdx.y, st = b.star0 + sl, t = blockIdx.x;
+    const int d = threadIdx.x, sl = blockIdx.y, st = b.stars[sl], t = blockIdx.x;
     const LineArgs g = star_view(gq, st);
     for (int k = threadIdx.x; k < b.B * g.nd; k += blockDim.x) {
         const int row = k / b.B, col = k - row * b.B;
@@ -533,9 +534,9 @@ template <int KE, bool FOUR>
 __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int box = blockIdx.x, sl = blockIdx.y, st = b.star0 + sl;
+    const int box = blockIdx.x, sl = blockIdx.y, st = b.stars[sl];
     const LineArgs g = star_view(gq, st);
-    const int32_t *start = gq.bstart + (int64_t)st * (kBoxSplit * b.nbox + 1) + kBoxSplit * box;
+    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * box;
     const int lo = start[0], hi = start[kBoxSplit];
     if (lo >= hi) return;
     // the block's layers dz .. dz + nd

@@ -54,10 +54,12 @@ struct LineArgs {
     const uint32_t *keep;                           // centre-test mask [nl][kKeepWords] or NULL (all kept)
     // box expansions (pz_box.cuh): pairs they sum are skipped by the far-wing kernels
     int tDC, tDS;                                   // layers per depth group and slab of the line records
-    int boxB, boxsh, s_lo, nbox;                    // box points (0: off) and log2, first source box, boxes
+    int boxB, boxsh, s_lo, nbox;                    // of the star: box points (0: off) and log2, first source box, boxes
+    const int4 *bgeo;                               // [S] the four above (NULL: off for every star)
+    int64_t brow;                                   // row of bstart
     float shrink;                                   // |v| >= |Delta| ln r shrink k over a window
     const int *nmin;                                // [S][nslab][4] nearest offset of each class
-    const int32_t *bstart;                          // [S][4 nbox + 1] first line of each quarter of a box
+    const int32_t *bstart;                          // [S][brow] first line of each quarter of a box
     uint32_t *wide;                                 // [4][nslab][wwords] lines of class >= 1..4
     int64_t wwords;
 };
@@ -82,6 +84,13 @@ __device__ __forceinline__ LineArgs star_view(const LineArgs &g, int s) {
     v.kline += s * g.bstride;
     v.knear += s * g.bstride;
     v.Gt += s * g.bstride;
+    if (g.bgeo) {
+        const int4 q = __ldg(g.bgeo + s);
+        v.boxB = q.x;
+        v.boxsh = q.y;
+        v.s_lo = q.z;
+        v.nbox = q.w;
+    }
     return v;
 }
 
@@ -508,7 +517,7 @@ template <class F>
 __device__ __forceinline__ void box_rings(const LineArgs &g, const BoxView &v, int st, int slab, int n0g, int t0, int T,
                                           int q, int P, const WarpStage &ws, int LC, int lane, F &&f) {
     if (!g.boxB || n0g >= kBoxNever) return;
-    const int32_t *bs = g.bstart + (int64_t)st * (kBoxQuarters * g.nbox + 1);
+    const int32_t *bs = g.bstart + (int64_t)st * g.brow;
     int below = n0g;
     for (int c = 1; c <= kBoxClasses; ++c) {
         const int n = box_nmin(v, c);

@@ -92,22 +92,33 @@ struct LineTable {
     float *dgrad = nullptr, *dg4 = nullptr;
 };
 
-// Box expansions of the far wings (pz_box.cuh): geometry, tables and workspace.  B = 0: off, the
-// far-wing kernels sum every pair of a line's window.
-struct BoxPlan {
+// Box expansions of the far wings (pz_box.cuh).  Whether a star uses them and its box size follow from
+// the star's own lines and widths, so that its sums do not change with the other stars of a batch.
+// The stars of one box size share geometry, tables and launches.
+struct BoxGroup {
     int B = 0;                  // grid points per box (a power of two; 32 J is a multiple of it)
     int sh = 0;                 // log2 B
     int omax = 0, rem = 0;      // widest whole offset; (W + 1) - (omax + 1) B
     int s_lo = 0, nbox = 0, ntb = 0;   // first source box, source boxes, target boxes
     int KE = 0;                 // moments kept per grid index for the window ends
+    int first = 0, count = 0;   // its stars: [first, first + count) of BoxPlan::stars
     int chunk = 0;              // stars per launch (bounds the workspace)
-    int *d_nmin = nullptr;      // [S][nslab][4] nearest offset of each separation class
-    int32_t *d_start = nullptr; // [S][4 nbox + 1] first line of each quarter of a box
     float *d_A = nullptr, *d_C = nullptr, *d_E = nullptr;
-    float *d_ws = nullptr;      // moments and prefixes, or the moments of G
-    uint32_t *d_wide = nullptr; // [4][nslab][words] lines of class >= 1..4, one bit per line
+};
+struct BoxPlan {
+    std::vector<BoxGroup> groups;      // empty: the far-wing kernels sum every pair of a line's window
+    std::vector<int> of;               // [S] group of each star (-1: none)
+    std::vector<int32_t> stars;        // stars in order of their groups
+    int64_t stride = 0;                // row of d_start: 4 nbox + 1 of the widest group
+    int32_t *d_stars = nullptr;
+    int4 *d_geo = nullptr;             // [S] (B, sh, s_lo, nbox), B = 0: none
+    int *d_nmin = nullptr;             // [S][nslab][4] nearest offset of each separation class
+    int32_t *d_start = nullptr;        // [S][stride] first line of each quarter of a box
+    float *d_ws = nullptr;             // moments, or the moments of G
+    uint32_t *d_wide = nullptr;        // [4][nslab][words] lines of class >= 1..4, one bit per line
     size_t wide_cap = 0;
     std::vector<int> h_nmin;
+    bool on(int star) const { return !of.empty() && of[star] >= 0; }
 };
 constexpr int kBoxQuarters = 4;      // parts of a box with a first line of their own
 constexpr int kBoxNever = 1 << 28;   // offset of a class that does not exist
@@ -325,8 +336,9 @@ bool tiling_supported(int J, int DS, int minb);
 bool tiling_fits(const Tiling &t);   // both far-wing chunks fit in shared memory
 size_t far_info_bytes(const pz_ctx *c);
 size_t box_wide_bytes(const pz_ctx *c);
-size_t box_workspace_floats(const pz_ctx *c, int stars);
-void box_choose(pz_ctx *c, double thr_max);          // geometry of the box expansions (host)
+size_t box_workspace_floats(const pz_ctx *c, const BoxGroup &b, int stars);
+// which stars use the box expansions, and their geometry (host); evals: (line, point, layer) terms per star
+void box_choose(pz_ctx *c, const std::vector<int64_t> &evals);
 cudaError_t launch_box_tables(pz_ctx *c);            // fills their device tables
 
 }  // namespace pz

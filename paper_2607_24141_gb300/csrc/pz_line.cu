@@ -172,12 +172,12 @@ __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, L
         }
         amask = (ok ? 1 << w : 0) | (wide ? 16 << w : 0) | (none ? 256 << w : 0);
         int cls = kBoxClasses;
-        if (gq.boxB) {
-            if (in) {
+        if (gq.bgeo) {
+            if (in && g.boxB) {
                 need *= 9.0f / (gq.lnr * gq.shrink);
                 const int *n = gq.nmin + ((int64_t)st * gq.nslab + grp * (DC / DS) + w) * 4;
                 for (int c = kBoxClasses - 1; c >= 0; --c)
-                    if (n[c] < kBoxNever && (float)((n[c] - 1) * gq.boxB) >= need) cls = c;
+                    if (n[c] < kBoxNever && (float)((n[c] - 1) * g.boxB) >= need) cls = c;
             }
             for (int c = 1; c <= kBoxClasses; ++c) {
                 const unsigned m = __ballot_sync(0xffffffffu, in && !none && cls >= c);
@@ -518,10 +518,9 @@ static LineArgs make_args(pz_ctx *c) {
     g.tstride = (int64_t)c->ns * c->nslab;
     g.tDC = c->tiling.depth_per_cta();
     g.tDS = c->tiling.DS;
-    g.boxB = c->box.B;
-    g.boxsh = c->box.sh;
-    g.s_lo = c->box.s_lo;
-    g.nbox = c->box.nbox;
+    g.boxB = g.boxsh = g.s_lo = g.nbox = 0;
+    g.bgeo = c->box.d_geo;
+    g.brow = c->box.stride;
     g.shrink = (float)std::max(0.5, 1.0 - 0.5 * (c->W + 1024.0) * c->lnr);
     g.nmin = c->box.d_nmin;
     g.bstart = c->box.d_start;
@@ -609,42 +608,61 @@ size_t far_info_bytes(const pz_ctx *c) {
 // ---- box expansions: host side -------------------------------------------------
 constexpr size_t kBoxWorkspace = (size_t)1 << 30;   // bytes per launch aimed at (stars are taken in chunks)
 
-// Geometry of the expansions.  A box of B points, a power of two near half the widest near zone
-// (thr_max: 20 Doppler widths in grid points), so that the nearest pairs are 3 or 4 boxes apart:
-// smaller boxes raise the pairs as 1/B^2, larger ones the points left to the direct sum.
-void box_choose(pz_ctx *c, double thr_max) {
-    BoxPlan &b = c->box;
-    b.B = b.sh = 0;
-    if (c->prec != PZ_MIXED || c->L.n == 0) return;
-    int sh = 2;
-    while (sh < 5 && thr_max >= 2.5 * (1 << sh)) ++sh;
-    const int B = 1 << sh;
-    const int64_t omax = (c->W + 1) / B - 1;
-    // the window ends' tables need a wide offset (few moments), and at least some whole boxes
-    if (omax < 8) return;
-    // the expansions cost a fixed amount per (point, layer) and some 0.1 ms of latency per pass:
-    // below about 200 lines per window, or 2e8 (line, point, layer) terms in all, the direct sum
-    // is as fast (574 points x 1,416 lines, 3.5e7 terms: 0.63 ms direct, 0.72 ms with boxes; 4,000 x
-    // 2,000, 2.5e8: 0.22 against 0.18 ms; 2,200 x 12,000, 1.7e9, with the reverse pass: 1.35 against
-    // 0.92 ms; 37,550 x 200,000, 4.3e10: 23.0 against 7.0 ms, near cores aside)
-    const double per_window = (double)c->L.n / c->S / (double)c->nlam * (2.0 * c->W + 1.0);
-    if (per_window < 200.0 || (double)c->n_evals < 2e8) return;
-    b.B = B;
-    b.sh = sh;
-    b.omax = (int)omax;
-    b.rem = c->W + 1 - (int)(omax + 1) * B;
-    b.s_lo = -((c->W + B - 1) / B);
-    b.nbox = (int)((c->nlam - 1 + c->W) / B) - b.s_lo + 1;
-    b.ntb = (int)((c->nlam + B - 1) / B);
-    b.KE = box_order((int)omax + 1) + 1 <= 5 ? 5 : 8;
-    b.chunk = 1;
-    while (b.chunk < c->S && box_workspace_floats(c, b.chunk + 1) * sizeof(float) <= kBoxWorkspace) ++b.chunk;
+// Which stars use the expansions, and their geometry.  A box of B points, a power of two near half
+// the star's widest near zone (20 Doppler widths in grid points), so that the nearest pairs are 3 or 4
+// boxes apart: smaller boxes raise the pairs as 1/B^2, larger ones the points left to the direct sum.
+void box_choose(pz_ctx *c, const std::vector<int64_t> &evals) {
+    BoxPlan &p = c->box;
+    p.of.assign(c->S, -1);
+    if (c->prec != PZ_MIXED) return;
+    std::vector<int> size(c->S, 0);      // log2 B of each star, 0: no boxes
+    const size_t row = (size_t)c->ns * c->nd;
+    for (int st = 0; st < c->S; ++st) {
+        // the expansions cost a fixed amount per (point, layer) and some 0.1 ms of latency per pass:
+        // below about 200 lines per window, or 2e8 (line, point, layer) terms, the direct sum
+        // is as fast (574 points x 1,416 lines, 3.5e7 terms: 0.63 ms direct, 0.72 ms with boxes; 4,000 x
+        // 2,000, 2.5e8: 0.22 against 0.18 ms; 2,200 x 12,000, 1.7e9, with the reverse pass: 1.35 against
+        // 0.92 ms; 37,550 x 200,000, 4.3e10: 23.0 against 7.0 ms, near cores aside)
+        const double lines = (double)(c->h_line_off[st + 1] - c->h_line_off[st]);
+        const double per_window = lines / (double)c->nlam * (2.0 * c->W + 1.0);
+        if (per_window < 200.0 || (double)evals[st] < 2e8) continue;
+        const auto inv = c->h_invdv.begin() + st * row;
+        const double thr = 20.0 / (kC * (double)*std::min_element(inv, inv + row) * c->lnr);
+        int sh = 2;
+        while (sh < 5 && thr >= 2.5 * (1 << sh)) ++sh;
+        // the window ends' tables need a wide offset (few moments), and at least some whole boxes
+        if ((c->W + 1) / (1 << sh) - 1 >= 8) size[st] = sh;
+    }
+    for (int sh = 2; sh <= 5; ++sh) {
+        BoxGroup b;
+        b.first = (int)p.stars.size();
+        for (int st = 0; st < c->S; ++st)
+            if (size[st] == sh) {
+                p.of[st] = (int)p.groups.size();
+                p.stars.push_back(st);
+            }
+        b.count = (int)p.stars.size() - b.first;
+        if (b.count == 0) continue;
+        b.sh = sh;
+        b.B = 1 << sh;
+        b.omax = (c->W + 1) / b.B - 1;
+        b.rem = c->W + 1 - (b.omax + 1) * b.B;
+        b.s_lo = -((c->W + b.B - 1) / b.B);
+        b.nbox = (int)((c->nlam - 1 + c->W) / b.B) - b.s_lo + 1;
+        b.ntb = (int)((c->nlam + b.B - 1) / b.B);
+        b.KE = box_order(b.omax + 1) + 1 <= 5 ? 5 : 8;
+        b.chunk = 1;
+        while (b.chunk < b.count && box_workspace_floats(c, b, b.chunk + 1) * sizeof(float) <= kBoxWorkspace) ++b.chunk;
+        p.stride = std::max<int64_t>(p.stride, (int64_t)kBoxSplit * b.nbox + 1);
+        p.groups.push_back(b);
+    }
 }
 
-static size_t box_moment_floats(const pz_ctx *c) { return (size_t)c->box.nbox * kBoxClasses * kBoxK * c->nd; }
-size_t box_workspace_floats(const pz_ctx *c, int stars) {
-    const BoxPlan &b = c->box;
-    const size_t fwd = box_moment_floats(c) + (size_t)b.nbox * b.B * b.KE * c->nd;
+static size_t box_moment_floats(const pz_ctx *c, const BoxGroup &b) {
+    return (size_t)b.nbox * kBoxClasses * kBoxK * c->nd;
+}
+size_t box_workspace_floats(const pz_ctx *c, const BoxGroup &b, int stars) {
+    const size_t fwd = box_moment_floats(c, b) + (size_t)b.nbox * b.B * b.KE * c->nd;
     const size_t bwd = (size_t)b.ntb * kBoxK * c->nd;
     return std::max(fwd, bwd) * stars;
 }
@@ -652,12 +670,11 @@ size_t box_wide_bytes(const pz_ctx *c) {
     return (size_t)kBoxClasses * c->nslab * (size_t)((c->L.n + 31) / 32) * sizeof(uint32_t);
 }
 
-cudaError_t launch_box_tables(pz_ctx *c) {
-    const BoxPlan &b = c->box;
+static cudaError_t launch_box_group_tables(pz_ctx *c, const BoxGroup &b) {
     k_box_tables<<<dim3(b.omax + 2, 2), 256>>>(b.B, c->lnr, b.omax, b.d_C);
     k_box_edges<<<dim3(b.B, 2, 2), 32>>>(b.B, b.omax, b.KE, b.d_C, b.d_E);
-    k_box_start<<<dim3(kBoxSplit * b.nbox / 256 + 1, c->S), 256>>>(kBoxSplit * b.nbox, b.s_lo, b.B, c->L.il32,
-                                                                 c->d_line_off, b.d_start);
+    k_box_start<<<dim3(kBoxSplit * b.nbox / 256 + 1, b.count), 256>>>(
+        kBoxSplit * b.nbox, b.s_lo, b.B, c->box.d_stars + b.first, c->L.il32, c->d_line_off, c->box.stride, c->box.d_start);
     // operators of f^2, f^3, f^4 on the Chebyshev basis: column k of (1/m)(d + p eps)(d + q eps)
     const double eps = 0.5 * b.B * c->lnr;
     std::vector<double> cur((size_t)kBoxK * kBoxK, 0.0);   // [k][j]: image of T_k as coefficients of T_j
@@ -684,8 +701,16 @@ cudaError_t launch_box_tables(pz_ctx *c) {
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-static BoxArgs box_args(const pz_ctx *c, int star0) {
-    const BoxPlan &p = c->box;
+cudaError_t launch_box_tables(pz_ctx *c) {
+    for (const BoxGroup &b : c->box.groups) {
+        const cudaError_t e = launch_box_group_tables(c, b);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// Arguments of the stars [first, ...) of BoxPlan::stars, all of group p.
+static BoxArgs box_args(const pz_ctx *c, const BoxGroup &p, int first) {
     BoxArgs b;
     b.B = p.B;
     b.omax = p.omax;
@@ -695,7 +720,7 @@ static BoxArgs box_args(const pz_ctx *c, int star0) {
     b.ntb = p.ntb;
     b.DC = c->tiling.depth_per_cta();
     b.DS = c->tiling.DS;
-    b.star0 = star0;
+    b.stars = c->box.d_stars + first;
     b.invh = 2.0f / p.B;
     b.ctr = 0.5f * (p.B - 1);
     const double eps = 0.5 * p.B * c->lnr;
@@ -703,21 +728,21 @@ static BoxArgs box_args(const pz_ctx *c, int star0) {
     b.A = p.d_A;
     b.C = p.d_C;
     b.E = p.d_E;
-    b.nmin = p.d_nmin;
-    b.M = p.d_ws;
-    b.PM = p.d_ws + (size_t)p.chunk * box_moment_floats(c);
-    b.N = p.d_ws;
+    b.nmin = c->box.d_nmin;
+    b.M = c->box.d_ws;
+    b.PM = c->box.d_ws + (size_t)p.chunk * box_moment_floats(c, p);
+    b.N = c->box.d_ws;
     return b;
 }
 
 // Fewer than two boxes per SM: the boxes' blocks are cut further (by indices of the box or layers).
-static bool box_few(const pz_ctx *c) {
-    return (int64_t)c->box.nbox * std::min(c->box.chunk, c->S) < 2 * (int64_t)c->n_sm;
+static bool box_few(const pz_ctx *c, const BoxGroup &p) {
+    return (int64_t)p.nbox * std::min(p.chunk, p.count) < 2 * (int64_t)c->n_sm;
 }
 
 // Forward: moments of the lines, then the far field of every point into knear.
 template <int KE, int NP>
-static cudaError_t launch_box_fwd_parts(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+static cudaError_t launch_box_fwd_parts(pz_ctx *c, const BoxGroup &p, const LineArgs &g, cudaStream_t s) {
     static std::atomic<bool> attr_set[kMaxDevices];
     if (!attr_set[c->device].load(std::memory_order_acquire)) {
         const cudaError_t e = cudaFuncSetAttribute(k_box_moments<KE, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -729,9 +754,9 @@ static cudaError_t launch_box_fwd_parts(pz_ctx *c, const LineArgs &g, cudaStream
         attr_set[c->device].store(true, std::memory_order_release);
     }
     const int thr_m = (NP * c->nd + 31) / 32 * 32, thr_f = (kBoxSplit * c->nd + 31) / 32 * 32;
-    for (int st = 0; st < c->S; st += c->box.chunk) {
-        const int n = std::min(c->box.chunk, c->S - st);
-        const BoxArgs b = box_args(c, st);
+    for (int k = 0; k < p.count; k += p.chunk) {
+        const int n = std::min(p.chunk, p.count - k);
+        const BoxArgs b = box_args(c, p, p.first + k);
         k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(c->nd), s>>>(g, b);
         k_box_field<KE><<<dim3(b.ntb, n), thr_f, box_field_smem(b.B, c->nd), s>>>(g, b);
         c->launches += 2;
@@ -739,17 +764,17 @@ static cudaError_t launch_box_fwd_parts(pz_ctx *c, const LineArgs &g, cudaStream
     return cudaGetLastError();
 }
 template <int KE>
-static cudaError_t launch_box_fwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
-    return box_few(c) ? launch_box_fwd_parts<KE, kBoxSplit>(c, g, s) : launch_box_fwd_parts<KE, 1>(c, g, s);
+static cudaError_t launch_box_fwd(pz_ctx *c, const BoxGroup &p, const LineArgs &g, cudaStream_t s) {
+    return box_few(c, p) ? launch_box_fwd_parts<KE, kBoxSplit>(c, p, g, s) : launch_box_fwd_parts<KE, 1>(c, p, g, s);
 }
 
 // Backward: moments of G, then every line's sums over the points its boxes reach, into gacc.
 template <int KE, bool FOUR>
-static cudaError_t launch_box_bwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) {
+static cudaError_t launch_box_bwd(pz_ctx *c, const BoxGroup &p, const LineArgs &g, cudaStream_t s) {
     const int thr = (c->nd + 31) / 32 * 32;
     // several blocks per box, each with part of the layers, where the lines fill few boxes
-    const int nz = box_few(c) ? std::min(3, c->nd) : 1;
-    const size_t smem = box_grad_smem(c->box.B, KE, (c->nd + nz - 1) / nz);
+    const int nz = box_few(c, p) ? std::min(3, c->nd) : 1;
+    const size_t smem = box_grad_smem(p.B, KE, (c->nd + nz - 1) / nz);
     static std::atomic<bool> attr_set[kMaxDevices];
     if (!attr_set[c->device].load(std::memory_order_acquire)) {
         const cudaError_t e = cudaFuncSetAttribute(k_box_grad<KE, FOUR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -757,9 +782,9 @@ static cudaError_t launch_box_bwd(pz_ctx *c, const LineArgs &g, cudaStream_t s) 
         if (e != cudaSuccess) return e;
         attr_set[c->device].store(true, std::memory_order_release);
     }
-    for (int st = 0; st < c->S; st += c->box.chunk) {
-        const int n = std::min(c->box.chunk, c->S - st);
-        const BoxArgs b = box_args(c, st);
+    for (int k = 0; k < p.count; k += p.chunk) {
+        const int n = std::min(p.chunk, p.count - k);
+        const BoxArgs b = box_args(c, p, p.first + k);
         k_box_gmoments<<<dim3(b.ntb, n), thr, sizeof(float) * c->nd * (b.B + 1), s>>>(g, b);
         k_box_grad<KE, FOUR><<<dim3(b.nbox, n, nz), 32 * kBoxGradWarps, smem, s>>>(g, b);
         c->launches += 2;
@@ -796,8 +821,8 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
     g.n_items = c->n_fitems;
     g.ngroups = ngroups;
     g.ctr = c->d_ctr + 1;
-    if (c->box.B) {
-        e = c->box.KE == 5 ? launch_box_fwd<5>(c, g, s) : launch_box_fwd<8>(c, g, s);
+    for (const BoxGroup &p : c->box.groups) {
+        e = p.KE == 5 ? launch_box_fwd<5>(c, p, g, s) : launch_box_fwd<8>(c, p, g, s);
         if (e != cudaSuccess) return e;
     }
     if (c->n_fsplit > 0) {
@@ -827,9 +852,9 @@ cudaError_t launch_line_bwd_mixed(pz_ctx *c, cudaStream_t s, bool four) {
             e = launch_far_info(c, gb, gb.ngroups, s);
             if (e != cudaSuccess) return e;
         }
-        if (c->box.B) {
-            e = c->box.KE == 5 ? (four ? launch_box_bwd<5, true>(c, gb, s) : launch_box_bwd<5, false>(c, gb, s))
-                               : (four ? launch_box_bwd<8, true>(c, gb, s) : launch_box_bwd<8, false>(c, gb, s));
+        for (const BoxGroup &p : c->box.groups) {
+            e = p.KE == 5 ? (four ? launch_box_bwd<5, true>(c, p, gb, s) : launch_box_bwd<5, false>(c, p, gb, s))
+                          : (four ? launch_box_bwd<8, true>(c, p, gb, s) : launch_box_bwd<8, false>(c, p, gb, s));
             if (e != cudaSuccess) return e;
         }
         const int NQ = four ? kNQB4 : kNQB, NS = four ? 2 : 1, LC = far_bwd_chunk(t, NQ, NS);

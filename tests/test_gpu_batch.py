@@ -63,9 +63,9 @@ def test_small_batch_forward_every_star(oracle, prec):
 
 
 def test_batch_forward_equals_single_star_contexts():
-    """Every output cell is computed by one work item with the same arithmetic as in a
-    single-star context; only the order of the near-core shared-memory accumulation
-    may differ (last-bit rounding), so a batch matches single-star runs to ~1e-7."""
+    """Every output cell is the same sum as in a single-star context (form, boxes and cuts follow
+    from the star's own lines); only the order of the partial sums of split items may differ
+    (last-bit rounding), so a batch matches single-star runs to ~1e-7."""
     b = I.small_batch(n_stars=4, span_nm=4.0, seed=23)
     s, kl, F, Fc, f = _run_batch(b)
     for k in range(b.n_stars):
@@ -155,8 +155,8 @@ def test_calib_step_graph_matches_eager_calls(prec):
     """pz_calib_step = corrections + forward + chi2 + backward + update in one graph
     launch; its loss and gradients equal the eager calls, its update is delta - lr g,
     and a replay sees the updated corrections.  The plain FP64 form matches to 1e-12;
-    the mixed path's near-core forward adds FP32 partial sums through shared-memory
-    atomics whose order changes from launch to launch, so two eager runs already
+    on short grids the mixed path's near-core forward adds FP32 partial sums of an item's
+    pieces by atomics whose order changes from launch to launch, so two eager runs already
     differ at FP32 rounding and the graph is held to the same bar."""
     import torch
     b = I.small_batch(n_stars=2, span_nm=3.0, seed=37)
@@ -202,7 +202,7 @@ def test_calib_step_graph_matches_eager_calls(prec):
         # FP64 throughout: only the order of FP64 atomic additions may differ
         assert d_ge < 1e-12 and g_ge < 1e-6     # gradients are returned in FP32
     else:
-        # FP32 near-core sums through shared-memory atomics: the launch-to-launch spread
+        # FP32 near-core sums added by atomics: the launch-to-launch spread
         assert d_ge < 1e-8 and d_ee < 1e-8 and g_ge < 1e-6
     for a, c in zip(g_s + [gab_s], g_e + [gab_e]):
         a, c = a.cpu().numpy().astype(np.float64), c.cpu().numpy().astype(np.float64)

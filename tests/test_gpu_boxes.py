@@ -101,3 +101,42 @@ def test_points_past_a_dominant_lines_window(W):
         assert err[:, side].max() < 2e-6
     # beyond every window: nothing at all
     assert np.all(got[0][:, 1536 + W:] == 0.0) and np.all(got[0][:, :1504 - W] == 0.0)
+
+
+def uneven_batch():
+    """Three stars on one list at R = 1e5: dense and narrow (boxes of 16), sparse (no boxes), dense and wide (32)."""
+    ns, W, grid = 10, 667, I.Grid(1600.0, 1e5, 1500)
+    at = [I.make_atmosphere(t, 4.5, ns, 5, log_abund_mean=-10.0, xi_kms=xi) for t, xi in ((4200.0, 1.0), (4500.0, 1.0),
+                                                                                       (4800.0, 15.0))]
+    rng = np.random.default_rng(8)
+    hi = float(I.grid_lambda_nm(grid)[-1])
+    n = 9000
+    ll = I._pack([I._atomic_lines(rng, n, 1600.0 * (1 - W / 1e5), hi * (1 + W / 1e5), np.arange(ns))], W)
+    subsets = [np.arange(n, dtype=np.int32), np.arange(0, n, 20, dtype=np.int32), np.arange(0, n, 2, dtype=np.int32)]
+    return I.Batch("uneven", at, grid, ll, [I.make_kappa_c(a, grid) for a in at], subsets)
+
+
+@pytest.mark.parametrize("make", [uneven_batch, lambda: I.small_batch(n_stars=4, span_nm=4.0, seed=23)],
+                         ids=["sizes and densities", "densities"])
+def test_a_star_takes_the_same_sums_in_a_batch(make):
+    """A star's form (boxes or the direct sum, and the box size) follows from its own lines and widths: in a batch
+    and alone it differs by the order of a few sums.  The two forms agree in 0.72 to 0.77 of all FP32 values, the
+    same form in another order in more than 0.95."""
+    import torch
+
+    def kappa(b):
+        s = pz.Synthesizer(b)
+        kl = torch.empty((b.n_stars, s.n_depth, s.n_lambda), dtype=torch.float32, device=s.device)
+        pz.pz_line_opacity(s.ctx, kl)
+        out = kl.cpu().numpy()
+        s.close()
+        return out
+
+    b = make()
+    together = kappa(b)
+    for k in range(b.n_stars):
+        alone = kappa(I.Batch("one", [b.atmos[k]], b.grid, b.lines, [b.kappa_c[k]], [b.subsets[k]]))[0]
+        same = np.mean(together[k] == alone)
+        print("star %d, %d lines: %.4f of the values equal" % (k, len(b.subsets[k]), same))
+        assert same > 0.9
+        assert np.max(np.abs(together[k] - alone) / np.maximum(alone, 1e-30)) < 6e-7
