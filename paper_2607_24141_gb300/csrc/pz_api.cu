@@ -451,18 +451,24 @@ static pz_status build_boxes(pz_ctx *c) {
     if (p.groups.empty()) return PZ_OK;
     const size_t K = 14, row = 16;   // moments per box, row of the tables
     std::vector<int4> geo(c->S, make_int4(0, 0, 0, 0));
-    size_t ws = 0;
     for (BoxGroup &b : p.groups) {
         PZ_TRY(dalloc(&b.d_C, (size_t)2 * (b.omax + 3) * K * row, "box tables"));
         PZ_TRY(dalloc(&b.d_E, (size_t)4 * b.B * b.KE, "box tables"));
         PZ_TRY(dalloc(&b.d_A, 3 * K * K, "box tables"));
         for (int k = 0; k < b.count; ++k) geo[p.stars[b.first + k]] = make_int4(b.B, b.sh, b.s_lo, b.nbox);
-        ws = std::max(ws, box_workspace_floats(c, b, b.chunk));
     }
     PZ_TRY(upload(&p.d_geo, geo, "box tables"));
     PZ_TRY(upload(&p.d_stars, p.stars, "box tables"));
     PZ_TRY(dalloc(&p.d_start, (size_t)c->S * p.stride, "box tables"));
-    PZ_TRY(dalloc(&p.d_ws, ws, "box workspace"));
+    // at most kBoxWorkspace, less where memory is short: the launches are cut to what there is
+    for (size_t want = kBoxWorkspace;; want /= 2) {
+        const size_t bytes = box_cut(c, want);
+        if (bytes == 0) return fail(PZ_ENOMEM, "box workspace: allocation failed");
+        if (dev_alloc((void **)&p.d_ws, bytes) == cudaSuccess) break;
+        p.d_ws = nullptr;
+        cudaGetLastError();
+        want = std::min(want, bytes);
+    }
     return cuda_check(launch_box_tables(c), "box tables");
 }
 

@@ -107,7 +107,8 @@ __global__ void k_box_start(int nq, int s_lo, int B, const int32_t *stars, const
 
 struct BoxArgs {
     int B, omax, rem;             // box, widest whole offset, (W + 1) - (omax + 1) B
-    int s_lo, nbox, ntb;          // first source box, source boxes, target boxes
+    int s_lo, nbox, ntb;          // first source box and source boxes of this launch, target boxes
+    int box0, tgt0;               // place of s_lo among the star's boxes, first target box of this launch
     int DC, DS;                   // tiling of the line records (class bits)
     const int32_t *stars;         // stars of this launch
     float invh, ctr;              // 2/B, (B - 1)/2
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(NP * 128) k_box_moments(LineArgs gq, BoxArgs b
     const bool live = part < NP;
     float *s_cls = reinterpret_cast<float *>(&sg + 1);          // [part][3][kBoxK][nd]: lines of classes 1..3
     float *s_m = s_cls + NP * 3 * kBoxK * nd;            // [part][kBoxK][nd]: class 0
-    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * box;
+    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * (b.box0 + box);
     const int i0 = (b.s_lo + box) * b.B;
     int most = 0;
 #pragma unroll
@@ -433,7 +434,7 @@ static size_t box_field_smem(int B, int nd) {
 template <int KE>
 __global__ void __maxnreg__(96) k_box_field(LineArgs gq, BoxArgs b) {
     extern __shared__ float smem_f[];         // [kBoxSplit][kBoxK][nd], then [kBoxSplit][B][nd + 1]
-    const int sl = blockIdx.y, st = b.stars[sl], t = blockIdx.x;
+    const int sl = blockIdx.y, st = b.stars[sl], t = b.tgt0 + blockIdx.x;
     const LineArgs g = star_view(gq, st);
     const int nd = g.nd, part = threadIdx.x / nd, d = threadIdx.x - part * nd;
     const bool live = part < kBoxSplit;
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(32 * kBoxGradWarps) k_box_grad(LineArgs gq, Bo
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int box = blockIdx.x, sl = blockIdx.y, st = b.stars[sl];
     const LineArgs g = star_view(gq, st);
-    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * box;
+    const int32_t *start = gq.bstart + (int64_t)st * gq.brow + kBoxSplit * (b.box0 + box);
     const int lo = start[0], hi = start[kBoxSplit];
     if (lo >= hi) return;
     // the block's layers dz .. dz + nd

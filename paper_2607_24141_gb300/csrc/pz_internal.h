@@ -102,7 +102,7 @@ struct BoxGroup {
     int s_lo = 0, nbox = 0, ntb = 0;   // first source box, source boxes, target boxes
     int KE = 0;                 // moments kept per grid index for the window ends
     int first = 0, count = 0;   // its stars: [first, first + count) of BoxPlan::stars
-    int chunk = 0;              // stars per launch (bounds the workspace)
+    int chunk = 0, span = 0;    // stars and source boxes per forward launch (bound the workspace)
     float *d_A = nullptr, *d_C = nullptr, *d_E = nullptr;
 };
 struct BoxPlan {
@@ -336,7 +336,9 @@ bool tiling_supported(int J, int DS, int minb);
 bool tiling_fits(const Tiling &t);   // both far-wing chunks fit in shared memory
 size_t far_info_bytes(const pz_ctx *c);
 size_t box_wide_bytes(const pz_ctx *c);
-size_t box_workspace_floats(const pz_ctx *c, const BoxGroup &b, int stars);
+// cuts the launches to a workspace of about `bytes`; returns its size, or 0 if they cannot be cut to it
+size_t box_cut(pz_ctx *c, size_t bytes);
+constexpr size_t kBoxWorkspace = (size_t)1 << 30;   // bytes of the box expansions' workspace aimed at
 // which stars use the box expansions, and their geometry (host); evals: (line, point, layer) terms per star
 void box_choose(pz_ctx *c, const std::vector<int64_t> &evals);
 cudaError_t launch_box_tables(pz_ctx *c);            // fills their device tables

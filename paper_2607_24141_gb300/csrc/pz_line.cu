@@ -606,8 +606,6 @@ size_t far_info_bytes(const pz_ctx *c) {
 }
 
 // ---- box expansions: host side -------------------------------------------------
-constexpr size_t kBoxWorkspace = (size_t)1 << 30;   // bytes per launch aimed at (stars are taken in chunks)
-
 // Which stars use the expansions, and their geometry.  A box of B points, a power of two near half
 // the star's widest near zone (20 Doppler widths in grid points), so that the nearest pairs are 3 or 4
 // boxes apart: smaller boxes raise the pairs as 1/B^2, larger ones the points left to the direct sum.
@@ -651,20 +649,27 @@ void box_choose(pz_ctx *c, const std::vector<int64_t> &evals) {
         b.nbox = (int)((c->nlam - 1 + c->W) / b.B) - b.s_lo + 1;
         b.ntb = (int)((c->nlam + b.B - 1) / b.B);
         b.KE = box_order(b.omax + 1) + 1 <= 5 ? 5 : 8;
-        b.chunk = 1;
-        while (b.chunk < b.count && box_workspace_floats(c, b, b.chunk + 1) * sizeof(float) <= kBoxWorkspace) ++b.chunk;
         p.stride = std::max<int64_t>(p.stride, (int64_t)kBoxSplit * b.nbox + 1);
         p.groups.push_back(b);
     }
 }
 
-static size_t box_moment_floats(const pz_ctx *c, const BoxGroup &b) {
-    return (size_t)b.nbox * kBoxClasses * kBoxK * c->nd;
-}
-size_t box_workspace_floats(const pz_ctx *c, const BoxGroup &b, int stars) {
-    const size_t fwd = box_moment_floats(c, b) + (size_t)b.nbox * b.B * b.KE * c->nd;
-    const size_t bwd = (size_t)b.ntb * kBoxK * c->nd;
-    return std::max(fwd, bwd) * stars;
+// Forward launches take whole stars while they fit, then parts of one star's source boxes (the field
+// of a part is added to the near-core sums as the whole's is); the reverse pass keeps the moments of
+// G of whole stars, 56 bytes per layer and box.
+size_t box_cut(pz_ctx *c, size_t bytes) {
+    constexpr int kLeastBoxes = 16;
+    size_t most = 0;
+    for (BoxGroup &b : c->box.groups) {
+        const size_t per_box = sizeof(float) * (kBoxClasses * kBoxK + (size_t)b.B * b.KE) * c->nd;
+        const size_t bwd = sizeof(float) * (size_t)b.ntb * kBoxK * c->nd, star = std::max(per_box * b.nbox, bwd);
+        b.chunk = (int)std::min<size_t>(b.count, std::max<size_t>(1, bytes / star));
+        b.span = (int)std::min<size_t>(b.nbox, std::max<size_t>(1, bytes / per_box));
+        const size_t need = std::max(per_box * b.span, bwd) * b.chunk;
+        if (need > bytes && b.span < std::min(kLeastBoxes, b.nbox)) return 0;
+        most = std::max(most, need);
+    }
+    return most;
 }
 size_t box_wide_bytes(const pz_ctx *c) {
     return (size_t)kBoxClasses * c->nslab * (size_t)((c->L.n + 31) / 32) * sizeof(uint32_t);
@@ -709,15 +714,17 @@ cudaError_t launch_box_tables(pz_ctx *c) {
     return cudaSuccess;
 }
 
-// Arguments of the stars [first, ...) of BoxPlan::stars, all of group p.
-static BoxArgs box_args(const pz_ctx *c, const BoxGroup &p, int first) {
+// Arguments of the stars [first, ...) of BoxPlan::stars, all of group p, and its source boxes [box0, box0 + nbox).
+static BoxArgs box_args(const pz_ctx *c, const BoxGroup &p, int first, int box0, int nbox) {
     BoxArgs b;
     b.B = p.B;
     b.omax = p.omax;
     b.rem = p.rem;
-    b.s_lo = p.s_lo;
-    b.nbox = p.nbox;
+    b.s_lo = p.s_lo + box0;
+    b.nbox = nbox;
     b.ntb = p.ntb;
+    b.box0 = box0;
+    b.tgt0 = std::max(0, b.s_lo - p.omax - 2);       // first box that the sources reach
     b.DC = c->tiling.depth_per_cta();
     b.DS = c->tiling.DS;
     b.stars = c->box.d_stars + first;
@@ -730,7 +737,7 @@ static BoxArgs box_args(const pz_ctx *c, const BoxGroup &p, int first) {
     b.E = p.d_E;
     b.nmin = c->box.d_nmin;
     b.M = c->box.d_ws;
-    b.PM = c->box.d_ws + (size_t)p.chunk * box_moment_floats(c, p);
+    b.PM = c->box.d_ws + (size_t)p.chunk * p.span * kBoxClasses * kBoxK * c->nd;
     b.N = c->box.d_ws;
     return b;
 }
@@ -754,13 +761,16 @@ static cudaError_t launch_box_fwd_parts(pz_ctx *c, const BoxGroup &p, const Line
         attr_set[c->device].store(true, std::memory_order_release);
     }
     const int thr_m = (NP * c->nd + 31) / 32 * 32, thr_f = (kBoxSplit * c->nd + 31) / 32 * 32;
-    for (int k = 0; k < p.count; k += p.chunk) {
-        const int n = std::min(p.chunk, p.count - k);
-        const BoxArgs b = box_args(c, p, p.first + k);
-        k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(c->nd), s>>>(g, b);
-        k_box_field<KE><<<dim3(b.ntb, n), thr_f, box_field_smem(b.B, c->nd), s>>>(g, b);
-        c->launches += 2;
-    }
+    for (int k = 0; k < p.count; k += p.chunk)
+        for (int box0 = 0; box0 < p.nbox; box0 += p.span) {
+            const int n = std::min(p.chunk, p.count - k);
+            const BoxArgs b = box_args(c, p, p.first + k, box0, std::min(p.span, p.nbox - box0));
+            const int tgt = std::min(p.ntb, b.s_lo + b.nbox + p.omax + 2) - b.tgt0;
+            if (tgt <= 0) continue;
+            k_box_moments<KE, NP><<<dim3(b.nbox, n), thr_m, box_moment_smem<NP>(c->nd), s>>>(g, b);
+            k_box_field<KE><<<dim3(tgt, n), thr_f, box_field_smem(b.B, c->nd), s>>>(g, b);
+            c->launches += 2;
+        }
     return cudaGetLastError();
 }
 template <int KE>
@@ -784,7 +794,7 @@ static cudaError_t launch_box_bwd(pz_ctx *c, const BoxGroup &p, const LineArgs &
     }
     for (int k = 0; k < p.count; k += p.chunk) {
         const int n = std::min(p.chunk, p.count - k);
-        const BoxArgs b = box_args(c, p, p.first + k);
+        const BoxArgs b = box_args(c, p, p.first + k, 0, p.nbox);
         k_box_gmoments<<<dim3(b.ntb, n), thr, sizeof(float) * c->nd * (b.B + 1), s>>>(g, b);
         k_box_grad<KE, FOUR><<<dim3(b.nbox, n, nz), 32 * kBoxGradWarps, smem, s>>>(g, b);
         c->launches += 2;

@@ -140,3 +140,29 @@ def test_a_star_takes_the_same_sums_in_a_batch(make):
         print("star %d, %d lines: %.4f of the values equal" % (k, len(b.subsets[k]), same))
         assert same > 0.9
         assert np.max(np.abs(together[k] - alone) / np.maximum(alone, 1e-30)) < 6e-7
+
+
+def test_launches_are_cut_where_memory_is_short():
+    """Where the workspace of a star's 188 boxes is refused the source boxes are taken in parts."""
+    import gc
+    gc.collect()                     # contexts that other tests left to the garbage collector
+    prob = problem(2999, 4100, 1500)
+    ref, _ = outputs(prob, pz.PZ_FP64, 0.0, None)
+    alloc, free = pz.torch_allocator()
+    whole = 4 * 188 * (4 * 14 + 32 * 5) * 72          # moments by class and by grid index
+    refused = []
+
+    def short(n, u):
+        if n in (whole, whole // 2 // (whole // 188) * (whole // 188)):      # the whole, then half of the boxes
+            refused.append(n)
+            return 0
+        return alloc(n, u)
+
+    pz.pz_set_allocator(short, free)
+    try:
+        got, launches = outputs(prob, pz.PZ_MIXED, 0.0, None)
+    finally:
+        pz.pz_set_allocator()
+    assert len(refused) == 2 and launches == 3 + 2 * 4          # a quarter: 47 boxes at a time
+    for a, b in zip(got, ref):
+        assert np.linalg.norm(a - b) < 2e-6 * np.linalg.norm(b)
