@@ -19,7 +19,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -272,14 +271,18 @@ __device__ __forceinline__ double interval(double ta, double tb, double Sa, doub
     return Sa * (e3a - e3b) + s * (e4a - e4b - D * e3b);
 }
 
-// Dynamic shared memory granted to a kernel so far, per device (slots 0-9: scattering kernels).
+// Dynamic shared memory granted to a kernel so far, per device (slots 0-9: scattering kernels).  The
+// sizes follow from the layers, so the check and the grant are one step: a smaller grant of another
+// thread's context must not come after a larger one.
 constexpr int kSmemFlux = 10, kSmemFlux64 = 11, kSmemAdj = 12, kSmemAdj64 = 13, kSmemSlots = 14;
 static cudaError_t smem_attr(pz_ctx *c, const void *fn, int slot, size_t smem) {
-    static std::atomic<size_t> granted[kMaxDevices][kSmemSlots];
+    static std::mutex mu;
+    static size_t granted[kMaxDevices][kSmemSlots];
     if (c->device < 0 || c->device >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (smem <= granted[c->device][slot].load()) return cudaSuccess;
+    std::lock_guard<std::mutex> lk(mu);
+    if (smem <= granted[c->device][slot]) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) granted[c->device][slot].store(smem);
+    if (e == cudaSuccess) granted[c->device][slot] = smem;
     return e;
 }
 
