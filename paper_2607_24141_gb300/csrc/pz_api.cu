@@ -224,6 +224,7 @@ constexpr double kNearCtasPerSm = 6.0;      // resident near-core CTAs per SM (e
 constexpr int kMinNearPieceLines = 64;      // lines of a near-core backward piece at least
 
 static pz_status build_items(pz_ctx *c) {
+    if (c->prec != PZ_MIXED) return PZ_OK;   // the plain FP64 kernels take no items
     const int T = c->tiling.lambda_per_tile();
     const int nt = (int)((c->nlam + T - 1) / T);
     const int DC = c->tiling.depth_per_cta();
@@ -369,7 +370,7 @@ static pz_status build_items(pz_ctx *c) {
     PZ_TRY(upload(&c->d_fitems, hf, "work items"));
     PZ_TRY(upload(&c->d_fext, hx, "work items"));
     PZ_TRY(upload(&c->d_bitems, hbf, "work items"));
-    if (c->prec == PZ_MIXED) PZ_TRY(upload(&c->d_bext, hbx, "work items"));
+    PZ_TRY(upload(&c->d_bext, hbx, "work items"));
     PZ_TRY(upload(&c->d_nitems_f, hn, "work items"));
     PZ_TRY(upload(&c->d_nitems_b, hb, "work items"));
     PZ_TRY(dalloc(&c->d_fcnt, (size_t)nsplit, "work items"));
@@ -397,6 +398,7 @@ static pz_status build_items(pz_ctx *c) {
 // depth of the slab, because |v| = |expm1(Delta ln r)| c/dv_D >= |Delta| ln r (1 - |Delta| ln r / 2) c/dv_D.
 // Slabs past the last layer (grid padding) get 0.
 static pz_status build_thresholds(pz_ctx *c) {
+    if (c->prec != PZ_MIXED) return PZ_OK;   // they serve the mixed form's kernels alone
     const int DS = c->tiling.DS, DC = c->tiling.depth_per_cta();
     const int nslab = ((c->nd + DC - 1) / DC) * c->tiling.GW;
     double shrink = 1.0 - 0.5 * (c->W + 1024.0) * c->lnr;
@@ -419,9 +421,8 @@ static pz_status build_thresholds(pz_ctx *c) {
     dfree(c->d_cut);
     c->d_thr = c->d_cut = nullptr;
     PZ_TRY(upload(&c->d_thr, thr, "thresholds"));
-    c->nslab = nslab;
-    if (c->prec != PZ_MIXED) return PZ_OK;   // the rest serves the mixed form's kernels
     PZ_TRY(upload(&c->d_cut, cut, "thresholds"));
+    c->nslab = nslab;
     // box expansions: nearest offset n_c of class c at each (star, slab): the points of boxes n_c
     // apart lie beyond 2^c times the widest species' threshold; kBoxNever if no whole box or
     // window end is that far.  Layers past the last one take the bounds of no line.

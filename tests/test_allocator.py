@@ -71,3 +71,30 @@ def test_allocation_failure_is_reported_and_nothing_leaks():
             assert not live, (limit, len(live))
         finally:
             pz.pz_set_allocator()
+
+
+@pytest.mark.gpu
+def test_plain_form_keeps_no_work_items():
+    """The plain FP64 kernels read no work items or thresholds: a change of tiling allocates nothing for them."""
+    import gc
+    gc.collect()
+    prob = I.small_config1(n_lambda_span_nm=1.0, seed=3)
+    alloc, free = pz.torch_allocator()
+    sizes = []
+
+    def record(n, u):
+        sizes.append(n)
+        return alloc(n, u)
+
+    for prec in (pz.PZ_FP64, pz.PZ_MIXED):
+        pz.pz_set_allocator(record, free)
+        try:
+            s = pz.Synthesizer(prob, prec)
+            del sizes[:]
+            pz.pz_set_tiling(s.ctx, 2, 8, 2, 16, 4)
+            taken = len(sizes)
+            s.forward()
+            s.close()
+        finally:
+            pz.pz_set_allocator()
+        assert (taken == 0) == (prec == pz.PZ_FP64), taken
