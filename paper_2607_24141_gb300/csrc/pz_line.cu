@@ -936,7 +936,8 @@ __device__ __forceinline__ LineTerm64 term64(const Fp64Args &g, int64_t l, int s
     const double g6n = exp10((double)g.lg_6[l] + (double)g.dg6[l]) * g.npert[sd];
     const double grad = exp10((double)g.lg_rad[l] + (double)g.dgrad[l]);
     const double g4n = exp10((double)g.lg_4[l] + (double)g.dg4[l]) * g.ne[sd];
-    q.a = (grad + g4n + g6n) * inv_dnu / (4.0 * kPI);
+    // (a^2 stays finite: voigt64 takes 1/(v^2 + a^2) by Newton's iteration, and H is zero there in any case)
+    q.a = fmin((grad + g4n + g6n) * inv_dnu / (4.0 * kPI), 1e150);
     q.a6 = (g.dsel == 0 ? g6n : (g.dsel == 1 ? grad : g4n)) * inv_dnu / (4.0 * kPI);
     q.kv = kC / dv;
     return q;

@@ -53,3 +53,18 @@ def test_wide_lines_against_the_plain_form(xi, teff, masses, mu, g4):
     assert np.linalg.norm(got[0] - ref[0]) < 2e-6 * np.linalg.norm(ref[0])
     for a, b in zip(got[2:], ref[2:]):
         assert np.linalg.norm(a - b) < 1e-5 * np.linalg.norm(b)
+
+
+def test_plain_form_with_unbounded_damping():
+    """A damping whose square leaves FP64 gives the line no profile, not NaN (the plain FP64 form)."""
+    prob = problem(1.0, 5000.0, (12.0, 60.0), -9.0, lines=300)
+    none = problem(1.0, 5000.0, (12.0, 60.0), -9.0, lines=300)
+    for k in (0, 7, 150):
+        prob.lines.log_gamma_rad[k] = 200.0       # a near 10^187
+        none.lines.log_gf[k] = -300.0             # the same lines without strength
+    got, ref = outputs(prob, pz.PZ_FP64), outputs(none, pz.PZ_FP64)
+    for a, b in zip(got[:2], ref[:2]):
+        assert np.all(np.isfinite(a))
+        assert np.array_equal(a, b)
+    for a in got[2:]:
+        assert np.all(np.isfinite(a))
