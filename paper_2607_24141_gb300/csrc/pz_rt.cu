@@ -12,10 +12,11 @@
 // (S extrapolated linearly from the first segment).  Nothing is added below
 // the bottom layer.  Total and continuum branches share the walk.  Bound by the
 // FP64 pipe on long grids and by the chain of Taylor series on short ones, where
-// one thread per wavelength walked all 72 layers: 4,000 points 0.465 -> 0.112 ms,
-// 2,200 points with the adjoint 0.63 -> 0.19 ms; 37,550 points (with ten instead of
-// fourteen Taylor terms and Newton reciprocals) flux 0.60 -> 0.49, adjoint 0.525 ->
-// 0.44 ms.
+// one thread per wavelength walked all 72 layers: 4,000 points 0.465 -> 0.117 ms,
+// 2,200 points with the adjoint 0.63 -> 0.19 ms; 37,550 points (ten instead of
+// fourteen Taylor terms) flux 0.60 -> 0.53, adjoint, whose 1/(tb - ta) is a Newton
+// reciprocal, 0.525 -> 0.44 ms.  The flux keeps its division: a product with the
+// reciprocal rounds twice (0.49 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -267,7 +268,7 @@ cudaError_t launch_planck_tables(pz_ctx *c, cudaStream_t s) {
 __device__ __forceinline__ double interval(double ta, double tb, double Sa, double Sb, double e3a, double e4a,
                                            double e3b, double e4b) {
     double D = tb - ta;
-    double s = (Sb - Sa) * rcp_newton(D);
+    double s = (Sb - Sa) / D;
     return Sa * (e3a - e3b) + s * (e4a - e4b - D * e3b);
 }
 
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(32 * kRtSegs) k_flux(FluxArgs g) {
                 if (d == 1) {
                     // top interval [0, tau_0], S linear through layers 0 and 1 (both in segment 0)
                     const FluxNode &n0 = last[br];
-                    const double s0 = (n.S - n0.S) * rcp_newton(n.tau - n0.tau);
+                    const double s0 = (n.S - n0.S) / (n.tau - n0.tau);
                     F[br] += interval(0.0, n0.tau, n0.S - s0 * n0.tau, n0.S, 0.5, 1.0 / 3.0, n0.e3, n0.e4);
                 }
                 last[br] = n;
@@ -1586,7 +1587,7 @@ __global__ void __launch_bounds__(32 * kRtSegs) k_rt_adjoint(RtAdjArgs g) {
                 interval_grad(last.tau, n.tau, last.S, n.S, last.e2, last.e3, last.e4, n.e2, n.e3, n.e4, da, db);
                 if (d == 1) {
                     // top interval: Sa = S0 - s0 tau0, s0 = (S1 - S0)/(tau1 - tau0)
-                    const double t0 = last.tau, iD = rcp_newton(n.tau - t0), s0 = (n.S - last.S) * iD, sp = s0 * iD;
+                    const double t0 = last.tau, D = n.tau - t0, s0 = (n.S - last.S) / D, sp = s0 / D;
                     const double Pt = 0.5 - last.e3, Bt = 1.0 / 3.0 - last.e4 - t0 * last.e3;
                     v += -s0 * Pt + sp * (Bt - t0 * Pt) + last.S * last.e2;
                     nv = -sp * (Bt - t0 * Pt);
