@@ -24,8 +24,9 @@
 // Which pairs: all boxes |o| >= n_c whose points lie inside the window of every line of the
 // source box (|o| <= omax = (W + 1)/B - 1).  n_c is the line's separation class at the slab
 // of layers: at distance (n_c - 1) B every |v| is at least 20 (the widest species) and 9 a,
-// where the dropped terms are below 3e-8; n_0 >= 3 keeps the expansions' truncation there
-// too.  Lines whose damping needs more than the widest class keep class 4 and are summed
+// where the dropped terms are at most 2.2e-8 of H and 2.1e-7 of dH/da (the first of them (a/v)^8 and
+// 9 (a/v)^8, at |v| = 9 a; a tenth of that at a = v/12); n_0 >= 3 keeps the expansions' truncation
+// below 1e-7.  Lines whose damping needs more than the widest class keep class 4 and are summed
 // directly over their whole window.  A window ends inside at most two further boxes on each
 // side; there f is almost constant over a box, a few k suffice, and the sharp end is kept by
 // moments of every grid index of the boxes by itself, which the points add up in the order in

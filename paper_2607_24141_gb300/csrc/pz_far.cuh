@@ -339,7 +339,7 @@ constexpr float kCoreV = 0.3f;       // distance threshold factor: |v| >= 0.3 x 
 constexpr float kFast3V = 1.5f;      // distance threshold factor: |v| >= 1.5 x 20
 constexpr float kFast2A2 = 1.5f;     // a^2 bound
 // Larger damping, a^2 <= 44 (a <= 20/3): the eight terms hold where |v| >= 20, so |v| >= 3a (H below
-// 3.5e-9, dH/da below 7e-8 of its scale); those lines keep the whole near zone, U < 400 K of the slab's
+// 3.6e-9, dH/da below 7e-8 of its scale); those lines keep the whole near zone, U < 400 K of the slab's
 // widest layer, in the near-core kernels.  They are few in giants but a third of the deepest layers'
 // lines in dwarfs, where the polynomial in t (two reciprocals per depth pair and cell, and a mask)
 // took most of the far-wing time: two-star fit on 10^5 lines, far
