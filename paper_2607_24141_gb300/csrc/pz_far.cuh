@@ -50,7 +50,6 @@ struct LineArgs {
     float rj[4], rm1j[4];                           // r^-j and (r^-j - 1) 2^uexp, j = 0..3 (r = 1 + 1/R)
     const int32_t *star;                            // [nl] star of each line
     const LineInfo *finfo;                          // far-wing line records [ngroups][nl] (k_far_info)
-    int *status;                                    // device status word (bounded-wait failures)
     const uint32_t *keep;                           // centre-test mask [nl][kKeepWords] or NULL (all kept)
     // box expansions (pz_box.cuh): pairs they sum are skipped by the far-wing kernels
     int tDC, tDS;                                   // layers per depth group and slab of the line records
@@ -94,8 +93,7 @@ __device__ __forceinline__ LineArgs star_view(const LineArgs &g, int s) {
     return v;
 }
 
-// Persistent work loop: every CTA takes the next item of the queue until it is empty
-// (or until f, if it returns a flag, returns false -- uniformly over the CTA).
+// Persistent work loop: every CTA takes the next item of the queue until it is empty.
 template <class F>
 __device__ __forceinline__ void for_each_item(const LineArgs &g, F &&f) {
     __shared__ int s_it;
@@ -106,22 +104,10 @@ __device__ __forceinline__ void for_each_item(const LineArgs &g, F &&f) {
         __syncthreads();
         if (it >= g.n_items) break;
         const int4 item = g.items[it];
-        using R = decltype(f(star_view(g, item.x), 0, 0, 0, 0, 0));
-        if constexpr (std::is_same<R, bool>::value) {
-            if (!f(star_view(g, item.x), item.y / g.ngroups, item.y % g.ngroups, item.z, item.w, it)) break;
-        } else {
-            f(star_view(g, item.x), item.y / g.ngroups, item.y % g.ngroups, item.z, item.w, it);
-        }
+        f(star_view(g, item.x), item.y / g.ngroups, item.y % g.ngroups, item.z, item.w, it);
     }
 }
 
-// Per-(line, depth) prefactors.  NP = 8 (forward), 16 (backward) or 18 (all damping families):
-//  [0] k = c/dv_D   [1] a^2   [2..6] B1..B5 = A a/sqrt(pi) x (1, 1.5, 3.75-2a^2, -15a^2, 12a^4)
-//  [7] A            (backward:) [8..13] C1..C6 = A a6/sqrt(pi) x (1, 1.5-2a^2, 3.75-12a^2,
-//  12a^4-67.5a^2, 180a^4, -120a^6)   [14] A a6   [15] a   [16] A a_rad   [17] A a_Stark
-// where a6 is the part of a that van der Waals broadening contributes, gamma6 n_pert/(4 pi dnu_D)
-// (Eq. 10 scales one family by 10^delta, so d a / d delta = ln10 a6), and a_rad, a_Stark those of
-// gamma_rad and gamma4 n_e.
 // Per-line scalars of the prefactors (one load per line, shared by its depths).
 struct LineScalars {
     int sp;
@@ -139,58 +125,38 @@ __device__ __forceinline__ LineScalars load_line(const LineArgs &g, int64_t l) {
     return L;
 }
 
+// Per-(line, depth) prefactors of the near-core kernels: k = c/dv_D, the damping parameter a and its square, the
+// strength A, and (NG > 0) A times the parts of a that the damping families contribute: van der Waals
+// gamma6 n_pert/(4 pi dnu_D) and (NG = 3) radiative gamma_rad and Stark gamma4 n_e alike (Eq. 10 scales
+// one family by 10^delta, so d a / d delta = ln10 a_family).  Layers past the last one: no width, no strength.
 // The damping products are rounded explicitly (no contraction), so that every kernel
 // that classifies a cell by |v|^2 + a^2 -- the far-wing and near-core passes -- forms
 // k and a^2 with identical roundings.
-template <int NP>
-__device__ __forceinline__ void depth_params(const LineArgs &g, const LineScalars &L, int d, float *out) {
-    if (d >= g.nd) {
-#pragma unroll
-        for (int k = 0; k < NP; ++k) out[k] = 0.0f;
-        out[1] = 1.0f;
-        return;
-    }
+struct DepthParams {
+    float k, a2, A, a, damp[3];
+};
+template <int NG>
+__device__ __forceinline__ DepthParams depth_params(const LineArgs &g, const LineScalars &L, int d) {
+    DepthParams q{0.0f, 1.0f, 0.0f, 0.0f, {0.0f, 0.0f, 0.0f}};
+    if (d >= g.nd) return q;
     const int id = L.sp * g.nd + d;
     const float invdv = __ldg(g.invdv + id);
     const float bh = __ldg(g.beta_hi + d), bl = __ldg(g.beta_lo + d);
     const float p = L.E * bh;
     const float r = fmaf(L.E, bh, -p) + L.E * bl;      // E beta = p + r
     const float boltz = expf(-p) * (1.0f - r);
-    const float A = L.Q * __ldg(g.R + id) * boltz;
     const float lw = __fmul_rn(__fmul_rn(L.lamcm, invdv), (float)(1.0 / (4.0 * kPI)));
     const float g6n = __fmul_rn(L.g6, __ldg(g.npert + d));
-    const float a = __fmul_rn(fmaf(L.g4, __ldg(g.ne + d), __fadd_rn(L.grad, g6n)), lw);
-    const float a2 = __fmul_rn(a, a);
-    const float B1 = A * a * kInvSqrtPiF;
-    out[0] = __fmul_rn((float)kC, invdv);
-    out[1] = a2;
-    out[2] = B1;
-    out[3] = 1.5f * B1;
-    out[4] = fmaf(-2.0f, a2, 3.75f) * B1;
-    out[5] = -15.0f * a2 * B1;
-    out[6] = 12.0f * a2 * a2 * B1;
-    out[7] = A;
-    if (NP >= 16) {
-        const float Aa6 = A * g6n * lw;
-        const float C1 = Aa6 * kInvSqrtPiF;
-        out[8] = C1;
-        out[9] = fmaf(-2.0f, a2, 1.5f) * C1;
-        out[10] = fmaf(-12.0f, a2, 3.75f) * C1;
-        out[11] = a2 * fmaf(12.0f, a2, -67.5f) * C1;
-        out[12] = 180.0f * a2 * a2 * C1;
-        out[13] = -120.0f * a2 * a2 * a2 * C1;
-        out[14] = Aa6;
-        out[15] = a;
-        if (NP == 18) {
-            out[16] = A * L.grad * lw;
-            out[17] = A * __fmul_rn(L.g4, __ldg(g.ne + d)) * lw;
-        }
+    q.a = __fmul_rn(fmaf(L.g4, __ldg(g.ne + d), __fadd_rn(L.grad, g6n)), lw);
+    q.a2 = __fmul_rn(q.a, q.a);
+    q.k = __fmul_rn((float)kC, invdv);
+    q.A = L.Q * __ldg(g.R + id) * boltz;
+    if (NG > 0) q.damp[0] = q.A * g6n * lw;
+    if (NG == 3) {
+        q.damp[1] = q.A * L.grad * lw;
+        q.damp[2] = q.A * __fmul_rn(L.g4, __ldg(g.ne + d)) * lw;
     }
-}
-
-template <int NP>
-__device__ __forceinline__ void line_params(const LineArgs &g, int64_t l, int d, float *out) {
-    depth_params<NP>(g, load_line(g, l), d, out);
+    return q;
 }
 
 // index-space frequency offset u = lambda_l/lambda_i - 1 = expm1(Delta ln r)
@@ -652,7 +618,7 @@ __device__ __forceinline__ float4 *comp_lo(float *s_comp, int dd, int tid, int n
     return reinterpret_cast<float4 *>(s_comp) + (size_t)(2 * dd + 1) * nthr + tid;
 }
 
-// Higher far-wing coefficients from a^2 and B1 (as depth_params forms them):
+// Coefficients of the polynomial in t from a^2 and B1 (B2 = 1.5 B1):
 // B3 = (3.75 - 2a^2) B1, B4 = -15 a^2 B1, B5 = 12 a^4 B1.
 __device__ __forceinline__ void far_b345(f2_t a2, f2_t B1, f2_t &B3, f2_t &B4, f2_t &B5) {
     B3 = f2_mul(f2_fma(a2, f2_splat(-2.0f), f2_splat(3.75f)), B1);
@@ -809,12 +775,11 @@ __device__ __forceinline__ void far_bwd_series(const ulonglong2 *par, const f2_t
     }
 }
 
-// Far-wing kernel (forward).  Every cell with |v|^2 + a^2 >= 400 inside its window is
-// evaluated here with the far polynomial; the near-core cells are summed by
-// k_line_near_fwd into knear, which this kernel adds before applying stim.
-// Returns false if a chunk never arrived (the kernel stops).
+// Far-wing kernel (forward).  The cells of a line outside its core (far_form) and nearer than the box
+// expansions' pairs are summed here; the cores' cells and the boxes' field are in knear already, which
+// this kernel adds before applying stim.
 template <int J, int DS, bool GATHER>
-__device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, const int tile, const int group,
+__device__ __forceinline__ void far_fwd_item(const LineArgs &g, const int st, const int tile, const int group,
                                              const int lo, const int hi, const int GW, const int LC,
                                              const WarpStage &ws, float *s_comp, const int4 ext) {
     static_assert(J == 2 || J == 4, "J must be 2 or 4");
@@ -1040,7 +1005,7 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
         __syncthreads();
         if (tid == 0) s_last = atomicAdd(g.fcnt + ext.z, 1) == ext.y - 1;
         __syncthreads();
-        if (!s_last) return true;
+        if (!s_last) return;
         __threadfence();
 #pragma unroll
         for (int dd = 0; dd < DS; ++dd) {
@@ -1091,7 +1056,6 @@ __device__ __forceinline__ bool far_fwd_item(const LineArgs &g, const int st, co
         else
             *reinterpret_cast<float2 *>(row) = make_float2(v[0], v[1 % J]);
     }
-    return true;
 }
 
 // Shared memory of the far-wing kernels: each warp's stage (warp_stage_quads), then
@@ -1108,7 +1072,7 @@ __global__ void __launch_bounds__(128, MINB) k_line_fwd(LineArgs g, int GW, int 
     const WarpStage ws = make_stage(mine, LC, DS, kNQF);
     float *s_comp = reinterpret_cast<float *>(smem4 + (size_t)GW * wq);
     for_each_item(g, [&](const LineArgs &v, int tile, int group, int lo, int hi, int it) {
-        return far_fwd_item<J, DS, GATHER>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_comp, g.fext[it]);
+        far_fwd_item<J, DS, GATHER>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_comp, g.fext[it]);
     });
 }
 
@@ -1184,7 +1148,7 @@ __device__ __forceinline__ int64_t far_row(int q) { return q < 2 ? q : 2 * q - 1
 // Far-wing kernel (backward): the per-line sums over the tile's far cells of
 // G stim A H and G stim A a6 dH/da, reduced over the CTA and added to gacc.
 template <int J, int DS, bool FOUR>
-__device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, const int tile, const int group,
+__device__ __forceinline__ void far_bwd_item(const LineArgs &g, const int st, const int tile, const int group,
                                              const int lo, const int hi, const int GW, const int LC,
                                              const WarpStage &ws, float2 *s_part, float2 *s_red2, unsigned &cc,
                                              const int4 ext) {
@@ -1366,7 +1330,6 @@ __device__ __forceinline__ bool far_bwd_item(const LineArgs &g, const int st, co
             atomicAdd(g.gacc + far_row(2 * q + 1) * g.nl + ws.idx[k], (double)a2);
         });
     });
-    return true;
 }
 
 template <int J, int DS, int MINB, bool FOUR>
@@ -1381,8 +1344,7 @@ __global__ void __launch_bounds__(128, MINB) k_line_bwd(LineArgs g, int GW, int 
     float2 *s_part = s_red2 + (size_t)2 * NS * LC * GW + (size_t)warp * NS * kBwdBatch * 32;
     unsigned cc = 0;
     for_each_item(g, [&](const LineArgs &v, int tile, int group, int lo, int hi, int it) {
-        return far_bwd_item<J, DS, FOUR>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_part, s_red2, cc,
-                                         g.fext[it]);
+        far_bwd_item<J, DS, FOUR>(v, g.items[it].x, tile, group, lo, hi, GW, LC, ws, s_part, s_red2, cc, g.fext[it]);
     });
 }
 

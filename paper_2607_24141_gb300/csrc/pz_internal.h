@@ -25,7 +25,7 @@ constexpr double kSQRTPI = 1.77245385090551602730;
 constexpr double kLN10 = 2.30258509299404568402;
 constexpr double kC2 = kH * kC / kKB;       // second radiation constant, cm K
 
-// Largest supported depth count (register/local arrays in the flux kernels).
+// Largest supported depth count (threads and shared memory of the transfer and box kernels).
 constexpr int kMaxDepth = 128;
 constexpr int kNearDepths = 8;       // layers per work item of the near-core kernels
 // Largest number of instrument taps per pixel.
@@ -35,7 +35,7 @@ constexpr int kMaxDevices = 64;
 
 // Far-wing / mid / core boundaries of the FP32 Voigt (|z|^2 thresholds).
 constexpr float kFar2 = 400.0f;   // |z| >= 20: asymptotic series, 2 corrections
-constexpr float kMid2 = 36.0f;    // 6 <= |z| < 20: asymptotic series, 8 corrections
+constexpr float kMid2 = 36.0f;    // 6 <= |z| < 20: asymptotic series, 6 corrections
 // |z| < 6: a < kCoreA -> Dawson-derivative Taylor table; else Weideman rational.
 constexpr float kCoreA = 0.5f;
 constexpr int kDawsonK = 16;      // Taylor order of the core table

@@ -162,12 +162,11 @@ __global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, L
             const LineScalars L = load_line(g, l);
             const int d1 = min(grp * DC + (w + 1) * DS, g.nd);
             for (int dd = grp * DC + w * DS; dd < d1; ++dd) {
-                float q[8];
-                depth_params<8>(g, L, dd, q);
-                ok = ok && q[1] <= kFast2A2;
-                wide = wide && q[1] <= kWideA2;
+                const DepthParams q = depth_params<0>(g, L, dd);
+                ok = ok && q.a2 <= kFast2A2;
+                wide = wide && q.a2 <= kWideA2;
                 none = none && !pair_kept(g.keep, l, dd);
-                need = fmaxf(need, sqrtf(q[1]) / q[0]);
+                need = fmaxf(need, sqrtf(q.a2) / q.k);
             }
         }
         amask = (ok ? 1 << w : 0) | (wide ? 16 << w : 0) | (none ? 256 << w : 0);
@@ -326,15 +325,14 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
             const LineScalars L = load_line(g, l);
             const float ilf = g.ilf[l], frac = g.frac[l];
             const bool wide = (e >> (12 + slab - sl0)) & 1, series = wide || ((e >> (8 + slab - sl0)) & 1);
-            float p[18];
-            depth_params<NG == 3 ? 18 : NG == 1 ? 16 : 8>(g, L, d, p);   // (zero strength and k past the last layer)
+            const DepthParams p = depth_params<NG>(g, L, d);
             // the points that may be near [lo, hi], and (series slabs) those that certainly are; |u| <= reach
             // there, and u = expm1(Delta ln r) differs from Delta ln r by less than 0.6 reach of it
             const float cut = (wide ? kWideCut : 1.0f) * __ldg(g.cut + L.sp * g.nslab + slab);
-            const float r2 = kFar2 - p[1];
-            const float reach = series ? sqrtf(cut * g.kunscale) : sqrtf(fmaxf(r2, 0.0f)) / p[0];
+            const float r2 = kFar2 - p.a2;
+            const float reach = series ? sqrtf(cut * g.kunscale) : sqrtf(fmaxf(r2, 0.0f)) / p.k;
             int lo = 1 << 30, hi = -(1 << 30), ilo = 0, in = -1;
-            if (have && p[0] > 0.0f && (series || r2 > 0.0f) && pair_kept(g.keep, l, d)) {
+            if (have && p.k > 0.0f && (series || r2 > 0.0f) && pair_kept(g.keep, l, d)) {
                 const float span = reach / g.lnr, m = fmaf(fmaf(0.6f, reach, 1e-3f), span, 0.01f);
                 const int ic = (int)ilf;
                 lo = max(max(t0, ic + (int)ceilf(frac - span - m)), ic - g.W);
@@ -344,17 +342,17 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
                     in = min(hi, ic + (int)floorf(frac + span - m)) - ilo;
                 }
             }
-            const float ma = D ? p[15] : sqrtf(p[1]), mcut = series ? cut : -1.0f;
+            const float ma = D ? p.a : sqrtf(p.a2), mcut = series ? cut : -1.0f;
             for (int q = 0; q < per; ++q) {
                 const int src = q * ND + lane % ND;
                 if (!__shfl_sync(0xffffffffu, (int)have, q * ND)) break;
                 const int lq = __shfl_sync(0xffffffffu, l, q * ND);
                 const float qil = __shfl_sync(0xffffffffu, ilf, q * ND), qfr = __shfl_sync(0xffffffffu, frac, q * ND);
-                const float k = __shfl_sync(0xffffffffu, p[0], src), a = __shfl_sync(0xffffffffu, ma, src);
-                const float a2 = __shfl_sync(0xffffffffu, p[1], src), A = __shfl_sync(0xffffffffu, p[7], src);
+                const float k = __shfl_sync(0xffffffffu, p.k, src), a = __shfl_sync(0xffffffffu, ma, src);
+                const float a2 = __shfl_sync(0xffffffffu, p.a2, src), A = __shfl_sync(0xffffffffu, p.A, src);
                 float damp[NG > 0 ? NG : 1];
 #pragma unroll
-                for (int f = 0; f < NG; ++f) damp[f] = __shfl_sync(0xffffffffu, p[f == 0 ? 14 : 15 + f], src);
+                for (int f = 0; f < NG; ++f) damp[f] = __shfl_sync(0xffffffffu, p.damp[f], src);
                 const float qcut = __shfl_sync(0xffffffffu, mcut, src);
                 const int qlo = __shfl_sync(0xffffffffu, lo, src), qhi = __shfl_sync(0xffffffffu, hi, src);
                 const int qilo = __shfl_sync(0xffffffffu, ilo, src), qin = __shfl_sync(0xffffffffu, in, src);
@@ -480,7 +478,6 @@ static LineArgs make_args(pz_ctx *c) {
     g.fpart = c->d_fpart;
     g.fcnt = c->d_fcnt;
     g.finfo = reinterpret_cast<const LineInfo *>(c->d_finfo);
-    g.status = c->d_status;
     g.keep = c->d_keep;
     g.lam0cm = (float)(c->lambda0_nm * 1e-7);
     g.ilf = c->L.ilf;
@@ -1338,7 +1335,7 @@ cudaError_t launch_probe_pipe(int kind, int iters, int blocks, float *out, cudaS
 }
 
 // Bounded-wait probe: one CTA waits on an mbarrier phase that nothing completes, gives
-// up after limit_ns and records the failure exactly as the far-wing kernels do.
+// up after limit_ns and records the failure in the status word.
 __global__ void k_probe_wait(uint64_t limit_ns, int32_t *status) {
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) {
