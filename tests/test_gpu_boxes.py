@@ -51,6 +51,9 @@ CASES = {
     "boxes of 16": (lambda: problem(1500, 8500, 667, R=1e5), 0.0, None),
     "boxes of 4": (lambda: problem(700, 53000, 67, R=1e4), 0.0, (4, 6, 4, 64, 4)),
     "7 layers": (lambda: problem(4000, 24000, 1500, nd=7), 0.0, None),
+    # more than two boxes per SM: one part per box and one block over all layers
+    "long grid, 8 moments at the ends": (lambda: problem(9701, 6000, 287, teff=4500.0, logg=2.5), 0.0, None),
+    "long grid, 5 moments at the ends": (lambda: problem(9600, 4000, 1500), 0.0, None),
     "grid narrower than the window": (lambda: problem(311, 21000, 1500), 0.0, None),
     "centre test": (lambda: problem(2500, 4600, 1400, teff=5000.0, logg=2.0), 1e-3, None),
     "three stars, one with a seventh of the lines": (lambda: I.small_batch(3, 5.0), 0.0, None),
