@@ -671,13 +671,34 @@ __device__ __forceinline__ void far_reduced_s(const LineArgs &g, const LineInfo 
     for (int j = 0; j < J; ++j) sq[j] = f2_mul(sp[j], sp[j]);
 }
 
+// U = 4^uexp u^2 of one point by itself (il_i = i_l - i, exact).  Within 20 Doppler widths of a line the
+// chain of far_scaled_u2 would carry the rounding of the lane's first point to points nearer the line
+// (on grids of R = 10^4, where a core is one point wide, F was 1.6e-8 from FP64 and is 1.1e-8).
+__device__ __forceinline__ float point_u2(const LineArgs &g, float il_i, float frac) {
+    const float u = offset_u(il_i + frac, g.lnr) * g.uscale;
+    return u * u;
+}
+// The same for two neighbouring points i, i + 1 (the packed operations round each half as the scalar ones).
+__device__ __forceinline__ f2_t point_u2(const LineArgs &g, const LineInfo &info, float lam) {
+    const f2_t d = f2_fma(f2_pack(lam, lam + 1.0f), f2_splat(-1.0f), f2_splat(info.ilf));
+    const f2_t y = f2_mul(f2_fma(d, f2_splat(1.0f), f2_splat(info.frac)), f2_splat(g.lnr));
+    const f2_t u = f2_mul(f2_fma(f2_mul(y, y), f2_fma(y, f2_splat(0.16666667f), f2_splat(0.5f)), y), f2_splat(g.uscale));
+    return f2_mul(u, u);
+}
+
 // Reciprocals s_j = 1/U_j at the thread's points for the series forms: zero outside the window,
 // below cut (the points left to the near-core kernels) and for lanes left to the box expansions.
 template <int J>
-__device__ __forceinline__ void far_series_s(const LineArgs &g, const LineInfo &info, bool full, bool near, float lamf,
+__device__ __forceinline__ void far_series_s(const LineArgs &g, const LineInfo &info, int form, bool near, float lamf,
                                              int lam_thr, float cut, f2_t (&sp)[J]) {
+    const bool full = form & kFormFull;
     float U[J];
-    far_scaled_u2<J>(g, info, lamf, U);
+    if ((form & 7) >= kFormEight) {
+#pragma unroll
+        for (int j = 0; j < J; j += 2) f2_unpack(point_u2(g, info, lamf + (float)j), U[j], U[j + 1]);
+    } else {
+        far_scaled_u2<J>(g, info, lamf, U);
+    }
     const int di0 = lam_thr - (int)info.ilf;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
@@ -856,7 +877,7 @@ __device__ __forceinline__ void far_fwd_item(const LineArgs &g, const int st, co
             const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
             if ((fl & 7) <= kFormWide) {
                 f2_t sp[J];
-                far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
+                far_series_s<J>(g, info, fl, near, lamf, lam_thr,
                                 far_cut(g, fl, info.sp, slab), sp);
                 if ((fl & 7) >= kFormEight)
                     far_fwd_series<J, DP, 8>(par, sp, acc);
@@ -1234,7 +1255,7 @@ __device__ __forceinline__ void far_bwd_item(const LineArgs &g, const int st, co
                     const bool near = box_near(g, bv, info, warp);   // the lane's points are summed here
                     if ((fl & 7) <= kFormWide) {
                         f2_t sp[J];
-                        far_series_s<J>(g, info, fl & kFormFull, near, lamf, lam_thr,
+                        far_series_s<J>(g, info, fl, near, lamf, lam_thr,
                                         far_cut(g, fl, info.sp, slab), sp);
                         if ((fl & 7) >= kFormEight)
                             far_bwd_series<J, DP, 8, FOUR>(par, sp, gv, R);

@@ -252,16 +252,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
 // lines x 1,500 points, forward items cut by lines: 0.090 -> 0.086, reverse 0.146 -> 0.086 ms).
 // ---------------------------------------------------------------------------
 
-// U = 4^uexp u^2 of point i as the far kernels form it, from their lane's first point (far_scaled_u2).
-template <int J>
-__device__ __forceinline__ float far_u2(const LineArgs &g, float ilf, float frac, int i) {
-    const int j = i & (J - 1);
-    const float u0 = offset_u((ilf - (float)(i - j)) + frac, g.lnr) * g.uscale;
-    const float rj = j == 1 ? g.rj[1] : j == 2 ? g.rj[2] : g.rj[3], rm = j == 1 ? g.rm1j[1] : j == 2 ? g.rm1j[2] : g.rm1j[3];
-    const float u = j == 0 ? u0 : fmaf(u0, rj, rm);
-    return u * u;
-}
-
 constexpr int kNearWarps = 8;        // warps per near-core CTA
 constexpr int kNearBatch = 512;      // lines looked at together
 struct NearList {
@@ -362,7 +352,7 @@ __device__ __forceinline__ void near_sweep(const LineArgs &g, int t0, int nlo, i
                     const float x = fabsf(offset_u((qil - (float)i) + qfr, g.lnr) * k);
                     const float z2 = fmaf(x, x, a2);
                     if (!own && i >= qlo && i <= qhi)
-                        own = qcut >= 0.0f ? far_u2<T / 32>(g, qil, qfr, i) < qcut : z2 < kFar2;
+                        own = qcut >= 0.0f ? point_u2(g, qil - (float)i, qfr) < qcut : z2 < kFar2;
                     if (own) {
                         float H, dH;
                         if (z2 < kMid2)
