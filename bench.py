@@ -45,12 +45,7 @@ WORKLOAD = ("64-star batched fwd+bwd: 64 stars (Teff U[3500,7000] K, log g U[1,5
             "abundances, update)")
 GOLDEN = os.path.join(ROOT, "tests", "golden")
 
-# Per-launch DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) and pipe counters of
-# the dominant kernel, from one ncu capture per (kernel, workload) written up under profiles/;
-# each entry is valid only while the library sources hash to the recorded value, and is
-# reported as null otherwise.
-TRAFFIC = {}
-NCU_PIPES = {}
+# sources whose hash goes with the line kernels' figures
 KERNEL_SOURCES = ("pz_line.cu", "pz_far.cuh", "pz_box.cuh", "pz_line_bwd.cu", "pz_line_bwd4.cu", "pz_voigt.cuh",
                   "pz_internal.h", "pz_api.cu")
 FMA_PER_EN = 27      # FP64 FMAs of one E_2/E_3/E_4 Taylor step (9 rounds of value + two derivatives)
@@ -175,11 +170,12 @@ def grad_rel(g, ref):
     return np.abs(g - ref) / np.maximum(np.abs(ref), floor)
 
 
-def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key, half_window=1500):
+def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, half_window=1500):
     """Roofline of the dominant far-wing line kernel from the profiler's kernel times
     {family: (ms, launches)}: FP32-pipe lane operations per second on the cells summed
-    directly (direct_cells) at the eight-term form's count against the measured FP32 pipe
-    peak.  The family's time includes the box expansions' kernels."""
+    directly (direct_cells, an assumed NEAR_POINTS per line whatever the star's damping or the
+    tiling) at the eight-term form's count against the measured FP32 pipe peak.  The family's
+    time includes the box expansions' kernels."""
     far = {"line_fwd": kt["line_fwd"][0] - kt["near_fwd"][0], "line_bwd": kt["line_bwd"][0] - kt["near_bwd"][0]}
     dom = max(far, key=far.get)
     t_dom = far[dom] * 1e-3 / max(kt[dom][1], 1)
@@ -191,20 +187,16 @@ def line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, workload_key, half_wi
     achieved = cells * ops["fp32"] / t_dom
     kname = "k_line_bwd" if dom == "line_bwd" else "k_line_fwd"
     hsh = source_hash()
-    tr = TRAFFIC.get((kname, workload_key))
-    np_ = NCU_PIPES.get((kname, workload_key))
     share = {k: v[0] for k, v in kt.items() if k not in ("near_fwd", "near_bwd", "step")}
     tot = sum(share.values())
     return {
         "bound": "alu", "kernel": kname + " (far wing)", "pipe": "fp32",
         "achieved": achieved * 1e-9, "peak": peak_fp32 * 1e-9, "unit": "Gop/s", "frac": achieved / peak_fp32,
-        "traffic": tr[0] if tr and tr[1] == hsh else None,
-        "ncu_pipes": np_[0] if np_ and np_[1] == hsh else None,
         "peak_source": ("measured: pz_probe_pipe packed-FMA throughput (%d SMs); 128-lane derivation %.0f Gop/s"
                         % (n_sm, peak_fp32_lanes * 1e-9)) if pipe_peaks.get("fp32") else
                        "derived: %d SMs x 128 FP32 lanes x %.0f MHz (max SM clock)" % (n_sm, clk_max),
         "evals_per_launch": evals, "ms_per_launch": t_dom * 1e3, "evals_per_s": evals / t_dom,
-        "direct_cells_per_launch": cells, "ops_per_direct_cell": ops,
+        "direct_cells_per_launch": cells, "direct_points_per_line_assumed": NEAR_POINTS, "ops_per_direct_cell": ops,
         "mufu_pipe_frac": cells * ops["mufu"] / t_dom / peak_mufu,
         "kernel_share": {k: round(v / tot, 4) for k, v in share.items() if tot > 0},
         "far_ms_per_launch": {k: v / max(kt[k][1], 1) for k, v in far.items()},
@@ -1086,7 +1078,7 @@ def run_config1(args, dev, pipe_peaks, clk_max):
     s.close()
     J = tune["tiling"][0] if tune else 4
     n_sm = torch.cuda.get_device_properties(dev.index).multi_processor_count
-    roof = line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max, "apogee")
+    roof = line_roofline(kt, evals, J, pipe_peaks, n_sm, clk_max)
     out = {"workload": "APOGEE-like fwd+bwd, one spectrum: 37,550 pts x 2e5 lines (40 species, 1/3 in bands) x "
                        "72 depths, W=1,500, instrument onto 8,575 px, chi^2, reverse pass; eager C-ABI calls, "
                        "256 MiB L2 flush between steps",
@@ -1274,7 +1266,7 @@ def main():
     hl = run_headline(args, dev, barrier, max_over_ranks, ws, rank, tiling, pipe_peaks, clk_max)
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count
     roof = line_roofline(hl["kernel_times"], hl["evals_per_step"], tiling[0] if tiling else 4, pipe_peaks, n_sm,
-                         clk_max, "batch64")
+                         clk_max)
     roof["hbm_gbs_peak"] = peaks.get("hbm_gbs")
     roof["timing"] = "CUDA events recorded inside the step graph around each kernel family, over the timed steps"
     roof["pipe_peaks_measured"] = {k: v * 1e-9 for k, v in pipe_peaks.items()}
