@@ -147,7 +147,7 @@ pz_status ensure_device_tables() {
 // consecutive lines, one word of wide (with one thread per line over all slabs a short list
 // waited on the chain of table loads: 11 -> 6 us at 5,300 lines; 50 us at 2 10^5 either way).
 constexpr int kInfoLines = 64;     // lines per block
-__global__ void __launch_bounds__(256) k_far_info(LineArgs gq, int DC, int DS, LineInfo *info) {
+__global__ void __launch_bounds__(256, 6) k_far_info(LineArgs gq, int DC, int DS, LineInfo *info) {
     __shared__ int s_mask[4][kInfoLines];
     const int grp = blockIdx.y, w = (threadIdx.x >> 5) & 3, col = (threadIdx.x & 31) + (threadIdx.x >> 7) * 32;
     const int64_t l = (int64_t)blockIdx.x * kInfoLines + col;
