@@ -1,14 +1,14 @@
 """CPU checks of the far-wing forms the line kernels evaluate in FP32.
 
-The far-wing kernels (cells with |z|^2 = v^2 + a^2 >= 400) use a five-term polynomial in
-t = 1/|z|^2 for H(a, v) and a six-term one for dH/da (Eqs. 4-5: the Voigt profile and the
-damping derivative of the line gradients).  Lines far from the whole wavelength tile take
-reduced forms in p = 1/v^2 instead, two terms at |v| >= 100 and three at |v| >= 30, both for
-a^2 <= 1.5.  These tests pin the stated truncation bounds in FP64: the polynomials against the
-Faddeeva function (scipy.special.wofz), and the reduced forms against the polynomials, over
-dense (a, v) lattices of the regions where the kernels use them.  They restate the series, so
-a dropped term or a wrong coefficient in either form fails here.  They do not call the CUDA
-path.
+Lines of large damping (a^2 > 44) take a five-term polynomial in t = 1/|z|^2 for H(a, v) and a
+six-term one for dH/da (Eqs. 4-5: the Voigt profile and the damping derivative of the line
+gradients) where |z|^2 = v^2 + a^2 >= 400.  All others take series in p = 1/v^2: of up to a^2 = 1.5 two
+terms at |v| >= 100 and three at |v| >= 30, pinned here; the four- and eight-term ones nearer the line
+and up to a^2 = 44 are pinned in test_box_forms.py.  These tests pin the stated truncation bounds
+in FP64: the polynomials against the Faddeeva function (scipy.special.wofz), and the two- and
+three-term series against the polynomials, over dense (a, v) lattices of the regions where the kernels
+use them.  They restate the series, so a dropped term or a wrong coefficient in either form fails
+here.  They do not call the CUDA path.
 """
 import numpy as np
 import pytest

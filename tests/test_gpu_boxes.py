@@ -56,7 +56,8 @@ CASES = {
     "long grid, 5 moments at the ends": (lambda: problem(9600, 4000, 1500), 0.0, None),
     "grid narrower than the window": (lambda: problem(311, 21000, 1500), 0.0, None),
     "centre test": (lambda: problem(2500, 4600, 1400, teff=5000.0, logg=2.0), 1e-3, None),
-    "three stars, one with a seventh of the lines": (lambda: I.small_batch(3, 5.0), 0.0, None),
+    "three stars, one with a seventh of the lines": (lambda: I.small_batch(3, 14.0), 0.0, None),
+    "three stars, the fullest with boxes": (lambda: I.small_batch(3, 5.0), 0.0, None),
 }
 
 
