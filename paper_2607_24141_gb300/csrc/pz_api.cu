@@ -358,21 +358,21 @@ static pz_status build_items(pz_ctx *c) {
                                      it.v.z + (int)((int64_t)n * (q + 1) / P)), it.cost / P});
     }
     std::vector<int4> hn = order(nfp), hb = order(nbp);
-    dfree(c->d_fitems);
-    dfree(c->d_fext);
-    dfree(c->d_bitems);
-    dfree(c->d_bext);
-    dfree(c->d_nitems_f);
-    dfree(c->d_nitems_b);
+    // the six lists in one buffer (an allocation and a copy each cost more than the lists are worth)
+    dfree(c->d_items);
     dfree(c->d_fcnt);
-    c->d_fitems = c->d_fext = c->d_bitems = c->d_bext = c->d_nitems_f = c->d_nitems_b = nullptr;
+    c->d_items = c->d_fitems = c->d_fext = c->d_bitems = c->d_bext = c->d_nitems_f = c->d_nitems_b = nullptr;
     c->d_fcnt = nullptr;
-    PZ_TRY(upload(&c->d_fitems, hf, "work items"));
-    PZ_TRY(upload(&c->d_fext, hx, "work items"));
-    PZ_TRY(upload(&c->d_bitems, hbf, "work items"));
-    PZ_TRY(upload(&c->d_bext, hbx, "work items"));
-    PZ_TRY(upload(&c->d_nitems_f, hn, "work items"));
-    PZ_TRY(upload(&c->d_nitems_b, hb, "work items"));
+    const std::vector<int4> *lists[6] = {&hf, &hx, &hbf, &hbx, &hn, &hb};
+    int4 **where[6] = {&c->d_fitems, &c->d_fext, &c->d_bitems, &c->d_bext, &c->d_nitems_f, &c->d_nitems_b};
+    std::vector<int4> all;
+    for (const auto *l : lists) all.insert(all.end(), l->begin(), l->end());
+    PZ_TRY(upload(&c->d_items, all, "work items"));
+    int4 *next = c->d_items;
+    for (int k = 0; k < 6; ++k) {
+        *where[k] = next;
+        next += lists[k]->size();
+    }
     PZ_TRY(dalloc(&c->d_fcnt, (size_t)nsplit, "work items"));
     PZ_CUDA(cudaMemset(c->d_fcnt, 0, sizeof(int) * std::max(nsplit, 1)), "work items");
     const size_t part = (size_t)nslot * slot_bytes;
@@ -490,8 +490,7 @@ static void destroy_ctx(pz_ctx *c) {
                     c->d_thr, c->d_cut, c->d_kc, c->d_B, c->d_stim, c->d_dab, c->d_mdgf, c->d_mdg6, c->d_eos, c->L.orig, c->L.star, c->L.ilf,
                     c->L.il32, c->L.frac, c->L.sp, c->L.E, c->L.lamcm, c->L.grad, c->L.g4, c->L.g6base, c->L.g6,
                     c->L.Q, c->L.Qbase, c->L.x64, c->L.lg_gf, c->L.lg_rad, c->L.lg_4, c->L.lg_6, c->L.dgf, c->L.dg6,
-                    c->d_line_off, c->d_fitems, c->d_fext, c->d_bitems, c->d_bext, c->d_fpart, c->d_fcnt, c->d_nitems_f,
-                    c->d_nitems_b, c->d_ctr, c->d_knear, c->d_kline,
+                    c->d_line_off, c->d_items, c->d_fpart, c->d_fcnt, c->d_ctr, c->d_knear, c->d_kline,
                     c->d_F, c->d_Fc, c->d_g, c->d_gc, c->d_tap0, c->d_ntap, c->d_tapw, c->d_dFbar, c->d_Gt,
                     c->d_Gt64, c->d_gacc, c->d_gline, c->d_gab, c->d_dLdf, c->d_finfo, c->d_status,
                     c->d_keep, c->L.gradbase, c->L.g4base, c->L.dgrad, c->L.dg4, c->d_mdgrad, c->d_mdg4,

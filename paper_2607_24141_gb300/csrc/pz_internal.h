@@ -204,6 +204,7 @@ struct pz_ctx {
     // work items (star, tile * groups + group, lo, hi), longest first
     // (far-wing items with many lines are split into pieces of their line range, so that
     // the queue holds several items per resident CTA; see build_items)
+    int4 *d_items = nullptr;        // the six lists that follow, in one buffer
     int4 *d_fitems = nullptr;       // far-wing forward pieces
     int4 *d_fext = nullptr;         // per forward piece: (first slot, pieces, item counter, piece)
     int4 *d_bitems = nullptr;       // far-wing backward pieces (those holding lines)
