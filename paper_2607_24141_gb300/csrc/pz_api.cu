@@ -363,6 +363,7 @@ static pz_status build_items(pz_ctx *c) {
     dfree(c->d_fcnt);
     c->d_items = c->d_fitems = c->d_fext = c->d_bitems = c->d_bext = c->d_nitems_f = c->d_nitems_b = nullptr;
     c->d_fcnt = nullptr;
+    c->n_fitems = c->n_bitems = c->n_nitems_f = c->n_nitems_b = 0;
     const std::vector<int4> *lists[6] = {&hf, &hx, &hbf, &hbx, &hn, &hb};
     int4 **where[6] = {&c->d_fitems, &c->d_fext, &c->d_bitems, &c->d_bext, &c->d_nitems_f, &c->d_nitems_b};
     std::vector<int4> all;
@@ -833,10 +834,13 @@ static pz_status apply_tiling(pz_ctx *c, const Tiling &t, const char *who) {
     drop_graph(c);
     c->finfo_valid = false;
     c->tiling = t;
+    c->n_fitems = 0;             // no launch before all tables fit the tiling (a failure leaves it so)
     PZ_TRY(build_thresholds(c));
     PZ_TRY(build_items(c));
-    if (c->prec == PZ_MIXED) PZ_TRY(ensure_far_tables(c));
-    return PZ_OK;
+    if (c->prec != PZ_MIXED) return PZ_OK;
+    const pz_status st = ensure_far_tables(c);
+    if (st != PZ_OK) c->n_fitems = 0;
+    return st;
 }
 
 // The backward stages after the objective's seed dL/df: instrument adjoint, transfer

@@ -791,6 +791,7 @@ static cudaError_t launch_box_bwd(pz_ctx *c, const BoxGroup &p, const LineArgs &
 
 template <int J, int DS, int MINB>
 static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
+    if (c->n_fitems == 0) return cudaErrorInvalidConfiguration;   // the tiling's tables could not be allocated
     const Tiling &t = c->tiling;
     LineArgs g = make_args(c);
     const int LC = far_fwd_chunk(t);
@@ -812,7 +813,7 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
         c->finfo_valid = true;
     }
     e = launch_near<32 * J, 0>(c, g, s);
-    if (e != cudaSuccess || c->n_fitems == 0) return e;
+    if (e != cudaSuccess) return e;
     g.items = c->d_fitems;
     g.fext = c->d_fext;
     g.n_items = c->n_fitems;
@@ -834,6 +835,7 @@ static cudaError_t launch_fwd_t(pz_ctx *c, cudaStream_t s) {
 
 // Reverse pass of the lines; four: with the radiative and Stark damping sums.
 cudaError_t launch_line_bwd_mixed(pz_ctx *c, cudaStream_t s, bool four) {
+    if (c->n_fitems == 0) return cudaErrorInvalidConfiguration;
     const Tiling &t = c->tiling;
     const LineArgs g = make_args(c);
     cudaError_t e = cudaMemsetAsync(c->d_ctr + 2, 0, 2 * sizeof(int), s);

@@ -98,3 +98,43 @@ def test_plain_form_keeps_no_work_items():
         finally:
             pz.pz_set_allocator()
         assert (taken == 0) == (prec == pz.PZ_FP64), taken
+
+
+@pytest.mark.gpu
+def test_a_tiling_without_memory_leaves_no_launch():
+    """Where a tiling's tables are refused the call fails, and so do the line kernels until a tiling fits."""
+    import gc
+
+    import torch
+    gc.collect()
+    prob = I.small_config1(n_lambda_span_nm=3.0, seed=3)
+    alloc, free = pz.torch_allocator()
+    budget = [None]                  # allocations still granted (None: all)
+
+    def limited(n, u):
+        if budget[0] is not None:
+            if budget[0] == 0:
+                return 0
+            budget[0] -= 1
+        return alloc(n, u)
+
+    for granted in range(5):         # thresholds, cuts, box offsets, items, counters
+        pz.pz_set_allocator(limited, free)
+        try:
+            s = pz.Synthesizer(prob)
+            f0 = s.forward().cpu()
+            budget[0] = granted
+            with pytest.raises(pz.PzError) as e:
+                pz.pz_set_tiling(s.ctx, 2, 8, 3, 32, 4)
+            status = e.value.status
+            with pytest.raises(pz.PzError):
+                pz.pz_line_opacity(s.ctx)
+            budget[0] = None
+            pz.pz_set_tiling(s.ctx, 4, 6, 2, 16, 4)
+            again = s.forward().cpu()
+            s.close()
+        finally:
+            budget[0] = None
+            pz.pz_set_allocator()
+        assert status == pz.PZ_ENOMEM
+        assert f0.numel() > 0 and torch.max(torch.abs(again - f0)) < 2e-7
