@@ -25,7 +25,7 @@ def test_allocation_failure_is_reported_and_nothing_leaks():
 
     import torch
     gc.collect()                     # contexts other tests left to the garbage collector
-    prob = I.small_config1(n_lambda_span_nm=1.0, seed=3)
+    prob = I.small_config1(n_lambda_span_nm=3.0, seed=3)     # (1 nm holds no pixel of the instrument)
     alloc, free = pz.torch_allocator()
     live = {}
 
@@ -60,7 +60,8 @@ def test_allocation_failure_is_reported_and_nothing_leaks():
         pz.pz_set_allocator(*make(None))
     assert e.value.status == pz.PZ_ESTATE
     s.close()
-    assert torch.equal(f0, f1)
+    # (on short grids the near cores' pieces are added by atomics: last bits of the opacity may differ)
+    assert f0.numel() > 0 and torch.max(torch.abs(f0 - f1)) < 2e-7
     # failure after a few allocations: PZ_ENOMEM from pz_create, nothing left behind
     for limit in (0, 3, 12):
         pz.pz_set_allocator(*make(limit))
