@@ -120,6 +120,20 @@ def uneven_batch():
     return I.Batch("uneven", at, grid, ll, [I.make_kappa_c(a, grid) for a in at], subsets)
 
 
+def test_stars_of_different_box_sizes_in_both_directions():
+    """Two box sizes and a star without boxes in one context: opacity, spectra and the four gradients."""
+    prob = uneven_batch()
+    got, launches = outputs(prob, pz.PZ_MIXED, 0.0, None)
+    ref, _ = outputs(prob, pz.PZ_FP64, 0.0, None)
+    assert launches == 7          # moments and field of either size
+    for k in range(prob.n_stars):
+        m = ref[0][k] > 0
+        assert np.max(np.abs(got[0][k][m] / ref[0][k][m] - 1)) < 3e-5
+        assert np.linalg.norm(got[0][k] - ref[0][k]) < 2e-6 * np.linalg.norm(ref[0][k])
+    for a, b in zip(got[1:], ref[1:]):
+        assert np.linalg.norm(a - b) < 2e-6 * np.linalg.norm(b)
+
+
 @pytest.mark.parametrize("make", [uneven_batch, lambda: I.small_batch(n_stars=4, span_nm=4.0, seed=23)],
                          ids=["sizes and densities", "densities"])
 def test_a_star_takes_the_same_sums_in_a_batch(make):
